@@ -61,7 +61,7 @@ typedef enum {
 } fstat_status;
 
 typedef enum {
-    FSTAT_FP64_PLAIN = 0,    /* every step in FP64, one cell at a time */
+    FSTAT_FP64_PLAIN = 0,    /* every step in FP64, cells in small batches */
     FSTAT_FP32_BATCHED = 1   /* FP32 resample/FFT/|F|^2; the delay in double-float
                                 (~48-bit) and the spindown phase in 64-bit fixed point,
                                 both reduced before any FP32 use; compensated sums;

@@ -233,6 +233,7 @@ void build_twiddles(Plan &p, const std::vector<int> &logs, int &n_alloc) {
         t.in1_f = df + o[0]; t.in2_f = df + o[1];
         t.lo_f = df + o[2]; t.hi_f = df + o[3];
         t.s1_f = df + o[4]; t.s2_f = df + o[5];
+        t.s1_d = dd + o[4]; t.s2_d = dd + o[5];
         if (log_n1(logs[i]) == 9) t.p512_f = reinterpret_cast<const float4 *>(df + o[6]);
         p.tw.push_back(t);
     }
@@ -323,6 +324,20 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
     }
     p.n_fft_max = max_nfft;
     build_twiddles(p, logs, n_alloc);
+    if (!fp32) {   // tables of the FP64 passes, for the lengths the bands search
+        double2 *ut = dalloc<double2>(p, (size_t)unit_table_entries(), n_alloc);
+        launch_unit_table(ut, s);
+        ++p.launches;
+        p.unit_tab = ut;
+        for (auto &t : p.tw) {
+            const bool used = std::any_of(p.bands.begin(), p.bands.end(), [&](const BandDev &b) { return b.logn == t.logn; });
+            if (!used || !inter_table_needed(t.logn)) continue;
+            double2 *it = dalloc<double2>(p, size_t(1) << t.logn, n_alloc);
+            launch_inter_table(it, t.logn, s);
+            ++p.launches;
+            t.inter_d = it;
+        }
+    }
 
     p.alpha = dalloc<double>(p, d->n_sky, n_alloc);
     p.delta = dalloc<double>(p, d->n_sky, n_alloc);
@@ -361,8 +376,10 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
     const int64_t nblk = (p.n_max + 255) / 256;
     // sky positions per batch: 64, or up to 256 when the spindowns are few, so that a
     // batch holds the 4096 cells of a launch pair
+    // FP64 form: up to 64 positions whose series (32 bytes a sample) fill 128 MiB: the FP64
+    // kernels are bound by their arithmetic, a batch only has to fill the SMs and hide latency
     p.sky_batch = fp32 ? std::min<int64_t>(d->n_sky, std::max<int64_t>(64, std::min<int64_t>(256, (4096 + d->n_spin - 1) / d->n_spin)))
-                       : 1;
+                       : std::min<int64_t>(d->n_sky, std::max<int64_t>(1, std::min<int64_t>(64, (int64_t(128) << 20) / (32 * p.w_stride))));
     if (fp32)
         if (const char *v = getenv("FSTAT_SKY_BATCH")) p.sky_batch = std::max<int64_t>(1, std::min<int64_t>(d->n_sky, atoll(v)));
     const size_t w_elem = fp32 ? 16 : 32;
@@ -390,8 +407,11 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
         p.cell_batch = std::min<int64_t>(p.cell_batch, p.sky_batch * d->n_spin);
         if (const char *v = getenv("FSTAT_CELL_BATCH")) p.cell_batch = std::max(1, std::min(65535, atoi(v)));
     } else {
+        // launches of many cells (scratch up to 512 MiB, 64 cells at 2^18): one cell of a short
+        // transform fills only a few SMs, and 2^18 leaves a sixth of them idle
         p.n_workers = 1;
-        p.cell_batch = 1;
+        p.cell_batch = std::max<int64_t>(1, std::min<int64_t>(4096, (int64_t(512) << 20) / (2 * max_nfft * (int64_t)tsz)));
+        p.cell_batch = std::min<int64_t>(p.cell_batch, p.sky_batch * d->n_spin);
     }
     // a worker's slot holds a launch's cells, or the ring of the fused launch
     if (fp32) {

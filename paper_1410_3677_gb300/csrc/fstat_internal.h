@@ -34,6 +34,9 @@ struct TwiddleSet {
     // second engine: stage-1 twiddles W_M^{r j} laid out [r][j], r < R1, j < R0
     // (float), for the rows (M = N1 = R0 R1, pass 2) and the columns (M = N2, pass 1)
     const float *s1_f = nullptr, *s2_f = nullptr;
+    const double *s1_d = nullptr, *s2_d = nullptr;   // the same in FP64
+    // FP64 form, 2^12 .. 2^20: W_N^{k1 l2} in the order of the FP64 scratch
+    const double2 *inter_d = nullptr;
     // packed passes (512-point rows, N_fft = 2^18 and 2^19): stage-1 twiddles of a
     // 512-point pass as pairs,
     // [r][k] = (cos a_2k, cos a_2k+1, -sin a_2k, -sin a_2k+1), a_j = 2 pi r j / 512
@@ -152,6 +155,7 @@ struct Plan {
     // twiddles, one set per transform length used
     std::vector<TwiddleSet> tw;
     void *tw_pool = nullptr;
+    const double2 *unit_tab = nullptr;   // FP64 form: e^{-2 pi i m / 2048}
 
     // candidates
     CandRecord *cand = nullptr;
@@ -258,6 +262,13 @@ int launch_reduce_norms(const Plan &p, const BandDev &b, int64_t ns, double *nor
 // counts; returns the buffer with the sorted records.
 CandRecord *launch_cand_sort(CandRecord *a, CandRecord *b, uint32_t *hist, int64_t n, uint32_t cell0,
                              uint64_t cell_span, int bin_bits, cudaStream_t s, int64_t *launches);
+
+// Tables of the FP64 form: unit phases, and the four-step twiddles of a length
+// 2^logn in the order its passes read them.
+int64_t unit_table_entries();
+bool inter_table_needed(int logn);
+void launch_unit_table(double2 *t, cudaStream_t s);
+void launch_inter_table(double2 *t, int logn, cudaStream_t s);
 
 // The two FFT passes of the search for cells [c0, c0 + nc) of band `band_idx`
 // (cells of this band: c = sky * n_spin + spin, skies relative to sky base s0).

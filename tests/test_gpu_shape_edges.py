@@ -1,0 +1,60 @@
+"""Every bin against the FP64 oracle at the edges of the launch rules: series just inside
+and just beyond the lengths where a kernel skips more of the zero padding, the shortest and
+longest transforms of each engine, and grids whose last sky batch and last launch are ragged.
+Tolerances as in test_gpu_parity: |F - F_ref| / max(F_ref, 2) <= 1e-10 (FP64), 1e-4 (FP32).
+"""
+import os
+
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1410_3677_gb300 import synth as S
+
+pytestmark = pytest.mark.gpu
+
+TOL = {0: 1e-10, 1: 1e-4}
+NTHREADS = os.cpu_count() or 4
+
+
+@pytest.fixture(scope="module")
+def fs():
+    from paper_1410_3677_gb300 import fstat
+    return fstat
+
+
+def _check(fs, form, n, n_fft, n_sky, n_spin, dt=2.0, f_off=100.5, full_range=False, full=False, U=2,
+           interbin=False, window=None):
+    """Every bin (or `window` bins at three places of the range) of every cell."""
+    alpha, delta = S.fibonacci_sky(n_sky)
+    fdot = S.spindown_grid(n_spin, -1e-8, 0.0)
+    b = S.make_band(n, dt, 31 + n, 1.0, alpha, delta, fdot, [], f_off=f_off, n_fft=n_fft)
+    top = n_fft - 1 if full_range else n_fft // 2 - 1
+    ranges = [(0 if full_range else 1, top)]
+    if window:
+        ranges = [(lo, lo + window - 1) for lo in (ranges[0][0], top // 2, top - window + 1)]
+    prm = O.params(S.LAT_DEFAULT, S.GAMMA_DEFAULT, U, 0.0, full, 0, interbin)
+    sky, spin = np.repeat(np.arange(n_sky), n_spin), np.tile(np.arange(n_spin), n_sky)
+    for lo, hi in ranges:
+        ref = O.cells_F(b, prm, alpha, delta, fdot, sky, spin, lo, hi, NTHREADS)
+        with fs.Plan([b], alpha, delta, fdot, -1.0, lat=S.LAT_DEFAULT, gamma=S.GAMMA_DEFAULT, upsample=U, form=form,
+                     bin_lo=lo, bin_hi=hi, cand_capacity=ref.size, full=full, interbin=interbin) as p:
+            p.search()
+            c, total = p.candidates()
+        assert total == ref.size
+        assert np.array_equal(c["bin"], np.tile(np.arange(lo, hi + 1), sky.size))
+        assert np.array_equal(c["sky"] * n_spin + c["spin"], np.repeat(np.arange(sky.size), hi - lo + 1))
+        err = np.abs(c["F"].reshape(ref.shape) - ref) / np.maximum(ref, 2.0)
+        assert err.max() <= TOL[form], (lo, hi, err.max(), np.unravel_index(np.argmax(err), err.shape))
+
+
+@pytest.mark.parametrize("n,n_fft,n_sky,n_spin,kw", [
+    (1900, 1 << 12, 70, 3, {}),                                  # shortest two-stage length, ragged sky batch
+    (2048, 1 << 12, 3, 2, dict(full_range=True)),                # n = N / 2, both halves of the spectrum
+    (1001, 1 << 11, 5, 3, {}),                                   # longest of the radix-8 engine, batched
+    (49152, 1 << 17, 2, 2, dict(full=True)),                     # n = 3N/8: five eighths of a column skipped
+    (49153, 1 << 17, 2, 2, dict(full_range=True)),               # one sample more: half skipped
+    (300001, 1 << 20, 3, 7, dict(dt=0.5, window=300)),           # longest, 1024-point rows, ragged last launch
+])
+def test_fp64_batches(fs, n, n_fft, n_sky, n_spin, kw):
+    _check(fs, fs.FP64_PLAIN, n, n_fft, n_sky, n_spin, **kw)
