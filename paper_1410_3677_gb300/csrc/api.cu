@@ -277,7 +277,8 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
 
     std::vector<int> logs;
     auto need = [&](int lg) { if (std::find(logs.begin(), logs.end(), lg) == logs.end()) logs.push_back(lg); };
-    int64_t max_m = 0, max_nfft = 0;
+    int64_t max_nfft = 0;
+    size_t up_scratch = 0;   // double2 of scratch the upsample needs
     p.n_max = 0;
     for (int i = 0; i < d->n_bands; ++i) {
         const fstat_band &hb = d->bands[i];
@@ -290,23 +291,16 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
         if (d->interpolation == FSTAT_INTERP_INTERBIN) need(b.logn - 1);
         if (d->bin_lo == 0 && d->bin_hi == 0) { b.lo = 1; b.hi = b.n_fft / 2 - 1; }
         else { b.lo = d->bin_lo; b.hi = d->bin_hi; }
-        // upsample transforms: a power of two >= 256 directly, else Bluestein
         if (U > 1) {
-            const int lgn = ilog2_exact(b.n);
-            if (lgn >= kMinLogN && lgn <= kMaxLogN) need(lgn);
-            else {
-                int lm = kMinLogN;
-                while ((int64_t(1) << lm) < 2 * b.n - 1) ++lm;
-                need(lm);
-                max_m = std::max<int64_t>(max_m, int64_t(1) << lm);
-            }
+            b.up.logh = upsample_logh(b.n);
+            need(b.up.logh);
+            up_scratch = std::max<size_t>(up_scratch, (size_t)upsample_scratch(b.up.logh, U));
         }
         max_nfft = std::max(max_nfft, b.n_fft);
         p.n_max = std::max(p.n_max, b.n);
         b.x = dalloc<double>(p, b.n, n_alloc);
         b.r = dalloc<double>(p, 3 * b.n, n_alloc);
         if (fp32) b.r2 = dalloc<DF>(p, 3 * b.n, n_alloc);
-        b.sigma2 = dalloc<double>(p, 1, n_alloc);
         b.xu = fp32 ? (void *)dalloc<float>(p, (size_t)U * b.n, n_alloc)
                     : (void *)dalloc<double>(p, (size_t)U * b.n, n_alloc);
         if (hb.x) {
@@ -391,6 +385,7 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
     p.dbuf = dalloc<double>(p, (size_t)p.sky_batch * p.n_max * (fp32 ? 2 : 1), n_alloc);
     p.partials = dalloc<double>(p, std::max<int64_t>((int64_t)p.sky_batch * nblk * 3, 256), n_alloc);
     p.S = dalloc<double>(p, 3 * p.sky_batch, n_alloc);
+    p.sigma_parts = dalloc<double>(p, kSigmaParts, n_alloc);
     for (int q = 0; q < 2; ++q) p.normbuf[q] = dalloc<double>(p, kNormStride * p.sky_batch, n_alloc);
 
     // FFT scratch: cell slots of 2 transforms; also hosts the generic FFT of the upsample
@@ -449,7 +444,7 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
     }
     p.slot_cells = (size_t)std::max<int64_t>(p.cell_batch, fp32 ? p.fused_slots : 1);
     size_t scratch_bytes = std::max<size_t>((size_t)p.n_workers * p.slot_cells * 2 * max_nfft * tsz,
-                                            (size_t)2 * std::max<int64_t>(max_m, p.n_max) * sizeof(double2) * 2);
+                                            up_scratch * sizeof(double2));
     if (fp32) {
         if (const char *v = getenv("FSTAT_PERSIST_BATCH")) p.pbatch = std::max(1, atoi(v));
         if (const char *v = getenv("FSTAT_PERSIST_SLOTS")) p.pslots = std::max(2, atoi(v));
@@ -466,8 +461,19 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
                                   n_alloc);
     }
     p.scratch = dalloc<unsigned char>(p, scratch_bytes, n_alloc);
-    p.bw_elems = 2 * p.n_max + 2 * max_m;
-    p.bw = dalloc<double>(p, 2 * (size_t)std::max<int64_t>(p.bw_elems, 1), n_alloc);
+    for (size_t i = 0; U > 1 && i < p.bands.size(); ++i) {   // bands of one length share the upsample's tables
+        BandDev &b = p.bands[i];
+        size_t j = 0;
+        while (j < i && p.bands[j].n != b.n) ++j;
+        if (j < i) { b.up = p.bands[j].up; continue; }
+        const size_t H = size_t(1) << b.up.logh;
+        const TwiddleSet *tw = p.twiddles(b.up.logh);
+        b.up.w_rows = tw->in1_d;
+        b.up.w_cols = tw->in2_d;
+        double2 *ab = dalloc<double2>(p, 2 * H * (size_t)(U - 1), n_alloc);
+        double2 *it = dalloc<double2>(p, H, n_alloc);
+        p.launches += launch_upsample_tables(b.n, U, b.up, ab, it, p.scratch, s);
+    }
 
     // worker streams (the FP64 plain form runs on the plan's stream alone)
     for (int q = 0; q < 2; ++q) {
@@ -589,9 +595,8 @@ void band_prologue(Plan &p, BandDev &b) {
     const bool t = stat_launch(p, idx, 0.0, (double)b.n * 8.0 * (1 + p.desc.upsample));
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (t) { e0 = ev_get(p); e1 = ev_get(p); rec_timing(e0, p.stream); }
-    p.launches += launch_sigma2(b.x, b.n, p.desc.sigma2, p.partials, b.sigma2, p.stream);
+    p.launches += launch_band_inputs(b, p.sigma_parts, p.stream);
     p.launches += launch_upsample(p, b, p.desc.upsample, b.xu, fp32, p.stream);
-    if (fp32) p.launches += launch_split_r(b, p.stream);
     if (t) { rec_timing(e1, p.stream); p.pending.push_back({idx, e0, e1}); }
 }
 

@@ -64,6 +64,18 @@ struct SkyConst {
     float nf[6];   // nx, ny, nz as double-float pairs (hi, lo) for the FP32 delay
 };
 
+// Tables of the FFT upsample of a series of n samples (upsample.cu), laid out once
+// per plan and length.
+struct UpsampleTables {
+    int logh = 0;                    // half of the convolution length: H = 2^logh complex points
+    const double2 *ab = nullptr;     // [U - 1][l2][l1][2]: the kernel's transform as (alpha, beta)
+    const double2 *tw = nullptr;     // W_H^{k1 l2}, [l2][k1]
+    const double *w_cols = nullptr, *w_rows = nullptr;   // W_N2^k, W_N1^k
+};
+
+// Partial sums of x^2 per band.
+constexpr int kSigmaParts = 256;
+
 // Band data resident on the device.
 struct BandDev {
     int64_t n = 0;
@@ -75,8 +87,8 @@ struct BandDev {
     float *x32 = nullptr;     // [n] staging of a float32 series (allocated on first use)
     double *r = nullptr;      // [3n]
     void *r2 = nullptr;       // FP32 form: r as double-float pairs (DF[3n]), redone per search
-    double *sigma2 = nullptr; // device scalar
     void *xu = nullptr;       // [U n]: double (FP64 form) or float (FP32 form)
+    UpsampleTables up;
 };
 
 struct Plan {
@@ -107,6 +119,7 @@ struct Plan {
     double *dbuf = nullptr;       // [sky_batch][n_max] per-sample delays
     double *partials = nullptr;   // [sky_batch][n_blocks_max][3]
     double *S = nullptr;          // [sky_batch][3]
+    double *sigma_parts = nullptr;   // [kSigmaParts] of the band being searched
     double *normbuf[2] = {nullptr, nullptr};   // [sky_batch][2]: 1/(sigma^2 S_aa), 1/(sigma^2 S_bb)
     int64_t n_max = 0;
 
@@ -147,10 +160,6 @@ struct Plan {
     bool p2_rows = true;           // 256-point rows (2^16, 2^17): two rows per warp, packed
     bool tma = true;               // two-stage pass 2: rows staged by bulk copies
     int p2_threads = 128;          // two-stage pass 2 with bulk copies: CTA size 256 or 128
-
-    // Bluestein / generic-FFT work buffers (double2)
-    double *bw = nullptr;
-    int64_t bw_elems = 0;
 
     // twiddles, one set per transform length used
     std::vector<TwiddleSet> tw;
@@ -226,23 +235,18 @@ struct CellBufs {
 // ---------------------------------------------------------------- launchers
 // Each returns the number of kernels it launched (for the plan's counter).
 
-// sigma^2 = (1/n) sum x^2, compensated, into *out (device); user_sigma2 > 0 overrides.
-// partials: >= 256 doubles.
-// FP32 form, per band and search: the ephemeris as double-float pairs (b.r2).
-int launch_split_r(const BandDev &b, cudaStream_t s);
-int launch_sigma2(const double *x, int64_t n, double user_sigma2, double *partials, double *out,
-                  cudaStream_t s);
+// Per band and search: partial sums of x^2 (kSigmaParts doubles; the variance is
+// finished with the norms) and, in the FP32 form, the ephemeris as double-float
+// pairs (b.r2).
+int launch_band_inputs(const BandDev &b, double *sigma_parts, cudaStream_t s);
 
-// Generic two-pass power-of-two FFT of `pairs` * 2 transforms of length 2^logn,
-// in[t] -> out[t] (t over 2*pairs contiguous transforms, interleaved complex).
-// dir = -1 forward, +1 inverse (unscaled).  FP64 or FP32 arithmetic.
-int launch_fft_generic(const TwiddleSet &tw, bool fp64, int dir, const void *in, void *out,
-                       int64_t n_transforms, void *scratch, cudaStream_t s);
-
-// Bluestein DFT of arbitrary length n (double2 in/out), using the generic FFT of
-// length M = 2^logm >= 2n - 1.  work holds 3*M double2.
-int launch_bluestein(const TwiddleSet &twm, int dir, const double *in, double *out, int64_t n,
-                     double *work, void *scratch, cudaStream_t s);
+// The upsample's tables for a series of n samples: log2 of its half length, the
+// double2 of scratch that building and running need, and the build itself (t.logh
+// and the w pointers set; ab holds 2 (U - 1) 2^logh, tw 2^logh double2).
+int upsample_logh(int64_t n);
+int64_t upsample_scratch(int logh, int U);
+int launch_upsample_tables(int64_t n, int U, UpsampleTables &t, double2 *ab, double2 *tw, void *scratch,
+                           cudaStream_t s);
 
 // U-fold FFT upsample of x[n] (double) into xu[U n] (double or float).
 int launch_upsample(const Plan &p, const BandDev &b, int U, void *xu, bool xu_fp32,

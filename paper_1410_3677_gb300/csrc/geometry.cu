@@ -1,6 +1,4 @@
-// Per-band and per-sky steps of the search (Sect. 2, Fig. 1):
-//   per band: noise variance, U-fold FFT upsample of the narrow-band series
-//             ("resampling ... using the FFT and splines");
+// Per-sky steps of the search (Sect. 2, Fig. 1; the per-band ones are in upsample.cu):
 //   per sky:  Roemer delay nhat . r, detector time of every barycentric sample,
 //             amplitude modulations a(t), b(t), Keys-cubic resampling and the
 //             band-offset phase demodulation ("amplitude and phase
@@ -10,6 +8,7 @@
 
 #include "dfloat.cuh"
 #include "fstat_internal.h"
+#include "reduce64.cuh"
 #include "unit_phase.cuh"
 
 namespace fstat {
@@ -18,37 +17,6 @@ namespace {
 
 constexpr double kTwoPi = 6.283185307179586476925286766559;
 constexpr double kOmegaR = kTwoPi / 86164.0905;   // sidereal rotation rate, rad/s
-
-struct KahanD {
-    double s = 0.0, c = 0.0;
-    __device__ void add(double v) {
-        double y = v - c;
-        double t = s + y;
-        c = (t - s) - y;
-        s = t;
-    }
-};
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// Sum of v over a 256-thread block into thread 0's return value.
-__device__ double block_sum256(double v, double *sh) {
-    v = warp_sum(v);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) sh[w] = v;
-    __syncthreads();
-    double r = 0.0;
-    if (w == 0) {
-        r = (l < (int)(blockDim.x >> 5)) ? sh[l] : 0.0;
-        r = warp_sum(r);
-    }
-    __syncthreads();
-    return r;
-}
 
 // The FP32 form's three S terms at once: each warp adds its 32 terms of each in
 // FP32 (relative error ~1e-7), one barrier, then three threads add the block's
@@ -76,26 +44,6 @@ __device__ void block_sum3_f(float a, float b, float c, double *sh, double *out)
         for (int i = 0; i < 8; ++i) t += sh[8 * threadIdx.x + i];
         out[threadIdx.x] = t;
     }
-}
-
-// ------------------------------------------------------------------ sigma^2
-__global__ void __launch_bounds__(256) k_sumsq(const double *__restrict__ x, int64_t n,
-                                               double *__restrict__ partials) {
-    __shared__ double sh[8];
-    KahanD k;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        k.add(x[i] * x[i]);
-    const double s = block_sum256(k.s - k.c, sh);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
-__global__ void k_sigma2_final(const double *__restrict__ partials, int nblk, int64_t n,
-                               double user_sigma2, double *__restrict__ out) {
-    KahanD k;
-    for (int i = threadIdx.x; i < nblk; i += 32) k.add(partials[i]);
-    double s = warp_sum(k.s - k.c);
-    if (threadIdx.x == 0) *out = user_sigma2 > 0.0 ? user_sigma2 : s / (double)n;
 }
 
 // ------------------------------------------------------------------ geometry
@@ -159,12 +107,6 @@ __global__ void __launch_bounds__(256) k_delays(const double *__restrict__ r,
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int sl = blockIdx.y;
     if (k < n) d[(int64_t)sl * stride + k] = delay_at(r, sky[s0 + sl], k);
-}
-
-// The ephemeris of a band as double-float pairs (once per search of the band).
-__global__ void k_split_r(const double *__restrict__ r, int64_t m, DF *__restrict__ r2) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < m) r2[i] = df_from_double(r[i]);
 }
 
 // Shift records of every sample of skies [s0, s0 + gridDim.y): the delay
@@ -380,15 +322,19 @@ __global__ void __launch_bounds__(256) k_geometry64(GeoArgs g) {
 // 1/(sigma^2 S_aa), 1/(sigma^2 S_bb).  Warp w adds term w % 3 over the w / 3-th
 // quarter of the partials: with one warp for all three terms the dependent FP64
 // chain over 337 partials took 10 us a launch.
+// A further warp finishes the noise variance from the band's partials.
 constexpr int kNormWarps = 12;
-__global__ void __launch_bounds__(32 * kNormWarps)
-k_reduce_norms(const double *__restrict__ partials, int nblk, const double *__restrict__ sigma2,
-               double *__restrict__ S, double *__restrict__ norm, int full) {
+__global__ void __launch_bounds__(32 * (kNormWarps + 1))
+k_reduce_norms(const double *__restrict__ partials, int nblk, const double *__restrict__ sigma_parts, int64_t n,
+               double user_sigma2, double *__restrict__ S, double *__restrict__ norm, int full) {
     const int sl = blockIdx.x;
-    __shared__ double sh[kNormWarps];
+    __shared__ double sh[kNormWarps + 1];
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     KahanD k;
-    for (int i = 32 * (w / 3) + l; i < nblk; i += 32 * (kNormWarps / 3)) k.add(partials[((int64_t)sl * nblk + i) * 3 + w % 3]);
+    if (w == kNormWarps)
+        for (int i = l; i < kSigmaParts; i += 32) k.add(sigma_parts[i]);
+    else
+        for (int i = 32 * (w / 3) + l; i < nblk; i += 32 * (kNormWarps / 3)) k.add(partials[((int64_t)sl * nblk + i) * 3 + w % 3]);
     const double v = warp_sum(k.s - k.c);
     if (l == 0) sh[w] = v;
     __syncthreads();
@@ -400,7 +346,7 @@ k_reduce_norms(const double *__restrict__ partials, int nblk, const double *__re
         for (int q = 0; q < kNormWarps / 3; ++q) out[c] += sh[3 * q + c];
     }
     if (threadIdx.x == 0) {
-        const double s2 = *sigma2;
+        const double s2 = user_sigma2 > 0.0 ? user_sigma2 : sh[kNormWarps] / (double)n;
         S[3 * sl] = out[0];
         S[3 * sl + 1] = out[1];
         S[3 * sl + 2] = out[2];
@@ -430,84 +376,6 @@ k_reduce_norms(const double *__restrict__ partials, int nblk, const double *__re
     }
 }
 
-// ------------------------------------------------------------------ FFT upsample
-__global__ void k_real_to_cplx(const double *__restrict__ x, int64_t n, double2 *__restrict__ z) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) z[i] = make_double2(x[i], 0.0);
-}
-
-// Bluestein: c_m = e^{dir i pi (m^2 mod 2n)/n}; A = in * c (zero beyond n);
-// B = conj(c) wrapped around M so that the circular convolution is linear.
-__global__ void k_blue_prep(const double2 *__restrict__ in, int64_t n, int64_t M, int dir,
-                            double2 *__restrict__ A, double2 *__restrict__ B) {
-    const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (m >= M) return;
-    double2 a = make_double2(0.0, 0.0), b = make_double2(0.0, 0.0);
-    int64_t mm = -1;
-    if (m < n) mm = m;
-    else if (m > M - n) mm = M - m;
-    if (mm >= 0) {
-        const int64_t q = (mm * mm) % (2 * n);
-        double s, c;
-        sincospi((double)dir * (double)q / (double)n, &s, &c);
-        b = make_double2(c, -s);
-        if (m < n) {
-            const double2 v = in[m];
-            a = make_double2(v.x * c - v.y * s, v.x * s + v.y * c);
-        }
-    }
-    A[m] = a;
-    B[m] = b;
-}
-
-__global__ void k_cmul_inplace(double2 *__restrict__ A, const double2 *__restrict__ B, int64_t M) {
-    const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (m >= M) return;
-    const double2 a = A[m], b = B[m];
-    A[m] = make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-
-__global__ void k_blue_post(const double2 *__restrict__ A, int64_t n, int64_t M, int dir,
-                            double2 *__restrict__ out) {
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const int64_t q = (k * k) % (2 * n);
-    double s, c;
-    sincospi((double)dir * (double)q / (double)n, &s, &c);
-    const double2 v = A[k];
-    const double inv = 1.0 / (double)M;
-    out[k] = make_double2((v.x * c - v.y * s) * inv, (v.x * s + v.y * c) * inv);
-}
-
-// Spectrum of the s-th sub-phase of the U-fold interpolant: Y_m = X_m e^{2 pi i m s/(U n)}
-// over signed frequencies; the Nyquist bin of an even n contributes X cos(pi s / U).
-__global__ void k_shift_spectrum(const double2 *__restrict__ X, int64_t n, int s, int U,
-                                 double2 *__restrict__ Y) {
-    const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (m >= n) return;
-    const double2 v = X[m];
-    if ((n % 2 == 0) && m == n / 2) {
-        double c = cospi((double)s / (double)U);
-        Y[m] = make_double2(v.x * c, v.y * c);
-        return;
-    }
-    const int64_t ms = (2 * m < n) ? m : m - n;
-    const int64_t un = (int64_t)U * n;
-    int64_t q = (ms * s) % un;
-    if (q < 0) q += un;
-    double sn, cs;
-    sincospi(2.0 * (double)q / (double)un, &sn, &cs);
-    Y[m] = make_double2(v.x * cs - v.y * sn, v.x * sn + v.y * cs);
-}
-
-template <typename TO>
-__global__ void k_scatter_sub(const double2 *__restrict__ z, const double *__restrict__ x, int64_t n,
-                              int U, int s, TO *__restrict__ xu) {
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    xu[(int64_t)U * k + s] = (TO)(s == 0 ? x[k] : z[k].x / (double)n);
-}
-
 inline unsigned blocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 // blocks of a geometry launch per sky position, each leaving one partial of the S sums
 inline int geo_blocks(int64_t n, bool fp32) { return (int)blocks(n, fp32 ? 256 : 256 * kGeo64); }
@@ -515,81 +383,6 @@ inline int geo_blocks(int64_t n, bool fp32) { return (int)blocks(n, fp32 ? 256 :
 }  // namespace
 
 // ================================================================== launchers
-int launch_split_r(const BandDev &b, cudaStream_t s) {
-    const int64_t m = 3 * b.n;
-    k_split_r<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(b.r, m, static_cast<DF *>(b.r2));
-    return 1;
-}
-
-int launch_sigma2(const double *x, int64_t n, double user_sigma2, double *partials,
-                  double *out, cudaStream_t s) {
-    constexpr int nblk = 256;
-    k_sumsq<<<nblk, 256, 0, s>>>(x, n, partials);
-    k_sigma2_final<<<1, 32, 0, s>>>(partials, nblk, n, user_sigma2, out);
-    return 2;
-}
-
-int launch_bluestein(const TwiddleSet &twm, int dir, const double *in, double *out, int64_t n,
-                     double *work, void *scratch, cudaStream_t s) {
-    const int64_t M = (int64_t)1 << twm.logn;
-    double2 *A = reinterpret_cast<double2 *>(work);
-    double2 *B = A + M;
-    int L = 0;
-    k_blue_prep<<<blocks(M, 256), 256, 0, s>>>(reinterpret_cast<const double2 *>(in), n, M, dir,
-                                                A, B);
-    ++L;
-    L += launch_fft_generic(twm, true, -1, A, A, 2, scratch, s);
-    k_cmul_inplace<<<blocks(M, 256), 256, 0, s>>>(A, B, M);
-    ++L;
-    L += launch_fft_generic(twm, true, +1, A, A, 1, scratch, s);
-    k_blue_post<<<blocks(n, 256), 256, 0, s>>>(A, n, M, dir, reinterpret_cast<double2 *>(out));
-    ++L;
-    return L;
-}
-
-static int dft_any(const Plan &p, int64_t n, int dir, double2 *z, double *work, cudaStream_t s) {
-    const bool pow2 = (n & (n - 1)) == 0 && n >= (1 << kMinLogN);
-    if (pow2) {
-        int lg = 0;
-        while ((int64_t(1) << lg) < n) ++lg;
-        return launch_fft_generic(*p.twiddles(lg), true, dir, z, z, 1, p.scratch, s);
-    }
-    int lm = kMinLogN;
-    while ((int64_t(1) << lm) < 2 * n - 1) ++lm;
-    return launch_bluestein(*p.twiddles(lm), dir, reinterpret_cast<double *>(z),
-                            reinterpret_cast<double *>(z), n, work, p.scratch, s);
-}
-
-int launch_upsample(const Plan &p, const BandDev &b, int U, void *xu, bool xu_fp32,
-                    cudaStream_t s) {
-    const int64_t n = b.n;
-    int L = 0;
-    if (U == 1) {
-        if (xu_fp32) k_scatter_sub<float><<<blocks(n, 256), 256, 0, s>>>(nullptr, b.x, n, 1, 0, (float *)xu);
-        else k_scatter_sub<double><<<blocks(n, 256), 256, 0, s>>>(nullptr, b.x, n, 1, 0, (double *)xu);
-        return 1;
-    }
-    double2 *X = reinterpret_cast<double2 *>(p.bw);
-    double2 *Y = X + p.n_max;
-    double *work = reinterpret_cast<double *>(Y + p.n_max);
-    k_real_to_cplx<<<blocks(n, 256), 256, 0, s>>>(b.x, n, X);
-    ++L;
-    L += dft_any(p, n, -1, X, work, s);
-    for (int sub = 0; sub < U; ++sub) {
-        if (sub > 0) {
-            k_shift_spectrum<<<blocks(n, 256), 256, 0, s>>>(X, n, sub, U, Y);
-            ++L;
-            L += dft_any(p, n, +1, Y, work, s);
-        }
-        if (xu_fp32)
-            k_scatter_sub<float><<<blocks(n, 256), 256, 0, s>>>(Y, b.x, n, U, sub, (float *)xu);
-        else
-            k_scatter_sub<double><<<blocks(n, 256), 256, 0, s>>>(Y, b.x, n, U, sub, (double *)xu);
-        ++L;
-    }
-    return L;
-}
-
 int launch_geometry(const Plan &p, const BandDev &b, int64_t s0, int64_t ns, bool fp32,
                     void *w, double *dbg_y, double *dbg_a, double *dbg_b, uint8_t *dbg_mask,
                     cudaStream_t s) {
@@ -633,9 +426,9 @@ int launch_geometry(const Plan &p, const BandDev &b, int64_t s0, int64_t ns, boo
 }
 
 int launch_reduce_norms(const Plan &p, const BandDev &b, int64_t ns, double *norm, cudaStream_t s) {
-    k_reduce_norms<<<(unsigned)ns, 32 * kNormWarps, 0, s>>>(p.partials, geo_blocks(b.n, p.desc.form == FSTAT_FP32_BATCHED),
-                                                            b.sigma2, p.S, norm,
-                                                            p.desc.statistic == FSTAT_F_FULL ? 1 : 0);
+    k_reduce_norms<<<(unsigned)ns, 32 * (kNormWarps + 1), 0, s>>>(
+        p.partials, geo_blocks(b.n, p.desc.form == FSTAT_FP32_BATCHED), p.sigma_parts, b.n, p.desc.sigma2, p.S, norm,
+        p.desc.statistic == FSTAT_F_FULL ? 1 : 0);
     return 1;
 }
 

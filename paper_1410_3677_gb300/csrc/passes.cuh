@@ -58,35 +58,6 @@ __device__ __forceinline__ void cmul_tw(T &xr, T &xi, T wr, T wi) {
 }
 
 // ------------------------------------------------------------------ pass 1 loaders
-// Generic: n_tr transforms of length N stored back to back; pair = blockIdx.y.
-template <typename T, class C>
-struct GenericLoad {
-    using V = typename Vec2<T>::type;
-    const V *in;
-    int64_t n_tr;
-    const V *a, *b;
-    bool has_b;
-    int k1_0;
-    __device__ void init() {
-        const int64_t p = blockIdx.y;
-        a = in + (2 * p) * (int64_t)C::N;
-        has_b = 2 * p + 1 < n_tr;
-        b = a + C::N;
-        k1_0 = blockIdx.x * C::F;
-    }
-    template <int R, int JPF>
-    __device__ __forceinline__ void load(int f, int j, T *ra, T *ia, T *rb, T *ib) const {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int k = k1_0 + f + C::N1 * (j + r * JPF);
-            V va = a[k];
-            ra[r] = va.x; ia[r] = va.y;
-            if (has_b) { V vb = b[k]; rb[r] = vb.x; ib[r] = vb.y; }
-            else { rb[r] = T(0); ib[r] = T(0); }
-        }
-    }
-};
-
 // Search, FP32: w[k] = (y_k a_k, y_k b_k) as float4 for one sky; z = w e^{-2 pi i phi_k},
 // phi_k = frac(fdot dt^2 k^2 / 2) from a 64-bit fixed-point product (exact mod 1
 // up to the rounding of the rate), zero for k >= n (the zero padding).
@@ -252,33 +223,6 @@ struct ScratchLoad {
 };
 
 // ------------------------------------------------------------------ pass 2 storers
-template <typename T, class C>
-struct GenericStore {
-    using V = typename Vec2<T>::type;
-    V *out;
-    int64_t n_tr;
-    V *a, *b;
-    bool has_b;
-    int l2_0;
-    __device__ void init() {
-        const int64_t p = blockIdx.y;
-        a = out + 2 * p * (int64_t)C::N;
-        b = a + C::N;
-        has_b = 2 * p + 1 < n_tr;
-        l2_0 = blockIdx.x * C::F;
-    }
-    template <int R, int JPF>
-    __device__ __forceinline__ void store(int f, int j, T *ra, T *ia, T *rb, T *ib) const {
-        const int l2 = l2_0 + f;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int l = C::N2 * (j + r * JPF) + l2;
-            a[l] = V{ra[r], ia[r]};
-            if (has_b) b[l] = V{rb[r], ib[r]};
-        }
-    }
-};
-
 // F = |F_a|^2/(sigma^2 S_aa) + |F_b|^2/(sigma^2 S_bb) per bin (Fig. 1,
 // "F-statistics calculation"), strict 2F > thr ("signals above the threshold
 // registered"), appended with one atomic per warp: the same offset arithmetic as
@@ -352,58 +296,6 @@ k_pass(LD ld, ST st, const T *__restrict__ tw) {
     ld.init();
     st.init();
     eng::run_pass<T, C::M, C::F, C::EH, DIR, MAPM>(ld, st, tw);
-}
-
-// Pass-1 output parked in the exchange area, in natural order, one row per
-// sequence (the group that transformed a column writes only its own row).
-template <typename T, class C>
-struct RowParkStore {
-    using V = typename Vec2<T>::type;
-    V *sd;
-    template <int R, int JPF>
-    __device__ __forceinline__ void store(int f, int j, T *ra, T *ia, T *rb, T *ib) const {
-        constexpr int RL = eng::row_ld(C::M);
-        V *pa = sd + f * RL, *pb = sd + (C::F + f) * RL;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int l2 = j + r * JPF;
-            pa[eng::pad(l2)] = V{ra[r], ia[r]};
-            pb[eng::pad(l2)] = V{rb[r], ib[r]};
-        }
-    }
-};
-
-// Search pass 1 with one sequence per thread group: each group gathers its
-// column, demodulates and transforms it with group-local synchronisation only,
-// parks the result in its shared-memory row; then the CTA writes the tile to
-// scratch row by row (coalesced), applying the inter-pass twiddle
-// W_N^{k1 l2} = hi[m >> log N1] lo[m & (N1 - 1)], m = k1 l2.
-template <typename T, int LOGN, int TS, class LD>
-__global__ void __launch_bounds__(Cfg<T, LOGN, 1, TS>::THREADS, Cfg<T, LOGN, 1, TS>::MIN_BLOCKS)
-k_search_pass1(LD ld, typename Vec2<T>::type *scratch, const T *__restrict__ lo,
-               const T *__restrict__ hi, const T *__restrict__ tw) {
-    using C = Cfg<T, LOGN, 1, TS>;
-    using V = typename Vec2<T>::type;
-    constexpr int RL = eng::row_ld(C::M);
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    V *sd = reinterpret_cast<V *>(smem_raw);
-    ld.init();
-    RowParkStore<T, C> st{sd};
-    eng::run_pass<T, C::M, C::F, C::EH, -1, eng::kMapW>(ld, st, tw);
-    __syncthreads();
-    V *base = scratch + (int64_t)blockIdx.y * 2 * C::N;
-    const int k1_0 = blockIdx.x * C::F;
-    for (int idx = threadIdx.x; idx < C::F * C::M; idx += C::THREADS) {
-        const int l2 = idx / C::F, f = idx - l2 * C::F;
-        const int k1 = k1_0 + f;
-        const int m = k1 * l2;
-        const V th = __ldg(reinterpret_cast<const V *>(hi) + (m >> C::LOGN1));
-        const V tl = __ldg(reinterpret_cast<const V *>(lo) + (m & (C::N1 - 1)));
-        const T wr = th.x * tl.x - th.y * tl.y, wi = th.x * tl.y + th.y * tl.x;
-        const V a = sd[f * RL + eng::pad(l2)], b = sd[(C::F + f) * RL + eng::pad(l2)];
-        base[(int64_t)l2 * C::N1 + k1] = V{a.x * wr - a.y * wi, a.x * wi + a.y * wr};
-        base[C::N + (int64_t)l2 * C::N1 + k1] = V{b.x * wr - b.y * wi, b.x * wi + b.y * wr};
-    }
 }
 
 template <class KernelPtr>

@@ -58,3 +58,30 @@ def _check(fs, form, n, n_fft, n_sky, n_spin, dt=2.0, f_off=100.5, full_range=Fa
 ])
 def test_fp64_batches(fs, n, n_fft, n_sky, n_spin, kw):
     _check(fs, fs.FP64_PLAIN, n, n_fft, n_sky, n_spin, **kw)
+
+
+@pytest.mark.parametrize("n,U", [(16, 2), (128, 3), (255, 2), (256, 2), (257, 5), (1024, 2), (2047, 8), (4097, 4),
+                                 (8191, 3), (65536, 2), (86165, 3), (262147, 2)])
+def test_upsample(fs, n, U):
+    """The FFT upsample at odd and even lengths, powers of two (circular convolution of that
+    length) and just beside them, and several factors, through the FP64 form's F at identity
+    resampling positions of the upsampled series: an ephemeris that moves the samples by a
+    constant j + s/U picks sub-phase s alone (s and U: s/U is a multiple of 1/U)."""
+    rng = np.random.default_rng(n + U)
+    nf = max(256, S.n_fft_auto(n))
+    x = rng.standard_normal(n)
+    one = np.zeros(1)
+    for s in {1, U // 2, U - 1}:
+        r = np.zeros((n, 3))
+        r[:, 0] = -2.0 * s / U          # nhat = (1, 0, 0): every sample read s/U later, dt = 2
+        b = S.Band(n=n, dt=2.0, f_off=0.0, x=x, r=r, phi0=0.3, eps=0.0, n_fft=nf, sigma=1.0)
+        prm = O.params(S.LAT_DEFAULT, S.GAMMA_DEFAULT, U, 1.0, False, 0)
+        lo, hi = 1, min(nf // 2 - 1, 3000)
+        ref = O.cells_F(b, prm, one, one, one, np.array([0]), np.array([0]), lo, hi, NTHREADS)
+        with fs.Plan([b], one, one, one, -1.0, lat=S.LAT_DEFAULT, gamma=S.GAMMA_DEFAULT, upsample=U, form=fs.FP64_PLAIN,
+                     sigma2=1.0, bin_lo=lo, bin_hi=hi, cand_capacity=ref.size) as p:
+            p.search()
+            c, total = p.candidates()
+        assert total == ref.size
+        err = np.abs(c["F"] - ref[0]) / np.maximum(ref[0], 2.0)
+        assert err.max() <= TOL[0], (s, err.max())
