@@ -203,6 +203,19 @@ void packed512_twiddles(std::vector<double> &o) {
             }
 }
 
+// The same for the stage 1 of a 1024-point row pass split by decimation in
+// frequency: [m][q] = (W_1024^{mq}, W_1024^{m(q+32)}), m < 16, q < 32.
+void packed1024_twiddles(std::vector<double> &o) {
+    o.assign(16 * 32 * 4, 0.0);
+    for (int m = 0; m < 16; ++m)
+        for (int q = 0; q < 32; ++q)
+            for (int e = 0; e < 2; ++e) {
+                const double a = kTwoPi * (double)((m * (q + 32 * e)) % 1024) / 1024.0;
+                o[(size_t)(4 * (m * 32 + q) + e)] = cos(a);
+                o[(size_t)(4 * (m * 32 + q) + 2 + e)] = -sin(a);
+            }
+}
+
 void build_twiddles(Plan &p, const std::vector<int> &logs, int &n_alloc) {
     std::vector<double> hd;
     std::vector<size_t> offs;
@@ -213,6 +226,7 @@ void build_twiddles(Plan &p, const std::vector<int> &logs, int &n_alloc) {
         stage1_twiddles(log_n1(lg), e);
         stage1_twiddles(log_n2(lg), f);
         if (log_n1(lg) == 9) packed512_twiddles(g);   // 512-point rows: N_fft = 2^18, 2^19
+        if (log_n1(lg) == 10) packed1024_twiddles(g);   // 1024-point rows: 2^20
         for (auto *v : {&a, &b, &c, &d, &e, &f, &g}) {
             while (hd.size() % 4) hd.push_back(0.0);   // 16-byte aligned float tables
             offs.push_back(hd.size());
@@ -235,6 +249,7 @@ void build_twiddles(Plan &p, const std::vector<int> &logs, int &n_alloc) {
         t.s1_f = df + o[4]; t.s2_f = df + o[5];
         t.s1_d = dd + o[4]; t.s2_d = dd + o[5];
         if (log_n1(logs[i]) == 9) t.p512_f = reinterpret_cast<const float4 *>(df + o[6]);
+        if (log_n1(logs[i]) == 10) t.p1024_f = reinterpret_cast<const float4 *>(df + o[6]);
         p.tw.push_back(t);
     }
 }
@@ -318,6 +333,15 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
     }
     p.n_fft_max = max_nfft;
     build_twiddles(p, logs, n_alloc);
+    for (auto &t : p.tw) {   // FP32 form: row factors of the packed rows, for the lengths the bands search
+        const bool used = std::any_of(p.bands.begin(), p.bands.end(),
+                                      [&](const BandDev &b) { return b.logn - (p.interbin ? 1 : 0) == t.logn; });
+        if (!fp32 || !used || row_twiddle_entries(t.logn) == 0) continue;
+        float4 *rt = dalloc<float4>(p, (size_t)row_twiddle_entries(t.logn), n_alloc);
+        launch_row_twiddles(rt, t.logn, s);
+        ++p.launches;
+        t.row_tw = rt;
+    }
     if (!fp32) {   // tables of the FP64 passes, for the lengths the bands search
         double2 *ut = dalloc<double2>(p, (size_t)unit_table_entries(), n_alloc);
         launch_unit_table(ut, s);

@@ -41,6 +41,10 @@ struct TwiddleSet {
     // 512-point pass as pairs,
     // [r][k] = (cos a_2k, cos a_2k+1, -sin a_2k, -sin a_2k+1), a_j = 2 pi r j / 512
     const float4 *p512_f = nullptr;
+    // 1024-point rows (2^20): [m][q] = (W_1024^{mq}, W_1024^{m(q+32)}) as packed pairs
+    // (cosines, then sines of the negative angles), m < 16, q < 32
+    const float4 *p1024_f = nullptr;
+    const float4 *row_tw = nullptr;   // FP32 packed rows: the rows' four-step factors
 };
 
 // Per-sky normaliser record: na, nb, nab, 0 in FP64 (doubles 0..3), then the
@@ -142,7 +146,7 @@ struct Plan {
     std::vector<cudaEvent_t> ev_done[2];
     std::vector<cudaEvent_t> ev_join;
     int elems_per_thread = 16;     // FP32 batched passes: 16 or 8 complex elements per thread
-    int engine = 2;                // FP32 batched passes, 2^12 .. 2^19: 2 = two-stage engine, 1 = radix-8 engine
+    int engine = 2;                // FP32 batched passes, 2^12 .. 2^20: 2 = two-stage engine, 1 = radix-8 engine
     bool fused = false;            // two-stage engine: both passes in one ticket-ordered launch
     bool interbin = false;         // FSTAT_INTERP_INTERBIN: half-length transforms + interbinning
     uint32_t *fctl = nullptr;      // per worker: 1 + 2 * cell_batch counters of the fused launch
@@ -267,6 +271,9 @@ int launch_reduce_norms(const Plan &p, const BandDev &b, int64_t ns, double *nor
 CandRecord *launch_cand_sort(CandRecord *a, CandRecord *b, uint32_t *hist, int64_t n, uint32_t cell0,
                              uint64_t cell_span, int bin_bits, cudaStream_t s, int64_t *launches);
 
+// Row factors of the four-step twiddle for the packed FP32 rows (0 entries: none used).
+int64_t row_twiddle_entries(int logn);
+void launch_row_twiddles(float4 *t, int logn, cudaStream_t s);
 // Tables of the FP64 form: unit phases, and the four-step twiddles of a length
 // 2^logn in the order its passes read them.
 int64_t unit_table_entries();

@@ -273,20 +273,23 @@ struct ScratchLoadTMA {
             ptx::bulk_g2s(const_cast<float2 *>(rows), src, bytes, bar);
         }
     }
+    // bounded wait for the copy
+    __device__ __forceinline__ void wait() const {
+        if (ptx::mbar_try_wait(bar, 0)) return;
+        const uint64_t t0 = ptx::globaltimer_ns();
+        bool late = false;
+        while (!ptx::mbar_try_wait(bar, 0)) {
+            const uint64_t dt = ptx::globaltimer_ns() - t0;
+            if (!late && dt > 1000000000ull) { atomicExch(err, 1u); late = true; }
+            if (dt > 2000000000ull) break;   // reported above; results are discarded
+        }
+    }
     template <int R, int JPF>
     __device__ __forceinline__ void load(const eng2::Job &q, float *re, float *im) const {
         // the twiddle factors load while the bulk copies are in flight
         const int l2 = l2_0 + q.f;
         const float2 w0 = tw.wn(l2 * q.j), st = tw.wn(l2 * JPF);
-        if (!ptx::mbar_try_wait(bar, 0)) {
-            const uint64_t t0 = ptx::globaltimer_ns();
-            bool late = false;
-            while (!ptx::mbar_try_wait(bar, 0)) {
-                const uint64_t dt = ptx::globaltimer_ns() - t0;
-                if (!late && dt > 1000000000ull) { atomicExch(err, 1u); late = true; }
-                if (dt > 2000000000ull) break;   // reported above; results are discarded
-            }
-        }
+        wait();
         const float2 *row = rows + 2 * (q.f * C::N1 + q.j) + q.t;
 #pragma unroll
         for (int r = 0; r < R; ++r) {

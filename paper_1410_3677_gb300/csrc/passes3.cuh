@@ -1,6 +1,7 @@
 // The FP32 search passes in packed arithmetic (packed.cuh) for passes of length
 // 512: both passes at N_fft = 2^18 (N1 = N2 = 512, the two-sidereal-day
-// segments), the rows (pass 2) at 2^19; and the 256-point rows of 2^16 and 2^17.  Same four-step split, scratch layout, tiles and
+// segments), the rows (pass 2) at 2^19; the 256-point rows of 2^16 and 2^17; and
+// the 1024-point rows of 2^20.  Same four-step split, scratch layout, tiles and
 // launch shapes as the second engine's passes (passes2.cuh); what changes is how
 // a thread's 32 elements are transformed:
 //
@@ -14,8 +15,7 @@
 //    its twiddles and the F epilogue run packed as well;
 //  - in pass 2 the four-step twiddle W_N^{k1 l2} of inputs m and m + 16 folds
 //    into the split: with T_m = W_N^{l2 (j + 16 m)} and c = W_N^{256 l2},
-//    a_m = T_m (s_m + c s_{m+16}) and b_m = T_m W_32^m (s_m - c s_{m+16}); the pair
-//    (T_m, T_m W_32^m) advances by the packed factor (W_N^{16 l2}, W_N^{16 l2} W_32).
+//    a_m = T_m (s_m + c s_{m+16}) and b_m = T_m W_32^m (s_m - c s_{m+16}).
 #pragma once
 
 #include "packed.cuh"
@@ -160,16 +160,54 @@ k_pass1h(SearchLoad2<Cfg2<LOGN, 1>> ld, ScratchStore2<Cfg2<LOGN, 1>> st, const f
     st.template store<16, kR0>(q1, re1, im1);
 }
 
+// --------------------------------------------------------------------- row twiddles
+// The four-step twiddle of element k1 = j + G m of row l2 is W_N^{l2 j} (the
+// thread's, from two table entries) times W_N^{G l2 m} (the row's).  The rows'
+// factors come from a table, 16 packed pairs (256 bytes) per row or row pair, which
+// a second bulk copy puts behind the staged rows; every lane reads the same word.
+// A recurrence over m in place of the table took as many instructions, but its
+// rounding error grew with m (a third of the error of F) and it chained 15
+// complex multiplies.  Measured at 2^18: pass 2 0.660 -> 0.648 us a cell, rms error of F
+// 6.5e-7 -> 3.2e-7.
+constexpr int kRowTw = 16;
+
+template <class C, int TILES_PER_ENTRY = 1>
+struct RowsTMA : ScratchLoadTMA<C> {
+    static constexpr int ENTRIES = C::F / TILES_PER_ENTRY;   // table rows per tile
+    static constexpr uint32_t TW_BYTES = ENTRIES * kRowTw * sizeof(float4);
+    static constexpr uint32_t ROW_BYTES = (uint32_t)(2 * C::F * C::N1 * sizeof(float2));
+    static constexpr size_t SMEM = ROW_BYTES + TW_BYTES + 16;   // rows, twiddles, mbarrier
+    const float4 *row_tw;   // [row or row pair][16]
+    const float4 *tws;      // in shared memory
+    __device__ void init(int tile, int64_t cell, int64_t slot) {
+        ScratchLoadTMA<C>::init(tile, cell, slot);
+        unsigned char *sm = eng2::dyn_smem();
+        tws = reinterpret_cast<const float4 *>(sm + ROW_BYTES);
+        this->bar = reinterpret_cast<uint64_t *>(sm + ROW_BYTES + TW_BYTES);
+        row_tw += (int64_t)tile * ENTRIES * kRowTw;
+    }
+    __device__ void stage() const {
+        if (threadIdx.x == 0) {
+            ptx::mbar_init(this->bar, 1);
+            ptx::fence_mbar_init();
+        }
+        if constexpr (C::THREADS == 32) __syncwarp(); else __syncthreads();
+        if (threadIdx.x == 0) {
+            ptx::mbar_arrive_expect_tx(this->bar, ROW_BYTES + TW_BYTES);
+            ptx::bulk_g2s(const_cast<float2 *>(this->rows), this->src, ROW_BYTES, this->bar);
+            ptx::bulk_g2s(const_cast<float4 *>(tws), row_tw, TW_BYTES, this->bar);
+        }
+    }
+    __device__ __forceinline__ PC tw_m(int entry, int m) const {
+        const float4 v = tws[entry * kRowTw + m];
+        return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+    }
+};
+
 // --------------------------------------------------------------------- pass 2
-// Dynamic shared memory of the packed pass 2 before its mbarrier (8 bytes after
-// it): the staged tile, F rows x 2 transforms x 512 complex floats.  Each warp's
-// exchange lies over the row it has staged: 2 transforms x 16 job pairs x 16
-// elements of 16 bytes, exactly the row's 8 KiB, so no warp waits for another
-// between the stages.
-template <class C>
-__host__ __device__ constexpr size_t pass2p_smem() {
-    return (size_t)2 * C::F * C::N1 * sizeof(float2);
-}
+// Each warp's exchange lies over the row it has staged: 2 transforms x 16 job
+// pairs x 16 elements of 16 bytes, exactly the row's 8 KiB, so no warp waits for
+// another between the stages.
 
 // Outputs p of a packed 16-point DFT that the F epilogue uses, halved: the bin
 // range below N/2 (LOWER) needs p < 8 only.
@@ -258,14 +296,13 @@ __device__ __forceinline__ void epilogue(const SearchEpi2<C, LOWER> &ep, int t, 
 // default) 24 CTAs share an SM and each waits only for its own 8 KiB copy.
 template <int LOGN, bool LOWER, int TS = 32>
 __global__ void __launch_bounds__(TS, 768 / TS)
-k_pass2p(ScratchLoadTMA<Cfg2<LOGN, 2, TS>> ld, SearchEpi2<Cfg2<LOGN, 2, TS>, LOWER> ep,
+k_pass2p(RowsTMA<Cfg2<LOGN, 2, TS>> ld, SearchEpi2<Cfg2<LOGN, 2, TS>, LOWER> ep,
          const float4 *__restrict__ tws) {
     using C = Cfg2<LOGN, 2, TS>;
     static_assert(C::M == kM && C::F == TS / 32 && C::SEQ == 2 * C::F && C::TPF == 16, "512-point rows, a warp per row");
     static_assert(2 * kR1 * kR1 * 16 == 2 * C::N1 * sizeof(float2), "a warp's exchange fills its staged row");
     ld.prefetch_ahead();
     ld.init(blockIdx.x, blockIdx.y, blockIdx.y);
-    ld.bar = reinterpret_cast<uint64_t *>(eng2::dyn_smem() + pass2p_smem<C>());   // after the staged tile
     const int w = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
     ep.init(blockIdx.x, blockIdx.y, blockIdx.y);
     ld.stage();
@@ -275,23 +312,11 @@ k_pass2p(ScratchLoadTMA<Cfg2<LOGN, 2, TS>> ld, SearchEpi2<Cfg2<LOGN, 2, TS>, LOW
     const int j = lane >> 1;           // stage-0 butterfly; stage-1 job pair (2j, 2j + 1)
     const int f = w;                   // tile row
     const int l2 = ld.l2_0 + f;
-    // four-step factors: T_0 = W^{l2 j}, step W^{16 l2}, c = W^{256 l2}
-    const float2 w0 = ld.tw.wn(l2 * j), stp = ld.tw.wn(16 * l2), cc = ld.tw.wn(256 * l2);
-    // (T_m, T_m W_32^m) advance by (stp, stp W_32)
-    PC T = {make_float2(w0.x, w0.x), make_float2(w0.y, w0.y)};
-    float s1r = stp.x, s1i = stp.y;
-    w32_scalar(1, s1r, s1i);
-    const PC S = {make_float2(stp.x, s1r), make_float2(stp.y, s1i)};
-    // wait for the tile's bulk copy (bounded, as ScratchLoadTMA::load)
-    if (!ptx::mbar_try_wait(ld.bar, 0)) {
-        const uint64_t t0 = ptx::globaltimer_ns();
-        bool late = false;
-        while (!ptx::mbar_try_wait(ld.bar, 0)) {
-            const uint64_t dt = ptx::globaltimer_ns() - t0;
-            if (!late && dt > 1000000000ull) { atomicExch(ld.err, 1u); late = true; }
-            if (dt > 2000000000ull) break;   // reported above; results are discarded
-        }
-    }
+    // four-step factors: T_0 = W^{l2 j}, c = W^{256 l2}; (W^{16 l2 m}, W^{16 l2 m} W_32^m)
+    // come with the row
+    const float2 w0 = ld.tw.wn(l2 * j), cc = ld.tw.wn(256 * l2);
+    const PC T = {make_float2(w0.x, w0.x), make_float2(w0.y, w0.y)};
+    ld.wait();
     PC P[16];
     {
         const float2 *row = ld.rows + 2 * (f * C::N1 + j) + t;   // element k1 at row[2 k1]
@@ -301,8 +326,7 @@ k_pass2p(ScratchLoadTMA<Cfg2<LOGN, 2, TS>> ld, SearchEpi2<Cfg2<LOGN, 2, TS>, LOW
             // u = c s_{m+16}; A = s_m + u, D = s_m - u
             const float ur = hi.x * cc.x - hi.y * cc.y, ui = hi.x * cc.y + hi.y * cc.x;
             const PC X = {make_float2(lo.x + ur, lo.x - ur), make_float2(lo.y + ui, lo.y - ui)};
-            P[m] = pk::cmul(X, T);
-            if (m + 1 < 16) T = pk::cmul(T, S);
+            P[m] = pk::cmul(X, m ? pk::cmul(T, ld.tw_m(f, m)) : T);
         }
     }
     pk::dft16<16>(P);   // P[k] = (X_{2k}, X_{2k+1}) of row l2
@@ -341,40 +365,28 @@ k_pass2p(ScratchLoadTMA<Cfg2<LOGN, 2, TS>> ld, SearchEpi2<Cfg2<LOGN, 2, TS>, LOW
 // giving l1 = q + 16 p.  The exchange lies over the warp's staged 8 KiB.
 template <int LOGN, bool LOWER>
 __global__ void __launch_bounds__(32, 24)
-k_pass2r(ScratchLoadTMA<Cfg2<LOGN, 2, 32>> ld, SearchEpi2<Cfg2<LOGN, 2, 32>, LOWER> ep,
+k_pass2r(RowsTMA<Cfg2<LOGN, 2, 32>, 2> ld, SearchEpi2<Cfg2<LOGN, 2, 32>, LOWER> ep,
          const float2 *__restrict__ w256) {
     using C = Cfg2<LOGN, 2, 32>;
     static_assert(C::M == 256 && C::F == 2 && C::THREADS == 32, "256-point rows, two per warp");
     ld.prefetch_ahead();
     ld.init(blockIdx.x, blockIdx.y, blockIdx.y);
-    ld.bar = reinterpret_cast<uint64_t *>(eng2::dyn_smem() + 2 * C::F * C::N1 * sizeof(float2));
     const int lane = (int)threadIdx.x & 31;
     ep.init(blockIdx.x, blockIdx.y, blockIdx.y);
     ld.stage();
     const int t = lane & 1, j = lane >> 1;
     const int l2 = ld.l2_0;   // rows l2 and l2 + 1
-    // four-step factors of the two rows: T_0 = W^{l2 j}, step W^{16 l2}
+    // four-step factors of the two rows: T_0 = W^{l2 j}; the pairs W^{16 l2 m} come with them
     const float2 wa = ld.tw.wn(l2 * j), wb = ld.tw.wn((l2 + 1) * j);
-    const float2 sa = ld.tw.wn(16 * l2), sb = ld.tw.wn(16 * (l2 + 1));
-    PC T = {make_float2(wa.x, wb.x), make_float2(wa.y, wb.y)};
-    const PC S = {make_float2(sa.x, sb.x), make_float2(sa.y, sb.y)};
-    if (!ptx::mbar_try_wait(ld.bar, 0)) {   // bounded wait, as ScratchLoadTMA::load
-        const uint64_t t0 = ptx::globaltimer_ns();
-        bool late = false;
-        while (!ptx::mbar_try_wait(ld.bar, 0)) {
-            const uint64_t dt = ptx::globaltimer_ns() - t0;
-            if (!late && dt > 1000000000ull) { atomicExch(ld.err, 1u); late = true; }
-            if (dt > 2000000000ull) break;   // reported above; results are discarded
-        }
-    }
+    const PC T = {make_float2(wa.x, wb.x), make_float2(wa.y, wb.y)};
+    ld.wait();
     PC P[16];
     {
         const float2 *ra = ld.rows + 2 * j + t, *rb = ra + 2 * C::N1;   // element k1 at r[2 k1]
 #pragma unroll
         for (int m = 0; m < 16; ++m) {
             const float2 a = ra[2 * 16 * m], b = rb[2 * 16 * m];
-            P[m] = pk::cmul({make_float2(a.x, b.x), make_float2(a.y, b.y)}, T);
-            if (m + 1 < 16) T = pk::cmul(T, S);
+            P[m] = pk::cmul({make_float2(a.x, b.x), make_float2(a.y, b.y)}, m ? pk::cmul(T, ld.tw_m(0, m)) : T);
         }
     }
     pk::dft16<16>(P);   // P[k] = Z_j[k] of both rows
@@ -402,6 +414,75 @@ k_pass2r(ScratchLoadTMA<Cfg2<LOGN, 2, 32>> ld, SearchEpi2<Cfg2<LOGN, 2, 32>, LOW
     // bins: output p = u + t H of job q for row l2 + e: l1 = q + 16 p, bin = N2 l1 + l2 + e
     constexpr int H = epi_half<LOWER>();
     epilogue<C, LOWER>(ep, t, C::N2 * (q + 16 * t * H) + l2, C::N2 * 16, 1, Q);
+}
+
+// --------------------------------------------------------------------- pass 2, 1024-point rows
+// The rows of N_fft = 2^20 (N1 = 1024 = 32 x 32), a row of both transforms per
+// 64-thread CTA: thread 2j + t takes the elements k1 = j + 32 m of transform t.
+// Both radix-32 stages are split by one decimation-in-frequency step into a packed
+// 16-point DFT, the stage's twiddle folded into the split as in k_pass2p: with
+// V_m the twiddle of input m and c = V_{m+16} / V_m (the same for every m),
+// a_m = V_m (x_m + c x_{m+16}), b_m = V_m W_32^m (x_m - c x_{m+16}); the outputs are
+// the pairs (X_2k, X_2k+1).  In stage 1 V_m = W_1024^{mq} and V_m W_32^m =
+// W_1024^{m(q+32)} come from one packed table.  A whole row per CTA (16 KiB, twelve
+// CTAs per SM) instead of the radix-8 engine's three stages and two exchanges.
+// Measured at N = 344 656 (768 cells): pass 1 and 2 together 13.4 -> 7.25 us a cell (pass 2
+// 5.36 -> 3.01 us).
+template <int LOGN, bool LOWER>
+__global__ void __launch_bounds__(64, 12)
+k_pass2q(RowsTMA<Cfg2<LOGN, 2, 64>> ld, SearchEpi2<Cfg2<LOGN, 2, 64>, LOWER> ep,
+         const float4 *__restrict__ tws, const float2 *__restrict__ w1024) {
+    using C = Cfg2<LOGN, 2, 64>;
+    static_assert(C::M == 1024 && C::F == 1 && C::THREADS == 64, "1024-point rows, one per CTA");
+    ld.init(blockIdx.x, blockIdx.y, blockIdx.y);
+    ep.init(blockIdx.x, blockIdx.y, blockIdx.y);
+    ld.stage();
+    const int t = (int)threadIdx.x & 1, j = (int)threadIdx.x >> 1;
+    const int l2 = ld.l2_0;
+    const float2 w0 = ld.tw.wn(l2 * j), cc = ld.tw.wn(512 * l2);
+    const PC T = {make_float2(w0.x, w0.x), make_float2(w0.y, w0.y)};
+    const float2 c1 = __ldg(w1024 + 16 * j);
+    ld.wait();
+    PC P[16];
+    {
+        const float2 *row = ld.rows + 2 * j + t;   // element k1 at row[2 k1]
+#pragma unroll
+        for (int m = 0; m < 16; ++m) {
+            const float2 lo = row[2 * 32 * m], hi = row[2 * 32 * (m + 16)];
+            const float ur = hi.x * cc.x - hi.y * cc.y, ui = hi.x * cc.y + hi.y * cc.x;
+            const PC X = {make_float2(lo.x + ur, lo.x - ur), make_float2(lo.y + ui, lo.y - ui)};
+            P[m] = pk::cmul(X, m ? pk::cmul(T, ld.tw_m(0, m)) : T);
+        }
+    }
+    pk::dft16<16>(P);   // P[k] = (X_{2k}, X_{2k+1}) of butterfly j
+    __syncthreads();    // the staged row has been read: the exchange may overwrite it
+    // element (output r, butterfly j) at 32 r + (j ^ r ^ 8 t): a half-warp holds 8 j (or,
+    // loading, 8 r) of both transforms and falls in 16 different 8-byte banks either way
+    float2 *ex = reinterpret_cast<float2 *>(eng2::dyn_smem()) + t * C::N1;
+    const int jx = j ^ (8 * t);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        ex[32 * (2 * k) + (jx ^ (2 * k))] = make_float2(P[k].re.x, P[k].im.x);
+        ex[32 * (2 * k + 1) + (jx ^ (2 * k + 1))] = make_float2(P[k].re.y, P[k].im.y);
+    }
+    __syncthreads();
+    // stage 1, job q = j: the butterflies of output q
+    const int q = j;
+    PC Q[16];
+#pragma unroll
+    for (int m = 0; m < 16; ++m) {
+        const float2 lo = ex[32 * q + (m ^ jx)], hi = ex[32 * q + ((m + 16) ^ jx)];
+        const float ur = hi.x * c1.x - hi.y * c1.y, ui = hi.x * c1.y + hi.y * c1.x;
+        Q[m] = {make_float2(lo.x + ur, lo.x - ur), make_float2(lo.y + ui, lo.y - ui)};
+    }
+#pragma unroll
+    for (int m = 1; m < 16; ++m) {
+        const float4 v = __ldg(tws + m * 32 + q);
+        Q[m] = pk::cmul(Q[m], PC{make_float2(v.x, v.y), make_float2(v.z, v.w)});
+    }
+    pk::dft16<16, LOWER>(Q);   // Q[k] = (Y_2k, Y_2k+1): l1 = q + 32 (2k + e)
+    constexpr int H = epi_half<LOWER>();
+    epilogue<C, LOWER>(ep, t, C::N2 * (q + 64 * t * H) + l2, C::N2 * 64, C::N2 * 32, Q);
 }
 
 }  // namespace p3

@@ -1,6 +1,6 @@
 // FP32 instantiations of the search passes (FSTAT_FP32_BATCHED): the two-stage
-// engine for transform lengths 2^12 .. 2^19 (both passes in one ticket-ordered
-// launch, or as two launches), the radix-8 engine otherwise (and whenever the
+// engine for transform lengths 2^12 .. 2^20 (as two launches, or up to 2^19 both
+// passes in one ticket-ordered launch), the radix-8 engine otherwise (and whenever the
 // plan selects it).
 #include <algorithm>
 
@@ -46,14 +46,15 @@ void launch_pass2p(const Plan &p, int band_idx, const BandDev &b, int64_t s0, in
                    cudaStream_t s, const CellBufs &cb, const ScratchLoad2<Cfg2<LOGN, 2>> &ld2,
                    const TwiddleSet *tw) {
     using D2 = Cfg2<LOGN, 2, TS>;
-    ScratchLoadTMA<D2> lt{};
+    p3::RowsTMA<D2> lt{};
     lt.scratch = ld2.scratch;
     lt.tw = ld2.tw;
     lt.pf_dist = p.pf_dist_pk;   // the paired pass gains nothing from L2 prefetch ahead
     lt.err = p.qerr;
+    lt.row_tw = tw->row_tw;
     const auto ep = make_epi<LOGN, LOWER, TS>(p, band_idx, b, c0, s0, cb);
     auto k2 = p3::k_pass2p<LOGN, LOWER, TS>;
-    constexpr size_t smem2 = p3::pass2p_smem<D2>() + 16;   // staged tile + mbarrier
+    constexpr size_t smem2 = p3::RowsTMA<D2>::SMEM;
     static bool attr2p = false;
     if (!attr2p) { set_smem(k2, smem2); attr2p = true; }
     k2<<<dim3(D2::TILES, (unsigned)nc), D2::THREADS, smem2, s>>>(lt, ep, tw->p512_f);
@@ -121,14 +122,15 @@ int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_
     if constexpr (LOGN == 16 || LOGN == 17) {   // 256-point rows: two per warp, packed
         if (p.packed >= 1 && p.tma && p.p2_threads != 256 && p.p2_rows) {
             using D2 = Cfg2<LOGN, 2, 32>;
-            ScratchLoadTMA<D2> lt{};
+            p3::RowsTMA<D2, 2> lt{};
             lt.scratch = ld2.scratch;
             lt.tw = ld2.tw;
             lt.pf_dist = 0;
             lt.err = p.qerr;
+            lt.row_tw = tw->row_tw;
             const auto ep = make_epi<LOGN, LOWER, 32>(p, band_idx, b, c0, s0, cb);
             auto k2 = p3::k_pass2r<LOGN, LOWER>;
-            constexpr size_t smem2 = (size_t)2 * D2::F * D2::N1 * sizeof(float2) + 16;   // staged rows + mbarrier
+            constexpr size_t smem2 = p3::RowsTMA<D2, 2>::SMEM;
             static bool attr2r = false;
             if (!attr2r) { set_smem(k2, smem2); attr2r = true; }
             k2<<<dim3(D2::TILES, (unsigned)nc), D2::THREADS, smem2, s>>>(
@@ -144,7 +146,23 @@ int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_
             return 2;
         }
     }
-    if (p.tma && p.p2_threads == 128) {   // smaller tiles, six CTAs per SM
+    if constexpr (LOGN == 20) {   // 1024-point rows: one per CTA, packed
+        using D2 = Cfg2<LOGN, 2, 64>;
+        p3::RowsTMA<D2> lt{};
+        lt.scratch = ld2.scratch;
+        lt.tw = ld2.tw;
+        lt.pf_dist = 0;
+        lt.err = p.qerr;
+        lt.row_tw = tw->row_tw;
+        const auto ep = make_epi<LOGN, LOWER, 64>(p, band_idx, b, c0, s0, cb);
+        auto k2 = p3::k_pass2q<LOGN, LOWER>;
+        constexpr size_t smem2 = p3::RowsTMA<D2>::SMEM;
+        static bool attr2q = false;
+        if (!attr2q) { set_smem(k2, smem2); attr2q = true; }
+        k2<<<dim3(D2::TILES, (unsigned)nc), D2::THREADS, smem2, s>>>(lt, ep, tw->p1024_f,
+                                                                     reinterpret_cast<const float2 *>(tw->in1_f));
+        return 2;
+    } else if (p.tma && p.p2_threads == 128) {   // smaller tiles, six CTAs per SM
         ScratchLoadTMA<Cfg2<LOGN, 2, 128>> lt{};
         lt.scratch = ld2.scratch;
         lt.tw = ld2.tw;
@@ -220,7 +238,7 @@ int launch_search2(const Plan &p, int band_idx, const BandDev &b, int64_t s0, in
     ld2.tw = {tw->lo_f, tw->hi_f};
     ld2.pf_dist = p.pf_dist;
     const bool lower = b.hi < (int64_t)C2::N / 2;
-    if (fused_supported(p, LOGN) && cb.ctl) {
+    if constexpr (LOGN < 20) if (fused_supported(p, LOGN) && cb.ctl) {
         return lower ? launch_fused<LOGN, true>(p, band_idx, b, s0, c0, nc, s, cb, ld1, st1, ld2, tw)
                      : launch_fused<LOGN, false>(p, band_idx, b, s0, c0, nc, s, cb, ld1, st1, ld2, tw);
     }
@@ -277,7 +295,35 @@ int launch_interbin(const Plan &p, int band_idx, const BandDev &b, int64_t s0, i
     return 2;
 }
 
+// Row factors of the four-step twiddle (RowsTMA): entry [i][m] holds the pair
+// (W_N^{G l2 m}, W_N^{G l2 m} W_32^m) of row l2 = i (512- and 1024-point rows, G = 16 and
+// 32), or (W_N^{16 l2 m}, W_N^{16 (l2+1) m}) of the rows l2 = 2i, 2i + 1 (256-point rows).
+__global__ void k_row_twiddles(float4 *t, int logn) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int n1 = logn / 2, n2 = logn - n1;
+    const bool pairs = n1 == 8;
+    if (i >= (p3::kRowTw << (pairs ? n2 - 1 : n2))) return;
+    const int e = i / p3::kRowTw, m = i % p3::kRowTw;
+    const double N = (double)(int64_t(1) << logn);
+    const int64_t g = n1 == 10 ? 32 : 16;
+    const double a = pairs ? (double)(g * 2 * e * m) / N : (double)(g * e * m) / N;
+    const double b = pairs ? (double)(g * (2 * e + 1) * m) / N : a + (double)m / 32.0;
+    double sa, ca, sb, cb;
+    sincospi(2.0 * a, &sa, &ca);
+    sincospi(2.0 * b, &sb, &cb);
+    t[i] = make_float4((float)ca, (float)cb, (float)-sa, (float)-sb);
+}
+
 }  // namespace
+
+int64_t row_twiddle_entries(int logn) {
+    const int n1 = logn / 2, n2 = logn - n1;
+    return n1 < 8 || n1 > 10 ? 0 : (int64_t)p3::kRowTw << (n1 == 8 ? n2 - 1 : n2);
+}
+
+void launch_row_twiddles(float4 *t, int logn, cudaStream_t s) {
+    k_row_twiddles<<<(unsigned)((row_twiddle_entries(logn) + 255) / 256), 256, 0, s>>>(t, logn);
+}
 
 bool interbin_supported(int logn) { return logn - 1 >= 12 && logn - 1 <= 19; }
 
@@ -311,6 +357,7 @@ int launch_search_cells_f32(const Plan &p, int band_idx, const BandDev &b, int64
             case 17: return launch_search2<17>(p, band_idx, b, s0, c0, nc, s, mid, cb);
             case 18: return launch_search2<18>(p, band_idx, b, s0, c0, nc, s, mid, cb);
             case 19: return launch_search2<19>(p, band_idx, b, s0, c0, nc, s, mid, cb);
+            case 20: return launch_search2<20>(p, band_idx, b, s0, c0, nc, s, mid, cb);
             default: break;
         }
     }

@@ -85,3 +85,13 @@ def test_upsample(fs, n, U):
         assert total == ref.size
         err = np.abs(c["F"] - ref[0]) / np.maximum(ref[0], 2.0)
         assert err.max() <= TOL[0], (s, err.max())
+
+
+@pytest.mark.parametrize("n,n_fft,n_sky,n_spin,kw", [
+    (300001, 1 << 20, 3, 5, dict(dt=0.5, window=2000)),
+    (393216, 1 << 20, 2, 2, dict(dt=0.5, window=2000, full=True)),          # n = 3N/8
+    (393217, 1 << 20, 2, 2, dict(dt=0.5, window=2000, full_range=True)),    # half of a column, both spectrum halves
+    (524288, 1 << 20, 1, 2, dict(dt=0.5, window=2000, f_off=0.0)),          # n = N / 2
+])
+def test_fp32_1024_point_rows(fs, n, n_fft, n_sky, n_spin, kw):
+    _check(fs, fs.FP32_BATCHED, n, n_fft, n_sky, n_spin, **kw)
