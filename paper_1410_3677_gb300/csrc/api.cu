@@ -95,8 +95,8 @@ SkyConst sky_const(double al, double de, double lat, double gamma) {
     c.ny = cd * sin(al);
     c.nz = sd;
     c.alpha = al;
-    const double nv[3] = {c.nx, c.ny, c.nz};
-    for (int i = 0; i < 3; ++i) {
+    const double nv[4] = {c.nx, c.ny, c.nz, al / kTwoPi};
+    for (int i = 0; i < 4; ++i) {
         const DF d = df_from_double(nv[i]);
         c.nf[2 * i] = d.hi;
         c.nf[2 * i + 1] = d.lo;
@@ -391,7 +391,7 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
         const int64_t n1 = int64_t(1) << log_n1(b.logn);
         p.w_stride = std::max<int64_t>(p.w_stride, (b.n + n1 - 1) / n1 * n1);
     }
-    const int64_t nblk = (p.n_max + 255) / 256;
+    const int64_t nblk = (p.n_max + 1023) / 1024;   // blocks of a geometry launch per position
     // sky positions per batch: 64, or up to 256 when the spindowns are few, so that a
     // batch holds the 4096 cells of a launch pair
     // FP64 form: up to 64 positions whose series (32 bytes a sample) fill 128 MiB: the FP64
@@ -405,8 +405,7 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
         p.wbuf[q] = dalloc<unsigned char>(p, (size_t)p.sky_batch * p.w_stride * w_elem, n_alloc);
         check(cudaMemsetAsync(p.wbuf[q], 0, (size_t)p.sky_batch * p.w_stride * w_elem, s), "memset");
     }
-    // per-sample delays (FP64 form) or 16-byte shift records (FP32 form)
-    p.dbuf = dalloc<double>(p, (size_t)p.sky_batch * p.n_max * (fp32 ? 2 : 1), n_alloc);
+    if (!fp32) p.dbuf = dalloc<double>(p, (size_t)p.sky_batch * p.n_max, n_alloc);   // per-sample delays
     p.partials = dalloc<double>(p, std::max<int64_t>((int64_t)p.sky_batch * nblk * 3, 256), n_alloc);
     p.S = dalloc<double>(p, 3 * p.sky_batch, n_alloc);
     p.sigma_parts = dalloc<double>(p, kSigmaParts, n_alloc);

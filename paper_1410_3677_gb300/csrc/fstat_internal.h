@@ -65,7 +65,7 @@ struct SkyConst {
     double nx, ny, nz, alpha;
     double A[5];
     double B[4];
-    float nf[6];   // nx, ny, nz as double-float pairs (hi, lo) for the FP32 delay
+    float nf[8];   // nx, ny, nz and alpha / 2 pi as double-float pairs (hi, lo) for the FP32 form
 };
 
 // Tables of the FFT upsample of a series of n samples (upsample.cu), laid out once
@@ -120,7 +120,7 @@ struct Plan {
     // geometry of the next sky batch can overlap the transforms of this one)
     int64_t sky_batch = 0;
     void *wbuf[2] = {nullptr, nullptr};   // FP32: float4 [sky_batch][w_stride]; FP64: {y a, y b} double2 pairs
-    double *dbuf = nullptr;       // [sky_batch][n_max] per-sample delays
+    double *dbuf = nullptr;       // FP64 form: [sky_batch][n_max] per-sample delays
     double *partials = nullptr;   // [sky_batch][n_blocks_max][3]
     double *S = nullptr;          // [sky_batch][3]
     double *sigma_parts = nullptr;   // [kSigmaParts] of the band being searched

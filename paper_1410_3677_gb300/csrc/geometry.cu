@@ -18,51 +18,14 @@ namespace {
 constexpr double kTwoPi = 6.283185307179586476925286766559;
 constexpr double kOmegaR = kTwoPi / 86164.0905;   // sidereal rotation rate, rad/s
 
-// The FP32 form's three S terms at once: each warp adds its 32 terms of each in
-// FP32 (relative error ~1e-7), one barrier, then three threads add the block's
-// warp sums in FP64 and write the block's partials (blockDim.x = 256); the
-// blocks' partials are then added with compensation.  The S sums thus keep FP64
-// accumulation where the term count is large, and spend no FP64 instructions per
-// sample.
-__device__ void block_sum3_f(float a, float b, float c, double *sh, double *out) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        b += __shfl_down_sync(0xffffffffu, b, o);
-        c += __shfl_down_sync(0xffffffffu, c, o);
-    }
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) {
-        sh[w] = (double)a;
-        sh[8 + w] = (double)b;
-        sh[16 + w] = (double)c;
-    }
-    __syncthreads();
-    if (threadIdx.x < 3) {
-        double t = 0.0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) t += sh[8 * threadIdx.x + i];
-        out[threadIdx.x] = t;
-    }
-}
-
 // ------------------------------------------------------------------ geometry
-// FP32 form: the delay of sample j reduced once, in double-float arithmetic
-// (FP64 runs at 1/64 of the FP32 rate on GB300), to the sample shift
-// d_j / dt = I + phi (integer part exact, fraction in FP32) and to the
-// band-offset phase f_off d_j mod 1 with its increment f_off (d_{j+1} - d_j), so
-// that the detector-time inversion and the phase interpolation run in integer
-// and FP32 arithmetic (positions and phases to ~1e-7 samples and cycles).
-struct DelayRec {
-    int I;
-    float phi, psi, dpsi;
-};
-
 struct GeoArgs {
-    const double *r;
-    const double *d;          // per-sample delays of the sky batch, [sky][stride]
-    const DelayRec *dr;       // FP32 form: the same as shift records
+    const double *d;          // FP64 form: per-sample delays of the sky batch, [sky][stride]
     int64_t d_stride;
+    const DF *r2;             // FP32 form: the ephemeris as double-float pairs
+    DF inv_dt2, f_off2;       // 1 / dt and f_off
+    DF phi0_turns, turn_dt;   // phi0 / 2 pi and Omega_r dt / 2 pi
+    float w_dt;               // Omega_r dt
     const void *xu;
     int64_t m_up;
     int U;
@@ -109,124 +72,182 @@ __global__ void __launch_bounds__(256) k_delays(const double *__restrict__ r,
     if (k < n) d[(int64_t)sl * stride + k] = delay_at(r, sky[s0 + sl], k);
 }
 
-// Shift records of every sample of skies [s0, s0 + gridDim.y): the delay
-// nhat . r_k and its reductions in double-float arithmetic (about 2^-46
-// relative: 1e-11 samples and 1e-9 cycles at the delays and offsets of a
-// search, against the 6e-8 of the FP32 results); d_{k+1} of the phase
-// increment comes from the next thread (the block's first thread evaluates
-// the one past the block).  The increment of the last sample is never used
-// (the interpolation segment index is <= n - 2).
-__global__ void __launch_bounds__(256) k_delays_split(const DF *__restrict__ r2,
-                                                      const SkyConst *__restrict__ sky, int64_t s0,
-                                                      int64_t n, int64_t stride, DF inv_dt, DF f_off,
-                                                      int phase, DelayRec *__restrict__ out) {
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int sl = blockIdx.y;
-    __shared__ DF dsh[257];
-    const float *nf = sky[s0 + sl].nf;
-    const DF nx{nf[0], nf[1]}, ny{nf[2], nf[3]}, nz{nf[4], nf[5]};
-    auto delay = [&](int64_t j) {
-        const DF *rj = r2 + 3 * j;
-        return df_add(df_add(df_mul(nx, rj[0]), df_mul(ny, rj[1])), df_mul(nz, rj[2]));
-    };
-    const DF dk = k < n ? delay(k) : DF{0.f, 0.f};
-    DelayRec o;
-    float phi;
-    o.I = (int)df_split_floor(df_mul(dk, inv_dt), &phi);
-    o.phi = phi;
-    o.psi = 0.f;
-    o.dpsi = 0.f;
-    if (phase) {   // uniform: no phase records for a band at zero offset
-        dsh[threadIdx.x] = dk;
-        if (threadIdx.x == 0) {
-            const int64_t kn = k + blockDim.x;
-            dsh[blockDim.x] = kn < n ? delay(kn) : DF{0.f, 0.f};
-        }
-        __syncthreads();
-        float psi;
-        df_split_floor(df_mul(f_off, dk), &psi);
-        o.psi = psi;
-        if (k + 1 < n) {
-            const DF dd = df_add(dsh[threadIdx.x + 1], df_neg(dk));
-            o.dpsi = (f_off.hi + f_off.lo) * (dd.hi + dd.lo);
-        }
-    }
-    if (k < n) out[(int64_t)sl * stride + k] = o;
+// FP32 form, one launch per sky batch: delay, detector time, a(t) and b(t), the
+// resampled and phase-demodulated series and the S sums of a tile of kGeo32
+// consecutive samples of one sky position.
+//
+// The delay n . r is evaluated in double-float arithmetic (about 2^-46 relative;
+// FP64 runs at 1/64 of the FP32 rate) at the tile's own samples, which only pick
+// the interpolation segments, and on the window of samples where those segments
+// lie, d/dt samples earlier and as long as the tile because the delay changes by
+// ~1e-4 per sample.  The window stays in shared memory: no delay records go
+// through memory, and the two dependent look-ups per sample are shared-memory
+// reads.  From d_j the detector-time inversion runs on d_j / dt = I + phi (I an exact
+// integer, phi in FP32) and the band-offset phase on f_off d_j mod 1 plus the FP32
+// increment, as before.  A segment outside the window (an ephemeris that moves
+// by more than the margin within a tile) is evaluated directly.
+// The hour angle is a rotation by the tile's reference angle (double-float, once
+// per tile) and the small angle from it (Taylor series), instead of a sincos.
+// Bound by instruction issue.  Measured at n = 86 164 per 64 positions, f_off != 0:
+// 121 -> 82 us (delay records through memory and one sincos per sample before).
+constexpr int kGeo32 = 1024;                 // samples per tile
+constexpr int kGeoThreads = 256, kGeoPer = kGeo32 / kGeoThreads;
+constexpr int kGeoMargin = 4;                // samples before the first segment
+constexpr int kGeoWin = kGeo32 + 12;         // window length
+
+__device__ __forceinline__ DF delay_df(const DF *__restrict__ r2, DF nx, DF ny, DF nz, int j) {
+    const DF *rj = r2 + 3 * j;
+    return df_dot3(nx, rj[0], ny, rj[1], nz, rj[2]);
 }
 
-__global__ void __launch_bounds__(256) k_geometry(GeoArgs g) {
-    __shared__ double sh[24];
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int sl = blockIdx.y;
-    float saa_f = 0.f, sbb_f = 0.f, sab_f = 0.f;
-    // the sky's constants in FP32, converted once per block
-    __shared__ float cf[12];
-    if (threadIdx.x < 12) {
-        const SkyConst &sc = g.sky[g.s0 + sl];
-        const int i = threadIdx.x;
-        cf[i] = i < 5 ? (float)sc.A[i] : i < 9 ? (float)sc.B[i - 5]
-              : i == 9 ? (float)(sc.alpha - g.phi0) : i == 10 ? (float)g.dt : 0.f;
+// Sums over the 32 lanes of the 16 values v[0 .. 15] at once: each step halves the
+// values a lane carries by trading the other half with lane ^ mask, 16 shuffles in
+// place of 80.  Value i ends in lanes with bits 4 .. 1 equal to i (low bit: either).
+__device__ __forceinline__ float warp_sum16(float *v) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int h = 8; h >= 1; h >>= 1) {
+        const bool up = (lane & (2 * h)) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const float keep = up ? v[i + h] : v[i], send = up ? v[i] : v[i + h];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * h);
+        }
+    }
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+__global__ void __launch_bounds__(kGeoThreads, 4) k_geometry(GeoArgs g) {
+    __shared__ DF win[kGeoWin];
+    __shared__ float cf[11];
+    __shared__ int s_js;
+    __shared__ float sums[3][kGeoThreads / 32 * kGeoPer];
+    const int n = (int)g.n, tid = threadIdx.x, sl = blockIdx.y;
+    const int k0 = blockIdx.x * kGeo32;
+    const SkyConst &sc = g.sky[g.s0 + sl];
+    const DF nx{sc.nf[0], sc.nf[1]}, ny{sc.nf[2], sc.nf[3]}, nz{sc.nf[4], sc.nf[5]};
+    const bool pow2 = g.dt_pow2 != 0;
+    auto in_samples = [&](DF d) {   // d / dt; a power of two scales both parts exactly
+        return pow2 ? DF{d.hi * g.inv_dt2.hi, d.lo * g.inv_dt2.hi} : df_mul(d, g.inv_dt2);
+    };
+    // segment start (before clamping) and fraction at the tile's own samples
+    int a0[kGeoPer];
+    float ph[kGeoPer];
+#pragma unroll
+    for (int i = 0; i < kGeoPer; ++i) {
+        const int k = min(k0 + tid + i * kGeoThreads, n - 1);
+        float phi;
+        a0[i] = k - (int)df_split_floor(in_samples(delay_df(g.r2, nx, ny, nz, k)), &phi);   // u0 = a0 - phi
+        ph[i] = phi;
+    }
+    if (tid == 0) s_js = min(max(a0[0] - 1 - kGeoMargin, -(kGeoWin - 4)), n - 4);
+    __syncthreads();
+    const int js = s_js;
+#pragma unroll
+    for (int i = 0; i < (kGeoWin + kGeoThreads - 1) / kGeoThreads; ++i) {
+        const int e = tid + i * kGeoThreads;
+        if (e < kGeoWin) win[e] = delay_df(g.r2, nx, ny, nz, min(max(js + e, 0), n - 1));
+    }
+    const int mc = js + kGeoWin / 2;   // reference sample of the hour angle
+    if (tid < 9) {
+        cf[tid] = tid < 5 ? (float)sc.A[tid] : (float)sc.B[tid - 5];
+    } else if (tid == 32) {
+        // h = alpha - phi0 - Omega_r dt mc, reduced in turns
+        float fr;
+        df_split_floor(df_add(df_add(DF{sc.nf[6], sc.nf[7]}, df_neg(g.phi0_turns)),
+                              df_neg(df_mul(g.turn_dt, DF{(float)mc, 0.f}))), &fr);
+        sincospif(2.f * fr, &cf[10], &cf[9]);
     }
     __syncthreads();
-    if (k < g.n) {
+    float sv[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) sv[i] = 0.f;
+#pragma unroll
+    for (int i = 0; i < kGeoPer; ++i) {
+        const int k = k0 + tid + i * kGeoThreads;
+        if (k >= n) break;
+        auto delay2 = [&](int j, DF &d0, DF &d1) {   // delays of samples j, j + 1
+            const int e = j - js;
+            if ((unsigned)e < (unsigned)(kGeoWin - 1)) {
+                d0 = win[e];
+                d1 = win[e + 1];
+            } else {
+                d0 = delay_df(g.r2, nx, ny, nz, j);
+                d1 = delay_df(g.r2, nx, ny, nz, j + 1);
+            }
+        };
         // detector time t of barycentric sample k, t = k dt - d(k dt - d(k dt)),
         // as u = t / dt = A - F1: A an exact integer, F1 an FP32 fraction
-        const int n = (int)g.n, kk = (int)k;
-        const DelayRec *dr = g.dr + (int64_t)sl * g.d_stride;
-        const DelayRec rk = dr[kk];
-        const int a0 = kk - rk.I;                       // u0 = a0 - phi_k
-        const int j0 = min(max(a0 - 1, 0), n - 2);
-        const float f0 = (float)(a0 - j0) - rk.phi;     // u0 - j0
-        const DelayRec p0 = dr[j0], p1 = dr[j0 + 1];
-        const float F1 = p0.phi + f0 * ((float)(p1.I - p0.I) + (p1.phi - p0.phi));
-        const int A = kk - p0.I;
+        const int j0 = min(max(a0[i] - 1, 0), n - 2);
+        const float f0 = (float)(a0[i] - j0) - ph[i];     // u0 - j0
+        DF d0, d1;
+        delay2(j0, d0, d1);
+        float phi0;
+        const int A = k - (int)df_split_floor(in_samples(d0), &phi0);
+        const float F1 = phi0 + f0 * (((d1.hi - d0.hi) + (d1.lo - d0.lo)) * g.inv_dt2.hi);
         const float fl1 = floorf(-F1);
         int j = A + (int)fl1;
         float f = -F1 - fl1;                            // u - j in [0, 1)
         const int jc = min(max(j, 0), n - 2);
         f += (float)(j - jc);
         j = jc;
-        const bool valid = F1 <= (float)A && F1 >= (float)(A - (n - 1));
-        // band-offset phase at t, cycles: psi_j + f dpsi_j (mod 1)
-        const DelayRec q0 = dr[j];
-        const float cyc = q0.psi + f * q0.dpsi;
-        const float frs = cyc - rintf(cyc);
-        // hour angle h = alpha - phi0 - Omega_r t (|h| < 20 rad, error ~1e-6 rad
-        // from t rounded to FP32)
-        const float uf = (float)A - F1;
-        const float hr = cf[9] - (float)kOmegaR * (uf * cf[10]);
-        float s1, c1;
-        sincosf(hr, &s1, &c1);
+        // Keys cubic (a = -1/2) at p = U u = U A - U F1 on the upsampled series; inside the
+        // window p lies in [0, U (n - 1)]
+        const float up = -(float)g.U * F1;
+        const float upf = floorf(up);
+        const int i0 = (int)((unsigned)g.U * (unsigned)A + (unsigned)(int)upf) - 1;
+        const bool valid = F1 <= (float)A && F1 >= (float)(A - (n - 1)) &&
+                           (unsigned)(i0 + 1) <= (unsigned)(g.U * (n - 1));
+        // hour angle: the reference rotated by -Omega_r dt (u - mc)
+        const float dl = g.w_dt * (F1 - (float)(A - mc));
+        float sd, cd;
+        if (fabsf(dl) <= 0.25f) {   // first terms left out: d^9/9! and d^8/8!, below 4e-10
+            const float q = dl * dl;
+            sd = dl * fmaf(q, fmaf(q, fmaf(q, -1.f / 5040.f, 1.f / 120.f), -1.f / 6.f), 1.f);
+            cd = fmaf(q, fmaf(q, fmaf(q, -1.f / 720.f, 1.f / 24.f), -0.5f), 1.f);
+        } else {
+            sincosf(dl, &sd, &cd);
+        }
+        const float c1 = cf[9] * cd - cf[10] * sd, s1 = cf[10] * cd + cf[9] * sd;
         const float c2 = c1 * c1 - s1 * s1, s2 = 2.f * s1 * c1;
         const float av = cf[0] * c2 + cf[1] * s2 + cf[2] * c1 + cf[3] * s1 + cf[4];
         const float bv = cf[5] * c2 + cf[6] * s2 + cf[7] * c1 + cf[8] * s1;
         float yr = 0.f, yi = 0.f;
         if (valid) {
-            // Keys cubic (a = -1/2) at p = U u = U A - U F1 on the upsampled series,
-            // periodic indexing (only tap -1 and taps >= U n wrap, a single step)
-            const float up = -(float)g.U * F1;
-            const float upf = floorf(up);
             const float mu = up - upf;
-            const int64_t i0 = (int64_t)g.U * A + (int64_t)upf - 1;
             const float w0 = ((-0.5f * mu + 1.f) * mu - 0.5f) * mu;
             const float w1 = (1.5f * mu - 2.5f) * mu * mu + 1.f;
             const float w2 = ((-1.5f * mu + 2.f) * mu + 0.5f) * mu;
             const float w3 = (0.5f * mu - 0.5f) * mu * mu;
             const float *xu = (const float *)g.xu;
+            const int m_up = (int)g.m_up;
             float x4[4];
+            if (i0 >= 0 && i0 + 3 < m_up) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int64_t v = i0 + q;
-                x4[q] = xu[v < 0 ? v + g.m_up : (v >= g.m_up ? v - g.m_up : v)];
+                for (int q = 0; q < 4; ++q) x4[q] = __ldg(xu + i0 + q);
+            } else {   // periodic: only tap -1 and taps >= U n wrap, a single step
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int v = i0 + q;
+                    x4[q] = __ldg(xu + (v < 0 ? v + m_up : (v >= m_up ? v - m_up : v)));
+                }
             }
             const float v = w0 * x4[0] + w1 * x4[1] + w2 * x4[2] + w3 * x4[3];
-            float sp, cp;
-            sincospif(2.f * frs, &sp, &cp);
-            yr = v * cp;
-            yi = -v * sp;
-            saa_f = av * av;
-            sbb_f = bv * bv;
-            sab_f = av * bv;
+            yr = v;
+            if (g.f_off2.hi != 0.f) {   // uniform: a band at zero offset has no phase
+                // band-offset phase at t, cycles: f_off d_j mod 1 + f f_off (d_{j+1} - d_j)
+                if (j != j0) delay2(j, d0, d1);
+                float psi;
+                df_split_floor(df_mul(g.f_off2, d0), &psi);
+                const float cyc = psi + f * (g.f_off2.hi * ((d1.hi - d0.hi) + (d1.lo - d0.lo)));
+                float sp, cp;
+                sincospif(2.f * (cyc - rintf(cyc)), &sp, &cp);
+                yr = v * cp;
+                yi = -v * sp;
+            }
+            sv[i] = av * av;
+            sv[4 + i] = bv * bv;
+            sv[8 + i] = av * bv;
         }
         float4 *w = (float4 *)g.w + (int64_t)sl * g.w_stride;
         w[k] = make_float4(yr * av, yi * av, yr * bv, yi * bv);
@@ -235,7 +256,16 @@ __global__ void __launch_bounds__(256) k_geometry(GeoArgs g) {
             g.dbg_a[k] = av; g.dbg_b[k] = bv; g.dbg_mask[k] = valid;
         }
     }
-    block_sum3_f(saa_f, sbb_f, sab_f, sh, g.partials + ((int64_t)sl * g.nblk + blockIdx.x) * 3);
+    static_assert(kGeoPer == 4, "twelve sums of a warp in the sixteen slots");
+    // S sums: each warp adds 32 terms in FP32 (relative error ~1e-7), the rest in FP64
+    const float ws = warp_sum16(sv);
+    const int lane = tid & 31, wp = tid >> 5, id = lane >> 1;
+    if (!(lane & 1) && id < 12) sums[id >> 2][4 * wp + (id & 3)] = ws;
+    __syncthreads();
+    if (wp < 3) {
+        const double t = warp_sum((double)sums[wp][lane]);
+        if (lane == 0) g.partials[((int64_t)sl * g.nblk + blockIdx.x) * 3 + wp] = t;
+    }
 }
 
 // FP64 form.  Bound by the FP64 units (1/64 of the FP32 rate), so it spends FP64
@@ -378,7 +408,8 @@ k_reduce_norms(const double *__restrict__ partials, int nblk, const double *__re
 
 inline unsigned blocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 // blocks of a geometry launch per sky position, each leaving one partial of the S sums
-inline int geo_blocks(int64_t n, bool fp32) { return (int)blocks(n, fp32 ? 256 : 256 * kGeo64); }
+static_assert(256 * kGeo64 == kGeo32, "both forms: 1024 samples a block");
+inline int geo_blocks(int64_t n) { return (int)blocks(n, kGeo32); }
 
 }  // namespace
 
@@ -387,9 +418,13 @@ int launch_geometry(const Plan &p, const BandDev &b, int64_t s0, int64_t ns, boo
                     void *w, double *dbg_y, double *dbg_a, double *dbg_b, uint8_t *dbg_mask,
                     cudaStream_t s) {
     GeoArgs g;
-    g.r = b.r;
     g.d = p.dbuf;
-    g.dr = reinterpret_cast<const DelayRec *>(p.dbuf);
+    g.r2 = static_cast<const DF *>(b.r2);
+    g.f_off2 = df_from_double(b.f_off);
+    g.inv_dt2 = df_from_double(1.0 / b.dt);
+    g.phi0_turns = df_from_double(b.phi0 / kTwoPi);
+    g.turn_dt = df_from_double(kOmegaR * b.dt / kTwoPi);
+    g.w_dt = (float)(kOmegaR * b.dt);
     g.d_stride = p.n_max;
     g.xu = b.xu;
     g.U = p.desc.upsample;
@@ -407,17 +442,15 @@ int launch_geometry(const Plan &p, const BandDev &b, int64_t s0, int64_t ns, boo
     g.w = w;
     g.w_stride = p.w_stride;
     g.partials = p.partials;
-    g.nblk = geo_blocks(b.n, fp32);
+    g.nblk = geo_blocks(b.n);
     g.dbg_y = dbg_y;
     g.dbg_a = dbg_a;
     g.dbg_b = dbg_b;
     g.dbg_mask = dbg_mask;
     dim3 grid(g.nblk, (unsigned)ns);
     if (fp32) {
-        k_delays_split<<<grid, 256, 0, s>>>(static_cast<const DF *>(b.r2), p.sky, s0, b.n, p.n_max,
-                                            df_from_double(g.inv_dt), df_from_double(b.f_off),
-                                            b.f_off != 0.0 ? 1 : 0, reinterpret_cast<DelayRec *>(p.dbuf));
-        k_geometry<<<grid, 256, 0, s>>>(g);
+        k_geometry<<<grid, kGeoThreads, 0, s>>>(g);
+        return 1;
     } else {
         k_delays<<<dim3(blocks(b.n, 256), (unsigned)ns), 256, 0, s>>>(b.r, p.sky, s0, b.n, p.n_max, p.dbuf);
         k_geometry64<<<grid, 256, 0, s>>>(g);
@@ -427,7 +460,7 @@ int launch_geometry(const Plan &p, const BandDev &b, int64_t s0, int64_t ns, boo
 
 int launch_reduce_norms(const Plan &p, const BandDev &b, int64_t ns, double *norm, cudaStream_t s) {
     k_reduce_norms<<<(unsigned)ns, 32 * (kNormWarps + 1), 0, s>>>(
-        p.partials, geo_blocks(b.n, p.desc.form == FSTAT_FP32_BATCHED), p.sigma_parts, b.n, p.desc.sigma2, p.S, norm,
+        p.partials, geo_blocks(b.n), p.sigma_parts, b.n, p.desc.sigma2, p.S, norm,
         p.desc.statistic == FSTAT_F_FULL ? 1 : 0);
     return 1;
 }

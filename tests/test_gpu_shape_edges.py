@@ -3,6 +3,7 @@ and just beyond the lengths where a kernel skips more of the zero padding, the s
 longest transforms of each engine, and grids whose last sky batch and last launch are ragged.
 Tolerances as in test_gpu_parity: |F - F_ref| / max(F_ref, 2) <= 1e-10 (FP64), 1e-4 (FP32).
 """
+import math
 import os
 
 import numpy as np
@@ -95,3 +96,31 @@ def test_upsample(fs, n, U):
 ])
 def test_fp32_1024_point_rows(fs, n, n_fft, n_sky, n_spin, kw):
     _check(fs, fs.FP32_BATCHED, n, n_fft, n_sky, n_spin, **kw)
+
+
+@pytest.mark.parametrize("n,dt,scale", [(1023, 2.0, 1.0), (1024, 2.0, 1.0), (1025, 0.5, 1.0), (3000, 0.3, 1.0), (5000, 60.0, 1.0),
+                                        (2049, 0.01, 1.0), (3000, 2.0, 8.0)])
+def test_fp32_sky_stage_tiles(fs, n, dt, scale):
+    """The per-sky stage around its 1024-sample tiles: sampling intervals that are no power of
+    two, long ones (the hour angle turns far within a tile), short ones (the delay is many tiles
+    long and most samples fall outside the window), and an orbit eight times too large, whose
+    delay drifts past the shared window's margin within a tile.  Tolerances of
+    test_sky_stage_matches_oracle; S on the scale of its own sum."""
+    nf = max(4096, S.n_fft_auto(n))
+    one = np.array([0.7]), np.array([0.4]), np.array([0.0])
+    b = S.make_band(n, dt, 5 + n, 1.0, *one, [], f_off=100.5, n_fft=nf)
+    b.r = b.r * scale + (0.02 * np.sin(np.arange(n) * 0.7)[:, None] if scale > 1 else 0.0)
+    prm = O.params(S.LAT_DEFAULT, S.GAMMA_DEFAULT, 2, 0.0)
+    xu = O.upsample(b.x, 2)
+    with fs.Plan([b], *one, 20.0, lat=S.LAT_DEFAULT, gamma=S.GAMMA_DEFAULT, form=fs.FP32_BATCHED) as p:
+        g = p.debug_sky(0, 0, n)
+    r = O.sky_prepare(b, prm, xu, float(one[0][0]), float(one[1][0]))
+    assert np.array_equal(g["mask"], r["mask"])
+    assert np.max(np.abs(g["a"] - r["a"])) < 2e-6 and np.max(np.abs(g["b"] - r["b"])) < 2e-6
+    # phase: 2 pi (FP32 rounding of the position, 1.2e-7 samples, times f_off d' dt plus 1e-7 cycles) and
+    # the interpolated series' slope (pi per sample) times the position's error, against 2e-5
+    assert np.max(np.abs(g["y"] - r["y"])) / max(1.0, np.max(np.abs(r["y"]))) < 2e-5
+    m = r["mask"]
+    if m.any():
+        sc = np.array([r["S"][0], r["S"][1], math.sqrt(r["S"][0] * r["S"][1])])
+        assert np.max(np.abs(g["S"] - r["S"]) / sc) < 1e-5
