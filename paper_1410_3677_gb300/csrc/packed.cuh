@@ -145,5 +145,35 @@ __device__ __forceinline__ void dft16(PC *x) {
     }
 }
 
+// 8-point DFT: 4-point DFTs of the even and odd inputs, twiddles W8^k, sums and
+// differences.  LOWER: only the outputs 0 .. 3.
+template <bool LOWER = false>
+__device__ __forceinline__ void dft8(PC *x) {
+    PC e0 = x[0], e1 = x[2], e2 = x[4], e3 = x[6], o0 = x[1], o1 = x[3], o2 = x[5], o3 = x[7];
+    dft4(e0, e1, e2, e3);
+    dft4(o0, o1, o2, o3);
+    o1 = mul_w16(o1, 2);
+    o3 = mul_w16(o3, 6);
+    x[0] = add(e0, o0);
+    x[1] = add(e1, o1);
+    x[2] = add_rot<3>(e2, o2);   // W8^2 = -i
+    x[3] = add(e3, o3);
+    if constexpr (!LOWER) {
+        x[4] = sub(e0, o0);
+        x[5] = sub(e1, o1);
+        x[6] = add_rot<1>(e2, o2);
+        x[7] = sub(e3, o3);
+    }
+}
+
+// R-point DFT, R = 4, 8 or 16; LOWER: the first half of the outputs only.
+template <int R, bool LOWER = false>
+__device__ __forceinline__ void dft(PC *x) {
+    static_assert(R == 4 || R == 8 || R == 16, "packed radices");
+    if constexpr (R == 16) dft16<16, LOWER>(x);
+    else if constexpr (R == 8) dft8<LOWER>(x);
+    else dft4<0, LOWER>(x[0], x[1], x[2], x[3]);
+}
+
 }  // namespace pk
 }  // namespace fstat

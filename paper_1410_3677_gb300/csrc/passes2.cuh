@@ -223,6 +223,19 @@ struct ScratchLoad2 {
     }
 };
 
+// Wait for an mbarrier's first phase, bounded: past 1 s the error word is set, past 2 s
+// the wait is given up (reported; the results are discarded).
+__device__ __forceinline__ void mbar_wait_bounded(uint64_t *bar, uint32_t *err) {
+    if (ptx::mbar_try_wait(bar, 0)) return;
+    const uint64_t t0 = ptx::globaltimer_ns();
+    bool late = false;
+    while (!ptx::mbar_try_wait(bar, 0)) {
+        const uint64_t dt = ptx::globaltimer_ns() - t0;
+        if (!late && dt > 1000000000ull) { atomicExch(err, 1u); late = true; }
+        if (dt > 2000000000ull) break;
+    }
+}
+
 // Pass 2 input staged by the TMA unit: the tile's rows are one contiguous run of
 // 2 F N1 complex floats in scratch (both transforms interleaved); one thread
 // copies it into the CTA's exchange area with a bulk copy completing on an
@@ -273,17 +286,7 @@ struct ScratchLoadTMA {
             ptx::bulk_g2s(const_cast<float2 *>(rows), src, bytes, bar);
         }
     }
-    // bounded wait for the copy
-    __device__ __forceinline__ void wait() const {
-        if (ptx::mbar_try_wait(bar, 0)) return;
-        const uint64_t t0 = ptx::globaltimer_ns();
-        bool late = false;
-        while (!ptx::mbar_try_wait(bar, 0)) {
-            const uint64_t dt = ptx::globaltimer_ns() - t0;
-            if (!late && dt > 1000000000ull) { atomicExch(err, 1u); late = true; }
-            if (dt > 2000000000ull) break;   // reported above; results are discarded
-        }
-    }
+    __device__ __forceinline__ void wait() const { mbar_wait_bounded(bar, err); }
     template <int R, int JPF>
     __device__ __forceinline__ void load(const eng2::Job &q, float *re, float *im) const {
         // the twiddle factors load while the bulk copies are in flight
@@ -488,15 +491,7 @@ struct ScratchLoadIBTMA {
     __device__ __forceinline__ void load(const eng2::Job &q, float *re, float *im) const {
         const int l2 = (l2_0 + q.f) & (C::N2 - 1);
         const float2 w0 = tw.wn(l2 * q.j), st = tw.wn(l2 * JPF);
-        if (!ptx::mbar_try_wait(bar, 0)) {
-            const uint64_t t0 = ptx::globaltimer_ns();
-            bool late = false;
-            while (!ptx::mbar_try_wait(bar, 0)) {
-                const uint64_t dt = ptx::globaltimer_ns() - t0;
-                if (!late && dt > 1000000000ull) { atomicExch(err, 1u); late = true; }
-                if (dt > 2000000000ull) break;   // reported above; results are discarded
-            }
-        }
+        mbar_wait_bounded(bar, err);
         const float2 *row = rows + 2 * (q.f * C::N1 + q.j) + q.t;
 #pragma unroll
         for (int r = 0; r < R; ++r) {

@@ -1,6 +1,6 @@
 // The FP32 search passes in packed arithmetic (packed.cuh) for passes of length
 // 512: both passes at N_fft = 2^18 (N1 = N2 = 512, the two-sidereal-day
-// segments), the rows (pass 2) at 2^19; the 256-point rows of 2^16 and 2^17; and
+// segments), the rows (pass 2) at 2^19; the shorter rows of 2^12 .. 2^17; and
 // the 1024-point rows of 2^20.  Same four-step split, scratch layout, tiles and
 // launch shapes as the second engine's passes (passes2.cuh); what changes is how
 // a thread's 32 elements are transformed:
@@ -171,13 +171,13 @@ k_pass1h(SearchLoad2<Cfg2<LOGN, 1>> ld, ScratchStore2<Cfg2<LOGN, 1>> st, const f
 // 6.5e-7 -> 3.2e-7.
 constexpr int kRowTw = 16;
 
-template <class C, int TILES_PER_ENTRY = 1>
+template <class C>
 struct RowsTMA : ScratchLoadTMA<C> {
-    static constexpr int ENTRIES = C::F / TILES_PER_ENTRY;   // table rows per tile
+    static constexpr int ENTRIES = C::F;                     // table rows per tile
     static constexpr uint32_t TW_BYTES = ENTRIES * kRowTw * sizeof(float4);
     static constexpr uint32_t ROW_BYTES = (uint32_t)(2 * C::F * C::N1 * sizeof(float2));
     static constexpr size_t SMEM = ROW_BYTES + TW_BYTES + 16;   // rows, twiddles, mbarrier
-    const float4 *row_tw;   // [row or row pair][16]
+    const float4 *row_tw;   // [row][16]
     const float4 *tws;      // in shared memory
     __device__ void init(int tile, int64_t cell, int64_t slot) {
         ScratchLoadTMA<C>::init(tile, cell, slot);
@@ -218,10 +218,10 @@ __host__ __device__ constexpr int epi_half() { return (LOWER ? 8 : 16) / 2; }
 // Lanes 2j (F_a) and 2j + 1 (F_b) hold the same bins; the a lane evaluates F on
 // the outputs p < H, the b lane on p >= H, each taking the partner's values for
 // its half with one shuffle per value.  Output u of this lane's half, pair member
-// e, is bin bin0 + u step_u + e step_e.
-template <class C, bool LOWER>
-__device__ __forceinline__ void epilogue(const SearchEpi2<C, LOWER> &ep, int t, int bin0, int step_u, int step_e,
-                                         const PC *Y) {
+// e, is bin bin0 + off(u) + e step_e; lanes with own = false register nothing.
+template <class C, bool LOWER, class Off>
+__device__ __forceinline__ void epilogue(const SearchEpi2<C, LOWER> &ep, int t, int bin0, Off off, int step_e,
+                                         const PC *Y, bool own = true) {
     constexpr int H = epi_half<LOWER>();
     const int lane = (int)threadIdx.x & 31;
     const bool full = ep.nab != 0.f;
@@ -262,9 +262,9 @@ __device__ __forceinline__ void epilogue(const SearchEpi2<C, LOWER> &ep, int t, 
     for (int u = 0; u < H; ++u)
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-            const int bin = bin0 + step_u * u + step_e * e;
+            const int bin = bin0 + off(u) + step_e * e;
             const float f = e ? Fv[u].y : Fv[u].x;
-            pr[2 * u + e] = ((unsigned)(bin - lo) <= span) && (f > ep.thr_half);
+            pr[2 * u + e] = own && ((unsigned)(bin - lo) <= span) && (f > ep.thr_half);
             any |= pr[2 * u + e];
         }
     if (!__any_sync(0xffffffffu, any)) return;
@@ -283,7 +283,7 @@ __device__ __forceinline__ void epilogue(const SearchEpi2<C, LOWER> &ep, int t, 
                     const unsigned long long idx = b0 + __popc(m & ((1u << lane) - 1u));
                     const float f = e ? Fv[u].y : Fv[u].x;
                     if (idx < ep.cap)
-                        ep.out[idx] = CandRecord{ep.cell, (uint32_t)(bin0 + step_u * u + step_e * e), (double)f};
+                        ep.out[idx] = CandRecord{ep.cell, (uint32_t)(bin0 + off(u) + step_e * e), (double)f};
                 }
             }
         }
@@ -352,68 +352,169 @@ k_pass2p(RowsTMA<Cfg2<LOGN, 2, TS>> ld, SearchEpi2<Cfg2<LOGN, 2, TS>, LOWER> ep,
     pk::dft16<16, LOWER>(Q);
     // bins: job 2j + e, output p = u + t H: l1 = 2j + e + 32 p, bin = N2 l1 + l2
     constexpr int H = epi_half<LOWER>();
-    epilogue<C, LOWER>(ep, t, C::N2 * (2 * j + kR0 * t * H) + l2, C::N2 * kR0, C::N2, Q);
+    epilogue<C, LOWER>(ep, t, C::N2 * (2 * j + kR0 * t * H) + l2, [](int u) { return C::N2 * kR0 * u; }, C::N2, Q);
 }
 
-// --------------------------------------------------------------------- pass 2, 256-point rows
-// The rows of N_fft = 2^16 and 2^17 (N1 = 256 = 16 x 16) with two adjacent rows
-// per warp and CTA, the rows packed in pairs: every operation is the same for
-// rows l2 and l2 + 1 except the four-step twiddle, which comes as a pair.
-// Lane 2j + t (t the transform) takes the elements k1 = j + 16 m of both rows;
-// stage 0 is a packed 16-point DFT over m (after the twiddle W_N^{l2 k1}),
-// stage 1 for job q the twiddle W_256^{j q} and a packed 16-point DFT over j,
-// giving l1 = q + 16 p.  The exchange lies over the warp's staged 8 KiB.
-template <int LOGN, bool LOWER>
-__global__ void __launch_bounds__(32, 24)
-k_pass2r(RowsTMA<Cfg2<LOGN, 2, 32>, 2> ld, SearchEpi2<Cfg2<LOGN, 2, 32>, LOWER> ep,
-         const float2 *__restrict__ w256) {
+// --------------------------------------------------------------------- pass 2, short rows
+// The rows of N1 = 64, 128 or 256 points (2^12 .. 2^17) in adjacent pairs (l2, l2 + 1)
+// packed in pairs: every operation is the same for the two rows except the four-step
+// twiddle, which comes as a pair.  A warp takes G = 256 / N1 row pairs (1024 complex
+// values of both transforms); lane t + 2 (g + G j) holds butterfly j of transform t of
+// pair g: the 16 elements k1 = j + R1 m, R1 = N1 / 16.  Stage 0 is a packed 16-point DFT
+// over m, stage 1 for each of G jobs q = j + R1 i the twiddle W_N1^{rq} and a packed
+// R1-point DFT over the butterflies r, giving l1 = q + 16 p.  The exchange lies over the
+// warp's staged rows (8 KiB) and no warp waits for another.
+//
+// IB, the interbinning form (transforms of N = n_fft / 2 points): bin 2k is X(k), bin
+// 2k + 1 (pi/4)(X(k) - X(k + 1)).  The neighbour of a pair's first row is its second, that
+// of the second the next pair's first row, traded through shared memory; the last pair of
+// a tile only serves as a neighbour, so tiles advance by one pair less than they hold.
+// After the last row comes row 0 at l1 + 1; where only the outputs l1 < N1/2 are formed
+// (LOWER), its X(N/2), the sum of stage-1 inputs with alternating signs, is formed aside.
+// Bound by issue and latency like the 512-point rows.  Measured, us per 2^18 points of both
+// transforms, against the scalar two-stage pass: 64-point rows 1.55 -> 0.79, 128-point
+// 1.08 -> 0.66; interbinning (per 2^18 bins) 64-point 1.12 -> 0.64, 128-point 0.76 -> 0.50,
+// 256-point 0.636 -> 0.492.
+template <int LOGN, int W>
+struct RowGeom {
+    static constexpr int N1 = 1 << (LOGN / 2), N2 = 1 << (LOGN - LOGN / 2), NP = N2 / 2;
+    static constexpr int R1 = N1 / 16, G = 256 / N1;
+    static constexpr int PAIRS = W * G;                       // row pairs per tile
+    // complex floats between a warp's staged pairs: the padding puts the lanes of the
+    // different pairs in different banks
+    static constexpr int PAIR_LD = 4 * N1 + (G == 2 ? 8 : G == 4 ? 4 : 0);
+    static constexpr uint32_t PAIR_BYTES = 4 * N1 * sizeof(float2), TW_BYTES = kRowTw * sizeof(float4);
+    static constexpr size_t WARP_BYTES = (size_t)G * PAIR_LD * sizeof(float2);
+    static constexpr size_t SMEM = W * WARP_BYTES + PAIRS * TW_BYTES + 8 * W;
+    static constexpr int STEP = PAIRS >= NP ? NP : PAIRS > 1 ? PAIRS - 1 : 1;   // pairs emitted per interbinning tile
+    static constexpr int TILES_IB = (NP + STEP - 1) / STEP, TILES = NP / PAIRS;
+    static_assert(N1 >= 64 && N1 <= 256, "short rows");
+};
+
+template <int LOGN, bool LOWER, bool IB, int W>
+__global__ void __launch_bounds__(32 * W, 24 / W)
+k_pass2rows(const float2 *__restrict__ scratch, InterTw<LOGN / 2> tw, const float4 *__restrict__ row_tw,
+            const float2 *__restrict__ s1, uint32_t *err, SearchEpi2<Cfg2<LOGN, 2, 32>, LOWER> ep) {
     using C = Cfg2<LOGN, 2, 32>;
-    static_assert(C::M == 256 && C::F == 2 && C::THREADS == 32, "256-point rows, two per warp");
-    ld.prefetch_ahead();
-    ld.init(blockIdx.x, blockIdx.y, blockIdx.y);
-    const int lane = (int)threadIdx.x & 31;
-    ep.init(blockIdx.x, blockIdx.y, blockIdx.y);
-    ld.stage();
-    const int t = lane & 1, j = lane >> 1;
-    const int l2 = ld.l2_0;   // rows l2 and l2 + 1
-    // four-step factors of the two rows: T_0 = W^{l2 j}; the pairs W^{16 l2 m} come with them
-    const float2 wa = ld.tw.wn(l2 * j), wb = ld.tw.wn((l2 + 1) * j);
-    const PC T = {make_float2(wa.x, wb.x), make_float2(wa.y, wb.y)};
-    ld.wait();
-    PC P[16];
-    {
-        const float2 *ra = ld.rows + 2 * j + t, *rb = ra + 2 * C::N1;   // element k1 at r[2 k1]
+    using Q = RowGeom<LOGN, W>;
+    constexpr int N1 = Q::N1, N2 = Q::N2, R1 = Q::R1, G = Q::G;
+    unsigned char *sm = eng2::dyn_smem();
+    const int w = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+    const int t = lane & 1, g = (lane >> 1) & (G - 1), j = lane / (2 * G);
+    const int pair0 = blockIdx.x * (IB ? Q::STEP : Q::PAIRS) + w * G;   // the warp's first pair
+    float2 *stage = reinterpret_cast<float2 *>(sm + w * Q::WARP_BYTES);
+    float4 *tws = reinterpret_cast<float4 *>(sm + W * Q::WARP_BYTES) + w * G * kRowTw;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + W * Q::WARP_BYTES + Q::PAIRS * Q::TW_BYTES) + w;
+    if (lane == 0) {
+        ptx::mbar_init(bar, 1);
+        ptx::fence_mbar_init();
+        ptx::mbar_arrive_expect_tx(bar, G * (Q::PAIR_BYTES + Q::TW_BYTES));
+        const float2 *src = scratch + (int64_t)blockIdx.y * 2 * C::N;
 #pragma unroll
-        for (int m = 0; m < 16; ++m) {
-            const float2 a = ra[2 * 16 * m], b = rb[2 * 16 * m];
-            P[m] = pk::cmul({make_float2(a.x, b.x), make_float2(a.y, b.y)}, m ? pk::cmul(T, ld.tw_m(0, m)) : T);
+        for (int i = 0; i < G; ++i) {
+            const int pr = (pair0 + i) & (Q::NP - 1);   // past the last row come the first ones
+            ptx::bulk_g2s(stage + i * Q::PAIR_LD, src + (int64_t)pr * 4 * N1, Q::PAIR_BYTES, bar);
+            ptx::bulk_g2s(tws + i * kRowTw, row_tw + pr * kRowTw, Q::TW_BYTES, bar);
         }
     }
-    pk::dft16<16>(P);   // P[k] = Z_j[k] of both rows
-    __syncwarp();       // the staged rows have been read: the exchange may overwrite them
-    float4 *ex = reinterpret_cast<float4 *>(eng2::dyn_smem()) + t * 256;
-    const int jx = j ^ (4 * t);
-#pragma unroll
-    for (int k = 0; k < 16; ++k) ex[k * 16 + (jx ^ k)] = make_float4(P[k].re.x, P[k].re.y, P[k].im.x, P[k].im.y);
     __syncwarp();
-    // stage 1, job q = j: the butterflies r of output q, twiddled by W_256^{r q}
-    const int q = j;
-    PC Q[16];
+    ep.init(0, blockIdx.y, blockIdx.y);
+    const int P = pair0 + g, l2 = 2 * (P & (Q::NP - 1));   // rows l2 and l2 + 1
+    // four-step factors of the two rows: T_0 = W^{l2 j}; the pairs W^{R1 l2 m} come with them
+    const float2 wa = tw.wn(l2 * j), wb = tw.wn((l2 + 1) * j);
+    const PC T = {make_float2(wa.x, wb.x), make_float2(wa.y, wb.y)};
+    mbar_wait_bounded(bar, err);
+    PC Pm[16];
+    {
+        const float2 *ra = stage + g * Q::PAIR_LD + 2 * j + t, *rb = ra + 2 * N1;   // element k1 at r[2 k1]
+        const float4 *tp = tws + g * kRowTw;
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
-        const float4 v = ex[q * 16 + (r ^ jx)];
-        Q[r] = {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+        for (int m = 0; m < 16; ++m) {
+            const float2 a = ra[2 * R1 * m], b = rb[2 * R1 * m];
+            PC F = T;
+            if (m) {
+                const float4 v = tp[m];
+                F = pk::cmul(T, PC{make_float2(v.x, v.y), make_float2(v.z, v.w)});
+            }
+            Pm[m] = pk::cmul({make_float2(a.x, b.x), make_float2(a.y, b.y)}, F);
+        }
     }
+    pk::dft16<16>(Pm);   // output k of butterfly j, both rows
+    __syncwarp();        // the staged rows have been read: the exchange may overwrite them
+    // element (output k, butterfly j) of (t, g) at word (k R1 + j) ^ X(k) of its N1 words;
+    // X sends the 8 lanes of a quarter-warp to 8 different 16-byte bank groups, storing
+    // (fixed k) and loading (fixed r)
+    constexpr int JL = 4 / G;   // butterflies per quarter-warp
+    float4 *ex = reinterpret_cast<float4 *>(stage) + (t * G + g) * N1;
+    const int x0 = (t * G + g) * JL;
 #pragma unroll
-    for (int r = 1; r < 16; ++r) {
-        const float2 w = __ldg(w256 + ((r * q) & 255));
-        Q[r] = {pk::pfma(Q[r].re, pk::bc(w.x), pk::pmul(Q[r].im, pk::bc(-w.y))),
-                pk::pfma(Q[r].re, pk::bc(w.y), pk::pmul(Q[r].im, pk::bc(w.x)))};
+    for (int k = 0; k < 16; ++k)
+        ex[(k * R1 + j) ^ (x0 ^ (k & (JL - 1)))] = make_float4(Pm[k].re.x, Pm[k].re.y, Pm[k].im.x, Pm[k].im.y);
+    __syncwarp();
+    constexpr int HR = LOWER ? R1 / 2 : R1;   // outputs kept per job
+    PC Y[G * HR];
+    PC top = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};   // IB, LOWER: X(N/2) of job 0
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+        const int q = j + R1 * i;
+        PC z[R1];
+#pragma unroll
+        for (int r = 0; r < R1; ++r) {
+            const float4 v = ex[(q * R1 + r) ^ (x0 ^ (q & (JL - 1)))];
+            z[r] = {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+        }
+#pragma unroll
+        for (int r = 1; r < R1; ++r) {
+            const float2 e = __ldg(s1 + (N1 == 64 ? ((r * q) & 63) : r * 16 + q));   // W_N1^{rq}
+            z[r] = {pk::pfma(z[r].re, pk::bc(e.x), pk::pmul(z[r].im, pk::bc(-e.y))),
+                    pk::pfma(z[r].re, pk::bc(e.y), pk::pmul(z[r].im, pk::bc(e.x)))};
+        }
+        if (IB && LOWER && i == 0) {
+            top = z[0];
+#pragma unroll
+            for (int r = 1; r < R1; ++r) top = r & 1 ? pk::sub(top, z[r]) : pk::add(top, z[r]);
+        }
+        pk::dft<R1, LOWER>(z);
+#pragma unroll
+        for (int p = 0; p < HR; ++p) Y[i * HR + p] = z[p];   // l1 = q + 16 p
     }
-    pk::dft16<16, LOWER>(Q);   // Y[q + 16 p], p < 8 (LOWER) or 16
-    // bins: output p = u + t H of job q for row l2 + e: l1 = q + 16 p, bin = N2 l1 + l2 + e
+    // output v = i HR + p: l1 = j + R1 i + 16 p; the b lane's half starts TO further on
     constexpr int H = epi_half<LOWER>();
-    epilogue<C, LOWER>(ep, t, C::N2 * (q + 16 * t * H) + l2, C::N2 * 16, 1, Q);
+    constexpr int TO = G == 1 ? 16 * H : R1 * G / 2;
+    auto l1_of = [](int v) { return R1 * (v / HR) + 16 * (v % HR); };
+    const int bin0 = N2 * (j + t * TO) + l2;
+    if constexpr (!IB) {
+        epilogue<C, LOWER>(ep, t, bin0, [&](int u) { return N2 * l1_of(u); }, 1, Y);
+    } else {
+        const int pl = w * G + g;                                   // pair within the tile
+        const bool own = pl < Q::STEP && P < Q::NP;
+        auto off2 = [&](int u) { return 2 * N2 * l1_of(u); };
+        epilogue<C, LOWER>(ep, t, 2 * bin0, off2, 2, Y, own);      // even bins
+        __syncthreads();                                            // every exchange has been read
+        constexpr int LD = (LOWER ? N1 / 2 : N1) + 8;
+        float2 *nb = reinterpret_cast<float2 *>(sm);                // [pair][t][LD]: first rows
+        static_assert(Q::PAIRS * 2 * LD * sizeof(float2) <= W * Q::WARP_BYTES, "neighbours fit the staged rows");
+#pragma unroll
+        for (int v = 0; v < G * HR; ++v)
+            nb[(2 * pl + t) * LD + j + l1_of(v)] = make_float2(Y[v].re.x, Y[v].im.x);
+        if (LOWER && j == 0) nb[(2 * pl + t) * LD + N1 / 2] = make_float2(top.re.x, top.im.x);
+        __syncthreads();
+        const int pn = pl + 1 < Q::PAIRS ? pl + 1 : 0;
+        const bool wrap = P + 1 >= Q::NP;                           // the next row is row 0, at l1 + 1
+#pragma unroll
+        for (int v = 0; v < G * HR; ++v) {
+            int l1 = j + l1_of(v) + (wrap ? 1 : 0);
+            if constexpr (!LOWER) l1 &= N1 - 1;
+            const float2 n = nb[(2 * pn + t) * LD + l1];
+            Y[v] = {make_float2(Y[v].re.x - Y[v].re.y, Y[v].re.y - n.x),
+                    make_float2(Y[v].im.x - Y[v].im.y, Y[v].im.y - n.y)};
+        }
+        constexpr float Q2 = 0.61685027506808491f;                 // (pi / 4)^2
+        ep.na *= Q2;
+        ep.nb *= Q2;
+        ep.nab *= Q2;
+        epilogue<C, LOWER>(ep, t, 2 * bin0 + 1, off2, 2, Y, own);  // odd bins
+    }
 }
 
 // --------------------------------------------------------------------- pass 2, 1024-point rows
@@ -482,7 +583,7 @@ k_pass2q(RowsTMA<Cfg2<LOGN, 2, 64>> ld, SearchEpi2<Cfg2<LOGN, 2, 64>, LOWER> ep,
     }
     pk::dft16<16, LOWER>(Q);   // Q[k] = (Y_2k, Y_2k+1): l1 = q + 32 (2k + e)
     constexpr int H = epi_half<LOWER>();
-    epilogue<C, LOWER>(ep, t, C::N2 * (q + 64 * t * H) + l2, C::N2 * 64, C::N2 * 32, Q);
+    epilogue<C, LOWER>(ep, t, C::N2 * (q + 64 * t * H) + l2, [](int u) { return C::N2 * 64 * u; }, C::N2 * 32, Q);
 }
 
 }  // namespace p3

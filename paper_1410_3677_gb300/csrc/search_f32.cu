@@ -60,6 +60,24 @@ void launch_pass2p(const Plan &p, int band_idx, const BandDev &b, int64_t s0, in
     k2<<<dim3(D2::TILES, (unsigned)nc), D2::THREADS, smem2, s>>>(lt, ep, tw->p512_f);
 }
 
+// Short rows (64 .. 256 points) in packed pairs, zero-padded or interbinning.
+bool rows_packed(const Plan &p) { return p.packed >= 1 && p.tma && p.p2_threads != 256 && p.p2_rows; }
+
+template <int LOGN, bool LOWER, bool IB, int W>
+void launch_rows(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_t c0, int64_t nc, cudaStream_t s,
+                 const CellBufs &cb, const TwiddleSet *tw) {
+    using Q = p3::RowGeom<LOGN, W>;
+    const auto ep = make_epi<LOGN, LOWER, 32>(p, band_idx, b, c0, s0, cb);
+    auto k2 = p3::k_pass2rows<LOGN, LOWER, IB, W>;
+    static bool attr = false;
+    if (!attr) { set_smem(k2, Q::SMEM); attr = true; }
+    // stage-1 twiddles [r][q], q < 16; the 64-point rows' table is in another order, they take W_64^m
+    const float *s1 = Q::N1 == 64 ? tw->in1_f : tw->s1_f;
+    k2<<<dim3(IB ? Q::TILES_IB : Q::TILES, (unsigned)nc), 32 * W, Q::SMEM, s>>>(
+        reinterpret_cast<const float2 *>(cb.scratch), InterTw<LOGN / 2>{tw->lo_f, tw->hi_f}, tw->row_tw,
+        reinterpret_cast<const float2 *>(s1), p.qerr, ep);
+}
+
 template <int LOGN, bool LOWER>
 int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_t c0, int64_t nc,
                cudaStream_t s, cudaEvent_t mid, const CellBufs &cb, const SearchLoad2<Cfg2<LOGN, 1>> &ld1,
@@ -119,22 +137,9 @@ int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_
         k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, C1::SMEM, s>>>(ld1, st1, tw->s2_f);
     }
     if (mid) record_timing_event(mid, s);
-    if constexpr (LOGN == 16 || LOGN == 17) {   // 256-point rows: two per warp, packed
-        if (p.packed >= 1 && p.tma && p.p2_threads != 256 && p.p2_rows) {
-            using D2 = Cfg2<LOGN, 2, 32>;
-            p3::RowsTMA<D2, 2> lt{};
-            lt.scratch = ld2.scratch;
-            lt.tw = ld2.tw;
-            lt.pf_dist = 0;
-            lt.err = p.qerr;
-            lt.row_tw = tw->row_tw;
-            const auto ep = make_epi<LOGN, LOWER, 32>(p, band_idx, b, c0, s0, cb);
-            auto k2 = p3::k_pass2r<LOGN, LOWER>;
-            constexpr size_t smem2 = p3::RowsTMA<D2, 2>::SMEM;
-            static bool attr2r = false;
-            if (!attr2r) { set_smem(k2, smem2); attr2r = true; }
-            k2<<<dim3(D2::TILES, (unsigned)nc), D2::THREADS, smem2, s>>>(
-                lt, ep, reinterpret_cast<const float2 *>(tw->in1_f));
+    if constexpr (LOGN <= 17) {   // rows of 64 .. 256 points: packed in pairs
+        if (rows_packed(p)) {
+            launch_rows<LOGN, LOWER, false, 1>(p, band_idx, b, s0, c0, nc, s, cb, tw);
             return 2;
         }
     }
@@ -270,6 +275,15 @@ int launch_interbin(const Plan &p, int band_idx, const BandDev &b, int64_t s0, i
     if (!attr1) { set_smem(k1, C1::SMEM); attr1 = true; }
     k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, C1::SMEM, s>>>(ld1, st1, tw->s2_f);
     if (mid) record_timing_event(mid, s);
+    if constexpr (LOGN <= 17) {
+        if (rows_packed(p)) {
+            // warps per tile: few enough rows computed twice (one pair per tile) at 24 warps per SM
+            constexpr int W = LOGN == 12 || LOGN == 15 ? 8 : LOGN <= 14 ? 6 : 12;
+            if (b.hi < (int64_t)C2::N) launch_rows<LOGN, true, true, W>(p, band_idx, b, s0, c0, nc, s, cb, tw);
+            else launch_rows<LOGN, false, true, W>(p, band_idx, b, s0, c0, nc, s, cb, tw);
+            return 2;
+        }
+    }
     if (p.tma) {   // 128-thread row tiles staged by bulk copies (8-byte mbarrier after the smem)
         using D2 = Cfg2<LOGN, 2, 128>;
         ScratchLoadIBTMA<D2> ld2{};
@@ -295,17 +309,17 @@ int launch_interbin(const Plan &p, int band_idx, const BandDev &b, int64_t s0, i
     return 2;
 }
 
-// Row factors of the four-step twiddle (RowsTMA): entry [i][m] holds the pair
-// (W_N^{G l2 m}, W_N^{G l2 m} W_32^m) of row l2 = i (512- and 1024-point rows, G = 16 and
-// 32), or (W_N^{16 l2 m}, W_N^{16 (l2+1) m}) of the rows l2 = 2i, 2i + 1 (256-point rows).
+// Row factors of the four-step twiddle: entry [i][m] holds the pair (W_N^{G l2 m},
+// W_N^{G l2 m} W_32^m) of row l2 = i (512- and 1024-point rows, G = 16 and 32), or
+// (W_N^{G l2 m}, W_N^{G (l2+1) m}) of the rows l2 = 2i, 2i + 1 (N1 <= 256, G = N1 / 16).
 __global__ void k_row_twiddles(float4 *t, int logn) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int n1 = logn / 2, n2 = logn - n1;
-    const bool pairs = n1 == 8;
+    const bool pairs = n1 <= 8;
     if (i >= (p3::kRowTw << (pairs ? n2 - 1 : n2))) return;
     const int e = i / p3::kRowTw, m = i % p3::kRowTw;
     const double N = (double)(int64_t(1) << logn);
-    const int64_t g = n1 == 10 ? 32 : 16;
+    const int64_t g = pairs ? 1 << (n1 - 4) : 1 << (n1 - 5);
     const double a = pairs ? (double)(g * 2 * e * m) / N : (double)(g * e * m) / N;
     const double b = pairs ? (double)(g * (2 * e + 1) * m) / N : a + (double)m / 32.0;
     double sa, ca, sb, cb;
@@ -318,7 +332,7 @@ __global__ void k_row_twiddles(float4 *t, int logn) {
 
 int64_t row_twiddle_entries(int logn) {
     const int n1 = logn / 2, n2 = logn - n1;
-    return n1 < 8 || n1 > 10 ? 0 : (int64_t)p3::kRowTw << (n1 == 8 ? n2 - 1 : n2);
+    return n1 < 6 || n1 > 10 ? 0 : (int64_t)p3::kRowTw << (n1 <= 8 ? n2 - 1 : n2);
 }
 
 void launch_row_twiddles(float4 *t, int logn, cudaStream_t s) {

@@ -124,3 +124,21 @@ def test_fp32_sky_stage_tiles(fs, n, dt, scale):
     if m.any():
         sc = np.array([r["S"][0], r["S"][1], math.sqrt(r["S"][0] * r["S"][1])])
         assert np.max(np.abs(g["S"] - r["S"]) / sc) < 1e-5
+
+
+@pytest.mark.parametrize("interbin", [False, True])
+@pytest.mark.parametrize("lg", [12, 13, 14, 15, 16, 17])
+@pytest.mark.parametrize("kw", [dict(), dict(full=True), dict(full_range=True)])
+def test_packed_short_rows(fs, lg, interbin, kw):
+    """Rows of 64, 128 and 256 points in packed pairs (transforms of 2^12 .. 2^17; for the
+    interbinning form n_fft is twice that), every bin: both statistics, the lower half and the
+    whole of the spectrum (the interbinning form's wrap from the last row to row 0)."""
+    nf = 1 << (lg + 1 if interbin else lg)
+    _check(fs, fs.FP32_BATCHED, nf // 3 + 7, nf, 2, 2, interbin=interbin, **kw)
+
+
+@pytest.mark.parametrize("n", [1 << 13, (1 << 13) - 1, 3 << 11, (3 << 11) + 1])
+def test_interbin_long_series(fs, n):
+    """Interbinning at n = N (no zero padding left in the half-length transform) and around
+    three quarters of it."""
+    _check(fs, fs.FP32_BATCHED, n, 1 << 14, 3, 2, interbin=True)
