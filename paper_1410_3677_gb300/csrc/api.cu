@@ -219,15 +219,15 @@ void packed1024_twiddles(std::vector<double> &o) {
 void build_twiddles(Plan &p, const std::vector<int> &logs, int &n_alloc) {
     std::vector<double> hd;
     std::vector<size_t> offs;
-    constexpr int kSets = 7;
+    constexpr int kSets = 8;
     for (int lg : logs) {
-        std::vector<double> a, b, c, d, e, f, g;
+        std::vector<double> a, b, c, d, e, f, g, h;
         host_twiddles(lg, a, b, c, d);
         stage1_twiddles(log_n1(lg), e);
         stage1_twiddles(log_n2(lg), f);
         if (log_n1(lg) == 9) packed512_twiddles(g);   // 512-point rows: N_fft = 2^18, 2^19
-        if (log_n1(lg) == 10) packed1024_twiddles(g);   // 1024-point rows: 2^20
-        for (auto *v : {&a, &b, &c, &d, &e, &f, &g}) {
+        if (log_n2(lg) == 10) packed1024_twiddles(h);   // 1024-point columns or rows: 2^19, 2^20
+        for (auto *v : {&a, &b, &c, &d, &e, &f, &g, &h}) {
             while (hd.size() % 4) hd.push_back(0.0);   // 16-byte aligned float tables
             offs.push_back(hd.size());
             hd.insert(hd.end(), v->begin(), v->end());
@@ -249,7 +249,7 @@ void build_twiddles(Plan &p, const std::vector<int> &logs, int &n_alloc) {
         t.s1_f = df + o[4]; t.s2_f = df + o[5];
         t.s1_d = dd + o[4]; t.s2_d = dd + o[5];
         if (log_n1(logs[i]) == 9) t.p512_f = reinterpret_cast<const float4 *>(df + o[6]);
-        if (log_n1(logs[i]) == 10) t.p1024_f = reinterpret_cast<const float4 *>(df + o[6]);
+        if (log_n2(logs[i]) == 10) t.p1024_f = reinterpret_cast<const float4 *>(df + o[7]);
         p.tw.push_back(t);
     }
 }

@@ -162,6 +162,63 @@ __device__ __forceinline__ void dft16z(T *re, T *im) {
     }
 }
 
+// 8-point DFT of x[0 .. 6) with x[6] = x[7] = 0 (not read).
+template <int DIR, typename T>
+__device__ __forceinline__ void dft8z6(T *re, T *im) {
+    const T h = T(0.70710678118654752440084436210485);
+    T er[4] = {re[0], re[2], re[4], T(0)}, ei[4] = {im[0], im[2], im[4], T(0)};
+    T orr[4] = {re[1], re[3], re[5], T(0)}, oi[4] = {im[1], im[3], im[5], T(0)};
+    dft4z<DIR, 3>(er[0], ei[0], er[1], ei[1], er[2], ei[2], er[3], ei[3]);
+    dft4z<DIR, 3>(orr[0], oi[0], orr[1], oi[1], orr[2], oi[2], orr[3], oi[3]);
+    // O_k *= W8^k
+    T wr = DIR < 0 ? orr[1] + oi[1] : orr[1] - oi[1], wi = DIR < 0 ? oi[1] - orr[1] : oi[1] + orr[1];
+    orr[1] = wr * h; oi[1] = wi * h;
+    wr = DIR < 0 ? oi[2] : -oi[2];
+    wi = DIR < 0 ? -orr[2] : orr[2];
+    orr[2] = wr; oi[2] = wi;
+    wr = DIR < 0 ? oi[3] - orr[3] : -orr[3] - oi[3];
+    wi = DIR < 0 ? -oi[3] - orr[3] : orr[3] - oi[3];
+    orr[3] = wr * h; oi[3] = wi * h;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        re[k] = er[k] + orr[k]; im[k] = ei[k] + oi[k];
+        re[k + 4] = er[k] - orr[k]; im[k + 4] = ei[k] - oi[k];
+    }
+}
+
+// R-point DFT of x[0 .. 3R/4) with the last quarter zero (not read).
+template <int R, int DIR, typename T>
+__device__ __forceinline__ void dft_quarter_zero(T *re, T *im) {
+    if constexpr (R == 8) {
+        dft8z6<DIR>(re, im);
+    } else if constexpr (R == 16) {
+        dft16z<DIR, 12>(re, im);
+    } else {
+        static_assert(R == 32, "radices of the first stage");
+        T sr[4][8], si[4][8];   // radix 4 over 8-point DFTs, as dft_r4
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+#pragma unroll
+            for (int m = 0; m < 6; ++m) { sr[q][m] = re[4 * m + q]; si[q][m] = im[4 * m + q]; }
+            dft8z6<DIR>(sr[q], si[q]);
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            T zr[4], zi[4];
+            zr[0] = sr[0][k]; zi[0] = si[0][k];
+#pragma unroll
+            for (int q = 1; q < 4; ++q) {
+                zr[q] = sr[q][k];
+                zi[q] = si[q][k];
+                mul_w32<DIR>(q * k, zr[q], zi[q]);
+            }
+            eng::dft4<DIR>(zr[0], zi[0], zr[1], zi[1], zr[2], zi[2], zr[3], zi[3]);
+#pragma unroll
+            for (int p = 0; p < 4; ++p) { re[k + 8 * p] = zr[p]; im[k + 8 * p] = zi[p]; }
+        }
+    }
+}
+
 // R-point DFT of x[0 .. NZ) with x[NZ .. R) = 0, NZ <= R/2: the even outputs are
 // the R/2-point DFT of x, the odd ones that of x_r W_R^r (the first radix-2
 // layer of a decimation in frequency, whose partners are all zero); below R/2
@@ -290,8 +347,8 @@ struct NoHook {
 // ZQ: the stage-0 inputs r >= R0 ZQ/8 (sequence elements >= M ZQ/8) are known
 // to be zero (the zero padding of a transform at least 8/ZQ times the series):
 // the loader is asked for R0 ZQ/8 elements and the first DFT skips the zeros
-// (ZQ = 8: none known; 4: the upper half known zero; 3: the upper five eighths
-// known zero, R0 = 32 only).
+// (ZQ = 8: none known; 6: the upper quarter known zero; 4: the upper half; 3: the
+// upper five eighths, R0 = 32 only).
 // TWFULL: tw is the full stage-1 table W_M^{r j} laid out [r][j] (r < R1, j < R0)
 // and the twiddles are read from it through L1 (one 8-byte load per element, a
 // half-warp reading 16 consecutive j); else tw is the table W_M^m, m < M, from
@@ -331,14 +388,15 @@ __device__ __forceinline__ void run_pass(LD &ld, ST &st, const T *__restrict__ t
     }
 
     T re[EH], im[EH];
-    static_assert(ZQ == 8 || ZQ == 4 || (ZQ == 3 && R0 == 32), "known-zero fraction of the first stage");
+    static_assert(ZQ == 8 || ZQ == 6 || ZQ == 4 || (ZQ == 3 && R0 == 32), "known-zero fraction of the first stage");
     constexpr int RL0 = R0 * ZQ / 8;   // stage-0 inputs that can be non-zero
 #pragma unroll
     for (int i = 0; i < NJ0; ++i) ld.template load<RL0, JPF0>(job<MAPM, SEQ, TPF, THREADS>(i), &re[i * R0], &im[i * R0]);
     hk.after_loads();
 #pragma unroll
     for (int i = 0; i < NJ0; ++i) {
-        if constexpr (ZQ < 8) dft_half_zero<R0, DIR, RL0>(&re[i * R0], &im[i * R0]);
+        if constexpr (ZQ == 6) dft_quarter_zero<R0, DIR>(&re[i * R0], &im[i * R0]);
+        else if constexpr (ZQ < 8) dft_half_zero<R0, DIR, RL0>(&re[i * R0], &im[i * R0]);
         else dft<R0, DIR>(&re[i * R0], &im[i * R0]);
     }
     if constexpr (R1 == 1) {

@@ -41,7 +41,7 @@ struct TwiddleSet {
     // 512-point pass as pairs,
     // [r][k] = (cos a_2k, cos a_2k+1, -sin a_2k, -sin a_2k+1), a_j = 2 pi r j / 512
     const float4 *p512_f = nullptr;
-    // 1024-point rows (2^20): [m][q] = (W_1024^{mq}, W_1024^{m(q+32)}) as packed pairs
+    // 1024-point columns and rows (2^19, 2^20): [m][q] = (W_1024^{mq}, W_1024^{m(q+32)}) as packed pairs
     // (cosines, then sines of the negative angles), m < 16, q < 32
     const float4 *p1024_f = nullptr;
     const float4 *row_tw = nullptr;   // FP32 packed rows: the rows' four-step factors

@@ -105,26 +105,31 @@ struct SearchLoad2S : SearchLoad2<C> {
             if (k < this->n) v = __ldg(this->ws + 2 * k + q.t);
             re[r] = v.x; im[r] = v.y;
         }
-        float cs[R / 2], sn[R / 2];
-        const int kt = kb + C::N1 * JPF * q.t;
-#pragma unroll
-        for (int i = 0; i < R / 2; ++i) {   // this lane's half of the phases
-            const uint32_t k = (uint32_t)(kt + C::N1 * JPF * 2 * i);
-            const uint64_t kk = (uint64_t)k * (uint64_t)k;
-            const int32_t top = (int32_t)((this->afx * kk) >> 32);   // cycles in [-1/2, 1/2)
-            __sincosf((float)top * 1.4629180792671596e-09f, &sn[i], &cs[i]);   // 2 pi / 2^32
-        }
         const int lane = (int)threadIdx.x & 31;
+        const int kt = kb + C::N1 * JPF * q.t;
+        // in groups of a few elements, so that only a group's phases are held beside the data
+        constexpr int GR = R % 8 == 0 && R > 16 ? 8 : R;
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int src = (lane & ~1) | (r & 1);   // the lane that evaluated element r
-            const float c = __shfl_sync(0xffffffffu, cs[r / 2], src);
-            const float sv = __shfl_sync(0xffffffffu, sn[r / 2], src);
-            const uint32_t k = (uint32_t)(kb + C::N1 * JPF * r);
-            if (k < (uint32_t)this->n) {
-                const float x = re[r], y = im[r];
-                re[r] = x * c + y * sv;
-                im[r] = y * c - x * sv;
+        for (int r0 = 0; r0 < R; r0 += GR) {
+            float cs[GR / 2], sn[GR / 2];
+#pragma unroll
+            for (int i = 0; i < GR / 2; ++i) {   // this lane's half of the phases
+                const uint32_t k = (uint32_t)(kt + C::N1 * JPF * (r0 + 2 * i));
+                const uint64_t kk = (uint64_t)k * (uint64_t)k;
+                const int32_t top = (int32_t)((this->afx * kk) >> 32);   // cycles in [-1/2, 1/2)
+                __sincosf((float)top * 1.4629180792671596e-09f, &sn[i], &cs[i]);   // 2 pi / 2^32
+            }
+#pragma unroll
+            for (int r = r0; r < r0 + GR; ++r) {
+                const int src = (lane & ~1) | (r & 1);   // the lane that evaluated element r
+                const float c = __shfl_sync(0xffffffffu, cs[(r - r0) / 2], src);
+                const float sv = __shfl_sync(0xffffffffu, sn[(r - r0) / 2], src);
+                const uint32_t k = (uint32_t)(kb + C::N1 * JPF * r);
+                if (k < (uint32_t)this->n) {
+                    const float x = re[r], y = im[r];
+                    re[r] = x * c + y * sv;
+                    im[r] = y * c - x * sv;
+                }
             }
         }
     }
@@ -393,7 +398,8 @@ struct SearchEpi2 {
 // elements k2 >= N2/2 lie at k >= N/2 >= n, in the zero padding; with
 // n <= 3N/8 and a radix-32 first stage only the first three eighths (Z1 = 3);
 // Z1 = 8: a transform only as long as the series allows (the half-length
-// transform of the interbinning form, N >= n but not N >= 2n).
+// transform of the interbinning form, N >= n but not N >= 2n), 6: the same with
+// n <= 3N/4.
 template <int LOGN, int PASS, int MAPM, class LD, class ST, int TS = 256, int Z1 = 4>
 __global__ void __launch_bounds__(TS, 768 / TS) k_pass2(LD ld, ST st, const float *__restrict__ tw) {
     using C = Cfg2<LOGN, PASS, TS>;

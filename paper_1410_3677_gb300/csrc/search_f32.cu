@@ -103,6 +103,21 @@ int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_
     }
     // columns known zero beyond 3/8 of their length (radix-32 first stage) or 1/2
     bool launched = pk1;
+    if constexpr (C1::M == 1024) {   // 1024-point columns (2^19, 2^20): packed
+        if (p.packed >= 1 && p.share_chirp && tw->p1024_f) {
+            SearchLoad2S<C1> l1s{};
+            static_cast<SearchLoad2<C1> &>(l1s) = ld1;
+            auto k3 = p3::k_pass1q<LOGN, 3>;
+            auto k4 = p3::k_pass1q<LOGN, 4>;
+            constexpr size_t smem1 = (size_t)C1::SEQ * p3::kCol1024Ld * sizeof(float2);
+            static bool attr1q = false;
+            if (!attr1q) { set_smem(k3, smem1); set_smem(k4, smem1); attr1q = true; }
+            auto k1 = 8 * b.n <= 3 * (int64_t)C1::N ? k3 : k4;
+            k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, smem1, s>>>(l1s, st1, tw->p1024_f,
+                                                                         reinterpret_cast<const float2 *>(tw->in2_f));
+            launched = true;
+        }
+    }
     if constexpr (eng2::radix0(C1::M) == 32) {
         if (!launched && 8 * b.n <= 3 * (int64_t)C1::N && p.share_chirp) {
             SearchLoad2S<C1> l1s{};
@@ -270,10 +285,24 @@ int launch_interbin(const Plan &p, int band_idx, const BandDev &b, int64_t s0, i
     ld1.s0 = s0;
     ScratchStore2<C1> st1{};
     st1.scratch = reinterpret_cast<float2 *>(cb.scratch);
-    auto k1 = k_pass2<LOGN, 1, eng2::kMapFJ, SearchLoad2<C1>, ScratchStore2<C1>, 256, 8>;
-    static bool attr1 = false;
-    if (!attr1) { set_smem(k1, C1::SMEM); attr1 = true; }
-    k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, C1::SMEM, s>>>(ld1, st1, tw->s2_f);
+    // The last quarter of a column is skipped when it lies beyond the series.  Lane pairs share
+    // the spindown phases with a radix-16 or smaller first stage; with radix 32 the 24 or 32
+    // inputs leave no registers for the exchange.  Measured (n_fft x cells = 2^30, shared against
+    // not): 256-point columns 1.90 against 1.99 ms with the quarter skipped, 2.41 against 2.54
+    // without; 512-point 1.95 against 1.91 and 2.43 against 2.34; 1024-point 2.61 against 2.47
+    // and 3.04 against 2.75.
+    const bool z6 = 4 * b.n <= 3 * (int64_t)C1::N;
+    constexpr bool kShare = eng2::radix0(C1::N2) < 32;
+    SearchLoad2S<C1> l1s{};
+    static_cast<SearchLoad2<C1> &>(l1s) = ld1;
+    auto run = [&](auto k1, const auto &ld) {
+        set_smem(k1, C1::SMEM);
+        k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, C1::SMEM, s>>>(ld, st1, tw->s2_f);
+    };
+    if (z6 && kShare && p.share_chirp) run(k_pass2<LOGN, 1, eng2::kMapFJ, SearchLoad2S<C1>, ScratchStore2<C1>, 256, 6>, l1s);
+    else if (z6) run(k_pass2<LOGN, 1, eng2::kMapFJ, SearchLoad2<C1>, ScratchStore2<C1>, 256, 6>, ld1);
+    else if (kShare && p.share_chirp) run(k_pass2<LOGN, 1, eng2::kMapFJ, SearchLoad2S<C1>, ScratchStore2<C1>, 256, 8>, l1s);
+    else run(k_pass2<LOGN, 1, eng2::kMapFJ, SearchLoad2<C1>, ScratchStore2<C1>, 256, 8>, ld1);
     if (mid) record_timing_event(mid, s);
     if constexpr (LOGN <= 17) {
         if (rows_packed(p)) {
