@@ -1,7 +1,7 @@
 // Candidate records put in (cell, bin) order on the device before they are read
 // back: a stable least-significant-digit radix sort, 8-bit digits, over the key
 // (cell - cell0) << bin_bits | bin of the searched range.  One pass is a digit
-// histogram per tile of 4096 records, an exclusive scan of the histograms in
+// histogram per tile of 1024 or 4096 records, an exclusive scan of the histograms in
 // digit-major order (the tile's first slot for each digit), and a scatter that
 // ranks each record among the equal digits before it in its tile (warp match,
 // per-warp counts in shared memory), so records with equal digits keep their
@@ -9,6 +9,8 @@
 // the scatter adds the totals of the smaller digits.  The candidate set of
 // Sect. 2 has no order of its own; the plan returns it sorted by (band, sky,
 // spin, bin).
+#include <algorithm>
+
 #include "fstat_internal.h"
 
 namespace fstat {
@@ -16,21 +18,24 @@ namespace fstat {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kRounds = 16;
-constexpr int kTile = kThreads * kRounds;
+// Rounds of 256 records per tile: 16, or 4 for fewer than 2^20 records, whose 4096-record
+// tiles would leave most SMs idle (69 632 records, three digits: 80 -> 60 us).
+constexpr int kRoundsLong = 16, kRoundsShort = 4;
+constexpr int64_t kShort = int64_t(1) << 20;
 
 __device__ __forceinline__ uint32_t digit_of(const CandRecord &r, uint32_t cell0, int bin_bits, int shift) {
     const uint64_t key = ((uint64_t)(r.cell - cell0) << bin_bits) | r.bin;
     return (uint32_t)(key >> shift) & 255u;
 }
 
+template <int kRounds>
 __global__ void __launch_bounds__(kThreads) k_digit_hist(const CandRecord *__restrict__ in, int64_t n,
                                                          uint32_t cell0, int bin_bits, int shift,
                                                          uint32_t *__restrict__ hist, int64_t nblk) {
     __shared__ uint32_t h[256];
     h[threadIdx.x] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kTile;
+    const int64_t base = (int64_t)blockIdx.x * (kThreads * kRounds);
 #pragma unroll 4
     for (int i = 0; i < kRounds; ++i) {
         const int64_t idx = base + i * kThreads + threadIdx.x;
@@ -81,6 +86,7 @@ __global__ void __launch_bounds__(1024) k_scan_rows(uint32_t *__restrict__ h, in
     if (t == 0) tot[blockIdx.x] = carry;
 }
 
+template <int kRounds>
 __global__ void __launch_bounds__(kThreads) k_digit_scatter(const CandRecord *__restrict__ in,
                                                             CandRecord *__restrict__ out, int64_t n,
                                                             uint32_t cell0, int bin_bits, int shift,
@@ -105,7 +111,7 @@ __global__ void __launch_bounds__(kThreads) k_digit_scatter(const CandRecord *__
     uint32_t smaller = x - v;
     for (int q = 0; q < w; ++q) smaller += wt[q];
     run[t] = smaller + off[(int64_t)t * nblk + blockIdx.x];
-    const int64_t base = (int64_t)blockIdx.x * kTile;
+    const int64_t base = (int64_t)blockIdx.x * (kThreads * kRounds);
     for (int i = 0; i < kRounds; ++i) {
 #pragma unroll
         for (int q = 0; q < kThreads / 32; ++q) wc[q][t] = 0;
@@ -135,36 +141,40 @@ __global__ void __launch_bounds__(kThreads) k_digit_scatter(const CandRecord *__
     }
 }
 
-}  // namespace
-
-int sort_bits(uint64_t v) {
-    int b = 0;
-    while (b < 64 && (v >> b) != 0) ++b;
-    return b;
-}
-
-// Sorts n records of `a` (using b as the other buffer of the ping-pong and hist
-// for 256 ceil(n / 4096) counts plus 256 totals); returns the buffer that holds
-// the result.
-// cell0 and the cell span are those of the searched range, bins < 2^bin_bits.
-CandRecord *launch_cand_sort(CandRecord *a, CandRecord *b, uint32_t *hist, int64_t n, uint32_t cell0,
-                             uint64_t cell_span, int bin_bits, cudaStream_t s, int64_t *launches) {
-    const int key_bits = sort_bits(cell_span > 0 ? cell_span - 1 : 0) + bin_bits;
+template <int kRounds>
+CandRecord *sort_t(CandRecord *a, CandRecord *b, uint32_t *hist, int64_t n, uint32_t cell0, int key_bits, int bin_bits,
+                   cudaStream_t s, int64_t *launches) {
     const int passes = (key_bits + 7) / 8;
-    const int64_t nblk = (n + kTile - 1) / kTile;
+    const int64_t tile = kThreads * kRounds, nblk = (n + tile - 1) / tile;
     CandRecord *src = a, *dst = b;
     for (int p = 0; p < passes; ++p) {
         const int shift = 8 * p;
-        k_digit_hist<<<(unsigned)nblk, kThreads, 0, s>>>(src, n, cell0, bin_bits, shift, hist, nblk);
+        k_digit_hist<kRounds><<<(unsigned)nblk, kThreads, 0, s>>>(src, n, cell0, bin_bits, shift, hist, nblk);
         k_scan_rows<<<256, 1024, 0, s>>>(hist, nblk, hist + 256 * nblk);
-        k_digit_scatter<<<(unsigned)nblk, kThreads, 0, s>>>(src, dst, n, cell0, bin_bits, shift, hist, nblk,
-                                                             hist + 256 * nblk);
+        k_digit_scatter<kRounds><<<(unsigned)nblk, kThreads, 0, s>>>(src, dst, n, cell0, bin_bits, shift, hist, nblk,
+                                                                     hist + 256 * nblk);
         *launches += 3;
         CandRecord *x = src;
         src = dst;
         dst = x;
     }
     return src;
+}
+
+}  // namespace
+
+// Counts of the tiles and 256 totals, for up to n records.
+int64_t cand_sort_hist(int64_t n) {
+    auto tiles = [](int64_t m, int64_t t) { return (m + t - 1) / t; };
+    return 256 * (std::max(tiles(std::min(n, kShort), kThreads * kRoundsShort), tiles(n, kThreads * kRoundsLong)) + 1);
+}
+
+// Sorts n records of `a` (using b as the other buffer of the ping-pong); returns the buffer
+// that holds the result.
+CandRecord *launch_cand_sort(CandRecord *a, CandRecord *b, uint32_t *hist, int64_t n, uint32_t cell0, int key_bits,
+                             int bin_bits, cudaStream_t s, int64_t *launches) {
+    return n < kShort ? sort_t<kRoundsShort>(a, b, hist, n, cell0, key_bits, bin_bits, s, launches)
+                      : sort_t<kRoundsLong>(a, b, hist, n, cell0, key_bits, bin_bits, s, launches);
 }
 
 }  // namespace fstat

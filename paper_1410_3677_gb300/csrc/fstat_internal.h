@@ -58,6 +58,9 @@ struct CandRecord {
     double F;
 };
 
+// Records that come to the host with the search's status (64 KiB).
+constexpr int64_t kEagerRecords = 4096;
+
 // Per-sky constants computed once per plan: unit vector and the coefficients of
 // a(h) = A0 cos2h + A1 sin2h + A2 cosh + A3 sinh + A4 and
 //       b(h) = B0 cos2h + B1 sin2h + B2 cosh + B3 sinh, h = alpha - LST.
@@ -176,8 +179,11 @@ struct Plan {
     int64_t cand_capacity = 0;
     // pinned host staging of the candidate records (read back and sorted there),
     // grown on demand and reused by later calls
-    CandRecord *h_rec = nullptr;           // pinned staging of the read-back
+    // pinned: {count, error word}, then the first kEagerRecords records, of the last search
+    uint64_t *h_status = nullptr;
+    CandRecord *h_rec = nullptr;           // pinned staging of longer read-backs
     std::vector<CandRecord> h_tmp;         // work array of the host sort (few records)
+    bool host_sorted = false;              // the host's copy of the last search is in order
     int64_t h_rec_cap = 0;
     // device sort of the records before the read-back: the other ping-pong buffer,
     // the digit counts, the cell range of the records and the sorted buffer (null
@@ -265,11 +271,12 @@ int launch_geometry(const Plan &p, const BandDev &b, int64_t s0, int64_t ns, boo
 
 // Per-sky S sums and normalisations for the ns skies of the last geometry launch.
 int launch_reduce_norms(const Plan &p, const BandDev &b, int64_t ns, double *norm, cudaStream_t s);
-// Stable device sort of n candidate records by (cell - cell0, bin), bins < 2^bin_bits,
-// cells in [cell0, cell0 + cell_span); a and b ping-pong, hist holds 256 (ceil(n / 4096) + 1)
-// counts; returns the buffer with the sorted records.
-CandRecord *launch_cand_sort(CandRecord *a, CandRecord *b, uint32_t *hist, int64_t n, uint32_t cell0,
-                             uint64_t cell_span, int bin_bits, cudaStream_t s, int64_t *launches);
+// Stable device sort of n candidate records by (cell - cell0, bin), bins < 2^bin_bits, a key
+// of key_bits bits; a and b ping-pong, hist holds cand_sort_hist(n) counts; returns the
+// buffer with the sorted records.
+int64_t cand_sort_hist(int64_t n);
+CandRecord *launch_cand_sort(CandRecord *a, CandRecord *b, uint32_t *hist, int64_t n, uint32_t cell0, int key_bits,
+                             int bin_bits, cudaStream_t s, int64_t *launches);
 
 // Row factors of the four-step twiddle for the packed FP32 rows (0 entries: none used).
 int64_t row_twiddle_entries(int logn);

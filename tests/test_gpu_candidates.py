@@ -82,3 +82,26 @@ def test_measured_roofline_denominators(fs):
     assert 0.5 * nominal < tf < 1.05 * nominal, (tf, nominal)
     l2 = fs.measure_l2_copy(32 << 20)
     assert l2 > 7000.0, l2
+
+
+@pytest.mark.parametrize("n_bins", [15, 64, 511, 512, 513, 1023, 1024, 1025, 2500])
+def test_read_back_paths(fs, n_bins):
+    """Read-backs of 8 cells x n_bins records on either side of the limits between the copy that
+    comes with the search, the host sort and the device sort (4096 and 8192 records): the order,
+    a limited read (cap), a second read, and the count."""
+    w = S.workload(1, n_sky=4, n_spin=2)
+    p = fs.Plan(w.bands, w.alpha, w.delta, w.fdot, -1.0, lat=w.lat, gamma=w.gamma, bin_lo=100, bin_hi=99 + n_bins,
+                form=fs.FP32_BATCHED, cand_capacity=1 << 16)
+    p.search()
+    n = 8 * n_bins
+    assert p.candidates_get_status(0)[2] == n
+    few, total = p.candidates(cap=min(37, n))
+    c, total2 = p.candidates()
+    again, _ = p.candidates()
+    p.close()
+    assert total == total2 == n == c.size
+    assert np.array_equal(c["sky"] * 2 + c["spin"], np.repeat(np.arange(8), n_bins))
+    assert np.array_equal(c["bin"], np.tile(np.arange(100, 100 + n_bins), 8))
+    assert np.array_equal(c["alpha"], w.alpha[c["sky"]]) and np.array_equal(c["fdot"], w.fdot[c["spin"]])
+    assert np.array_equal(c["freq"], w.bands[0].f_off + c["bin"] / (w.bands[0].n_fft * w.bands[0].dt))
+    assert np.array_equal(few, c[:few.size]) and np.array_equal(again, c)
