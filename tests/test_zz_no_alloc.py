@@ -94,3 +94,29 @@ def test_noalloc_allocates_no_device_memory():
     assert torch.cuda.mem_get_info()[0] == free0
     assert torch.equal(out, first)                      # the shared scratch keeps no state
     del first
+
+
+@pytest.mark.parametrize("lg", range(12, 19))
+@pytest.mark.parametrize("frac,whole", [(0.33, False), (0.5, True)])
+def test_noalloc_every_length(lg, frac, whole):
+    """Every length, both column variants (n <= 3N/8 and n = N/2), half and whole bin range,
+    an odd output window: against an FP64 transform of the same series."""
+    import torch
+    from paper_1410_3677_gb300 import fstat as fs
+    N = 1 << lg
+    n = int(frac * N)
+    rng = np.random.default_rng(lg)
+    w = rng.standard_normal((n, 4)).astype(np.float32)
+    rate, na, nb = -1.7e-8, 1.0 / n, 2.0 / n
+    k = np.arange(n, dtype=np.float64)
+    ph = np.exp(-2j * np.pi * np.mod(rate * k * k, 1.0))
+    A = np.fft.fft((w[:, 0] + 1j * w[:, 1].astype(np.float64)) * ph, N)
+    B = np.fft.fft((w[:, 2] + 1j * w[:, 3].astype(np.float64)) * ph, N)
+    lo, hi = (3, N - 2) if whole else (1, N // 2 - 1)
+    ref = (np.abs(A) ** 2 * na + np.abs(B) ** 2 * nb)[lo:hi + 1]
+    wd = torch.from_numpy(w).cuda()
+    out = torch.full((hi - lo + 3,), -1.0, dtype=torch.float32, device="cuda")
+    assert fs.cell_F_noalloc(wd.data_ptr(), n, N, rate, na, nb, lo, hi, out.data_ptr() + 4) == fs.FSTAT_OK
+    got = out.cpu().numpy()
+    assert got[0] == -1.0 and got[-1] == -1.0            # nothing outside the window
+    assert np.max(np.abs(got[1:-1] - ref) / np.maximum(ref, 2.0)) <= 1e-4
