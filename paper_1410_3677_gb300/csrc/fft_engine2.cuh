@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fft_codelets.cuh"
 #include "fft_engine.cuh"
 
 namespace fstat {
@@ -43,10 +44,6 @@ __host__ __device__ constexpr double w32_im(int k) {   // -sin(2 pi k / 32)
 }
 
 // ------------------------------------------------------------------ register DFTs
-// Natural order in and out; DIR = -1 is the forward transform.
-template <int R, int DIR, typename T>
-__device__ __forceinline__ void dft(T *re, T *im);
-
 // x <- x W_32^e (DIR = -1) or x conj(W_32^e), e known at compile time once the
 // callers' loops are unrolled: the quarter turns are swaps and negations, so
 // no multiplication by 0 or 1 is left for the compiler to keep.
@@ -69,183 +66,16 @@ __device__ __forceinline__ void mul_w32(int e, T &xr, T &xi) {
     xr = r;
 }
 
-// Radix-4 decimation in time: 4 sub-DFTs of length R/4 over x[4m + q], then for
-// each k < R/4 the twiddles W_R^{q k} and a 4-point DFT across q.
-template <int R, int DIR, typename T>
-__device__ __forceinline__ void dft_r4(T *re, T *im) {
-    constexpr int n = R / 4;
-    T sr[4][n], si[4][n];
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int m = 0; m < n; ++m) { sr[q][m] = re[4 * m + q]; si[q][m] = im[4 * m + q]; }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) dft<n, DIR>(sr[q], si[q]);
-#pragma unroll
-    for (int k = 0; k < n; ++k) {
-        T zr[4], zi[4];
-        zr[0] = sr[0][k]; zi[0] = si[0][k];
-#pragma unroll
-        for (int q = 1; q < 4; ++q) {
-            zr[q] = sr[q][k];
-            zi[q] = si[q][k];
-            mul_w32<DIR>((32 / R) * q * k, zr[q], zi[q]);   // W_R^{q k} = W_32^{(32/R) q k}
-        }
-        eng::dft4<DIR>(zr[0], zi[0], zr[1], zi[1], zr[2], zi[2], zr[3], zi[3]);
-#pragma unroll
-        for (int p = 0; p < 4; ++p) { re[k + n * p] = zr[p]; im[k + n * p] = zi[p]; }
-    }
-}
-
-template <int R, int DIR, typename T>
+// R-point DFT of x[0 .. NZ) on split arrays, the rest zero (fft_codelets.cuh).
+template <int R, int DIR, int NZ = R, typename T>
 __device__ __forceinline__ void dft(T *re, T *im) {
-    if constexpr (R == 32 || R == 16) dft_r4<R, DIR>(re, im);
-    else eng::dft<R, DIR>(re, im);
-}
-
-// 4-point DFT whose inputs from index NZ on are known to be zero: the terms
-// with a zero partner are left out (the compiler may not drop x + 0 itself,
-// since -0 + 0 = +0 under IEEE rules).
-template <int DIR, int NZ, typename T>
-__device__ __forceinline__ void dft4z(T &r0, T &i0, T &r1, T &i1, T &r2, T &i2, T &r3, T &i3) {
-    static_assert(NZ >= 1 && NZ <= 4, "non-zero inputs");
-    if constexpr (NZ == 4) {
-        eng::dft4<DIR>(r0, i0, r1, i1, r2, i2, r3, i3);
-    } else {
-        // t0 = x0 + x2, t1 = x0 - x2, t2 = t3 = x1 (x3 = 0); u = (DIR i) x1
-        const T t0r = NZ >= 3 ? r0 + r2 : r0, t0i = NZ >= 3 ? i0 + i2 : i0;
-        const T t1r = NZ >= 3 ? r0 - r2 : r0, t1i = NZ >= 3 ? i0 - i2 : i0;
-        if constexpr (NZ == 1) {
-            r1 = r2 = r3 = r0;
-            i1 = i2 = i3 = i0;
-        } else {
-            const T ur = DIR < 0 ? i1 : -i1, ui = DIR < 0 ? -r1 : r1;
-            const T x1r = r1, x1i = i1;
-            r0 = t0r + x1r; i0 = t0i + x1i;
-            r2 = t0r - x1r; i2 = t0i - x1i;
-            r1 = t1r + ur;  i1 = t1i + ui;
-            r3 = t1r - ur;  i3 = t1i - ui;
-        }
-    }
-}
-
-// 16-point DFT (radix-4 decimation in time, as dft_r4) of x[0 .. NZ) with
-// x[NZ .. 16) = 0: the sub-DFT over x[4m + q] keeps its ceil((NZ - q)/4)
-// non-zero inputs; the elements from NZ on are not read.
-template <int DIR, int NZ, typename T>
-__device__ __forceinline__ void dft16z(T *re, T *im) {
-    static_assert(NZ >= 4 && NZ <= 16, "each sub-DFT keeps an input");
-    T sr[4][4], si[4][4];
+    static_assert(DIR == -1, "forward transforms");
+    cod::SC<T> x[R];
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int r = 0; r < NZ; ++r) x[r] = {re[r], im[r]};
+    cod::dft<R, NZ>(x);
 #pragma unroll
-        for (int m = 0; m < 4; ++m)
-            if (4 * m + q < NZ) { sr[q][m] = re[4 * m + q]; si[q][m] = im[4 * m + q]; }
-            else { sr[q][m] = T(0); si[q][m] = T(0); }   // never read below
-    dft4z<DIR, (NZ + 3) / 4>(sr[0][0], si[0][0], sr[0][1], si[0][1], sr[0][2], si[0][2], sr[0][3], si[0][3]);
-    dft4z<DIR, (NZ + 2) / 4>(sr[1][0], si[1][0], sr[1][1], si[1][1], sr[1][2], si[1][2], sr[1][3], si[1][3]);
-    dft4z<DIR, (NZ + 1) / 4>(sr[2][0], si[2][0], sr[2][1], si[2][1], sr[2][2], si[2][2], sr[2][3], si[2][3]);
-    dft4z<DIR, NZ / 4>(sr[3][0], si[3][0], sr[3][1], si[3][1], sr[3][2], si[3][2], sr[3][3], si[3][3]);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        T zr[4], zi[4];
-        zr[0] = sr[0][k]; zi[0] = si[0][k];
-#pragma unroll
-        for (int q = 1; q < 4; ++q) {
-            zr[q] = sr[q][k];
-            zi[q] = si[q][k];
-            mul_w32<DIR>(2 * q * k, zr[q], zi[q]);   // W_16^{q k} = W_32^{2 q k}
-        }
-        eng::dft4<DIR>(zr[0], zi[0], zr[1], zi[1], zr[2], zi[2], zr[3], zi[3]);
-#pragma unroll
-        for (int p = 0; p < 4; ++p) { re[k + 4 * p] = zr[p]; im[k + 4 * p] = zi[p]; }
-    }
-}
-
-// 8-point DFT of x[0 .. 6) with x[6] = x[7] = 0 (not read).
-template <int DIR, typename T>
-__device__ __forceinline__ void dft8z6(T *re, T *im) {
-    const T h = T(0.70710678118654752440084436210485);
-    T er[4] = {re[0], re[2], re[4], T(0)}, ei[4] = {im[0], im[2], im[4], T(0)};
-    T orr[4] = {re[1], re[3], re[5], T(0)}, oi[4] = {im[1], im[3], im[5], T(0)};
-    dft4z<DIR, 3>(er[0], ei[0], er[1], ei[1], er[2], ei[2], er[3], ei[3]);
-    dft4z<DIR, 3>(orr[0], oi[0], orr[1], oi[1], orr[2], oi[2], orr[3], oi[3]);
-    // O_k *= W8^k
-    T wr = DIR < 0 ? orr[1] + oi[1] : orr[1] - oi[1], wi = DIR < 0 ? oi[1] - orr[1] : oi[1] + orr[1];
-    orr[1] = wr * h; oi[1] = wi * h;
-    wr = DIR < 0 ? oi[2] : -oi[2];
-    wi = DIR < 0 ? -orr[2] : orr[2];
-    orr[2] = wr; oi[2] = wi;
-    wr = DIR < 0 ? oi[3] - orr[3] : -orr[3] - oi[3];
-    wi = DIR < 0 ? -oi[3] - orr[3] : orr[3] - oi[3];
-    orr[3] = wr * h; oi[3] = wi * h;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        re[k] = er[k] + orr[k]; im[k] = ei[k] + oi[k];
-        re[k + 4] = er[k] - orr[k]; im[k + 4] = ei[k] - oi[k];
-    }
-}
-
-// R-point DFT of x[0 .. 3R/4) with the last quarter zero (not read).
-template <int R, int DIR, typename T>
-__device__ __forceinline__ void dft_quarter_zero(T *re, T *im) {
-    if constexpr (R == 8) {
-        dft8z6<DIR>(re, im);
-    } else if constexpr (R == 16) {
-        dft16z<DIR, 12>(re, im);
-    } else {
-        static_assert(R == 32, "radices of the first stage");
-        T sr[4][8], si[4][8];   // radix 4 over 8-point DFTs, as dft_r4
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-#pragma unroll
-            for (int m = 0; m < 6; ++m) { sr[q][m] = re[4 * m + q]; si[q][m] = im[4 * m + q]; }
-            dft8z6<DIR>(sr[q], si[q]);
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            T zr[4], zi[4];
-            zr[0] = sr[0][k]; zi[0] = si[0][k];
-#pragma unroll
-            for (int q = 1; q < 4; ++q) {
-                zr[q] = sr[q][k];
-                zi[q] = si[q][k];
-                mul_w32<DIR>(q * k, zr[q], zi[q]);
-            }
-            eng::dft4<DIR>(zr[0], zi[0], zr[1], zi[1], zr[2], zi[2], zr[3], zi[3]);
-#pragma unroll
-            for (int p = 0; p < 4; ++p) { re[k + 8 * p] = zr[p]; im[k + 8 * p] = zi[p]; }
-        }
-    }
-}
-
-// R-point DFT of x[0 .. NZ) with x[NZ .. R) = 0, NZ <= R/2: the even outputs are
-// the R/2-point DFT of x, the odd ones that of x_r W_R^r (the first radix-2
-// layer of a decimation in frequency, whose partners are all zero); below R/2
-// non-zero inputs the half-length DFTs skip their zero inputs too (R = 32).
-template <int R, int DIR, int NZ = R / 2, typename T>
-__device__ __forceinline__ void dft_half_zero(T *re, T *im) {
-    constexpr int H = R / 2;
-    static_assert(NZ <= H && (NZ == H || H == 16), "pruned half-length DFTs are 16-point");
-    T er[H], ei[H], orr[H], oi[H];
-#pragma unroll
-    for (int r = 0; r < NZ; ++r) {
-        er[r] = re[r]; ei[r] = im[r];
-        orr[r] = re[r]; oi[r] = im[r];
-        mul_w32<DIR>((32 / R) * r, orr[r], oi[r]);
-    }
-    if constexpr (NZ < H) {
-        dft16z<DIR, NZ>(er, ei);
-        dft16z<DIR, NZ>(orr, oi);
-    } else if constexpr (H > 1) {
-        dft<H, DIR>(er, ei);
-        dft<H, DIR>(orr, oi);
-    }
-#pragma unroll
-    for (int p = 0; p < H; ++p) {
-        re[2 * p] = er[p]; im[2 * p] = ei[p];
-        re[2 * p + 1] = orr[p]; im[2 * p + 1] = oi[p];
-    }
+    for (int r = 0; r < R; ++r) { re[r] = x[r].re; im[r] = x[r].im; }
 }
 
 // ------------------------------------------------------------------ plan
@@ -395,9 +225,7 @@ __device__ __forceinline__ void run_pass(LD &ld, ST &st, const T *__restrict__ t
     hk.after_loads();
 #pragma unroll
     for (int i = 0; i < NJ0; ++i) {
-        if constexpr (ZQ == 6) dft_quarter_zero<R0, DIR>(&re[i * R0], &im[i * R0]);
-        else if constexpr (ZQ < 8) dft_half_zero<R0, DIR, RL0>(&re[i * R0], &im[i * R0]);
-        else dft<R0, DIR>(&re[i * R0], &im[i * R0]);
+        dft<R0, DIR, RL0>(&re[i * R0], &im[i * R0]);
     }
     if constexpr (R1 == 1) {
 #pragma unroll

@@ -7,7 +7,7 @@
 // the tiles are small (64 or 128 threads: 8 to 128 CTAs instead of 2 to 64), the second
 // launch is a programmatic dependent of the first (its launch and prologue run under the
 // first pass) and a length's function attributes are set once.  Measured, per call
-// from Python with the wait: 2^13 23.1 -> 16.1 us, 2^18 25.1 -> 19.0 us.
+// from Python with the wait: 2^13 22.8 -> 15.7 us, 2^18 25.1 -> 19.2 us.
 #include <mutex>
 
 #include "passes2.cuh"

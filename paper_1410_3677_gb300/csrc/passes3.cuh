@@ -79,7 +79,7 @@ k_pass1p(SearchLoad2<Cfg2<LOGN, 1>> ld, ScratchStore2<Cfg2<LOGN, 1>> st, const f
             }
         }
     }
-    pk::dft16<NZ>(P);   // P[k] = (X_{2k}, X_{2k+1})
+    cod::dft16<NZ>(P);   // P[k] = (X_{2k}, X_{2k+1})
     {
         float4 *p4 = reinterpret_cast<float4 *>(sd + s * RL + eng2::pad16(j * kR0));
 #pragma unroll
@@ -98,7 +98,7 @@ k_pass1p(SearchLoad2<Cfg2<LOGN, 1>> ld, ScratchStore2<Cfg2<LOGN, 1>> st, const f
     }
 #pragma unroll
     for (int r = 1; r < 16; ++r) Q[r] = pk::cmul(Q[r], tw1(tws, r, j));
-    pk::dft16<16>(Q);
+    cod::dft16<16>(Q);
     // outputs l2 = job + 32 p of the two jobs, one transposed store each
     float re0[16], im0[16], re1[16], im1[16];
 #pragma unroll
@@ -132,7 +132,7 @@ k_pass1h(SearchLoad2<Cfg2<LOGN, 1>> ld, ScratchStore2<Cfg2<LOGN, 1>> st, const f
     {
         float re[kR0], im[kR0];
         ld.template load<NZ, 16>(q, re, im);
-        eng2::dft_half_zero<kR0, -1, NZ>(re, im);
+        eng2::dft<kR0, -1, NZ>(re, im);
         float4 *p4 = reinterpret_cast<float4 *>(sd + s * RL + eng2::pad16(j * kR0));
 #pragma unroll
         for (int k = 0; k < 16; ++k) p4[k] = make_float4(re[2 * k], re[2 * k + 1], im[2 * k], im[2 * k + 1]);
@@ -149,7 +149,7 @@ k_pass1h(SearchLoad2<Cfg2<LOGN, 1>> ld, ScratchStore2<Cfg2<LOGN, 1>> st, const f
     }
 #pragma unroll
     for (int r = 1; r < 16; ++r) Q[r] = pk::cmul(Q[r], tw1(tws, r, j));
-    pk::dft16<16>(Q);
+    cod::dft16<16>(Q);
     float re0[16], im0[16], re1[16], im1[16];
 #pragma unroll
     for (int p = 0; p < 16; ++p) {
@@ -192,7 +192,7 @@ k_pass1q(SearchLoad2S<Cfg2<LOGN, 1>> ld, ScratchStore2<Cfg2<LOGN, 1>> st, const 
             P[m] = {make_float2(re[m], br), make_float2(im[m], bi)};
         }
     }
-    pk::dft16<NZ>(P);   // P[k] = (X_{2k}, X_{2k+1})
+    cod::dft16<NZ>(P);   // P[k] = (X_{2k}, X_{2k+1})
     // element (output r, butterfly j) at 32 r + (j ^ (r & 1)), rows 2 mod 16 elements apart: a
     // half-warp (8 sequences, 2 butterflies or 2 jobs) falls in 16 different 8-byte banks
 #pragma unroll
@@ -216,7 +216,7 @@ k_pass1q(SearchLoad2S<Cfg2<LOGN, 1>> ld, ScratchStore2<Cfg2<LOGN, 1>> st, const 
         const float4 v = __ldg(tws + m * 32 + j);
         Q[m] = pk::cmul(Q[m], PC{make_float2(v.x, v.y), make_float2(v.z, v.w)});
     }
-    pk::dft16<16>(Q);   // Q[k] = (Y_2k, Y_2k+1): l2 = j + 32 (2k + e)
+    cod::dft16<16>(Q);   // Q[k] = (Y_2k, Y_2k+1): l2 = j + 32 (2k + e)
     float re[32], im[32];
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
@@ -395,7 +395,7 @@ k_pass2p(RowsTMA<Cfg2<LOGN, 2, TS>> ld, SearchEpi2<Cfg2<LOGN, 2, TS>, LOWER> ep,
             P[m] = pk::cmul(X, m ? pk::cmul(T, ld.tw_m(f, m)) : T);
         }
     }
-    pk::dft16<16>(P);   // P[k] = (X_{2k}, X_{2k+1}) of row l2
+    cod::dft16<16>(P);   // P[k] = (X_{2k}, X_{2k+1}) of row l2
     // the warp's exchange covers exactly the row f it has just read: only its own
     // lanes have to be done reading
     __syncwarp();
@@ -415,7 +415,7 @@ k_pass2p(RowsTMA<Cfg2<LOGN, 2, TS>> ld, SearchEpi2<Cfg2<LOGN, 2, TS>, LOWER> ep,
     }
 #pragma unroll
     for (int r = 1; r < 16; ++r) Q[r] = pk::cmul(Q[r], tw1(tws, r, j));
-    pk::dft16<16, LOWER>(Q);
+    cod::dft16<16, LOWER>(Q);
     // bins: job 2j + e, output p = u + t H: l1 = 2j + e + 32 p, bin = N2 l1 + l2
     constexpr int H = epi_half<LOWER>();
     epilogue<C, LOWER>(ep, t, C::N2 * (2 * j + kR0 * t * H) + l2, [](int u) { return C::N2 * kR0 * u; }, C::N2, Q);
@@ -505,7 +505,7 @@ k_pass2rows(const float2 *__restrict__ scratch, InterTw<LOGN / 2> tw, const floa
             Pm[m] = pk::cmul({make_float2(a.x, b.x), make_float2(a.y, b.y)}, F);
         }
     }
-    pk::dft16<16>(Pm);   // output k of butterfly j, both rows
+    cod::dft16<16>(Pm);   // output k of butterfly j, both rows
     __syncwarp();        // the staged rows have been read: the exchange may overwrite them
     // element (output k, butterfly j) of (t, g) at word (k R1 + j) ^ X(k) of its N1 words;
     // X sends the 8 lanes of a quarter-warp to 8 different 16-byte bank groups, storing
@@ -540,7 +540,7 @@ k_pass2rows(const float2 *__restrict__ scratch, InterTw<LOGN / 2> tw, const floa
 #pragma unroll
             for (int r = 1; r < R1; ++r) top = r & 1 ? pk::sub(top, z[r]) : pk::add(top, z[r]);
         }
-        pk::dft<R1, LOWER>(z);
+        cod::dft<R1, R1, LOWER>(z);
 #pragma unroll
         for (int p = 0; p < HR; ++p) Y[i * HR + p] = z[p];   // l1 = q + 16 p
     }
@@ -621,7 +621,7 @@ k_pass2q(RowsTMA<Cfg2<LOGN, 2, 64>> ld, SearchEpi2<Cfg2<LOGN, 2, 64>, LOWER> ep,
             P[m] = pk::cmul(X, m ? pk::cmul(T, ld.tw_m(0, m)) : T);
         }
     }
-    pk::dft16<16>(P);   // P[k] = (X_{2k}, X_{2k+1}) of butterfly j
+    cod::dft16<16>(P);   // P[k] = (X_{2k}, X_{2k+1}) of butterfly j
     __syncthreads();    // the staged row has been read: the exchange may overwrite it
     // element (output r, butterfly j) at 32 r + (j ^ r ^ 8 t): a half-warp holds 8 j (or,
     // loading, 8 r) of both transforms and falls in 16 different 8-byte banks either way
@@ -647,7 +647,7 @@ k_pass2q(RowsTMA<Cfg2<LOGN, 2, 64>> ld, SearchEpi2<Cfg2<LOGN, 2, 64>, LOWER> ep,
         const float4 v = __ldg(tws + m * 32 + q);
         Q[m] = pk::cmul(Q[m], PC{make_float2(v.x, v.y), make_float2(v.z, v.w)});
     }
-    pk::dft16<16, LOWER>(Q);   // Q[k] = (Y_2k, Y_2k+1): l1 = q + 32 (2k + e)
+    cod::dft16<16, LOWER>(Q);   // Q[k] = (Y_2k, Y_2k+1): l1 = q + 32 (2k + e)
     constexpr int H = epi_half<LOWER>();
     epilogue<C, LOWER>(ep, t, C::N2 * (q + 64 * t * H) + l2, [](int u) { return C::N2 * 64 * u; }, C::N2 * 32, Q);
 }
