@@ -489,8 +489,8 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
         if (j < i) { b.up = p.bands[j].up; continue; }
         const size_t H = size_t(1) << b.up.logh;
         const TwiddleSet *tw = p.twiddles(b.up.logh);
-        b.up.w_rows = tw->in1_d;
-        b.up.w_cols = tw->in2_d;
+        b.up.w_rows = reinterpret_cast<const double2 *>(tw->in1_d);
+        b.up.w_cols = reinterpret_cast<const double2 *>(tw->in2_d);
         double2 *ab = dalloc<double2>(p, 2 * H * (size_t)(U - 1), n_alloc);
         double2 *it = dalloc<double2>(p, H, n_alloc);
         p.launches += launch_upsample_tables(b.n, U, b.up, ab, it, p.scratch, s);

@@ -77,7 +77,7 @@ struct UpsampleTables {
     int logh = 0;                    // half of the convolution length: H = 2^logh complex points
     const double2 *ab = nullptr;     // [U - 1][l2][l1][2]: the kernel's transform as (alpha, beta)
     const double2 *tw = nullptr;     // W_H^{k1 l2}, [l2][k1]
-    const double *w_cols = nullptr, *w_rows = nullptr;   // W_N2^k, W_N1^k
+    const double2 *w_cols = nullptr, *w_rows = nullptr;   // W_N2^k, W_N1^k
 };
 
 // Partial sums of x^2 per band.

@@ -20,16 +20,14 @@
 // Three launches, H = N1 N2: columns (k2 -> l2); pairs of rows (l2, N2 - l2), which
 // hold each other's partners: k1 -> l1, the product, and straight back l1 -> k1;
 // columns (l2 -> k2) and the interleaved store.
-// The FP64 units (1/64 of the FP32 rate) bound the three; the tiles are one warp's
-// work or two, so that even short series spread over the SMs.
+// The FP64 units (1/64 of the FP32 rate) bound the three.
 // Measured on GB300 for a band of a search (with k_band_inputs), U = 2, against a
-// Bluestein transform each way (23 launches): n = 86 164 390 -> 92 us, n = 344 656
-// 1521 -> 188 us, n = 4096 113 -> 55 us.
+// Bluestein transform each way (23 launches): n = 86 164 390 -> 54 us, n = 344 656
+// 1521 -> 186 us, n = 4096 113 -> 26 us.
 #include <math.h>
 
 #include <algorithm>
 
-#include "fft_engine.cuh"
 #include "dfloat.cuh"
 #include "fstat_internal.h"
 #include "reduce64.cuh"
@@ -38,261 +36,206 @@ namespace fstat {
 
 namespace {
 
-constexpr int kTS = 32;            // target threads per CTA
+constexpr int kTS = 128;           // target threads per CTA
 constexpr int kMinLogH = kMinLogN - 1, kMaxLogH = kMaxLogN - 1;
 
+// Sequences of length M on M / 4 threads each, 4 elements per thread: 2^17 points make a
+// thousand warps, enough for the FP64 units of all SM quarters (16 elements per thread
+// made 256 warps and left half of the units idle).
 template <int LOGH, int PASS>      // PASS 1: columns (length N2), 2: rows (length N1)
 struct CfgU {
     static constexpr int N1 = 1 << (LOGH / 2), N2 = 1 << (LOGH - LOGH / 2), H = 1 << LOGH;
     static constexpr int M = PASS == 1 ? N2 : N1;
-    static constexpr int PAIRS = (PASS == 1 ? N1 : N2) / 2;
-    static constexpr int EH = 8;
-    static constexpr int F0 = kTS * EH / M;
-    static constexpr int F = F0 < 1 ? 1 : (F0 < PAIRS ? F0 : PAIRS);   // pairs per tile
-    static constexpr int THREADS = F * M / EH;
-    static constexpr int TILES = PAIRS / F;
-    static constexpr size_t PASS_SMEM = eng::smem_bytes<double, M, F>();
-    static constexpr size_t SMEM = PASS_SMEM + (PASS == 2 ? 2 * F * M * sizeof(double2) : 0);
+    static constexpr int TPS = M / 4;                                    // threads per sequence
+    static constexpr int COUNT = PASS == 1 ? N1 : N2;                    // sequences
+    static constexpr int F0 = kTS / TPS, F1 = F0 < COUNT ? F0 : COUNT;
+    static constexpr int F = F1 < PASS ? PASS : F1;                      // sequences per CTA (rows: pairs)
+    static constexpr int THREADS = F * TPS;
+    static constexpr int TILES = COUNT / F;
+    static constexpr int LD = M + M / 8;                                 // exchange row
+    static constexpr size_t SMEM = (size_t)F * (LD + (PASS == 2 ? M : 0)) * sizeof(double2);
+    static_assert(M >= 8 && THREADS <= 1024, "tile shape");
 };
 
-// Columns 2f, 2f + 1 of the tile: z[m] = x[2m] + i x[2m + 1], zero beyond n.
-template <class C>
-struct SeriesLoad {
-    const double *x;
-    int64_t n;
-    int c0;
-    __device__ __forceinline__ double2 z(int64_t m) const {
-        if (2 * m + 1 < n) return __ldg(reinterpret_cast<const double2 *>(x) + m);
-        return make_double2(2 * m < n ? __ldg(x + 2 * m) : 0.0, 0.0);
+__device__ __forceinline__ int padu(int i) { return i + (i >> 3); }
+__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
+    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+__device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ double2 conj_if(bool c, double2 a) { return c ? make_double2(a.x, -a.y) : a; }
+
+// DFT of one sequence (direction DIR), Stockham radix 4 and a last radix 2 for odd log2 M:
+// ld(i) gives element i, st(i, v) takes output i; thread j < M / 4; w[k] = e^{-2 pi i k / M};
+// ex is the sequence's exchange row.  HALF: the upper half of the inputs is zero (not read).
+template <int M, int DIR, class LD, class ST>
+__device__ __forceinline__ void dft_seq(int j, const double2 *__restrict__ w, double2 *ex, bool half, LD ld, ST st) {
+    constexpr int Q = M / 4;
+    double2 x[4];
+    x[0] = ld(j);
+    x[1] = ld(j + Q);
+    if (half) {
+        const double2 t = DIR < 0 ? make_double2(x[1].y, -x[1].x) : make_double2(-x[1].y, x[1].x);   // DIR i x1
+        const double2 a = x[0], b = x[1];
+        x[0] = cadd(a, b);
+        x[1] = cadd(a, t);
+        x[2] = csub(a, b);
+        x[3] = csub(a, t);
+    } else {
+        x[2] = ld(j + 2 * Q);
+        x[3] = ld(j + 3 * Q);
     }
-    template <int R, int JPF>
-    __device__ __forceinline__ void load(int f, int j, double *ra, double *ia, double *rb, double *ib) const {
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int64_t m = c0 + 2 * f + (int64_t)C::N1 * (j + r * JPF);
-            const double2 a = z(m), b = z(m + 1);
-            ra[r] = a.x; ia[r] = a.y; rb[r] = b.x; ib[r] = b.y;
-        }
-    }
-};
-
-// Transposed store A[l2][k1] with the four-step twiddle W_H^{k1 l2} (table in the
-// same order).
-template <class C>
-struct ColumnStore {
-    double2 *A;
-    const double2 *tw;
-    int c0;
-    template <int R, int JPF>
-    __device__ __forceinline__ void store(int f, int j, double *ra, double *ia, double *rb, double *ib) const {
+    for (int Ns = 1; Ns <= Q; Ns *= 4) {
+        const int k = j & (Ns - 1);
+        if (Ns > 1) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int64_t i = (int64_t)(j + r * JPF) * C::N1 + c0 + 2 * f;
-            const double2 ta = __ldg(tw + i), tb = __ldg(tw + i + 1);
-            A[i] = make_double2(ra[r] * ta.x - ia[r] * ta.y, ra[r] * ta.y + ia[r] * ta.x);
-            A[i + 1] = make_double2(rb[r] * tb.x - ib[r] * tb.y, rb[r] * tb.y + ib[r] * tb.x);
-        }
-    }
-};
-
-// Rows of pair p: p and N2 - p, or the two that are their own partners, 0 and N2/2.
-template <class C>
-struct RowPair {
-    int p0;
-    __device__ __forceinline__ int a(int f) const { return p0 + f; }
-    __device__ __forceinline__ int b(int f) const { return p0 + f == 0 ? C::N2 / 2 : C::N2 - (p0 + f); }
-};
-
-template <class C>
-struct RowLoad {
-    const double2 *A;
-    RowPair<C> rows;
-    template <int R, int JPF>
-    __device__ __forceinline__ void load(int f, int j, double *ra, double *ia, double *rb, double *ib) const {
-        const double2 *a = A + (int64_t)rows.a(f) * C::N1, *b = A + (int64_t)rows.b(f) * C::N1;
+            for (int r = 0; r < 4; ++r) x[r] = ex[padu(j + r * Q)];
+            __syncthreads();
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const double2 va = a[j + r * JPF], vb = b[j + r * JPF];
-            ra[r] = va.x; ia[r] = va.y; rb[r] = vb.x; ib[r] = vb.y;
+            for (int r = 1; r < 4; ++r) x[r] = cmul(x[r], conj_if(DIR > 0, __ldg(w + k * r * (Q / Ns))));
         }
-    }
-};
-
-// Row transforms parked in shared memory (natural order).
-template <class C>
-struct RowPark {
-    double2 *z;   // [2 f + (0: a, 1: b)][N1]
-    template <int R, int JPF>
-    __device__ __forceinline__ void store(int f, int j, double *ra, double *ia, double *rb, double *ib) const {
+        if (Ns > 1 || !half) {
+            const double2 t0 = cadd(x[0], x[2]), t1 = csub(x[0], x[2]), t2 = cadd(x[1], x[3]), d = csub(x[1], x[3]);
+            const double2 t3 = DIR < 0 ? make_double2(d.y, -d.x) : make_double2(-d.y, d.x);
+            x[0] = cadd(t0, t2);
+            x[1] = cadd(t1, t3);
+            x[2] = csub(t0, t2);
+            x[3] = csub(t1, t3);
+        }
+        const int o = (j - k) * 4 + k;
+        if (Ns * 4 == M) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            z[(2 * f) * C::N1 + j + r * JPF] = make_double2(ra[r], ia[r]);
-            z[(2 * f + 1) * C::N1 + j + r * JPF] = make_double2(rb[r], ib[r]);
-        }
-    }
-};
-
-// alpha Z + beta conj(Z[H - k]); with k = N2 l1 + l2 the partner of (l2, l1) is
-// (N2 - l2, N1 - 1 - l1), or (0, -l1 mod N1) in row 0.
-template <class C>
-struct ProductLoad {
-    const double2 *z;
-    const double2 *ab;   // [l2][l1][2]
-    RowPair<C> rows;
-    __device__ __forceinline__ double2 one(double2 z0, double2 q, const double2 *t) const {
-        const double2 al = __ldg(t), be = __ldg(t + 1);
-        return make_double2(al.x * z0.x - al.y * z0.y + be.x * q.x + be.y * q.y,
-                            al.x * z0.y + al.y * z0.x + be.y * q.x - be.x * q.y);
-    }
-    template <int R, int JPF>
-    __device__ __forceinline__ void load(int f, int j, double *ra, double *ia, double *rb, double *ib) const {
-        const double2 *za = z + (2 * f) * C::N1, *zb = za + C::N1;
-        const int la = rows.a(f), lb = rows.b(f);
-        const bool self = la == 0;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int l1 = j + r * JPF;
-            const double2 qa = self ? za[(C::N1 - l1) & (C::N1 - 1)] : zb[C::N1 - 1 - l1];
-            const double2 qb = self ? zb[C::N1 - 1 - l1] : za[C::N1 - 1 - l1];
-            const double2 a = one(za[l1], qa, ab + 2 * ((int64_t)la * C::N1 + l1));
-            const double2 b = one(zb[l1], qb, ab + 2 * ((int64_t)lb * C::N1 + l1));
-            ra[r] = a.x; ia[r] = a.y; rb[r] = b.x; ib[r] = b.y;
-        }
-    }
-};
-
-// Inverse rows back to global memory, times conj(W_H^{k1 l2}).
-template <class C>
-struct RowStore {
-    double2 *B;
-    const double2 *tw;
-    RowPair<C> rows;
-    template <int R, int JPF>
-    __device__ __forceinline__ void store(int f, int j, double *ra, double *ia, double *rb, double *ib) const {
-        const int64_t a = (int64_t)rows.a(f) * C::N1, b = (int64_t)rows.b(f) * C::N1;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int k1 = j + r * JPF;
-            const double2 ta = __ldg(tw + a + k1), tb = __ldg(tw + b + k1);
-            B[a + k1] = make_double2(ra[r] * ta.x + ia[r] * ta.y, ia[r] * ta.x - ra[r] * ta.y);
-            B[b + k1] = make_double2(rb[r] * tb.x + ib[r] * tb.y, ib[r] * tb.x - rb[r] * tb.y);
-        }
-    }
-};
-
-template <class C>
-struct ColumnLoad {
-    const double2 *B;
-    int c0;
-    template <int R, int JPF>
-    __device__ __forceinline__ void load(int f, int j, double *ra, double *ia, double *rb, double *ib) const {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int64_t i = (int64_t)(j + r * JPF) * C::N1 + c0 + 2 * f;
-            const double2 a = B[i], b = B[i + 1];
-            ra[r] = a.x; ia[r] = a.y; rb[r] = b.x; ib[r] = b.y;
-        }
-    }
-};
-
-// xu[U k + s] = y[k]; the launch of sub-phase 1 also stores sub-phase 0, x itself.
-template <class C, typename TO>
-struct SeriesStore {
-    const double *x;
-    TO *xu;
-    int64_t n;
-    int U, s, c0;
-    __device__ __forceinline__ void put(int64_t m, double ye, double yo) const {
-        const int64_t k = 2 * m;
-        if (k >= n) return;
-        const bool odd = k + 1 < n;
-        if (U == 2 && odd) {   // four neighbours of the upsampled series
-            const double2 v = __ldg(reinterpret_cast<const double2 *>(x) + m);
-            if constexpr (sizeof(TO) == 4) {
-                reinterpret_cast<float4 *>(xu)[m] = make_float4((float)v.x, (float)ye, (float)v.y, (float)yo);
-            } else {
-                reinterpret_cast<double2 *>(xu)[2 * m] = make_double2(v.x, ye);
-                reinterpret_cast<double2 *>(xu)[2 * m + 1] = make_double2(v.y, yo);
-            }
+            for (int r = 0; r < 4; ++r) st(o + r * Ns, x[r]);
             return;
         }
-        xu[U * k + s] = (TO)ye;
-        if (odd) xu[U * (k + 1) + s] = (TO)yo;
-        if (s == 1) {
-            xu[U * k] = (TO)__ldg(x + k);
-            if (odd) xu[U * (k + 1)] = (TO)__ldg(x + k + 1);
-        }
-    }
-    template <int R, int JPF>
-    __device__ __forceinline__ void store(int f, int j, double *ra, double *ia, double *rb, double *ib) const {
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int64_t m = c0 + 2 * f + (int64_t)C::N1 * (j + r * JPF);
-            put(m, ra[r], ia[r]);
-            put(m + 1, rb[r], ib[r]);
-        }
+        for (int r = 0; r < 4; ++r) ex[padu(o + r * Ns)] = x[r];
+        __syncthreads();
     }
-};
-
-__device__ __forceinline__ unsigned char *up_smem() {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    return smem_raw;
+    // last stage of radix 2 (Ns = M / 2): butterflies j and j + M / 4
+    double2 y[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int k = j + h * Q;
+        const double2 a = ex[padu(k)], b = cmul(ex[padu(k + 2 * Q)], conj_if(DIR > 0, __ldg(w + k)));
+        y[h] = csub(a, b);
+        x[h] = cadd(a, b);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        st(j + h * Q, x[h]);
+        st(j + h * Q + 2 * Q, y[h]);
+    }
 }
 
+__device__ __forceinline__ double2 *up_smem() {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    return reinterpret_cast<double2 *>(smem_raw);
+}
+
+// Columns c of z[m] = x[2m] + i x[2m + 1] (zero beyond n), times W_H^{c l2}, to A[l2][c].
 template <int LOGH>
 __global__ void __launch_bounds__(CfgU<LOGH, 1>::THREADS)
 k_up_columns(const double *__restrict__ x, int64_t n, double2 *__restrict__ A, const double2 *__restrict__ tw,
-             const double *__restrict__ w) {
+             const double2 *__restrict__ w) {
     using C = CfgU<LOGH, 1>;
-    const int c0 = blockIdx.x * 2 * C::F;
-    SeriesLoad<C> ld{x, n, c0};
-    ColumnStore<C> st{A, tw, c0};
-    eng::run_pass<double, C::M, C::F, C::EH, -1, eng::kMapFJ>(ld, st, w);
+    const int f = (int)threadIdx.x % C::F, j = (int)threadIdx.x / C::F;   // consecutive threads: adjacent columns
+    const int c = blockIdx.x * C::F + f;
+    auto ld = [&](int i) {
+        const int64_t m = c + (int64_t)C::N1 * i;
+        if (2 * m + 1 < n) return __ldg(reinterpret_cast<const double2 *>(x) + m);
+        return make_double2(2 * m < n ? __ldg(x + 2 * m) : 0.0, 0.0);
+    };
+    auto st = [&](int i, double2 v) {
+        const int64_t q = (int64_t)i * C::N1 + c;
+        A[q] = cmul(v, __ldg(tw + q));
+    };
+    // z[m] = 0 from m = H / 2 on when n <= M / 2 (M = 2 H)
+    dft_seq<C::M, -1>(j, w, up_smem() + f * C::LD, n <= C::H, ld, st);
 }
 
-// grid.z: sub-phases.  A is read by every sub-phase, B holds one region each.
+// Rows: a CTA holds pairs p of rows, p and N2 - p, or the two that are their own partners, 0
+// and N2 / 2; sequence 2 q is the first row of its q-th pair, 2 q + 1 the second.
+template <class C>
+__device__ __forceinline__ int row_of(int tile, int f) {
+    const int p = tile * (C::F / 2) + (f >> 1);
+    return (f & 1) == 0 ? p : p == 0 ? C::N2 / 2 : C::N2 - p;
+}
+
+// k1 -> l1 of the pairs, alpha Z + beta conj(Z[H - k]), l1 -> k1 times conj(W_H^{k1 l2}).
+// With k = N2 l1 + l2 the partner of (l2, l1) is (N2 - l2, N1 - 1 - l1), or (0, -l1 mod N1)
+// in row 0.  grid.z: sub-phases; A is read by every one, B holds one region each.
 template <int LOGH>
 __global__ void __launch_bounds__(CfgU<LOGH, 2>::THREADS)
 k_up_rows(const double2 *__restrict__ A, double2 *__restrict__ B, const double2 *__restrict__ ab,
-          const double2 *__restrict__ tw, const double *__restrict__ w) {
+          const double2 *__restrict__ tw, const double2 *__restrict__ w) {
     using C = CfgU<LOGH, 2>;
-    const RowPair<C> rows{(int)blockIdx.x * C::F};
-    double2 *z = reinterpret_cast<double2 *>(up_smem() + C::PASS_SMEM);
-    RowLoad<C> ld{A, rows};
-    RowPark<C> park{z};
-    eng::run_pass<double, C::M, C::F, C::EH, -1, eng::kMapJ>(ld, park, w);
+    const int f = (int)threadIdx.x / C::TPS, j = (int)threadIdx.x % C::TPS;
+    const int l2 = row_of<C>(blockIdx.x, f);
+    double2 *ex = up_smem() + f * C::LD, *Z = up_smem() + C::F * C::LD;   // Z: [f][N1]
+    const int64_t row = (int64_t)l2 * C::N1;
+    dft_seq<C::M, -1>(j, w, ex, false, [&](int i) { return A[row + i]; }, [&](int i, double2 v) { Z[f * C::N1 + i] = v; });
     __syncthreads();
-    ProductLoad<C> pl{z, ab + 2 * (int64_t)C::H * blockIdx.z, rows};
-    RowStore<C> st{B + (int64_t)C::H * blockIdx.z, tw, rows};
-    eng::run_pass<double, C::M, C::F, C::EH, 1, eng::kMapJ>(pl, st, w);
+    const bool self = l2 == 0 || l2 == C::N2 / 2;
+    const double2 *mine = Z + f * C::N1, *other = self ? mine : Z + (f ^ 1) * C::N1;
+    const double2 *t = ab + 2 * ((int64_t)C::H * blockIdx.z + row);
+    auto ld = [&](int i) {
+        const double2 z = mine[i], q = other[l2 == 0 ? (C::N1 - i) & (C::N1 - 1) : C::N1 - 1 - i];
+        const double2 al = __ldg(t + 2 * i), be = __ldg(t + 2 * i + 1);
+        return make_double2(al.x * z.x - al.y * z.y + be.x * q.x + be.y * q.y,
+                            al.x * z.y + al.y * z.x + be.y * q.x - be.x * q.y);
+    };
+    double2 *out = B + (int64_t)C::H * blockIdx.z + row;
+    dft_seq<C::M, 1>(j, w, ex, false, ld, [&](int i, double2 v) {
+        const double2 e = __ldg(tw + row + i);
+        out[i] = make_double2(v.x * e.x + v.y * e.y, v.y * e.x - v.x * e.y);
+    });
 }
 
 // Plan time: the kernel's transform in the rows' order.
 template <int LOGH>
 __global__ void __launch_bounds__(CfgU<LOGH, 2>::THREADS)
-k_up_rows_forward(const double2 *__restrict__ A, double2 *__restrict__ Z, const double *__restrict__ w) {
+k_up_rows_forward(const double2 *__restrict__ A, double2 *__restrict__ Z, const double2 *__restrict__ w) {
     using C = CfgU<LOGH, 2>;
-    const RowPair<C> rows{(int)blockIdx.x * C::F};
-    double2 *z = reinterpret_cast<double2 *>(up_smem() + C::PASS_SMEM);
-    RowLoad<C> ld{A, rows};
-    RowPark<C> park{z};
-    eng::run_pass<double, C::M, C::F, C::EH, -1, eng::kMapJ>(ld, park, w);
-    __syncthreads();
-    for (int i = threadIdx.x; i < 2 * C::F * C::N1; i += C::THREADS) {
-        const int q = i / C::N1, l1 = i % C::N1;
-        Z[(int64_t)(q & 1 ? rows.b(q >> 1) : rows.a(q >> 1)) * C::N1 + l1] = z[i];
-    }
+    const int f = (int)threadIdx.x / C::TPS, j = (int)threadIdx.x % C::TPS;
+    const int64_t row = (int64_t)row_of<C>(blockIdx.x, f) * C::N1;
+    dft_seq<C::M, -1>(j, w, up_smem() + f * C::LD, false, [&](int i) { return A[row + i]; },
+                      [&](int i, double2 v) { Z[row + i] = v; });
 }
 
+// l2 -> k2 of the columns and the interleaved store xu[U k + s]; the launch's sub-phase 1
+// also stores sub-phase 0, x itself.
 template <int LOGH, typename TO>
 __global__ void __launch_bounds__(CfgU<LOGH, 1>::THREADS)
 k_up_output(const double2 *__restrict__ B, const double *__restrict__ x, TO *__restrict__ xu, int64_t n, int U,
-            const double *__restrict__ w) {
+            const double2 *__restrict__ w) {
     using C = CfgU<LOGH, 1>;
-    const int c0 = blockIdx.x * 2 * C::F;
-    ColumnLoad<C> ld{B + (int64_t)C::H * blockIdx.z, c0};
-    SeriesStore<C, TO> st{x, xu, n, U, (int)blockIdx.z + 1, c0};
-    eng::run_pass<double, C::M, C::F, C::EH, 1, eng::kMapFJ>(ld, st, w);
+    const int f = (int)threadIdx.x % C::F, j = (int)threadIdx.x / C::F;
+    const int c = blockIdx.x * C::F + f, s = (int)blockIdx.z + 1;
+    const double2 *in = B + (int64_t)C::H * blockIdx.z + c;
+    auto st = [&](int i, double2 y) {
+        const int64_t m = c + (int64_t)C::N1 * i, k = 2 * m;
+        if (k >= n) return;
+        const bool odd = k + 1 < n;
+        if (U == 2 && odd) {   // four neighbours of the upsampled series
+            const double2 v = __ldg(reinterpret_cast<const double2 *>(x) + m);
+            if constexpr (sizeof(TO) == 4) {
+                reinterpret_cast<float4 *>(xu)[m] = make_float4((float)v.x, (float)y.x, (float)v.y, (float)y.y);
+            } else {
+                reinterpret_cast<double2 *>(xu)[2 * m] = make_double2(v.x, y.x);
+                reinterpret_cast<double2 *>(xu)[2 * m + 1] = make_double2(v.y, y.y);
+            }
+            return;
+        }
+        xu[U * k + s] = (TO)y.x;
+        if (odd) xu[U * (k + 1) + s] = (TO)y.y;
+        if (s == 1) {
+            xu[U * k] = (TO)__ldg(x + k);
+            if (odd) xu[U * (k + 1)] = (TO)__ldg(x + k + 1);
+        }
+    };
+    dft_seq<C::M, 1>(j, w, up_smem() + f * C::LD, false, [&](int i) { return in[(int64_t)i * C::N1]; }, st);
 }
 
 template <typename TO>
