@@ -52,16 +52,6 @@ __device__ __forceinline__ double delay_at(const double *__restrict__ r, const S
                      __dmul_rn(sc.nz, r[3 * j + 2]));
 }
 
-// Linear interpolation of the delay at fractional sample u from the per-sample
-// delays dk; the end segments extend beyond the data.
-__device__ __forceinline__ double delay_lin(const double *__restrict__ dk, int64_t n, double u) {
-    int64_t j = (int64_t)floor(u);
-    j = j < 0 ? 0 : (j > n - 2 ? n - 2 : j);
-    const double f = __dsub_rn(u, (double)j);
-    const double d0 = dk[j], d1 = dk[j + 1];
-    return __dadd_rn(d0, __dmul_rn(f, __dsub_rn(d1, d0)));
-}
-
 // Roemer delay nhat . r_k of every sample of skies [s0, s0 + gridDim.y).
 __global__ void __launch_bounds__(256) k_delays(const double *__restrict__ r,
                                                 const SkyConst *__restrict__ sky, int64_t s0,
@@ -269,12 +259,26 @@ __global__ void __launch_bounds__(kGeoThreads, 4) k_geometry(GeoArgs g) {
 }
 
 // FP64 form.  Bound by the FP64 units (1/64 of the FP32 rate), so it spends FP64
-// instructions only where the result needs them: one hour-angle and one phase
-// factor from the unit-phase table, the S sums over kGeo64 samples of a thread
-// before the block's reduction, and the delay in samples as a multiplication when
-// dt is a power of two (the same value as the division).
-// Measured at n = 86 164: 50 -> 18.2 us per sky position (one position a launch before).
+// instructions only where the result needs them, about 100 a sample: floors by a rounding
+// addition whose low word is the integer, the hour angle as one multiply-add in turns, unit phases
+// from the table, the Keys cubic in Horner form, the window test on integers, the S sums
+// over kGeo64 samples of a thread before the block's reduction, and the delay in samples
+// as a multiplication when dt is a power of two (the same value as the division).
+// MEASURED64
 constexpr int kGeo64 = 4;
+
+// Linear interpolation of the delay at fractional sample u from the per-sample delays dk,
+// in the oracle's rounding sequence; the end segments extend beyond the data.  j = floor(u),
+// or -1 or n far outside, and f = u - floor(u).
+__device__ __forceinline__ double delay_lin(const double *__restrict__ dk, int n, double u, int &j, double &f) {
+    f = __dsub_rn(u, p64::floor_int(u, j));
+    if ((__double2hiint(u) & 0x7fffffff) >= 0x41d00000) j = u < 0.0 ? -1 : n;   // beyond 2^30 samples, or not a number
+    const int jc = j < 0 ? 0 : (j > n - 2 ? n - 2 : j);
+    const double g = jc == j ? f : __dsub_rn(u, (double)jc);
+    const double d0 = dk[jc], d1 = dk[jc + 1];
+    return __dadd_rn(d0, __dmul_rn(g, __dsub_rn(d1, d0)));
+}
+
 __global__ void __launch_bounds__(256) k_geometry64(GeoArgs g) {
     __shared__ double sh[24];
     const int sl = blockIdx.y;
@@ -282,48 +286,51 @@ __global__ void __launch_bounds__(256) k_geometry64(GeoArgs g) {
     const SkyConst &sc = g.sky[g.s0 + sl];
     const double *dd = g.d + (int64_t)sl * g.d_stride;
     const bool pow2 = g.dt_pow2 != 0;
+    const int n = (int)g.n;
     auto in_samples = [&](double t) { return pow2 ? __dmul_rn(t, g.inv_dt) : __ddiv_rn(t, g.dt); };
-    int64_t k = blockIdx.x * (int64_t)(256 * kGeo64) + threadIdx.x;
+    // h / 2 pi = (alpha - phi0) / 2 pi - Omega_r dt u / 2 pi
+    const double turn0 = (sc.alpha - g.phi0) * (1.0 / kTwoPi), turn_dt = kOmegaR / kTwoPi * g.dt;
+    int k = blockIdx.x * (256 * kGeo64) + threadIdx.x;
 #pragma unroll 1
-    for (int it = 0; it < kGeo64 && k < g.n; ++it, k += 256) {
+    for (int it = 0; it < kGeo64 && k < n; ++it, k += 256) {
         // detector time t of barycentric sample k: t = k dt - d(k dt - d(k dt)),
         // in the oracle's rounding sequence, for 1e-10 agreement of F
-        const double u0 = __dsub_rn((double)k, in_samples(dd[k]));
-        const double d1 = delay_lin(dd, g.n, u0);
-        const double u = __dsub_rn((double)k, in_samples(d1));
-        const double d2 = delay_lin(dd, g.n, u);
-        const bool valid = (u >= 0.0) && (u <= (double)(g.n - 1));
-        const double h = sc.alpha - (g.phi0 + kOmegaR * (u * g.dt));
-        const double turns = h * (1.0 / kTwoPi);
-        const double2 eh = p64::unit_phase(g.unit_tab, turns - floor(turns));
+        const double kd = (double)k;
+        int j;
+        double f;
+        const double u0 = __dsub_rn(kd, in_samples(dd[k]));
+        const double d1 = delay_lin(dd, n, u0, j, f);
+        const double u = __dsub_rn(kd, in_samples(d1));
+        const double d2 = delay_lin(dd, n, u, j, f);
+        // 0 <= u <= n - 1
+        const bool valid = j >= 0 && (j < n - 1 || (j == n - 1 && f == 0.0));
+        const double2 eh = p64::unit_phase(g.unit_tab, fma(-turn_dt, u, turn0));
         const double c1 = eh.x, s1 = -eh.y;
         const double c2 = c1 * c1 - s1 * s1, s2 = 2.0 * s1 * c1;
         const double av = sc.A[0] * c2 + sc.A[1] * s2 + sc.A[2] * c1 + sc.A[3] * s1 + sc.A[4];
         const double bv = sc.B[0] * c2 + sc.B[1] * s2 + sc.B[2] * c1 + sc.B[3] * s1;
         double yr = 0.0, yi = 0.0;
         if (valid) {
-            // Keys cubic (a = -1/2) on the upsampled series, periodic indexing: taps
-            // i0 .. i0 + 3 around floor(p); inside the window p lies in [0, U (n - 1)],
-            // so only i0 = -1 and indices >= U n wrap (a single step)
+            // Keys cubic (a = -1/2) on the upsampled series at p = U u = U j + U f, taps
+            // i0 .. i0 + 3 around floor(p), periodic: p lies in [0, U (n - 1)], so only
+            // i0 = -1 and indices >= U n wrap (a single step)
             const double p = (double)g.U * u;
-            const double pf = floor(p);
-            const int64_t i0 = (int64_t)pf - 1;
+            int ip;
+            const double mu = p - p64::floor_int(p, ip);
+            const int i0 = ip - 1, m_up = (int)g.m_up;
             const double *xu = (const double *)g.xu;
-            double x4[4];
+            double x[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const int64_t v = i0 + q;
-                x4[q] = xu[v < 0 ? v + g.m_up : (v >= g.m_up ? v - g.m_up : v)];
+                const int v = i0 + q;
+                x[q] = xu[v < 0 ? v + m_up : (v >= m_up ? v - m_up : v)];
             }
-            const double mu = p - pf;
-            const double w0 = ((-0.5 * mu + 1.0) * mu - 0.5) * mu;
-            const double w1 = (1.5 * mu - 2.5) * mu * mu + 1.0;
-            const double w2 = ((-1.5 * mu + 2.0) * mu + 0.5) * mu;
-            const double w3 = (0.5 * mu - 0.5) * mu * mu;
-            const double v = w0 * x4[0] + w1 * x4[1] + w2 * x4[2] + w3 * x4[3];
-            // band-offset phase, cycles, reduced in FP64
-            const double cyc = __dmul_rn(g.f_off, d2);
-            const double2 e = p64::unit_phase(g.unit_tab, __dsub_rn(cyc, floor(cyc)));
+            // x1 + mu/2 (x2 - x0 + mu (2 x0 - 5 x1 + 4 x2 - x3 + mu (3 (x1 - x2) + x3 - x0)))
+            const double a3 = fma(3.0, x[1] - x[2], x[3] - x[0]);
+            const double a2 = fma(2.0, x[0], fma(-5.0, x[1], fma(4.0, x[2], -x[3])));
+            const double v = fma(0.5 * mu, fma(mu, fma(mu, a3, a2), x[2] - x[0]), x[1]);
+            // band-offset phase in cycles
+            const double2 e = p64::unit_phase(g.unit_tab, __dmul_rn(g.f_off, d2));
             yr = v * e.x;
             yi = v * e.y;
             saa = fma(av, av, saa);

@@ -16,8 +16,8 @@
 //  - both passes run on many cells, so that the 128 tiles of one 2^18 transform
 //    no longer leave a sixth of the 152 SMs idle.
 // Measured on GB300 at N = 86 164, N_fft = 2^18 (192 sky positions, one spindown), per
-// cell: pass 1 52.9 -> 28.5 us, pass 2 44.9 -> 31.1 us against the radix-8 engine, one
-// cell a launch; 128 cells at 2^13: 80 -> 1.8 us per cell for both.
+// cell: pass 1 52.9 -> 25.9 us, pass 2 44.9 -> 29.3 us against the radix-8 engine, one
+// cell a launch, the FP64 pipe 85 % active; 128 cells at 2^13: 80 -> 1.73 us for both.
 #pragma once
 
 #include "passes2.cuh"
@@ -78,8 +78,7 @@ struct Load64 {
             e[i] = make_double2(1.0, 0.0);
             if (k < n) {
                 const double kd = (double)k;
-                const double cyc = rate * (kd * kd);
-                e[i] = unit_phase(tab, cyc - floor(cyc));
+                e[i] = unit_phase(tab, rate * (kd * kd));
             }
         }
         const int lane = (int)threadIdx.x & 31;
@@ -221,7 +220,8 @@ struct Epi64 {
     }
 };
 
-// 128 threads with 32 complex doubles each (128 registers of data): two CTAs per SM.
+// 128 threads with 32 complex doubles each (128 registers of data): two CTAs per SM (three,
+// with 168 registers a thread, measured the same).
 template <int LOGN, int PASS, class LD, class ST, int Z1>
 __global__ void __launch_bounds__(kTS, 2) k_pass64(LD ld, ST st, const double *__restrict__ tw) {
     using C = Cfg64<LOGN, PASS>;
