@@ -392,11 +392,20 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
         p.w_stride = std::max<int64_t>(p.w_stride, (b.n + n1 - 1) / n1 * n1);
     }
     const int64_t nblk = (p.n_max + 1023) / 1024;   // blocks of a geometry launch per position
-    // sky positions per batch: 64, or up to 256 when the spindowns are few, so that a
-    // batch holds the 4096 cells of a launch pair
+    // sky positions per batch: 64, or up to 1024 when the spindowns are few, so that a batch
+    // holds the 4096 cells of a launch pair; above 256 as far as both w buffers stay within
+    // 2 GiB; batches of equal size.  Measured with one spindown, 1024 positions of N = 86 164:
+    // batches of 64 3.25 ms, 256 2.84, 512 2.79, 1024 2.77.
+    auto fp32_batch = [&]() -> int64_t {
+        const int64_t fill = (4096 + d->n_spin - 1) / d->n_spin;
+        const int64_t room = std::max<int64_t>(256, (int64_t(1) << 31) / (2 * 16 * p.w_stride));
+        const int64_t most = std::max<int64_t>(64, std::min<int64_t>(std::min<int64_t>(1024, room), fill));
+        const int64_t batches = (d->n_sky + most - 1) / most;
+        return (d->n_sky + batches - 1) / batches;
+    };
     // FP64 form: up to 64 positions whose series (32 bytes a sample) fill 128 MiB: the FP64
     // kernels are bound by their arithmetic, a batch only has to fill the SMs and hide latency
-    p.sky_batch = fp32 ? std::min<int64_t>(d->n_sky, std::max<int64_t>(64, std::min<int64_t>(256, (4096 + d->n_spin - 1) / d->n_spin)))
+    p.sky_batch = fp32 ? fp32_batch()
                        : std::min<int64_t>(d->n_sky, std::max<int64_t>(1, std::min<int64_t>(64, (int64_t(128) << 20) / (32 * p.w_stride))));
     if (fp32)
         if (const char *v = getenv("FSTAT_SKY_BATCH")) p.sky_batch = std::max<int64_t>(1, std::min<int64_t>(d->n_sky, atoll(v)));

@@ -93,7 +93,7 @@ struct BandDev {
     double *x = nullptr;      // [n] float64 (converted from float32 when needed)
     float *x32 = nullptr;     // [n] staging of a float32 series (allocated on first use)
     double *r = nullptr;      // [3n]
-    void *r2 = nullptr;       // FP32 form: r as double-float pairs (DF[3n]), redone per search
+    void *r2 = nullptr;       // FP32 form: r as double-float pairs, DF[3][n], redone per search
     void *xu = nullptr;       // [U n]: double (FP64 form) or float (FP32 form)
     UpsampleTables up;
 };

@@ -85,9 +85,36 @@ constexpr int kGeoThreads = 256, kGeoPer = kGeo32 / kGeoThreads;
 constexpr int kGeoMargin = 4;                // samples before the first segment
 constexpr int kGeoWin = kGeo32 + 12;         // window length
 
-__device__ __forceinline__ DF delay_df(const DF *__restrict__ r2, DF nx, DF ny, DF nz, int j) {
-    const DF *rj = r2 + 3 * j;
-    return df_dot3(nx, rj[0], ny, rj[1], nz, rj[2]);
+// r2: the x, y and z of every sample, one component after the other (coalesced).
+__device__ __forceinline__ DF delay_df(const DF *__restrict__ r2, int n, DF nx, DF ny, DF nz, int j) {
+    return df_dot3(nx, r2[j], ny, r2[n + j], nz, r2[2 * n + j]);
+}
+
+// x = I + f: I the integer nearest to the high part, |f| <= 1/2 up to the low part.
+__device__ __forceinline__ int df_split_near(DF x, float &f) {
+    const float r = rintf(x.hi);
+    f = (x.hi - r) + x.lo;
+    return (int)r;
+}
+
+// cos and sin of 2 pi c: the nearest quarter turn and Taylor series in the rest, |r| <= 1/8
+// (first terms left out: 2 pi r ^11/11! and ^10/10!, below 2.5e-8), |c| < 2^20.
+__device__ __forceinline__ void unit_f(float c, float &cs, float &sn) {
+    constexpr float magic = 12582912.f;   // 1.5 2^23: the low bits of the sum are the integer
+    const float qm = fmaf(c, 4.f, magic);
+    const int q = __float_as_int(qm);
+    const float r = fmaf(qm - magic, -0.25f, c), r2 = r * r;
+    constexpr double T = 6.283185307179586476925286766559, T2 = T * T;
+    const float s = r * fmaf(r2, fmaf(r2, fmaf(r2, fmaf(r2, (float)(T * T2 * T2 * T2 * T2 / 362880.0),
+                                                        (float)(-T * T2 * T2 * T2 / 5040.0)),
+                                               (float)(T * T2 * T2 / 120.0)), (float)(-T * T2 / 6.0)), (float)T);
+    const float k = fmaf(r2, fmaf(r2, fmaf(r2, fmaf(r2, (float)(T2 * T2 * T2 * T2 / 40320.0),
+                                                    (float)(-T2 * T2 * T2 / 720.0)),
+                                           (float)(T2 * T2 / 24.0)), (float)(-T2 / 2.0)), 1.f);
+    const bool odd = q & 1;
+    const float a = odd ? s : k, b = odd ? k : s;
+    cs = __int_as_float(__float_as_int(a) ^ (((q + 1) & 2) << 30));
+    sn = __int_as_float(__float_as_int(b) ^ ((q & 2) << 30));
 }
 
 // Sums over the 32 lanes of the 16 values v[0 .. 15] at once: each step halves the
@@ -109,7 +136,7 @@ __device__ __forceinline__ float warp_sum16(float *v) {
 
 __global__ void __launch_bounds__(kGeoThreads, 4) k_geometry(GeoArgs g) {
     __shared__ DF win[kGeoWin];
-    __shared__ float cf[11];
+    __shared__ float4 cf[3];   // A0 .. A4, B0 .. B3, cos and sin of the reference angle
     __shared__ int s_js;
     __shared__ float sums[3][kGeoThreads / 32 * kGeoPer];
     const int n = (int)g.n, tid = threadIdx.x, sl = blockIdx.y;
@@ -120,15 +147,13 @@ __global__ void __launch_bounds__(kGeoThreads, 4) k_geometry(GeoArgs g) {
     auto in_samples = [&](DF d) {   // d / dt; a power of two scales both parts exactly
         return pow2 ? DF{d.hi * g.inv_dt2.hi, d.lo * g.inv_dt2.hi} : df_mul(d, g.inv_dt2);
     };
-    // segment start (before clamping) and fraction at the tile's own samples
+    // u0 = k - d_k / dt = a0 - ph at the tile's own samples
     int a0[kGeoPer];
     float ph[kGeoPer];
 #pragma unroll
     for (int i = 0; i < kGeoPer; ++i) {
         const int k = min(k0 + tid + i * kGeoThreads, n - 1);
-        float phi;
-        a0[i] = k - (int)df_split_floor(in_samples(delay_df(g.r2, nx, ny, nz, k)), &phi);   // u0 = a0 - phi
-        ph[i] = phi;
+        a0[i] = k - df_split_near(in_samples(delay_df(g.r2, n, nx, ny, nz, k)), ph[i]);
     }
     if (tid == 0) s_js = min(max(a0[0] - 1 - kGeoMargin, -(kGeoWin - 4)), n - 4);
     __syncthreads();
@@ -136,17 +161,18 @@ __global__ void __launch_bounds__(kGeoThreads, 4) k_geometry(GeoArgs g) {
 #pragma unroll
     for (int i = 0; i < (kGeoWin + kGeoThreads - 1) / kGeoThreads; ++i) {
         const int e = tid + i * kGeoThreads;
-        if (e < kGeoWin) win[e] = delay_df(g.r2, nx, ny, nz, min(max(js + e, 0), n - 1));
+        if (e < kGeoWin) win[e] = delay_df(g.r2, n, nx, ny, nz, min(max(js + e, 0), n - 1));
     }
     const int mc = js + kGeoWin / 2;   // reference sample of the hour angle
+    float *cs = reinterpret_cast<float *>(cf);
     if (tid < 9) {
-        cf[tid] = tid < 5 ? (float)sc.A[tid] : (float)sc.B[tid - 5];
+        cs[tid] = tid < 5 ? (float)sc.A[tid] : (float)sc.B[tid - 5];
     } else if (tid == 32) {
         // h = alpha - phi0 - Omega_r dt mc, reduced in turns
         float fr;
         df_split_floor(df_add(df_add(DF{sc.nf[6], sc.nf[7]}, df_neg(g.phi0_turns)),
                               df_neg(df_mul(g.turn_dt, DF{(float)mc, 0.f}))), &fr);
-        sincospif(2.f * fr, &cf[10], &cf[9]);
+        sincospif(2.f * fr, &cs[10], &cs[9]);
     }
     __syncthreads();
     float sv[16];
@@ -162,18 +188,18 @@ __global__ void __launch_bounds__(kGeoThreads, 4) k_geometry(GeoArgs g) {
                 d0 = win[e];
                 d1 = win[e + 1];
             } else {
-                d0 = delay_df(g.r2, nx, ny, nz, j);
-                d1 = delay_df(g.r2, nx, ny, nz, j + 1);
+                d0 = delay_df(g.r2, n, nx, ny, nz, j);
+                d1 = delay_df(g.r2, n, nx, ny, nz, j + 1);
             }
         };
         // detector time t of barycentric sample k, t = k dt - d(k dt - d(k dt)),
         // as u = t / dt = A - F1: A an exact integer, F1 an FP32 fraction
-        const int j0 = min(max(a0[i] - 1, 0), n - 2);
+        const int j0 = min(max(a0[i] - (ph[i] > 0.f ? 1 : 0), 0), n - 2);
         const float f0 = (float)(a0[i] - j0) - ph[i];     // u0 - j0
         DF d0, d1;
         delay2(j0, d0, d1);
         float phi0;
-        const int A = k - (int)df_split_floor(in_samples(d0), &phi0);
+        const int A = k - df_split_near(in_samples(d0), phi0);
         const float F1 = phi0 + f0 * (((d1.hi - d0.hi) + (d1.lo - d0.lo)) * g.inv_dt2.hi);
         const float fl1 = floorf(-F1);
         int j = A + (int)fl1;
@@ -198,17 +224,14 @@ __global__ void __launch_bounds__(kGeoThreads, 4) k_geometry(GeoArgs g) {
         } else {
             sincosf(dl, &sd, &cd);
         }
-        const float c1 = cf[9] * cd - cf[10] * sd, s1 = cf[10] * cd + cf[9] * sd;
+        const float4 q0 = cf[0], q1 = cf[1], q2 = cf[2];
+        const float c1 = q2.y * cd - q2.z * sd, s1 = q2.z * cd + q2.y * sd;
         const float c2 = c1 * c1 - s1 * s1, s2 = 2.f * s1 * c1;
-        const float av = cf[0] * c2 + cf[1] * s2 + cf[2] * c1 + cf[3] * s1 + cf[4];
-        const float bv = cf[5] * c2 + cf[6] * s2 + cf[7] * c1 + cf[8] * s1;
+        const float av = q0.x * c2 + q0.y * s2 + q0.z * c1 + q0.w * s1 + q1.x;
+        const float bv = q1.y * c2 + q1.z * s2 + q1.w * c1 + q2.x * s1;
         float yr = 0.f, yi = 0.f;
         if (valid) {
             const float mu = up - upf;
-            const float w0 = ((-0.5f * mu + 1.f) * mu - 0.5f) * mu;
-            const float w1 = (1.5f * mu - 2.5f) * mu * mu + 1.f;
-            const float w2 = ((-1.5f * mu + 2.f) * mu + 0.5f) * mu;
-            const float w3 = (0.5f * mu - 0.5f) * mu * mu;
             const float *xu = (const float *)g.xu;
             const int m_up = (int)g.m_up;
             float x4[4];
@@ -222,16 +245,19 @@ __global__ void __launch_bounds__(kGeoThreads, 4) k_geometry(GeoArgs g) {
                     x4[q] = __ldg(xu + (v < 0 ? v + m_up : (v >= m_up ? v - m_up : v)));
                 }
             }
-            const float v = w0 * x4[0] + w1 * x4[1] + w2 * x4[2] + w3 * x4[3];
+            // x1 + mu/2 (x2 - x0 + mu (2 x0 - 5 x1 + 4 x2 - x3 + mu (3 (x1 - x2) + x3 - x0)))
+            const float a3 = fmaf(3.f, x4[1] - x4[2], x4[3] - x4[0]);
+            const float a2 = fmaf(2.f, x4[0], fmaf(-5.f, x4[1], fmaf(4.f, x4[2], -x4[3])));
+            const float v = fmaf(0.5f * mu, fmaf(mu, fmaf(mu, a3, a2), x4[2] - x4[0]), x4[1]);
             yr = v;
             if (g.f_off2.hi != 0.f) {   // uniform: a band at zero offset has no phase
                 // band-offset phase at t, cycles: f_off d_j mod 1 + f f_off (d_{j+1} - d_j)
                 if (j != j0) delay2(j, d0, d1);
-                float psi;
-                df_split_floor(df_mul(g.f_off2, d0), &psi);
-                const float cyc = psi + f * (g.f_off2.hi * ((d1.hi - d0.hi) + (d1.lo - d0.lo)));
+                const float p = __fmul_rn(g.f_off2.hi, d0.hi);
+                const float e = fmaf(g.f_off2.lo, d0.hi, fmaf(g.f_off2.hi, d0.lo, fmaf(g.f_off2.hi, d0.hi, -p)));
+                const float psi = (p - rintf(p)) + e;
                 float sp, cp;
-                sincospif(2.f * (cyc - rintf(cyc)), &sp, &cp);
+                unit_f(psi + f * (g.f_off2.hi * ((d1.hi - d0.hi) + (d1.lo - d0.lo))), cp, sp);
                 yr = v * cp;
                 yi = -v * sp;
             }

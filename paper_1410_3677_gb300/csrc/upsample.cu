@@ -303,8 +303,9 @@ __global__ void __launch_bounds__(256) k_band_inputs(const double *__restrict__ 
                                                      DF *__restrict__ r2) {
     __shared__ double sh[8];
     if (r2)
-        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 3 * n; i += (int64_t)gridDim.x * blockDim.x)
-            r2[i] = df_from_double(r[i]);
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) r2[c * n + i] = df_from_double(r[3 * i + c]);
     if (blockIdx.x >= kSigmaParts) return;
     KahanD k;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)kSigmaParts * blockDim.x)
@@ -413,7 +414,7 @@ int launch_upsample_tables(int64_t n, int U, UpsampleTables &t, double2 *ab, dou
 }
 
 int launch_band_inputs(const BandDev &b, double *sigma_parts, cudaStream_t s) {
-    const unsigned grid = b.r2 ? std::max<unsigned>(kSigmaParts, std::min<unsigned>(1024, blocks(3 * b.n, 256))) : kSigmaParts;
+    const unsigned grid = b.r2 ? std::max<unsigned>(kSigmaParts, std::min<unsigned>(1024, blocks(b.n, 256))) : kSigmaParts;
     k_band_inputs<<<grid, 256, 0, s>>>(b.x, b.n, sigma_parts, b.r, static_cast<DF *>(b.r2));
     return 1;
 }
