@@ -44,22 +44,37 @@ void check(cudaError_t e, const char *what) {
 struct OomError {};
 struct TimeoutError {};
 
+// Device memory of the plan.  Small arrays are cut from 1 MiB slabs: a cudaMalloc takes
+// about 10 us, and a plan holds some thirty tables and counters.  own: an allocation of its
+// own, which the caller frees before the plan does.
+constexpr size_t kSlab = size_t(1) << 20, kSmall = kSlab / 8;
 template <typename T>
-T *dalloc(Plan &p, size_t count, int &n_alloc) {
+T *dalloc(Plan &p, size_t count, int &n_alloc, bool own = false) {
     ++n_alloc;
     const int fail = alloc_fail_at();
     if (fail > 0 && n_alloc == fail) throw OomError{};
-    void *ptr = nullptr;
     const size_t bytes = std::max<size_t>(count * sizeof(T), 16);
-    cudaError_t e = cudaMalloc(&ptr, bytes);
-    if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        throw OomError{};
+    const bool small = !own && bytes <= kSmall;
+    const size_t room = (bytes + 255) / 256 * 256;
+    if (!small || p.slab_left < room) {
+        void *ptr = nullptr;
+        const size_t want = small ? kSlab : bytes;
+        cudaError_t e = cudaMalloc(&ptr, want);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            throw OomError{};
+        }
+        check(e, "cudaMalloc");
+        p.allocs.push_back(ptr);
+        p.device_bytes += (int64_t)want;
+        if (!small) return reinterpret_cast<T *>(ptr);
+        p.slab = static_cast<unsigned char *>(ptr);
+        p.slab_left = kSlab;
     }
-    check(e, "cudaMalloc");
-    p.allocs.push_back(ptr);
-    p.device_bytes += (int64_t)bytes;
-    return reinterpret_cast<T *>(ptr);
+    T *out = reinterpret_cast<T *>(p.slab);
+    p.slab += room;
+    p.slab_left -= room;
+    return out;
 }
 
 int ilog2_exact(int64_t v) {
@@ -1172,10 +1187,10 @@ fstat_status fstat_debug_sky(fstat_plan *p, int band, int64_t sky, double *y, do
         const size_t before = p->allocs.size();
         const int64_t bytes_before = p->device_bytes;
         try {
-            dy = dalloc<double>(*p, 2 * n, n_alloc);
-            da = dalloc<double>(*p, n, n_alloc);
-            db = dalloc<double>(*p, n, n_alloc);
-            dm = dalloc<uint8_t>(*p, n, n_alloc);
+            dy = dalloc<double>(*p, 2 * n, n_alloc, true);
+            da = dalloc<double>(*p, n, n_alloc, true);
+            db = dalloc<double>(*p, n, n_alloc, true);
+            dm = dalloc<uint8_t>(*p, n, n_alloc, true);
         } catch (...) {
             for (size_t i = before; i < p->allocs.size(); ++i) cudaFree(p->allocs[i]);
             p->allocs.resize(before);

@@ -110,6 +110,8 @@ struct Plan {
     int64_t launches = 0;
     int64_t device_bytes = 0;
     std::vector<void *> allocs;
+    unsigned char *slab = nullptr;   // rest of the slab that small arrays are cut from
+    size_t slab_left = 0;
 
     // grids (device, and host copies for candidate retrieval)
     double *alpha = nullptr, *delta = nullptr, *fdot = nullptr;
