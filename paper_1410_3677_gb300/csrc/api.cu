@@ -175,7 +175,7 @@ fstat_status validate(const fstat_plan_desc *d, std::string &err) {
 
 void host_twiddles(int logn, std::vector<double> &in1, std::vector<double> &in2,
                    std::vector<double> &lo, std::vector<double> &hi) {
-    const int64_t N = int64_t(1) << logn;
+    const int64_t N = int64_t(1) << log_n(logn);
     const int64_t N1 = int64_t(1) << log_n1(logn), N2 = int64_t(1) << log_n2(logn);
     auto w = [](int64_t k, int64_t M, double *o) {
         // e^{-2 pi i k / M} with k reduced to the first octant-free form
@@ -241,7 +241,7 @@ void build_twiddles(Plan &p, const std::vector<int> &logs, int &n_alloc) {
         stage1_twiddles(log_n1(lg), e);
         stage1_twiddles(log_n2(lg), f);
         if (log_n1(lg) == 9) packed512_twiddles(g);   // 512-point rows: N_fft = 2^18, 2^19
-        if (log_n2(lg) == 10) packed1024_twiddles(h);   // 1024-point columns or rows: 2^19, 2^20
+        if (log_n1(lg) == 10 || log_n2(lg) == 10) packed1024_twiddles(h);   // 1024-point columns or rows: 2^19, 2^20
         for (auto *v : {&a, &b, &c, &d, &e, &f, &g, &h}) {
             while (hd.size() % 4) hd.push_back(0.0);   // 16-byte aligned float tables
             offs.push_back(hd.size());
@@ -264,7 +264,7 @@ void build_twiddles(Plan &p, const std::vector<int> &logs, int &n_alloc) {
         t.s1_f = df + o[4]; t.s2_f = df + o[5];
         t.s1_d = dd + o[4]; t.s2_d = dd + o[5];
         if (log_n1(logs[i]) == 9) t.p512_f = reinterpret_cast<const float4 *>(df + o[6]);
-        if (log_n2(logs[i]) == 10) t.p1024_f = reinterpret_cast<const float4 *>(df + o[7]);
+        if (log_n1(logs[i]) == 10 || log_n2(logs[i]) == 10) t.p1024_f = reinterpret_cast<const float4 *>(df + o[7]);
         p.tw.push_back(t);
     }
 }
@@ -318,6 +318,7 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
         if (b.n_fft == 0) { b.n_fft = 1; while (b.n_fft < 2 * b.n) b.n_fft <<= 1; }
         b.logn = ilog2_exact(b.n_fft);
         need(b.logn);
+        if (fp32 && !p.interbin && b.logn == 19) need(kTall + b.logn);
         if (d->interpolation == FSTAT_INTERP_INTERBIN) need(b.logn - 1);
         if (d->bin_lo == 0 && d->bin_hi == 0) { b.lo = 1; b.hi = b.n_fft / 2 - 1; }
         else { b.lo = d->bin_lo; b.hi = d->bin_hi; }
@@ -350,7 +351,7 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
     build_twiddles(p, logs, n_alloc);
     for (auto &t : p.tw) {   // FP32 form: row factors of the packed rows, for the lengths the bands search
         const bool used = std::any_of(p.bands.begin(), p.bands.end(),
-                                      [&](const BandDev &b) { return b.logn - (p.interbin ? 1 : 0) == t.logn; });
+                                      [&](const BandDev &b) { return b.logn - (p.interbin ? 1 : 0) == log_n(t.logn); });
         if (!fp32 || !used || row_twiddle_entries(t.logn) == 0) continue;
         float4 *rt = dalloc<float4>(p, (size_t)row_twiddle_entries(t.logn), n_alloc);
         launch_row_twiddles(rt, t.logn, s);
@@ -399,11 +400,11 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
     check(cudaMemcpy(p.chirp_fx, cfx.data(), cfx.size() * sizeof(uint64_t), cudaMemcpyHostToDevice), "chirp");
     check(cudaMemcpy(p.chirp_d, cd.data(), cd.size() * sizeof(double), cudaMemcpyHostToDevice), "chirp");
 
-    // per-sky-batch buffers; w rows padded to a multiple of each band's N1 so that
+    // per-sky-batch buffers; w rows padded to a multiple of each band's longer factor so that
     // column tiles of the first FFT pass never read past a sky's stretch
     p.w_stride = p.n_max;
     for (auto &b : p.bands) {
-        const int64_t n1 = int64_t(1) << log_n1(b.logn);
+        const int64_t n1 = int64_t(1) << log_n2(b.logn);   // the longer factor, whichever the columns take
         p.w_stride = std::max<int64_t>(p.w_stride, (b.n + n1 - 1) / n1 * n1);
     }
     const int64_t nblk = (p.n_max + 1023) / 1024;   // blocks of a geometry launch per position
@@ -693,7 +694,8 @@ void enqueue_search(Plan &p, int64_t begin, int64_t end) {
         // transform length of the search (half of n_fft when interbinning)
         const int tlog = p.interbin ? b.logn - 1 : b.logn;
         const double nfft = (double)(int64_t(1) << tlog);
-        const double lg1 = (double)log_n1(tlog), lg2 = (double)log_n2(tlog);
+        const int key = fp32 ? search_key_f32(p, tlog) : tlog;
+        const double lg1 = (double)log_n1(key), lg2 = (double)log_n2(key);
         const int i_geo = stat_index(p, "geometry_resample");
         const int i_p1 = stat_index(p, fp32 ? "fft_pass1_f32" : "fft_pass1_f64");
         const int i_p2 = stat_index(p, fp32 ? "fft_pass2_fstat_f32" : "fft_pass2_fstat_f64");

@@ -22,12 +22,16 @@ constexpr int kMaxLogN = 20;   // n_fft <= 2^20
 // Split of a power-of-two transform length N = N1 * N2 into the two passes of
 // the four-step FFT: pass 1 transforms the N1 strided columns (length N2), pass
 // 2 the N2 rows (length N1).
-inline int log_n1(int logn) { return logn / 2; }
-inline int log_n2(int logn) { return logn - logn / 2; }
+// kTall + logn names the same length with the longer factor in the rows: the FP32 search of
+// 2^19 points runs 512-point columns and 1024-point rows (see launch_search_cells_f32).
+constexpr int kTall = 100;
+__host__ __device__ constexpr int log_n(int key) { return key % kTall; }
+__host__ __device__ constexpr int log_n1(int key) { return key < kTall ? key / 2 : log_n(key) - log_n(key) / 2; }
+__host__ __device__ constexpr int log_n2(int key) { return log_n(key) - log_n1(key); }
 
-// Twiddle tables of one transform length, forward direction e^{-2 pi i k / M}.
+// Twiddle tables of one transform length and split, forward direction e^{-2 pi i k / M}.
 struct TwiddleSet {
-    int logn = 0;
+    int logn = 0;   // the key: log2 N, or kTall + log2 N
     // device pointers, interleaved (re, im); float and double copies
     const double *in1_d = nullptr, *in2_d = nullptr, *lo_d = nullptr, *hi_d = nullptr;
     const float *in1_f = nullptr, *in2_f = nullptr, *lo_f = nullptr, *hi_f = nullptr;
@@ -311,6 +315,8 @@ inline cudaError_t record_timing_event(cudaEvent_t e, cudaStream_t s) {
 // Whether a band of transform length 2^logn (the n_fft bin grid) can run in the
 // interbinning form (a half-length transform of 2^12 .. 2^19).
 bool interbin_supported(int logn);
+// The split (log2 N, or kTall + log2 N) an FP32 search of length 2^logn runs with.
+int search_key_f32(const Plan &p, int logn);
 // Whether the FP32 cells of a band of length 2^logn run as one fused launch.
 bool fused_supported(const Plan &p, int logn);
 // `mid` (may be null) is recorded between the two passes.

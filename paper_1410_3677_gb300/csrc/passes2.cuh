@@ -20,11 +20,11 @@ namespace fstat {
 
 template <int LOGN, int PASS, int TS = 256>
 struct Cfg2 {
-    static constexpr int LOGN1 = LOGN / 2;
-    static constexpr int LOGN2 = LOGN - LOGN / 2;
+    static constexpr int LOGN1 = log_n1(LOGN);
+    static constexpr int LOGN2 = log_n2(LOGN);
     static constexpr int N1 = 1 << LOGN1;
     static constexpr int N2 = 1 << LOGN2;
-    static constexpr int N = 1 << LOGN;
+    static constexpr int N = 1 << log_n(LOGN);
     static constexpr int M = PASS == 1 ? N2 : N1;        // length of this pass's FFTs
     static constexpr int OTHER = PASS == 1 ? N1 : N2;    // number of such FFTs per transform
     static constexpr int EH = 32;

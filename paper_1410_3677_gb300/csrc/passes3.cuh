@@ -1,7 +1,7 @@
 // The FP32 search passes in packed arithmetic (packed.cuh) for passes of length
 // 512: both passes at N_fft = 2^18 (N1 = N2 = 512, the two-sidereal-day
-// segments), the rows (pass 2) at 2^19; the shorter rows of 2^12 .. 2^17; and
-// the 1024-point rows of 2^20.  Same four-step split, scratch layout, tiles and
+// segments), the shorter rows of 2^12 .. 2^17; and
+// the 1024-point rows of 2^19 and 2^20 and the 1024-point columns of 2^20.  Same four-step split, scratch layout, tiles and
 // launch shapes as the second engine's passes (passes2.cuh); what changes is how
 // a thread's 32 elements are transformed:
 //
@@ -161,12 +161,12 @@ k_pass1h(SearchLoad2<Cfg2<LOGN, 1>> ld, ScratchStore2<Cfg2<LOGN, 1>> st, const f
     st.template store<16, kR0>(q1, re1, im1);
 }
 
-// The columns of 1024 points (N_fft = 2^19 and 2^20): 256 threads, 4 columns x 2
+// The columns of 1024 points (N_fft = 2^20): 256 threads, 4 columns x 2
 // transforms, 32 threads per sequence.  Both radix-32 stages packed by one
 // decimation-in-frequency split each: stage 0 as in k_pass1p, stage 1 (one 32-point job
 // per thread) with its twiddle folded into the split as in k_pass2q below.
-// Measured per 2^18 points: 1.045 -> 1.014 us at 2^19, 1.056 -> 1.008 us at 2^20 (a third fewer
-// instructions than the scalar pass; the 64-byte runs of its loads and stores bound it now).
+// Measured per 2^18 points: 1.056 -> 0.961 us (a third fewer instructions than the scalar pass;
+// the 64-byte runs of its loads and stores cost it the rest against the 512-point columns).
 template <int LOGN, int Z1>
 __global__ void __launch_bounds__(256, 3)
 k_pass1q(SearchLoad2S<Cfg2<LOGN, 1>> ld, ScratchStore2<Cfg2<LOGN, 1>> st, const float4 *__restrict__ tws,
@@ -584,7 +584,7 @@ k_pass2rows(const float2 *__restrict__ scratch, InterTw<LOGN / 2> tw, const floa
 }
 
 // --------------------------------------------------------------------- pass 2, 1024-point rows
-// The rows of N_fft = 2^20 (N1 = 1024 = 32 x 32), a row of both transforms per
+// The rows of N_fft = 2^19 and 2^20 (N1 = 1024 = 32 x 32), a row of both transforms per
 // 64-thread CTA: thread 2j + t takes the elements k1 = j + 32 m of transform t.
 // Both radix-32 stages are split by one decimation-in-frequency step into a packed
 // 16-point DFT, the stage's twiddle folded into the split as in k_pass2p: with
@@ -593,8 +593,7 @@ k_pass2rows(const float2 *__restrict__ scratch, InterTw<LOGN / 2> tw, const floa
 // the pairs (X_2k, X_2k+1).  In stage 1 V_m = W_1024^{mq} and V_m W_32^m =
 // W_1024^{m(q+32)} come from one packed table.  A whole row per CTA (16 KiB, twelve
 // CTAs per SM) instead of the radix-8 engine's three stages and two exchanges.
-// Measured at N = 344 656 (768 cells): pass 1 and 2 together 13.4 -> 7.25 us a cell (pass 2
-// 5.36 -> 3.01 us).
+// Measured at N = 344 656 (768 cells): pass 2 5.36 -> 2.93 us a cell.
 template <int LOGN, bool LOWER>
 __global__ void __launch_bounds__(64, 12)
 k_pass2q(RowsTMA<Cfg2<LOGN, 2, 64>> ld, SearchEpi2<Cfg2<LOGN, 2, 64>, LOWER> ep,

@@ -166,7 +166,7 @@ int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_
             return 2;
         }
     }
-    if constexpr (LOGN == 20) {   // 1024-point rows: one per CTA, packed
+    if constexpr (C2::M == 1024) {   // 1024-point rows: one per CTA, packed
         using D2 = Cfg2<LOGN, 2, 64>;
         p3::RowsTMA<D2> lt{};
         lt.scratch = ld2.scratch;
@@ -343,11 +343,11 @@ int launch_interbin(const Plan &p, int band_idx, const BandDev &b, int64_t s0, i
 // (W_N^{G l2 m}, W_N^{G (l2+1) m}) of the rows l2 = 2i, 2i + 1 (N1 <= 256, G = N1 / 16).
 __global__ void k_row_twiddles(float4 *t, int logn) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int n1 = logn / 2, n2 = logn - n1;
+    const int n1 = log_n1(logn), n2 = log_n2(logn);
     const bool pairs = n1 <= 8;
     if (i >= (p3::kRowTw << (pairs ? n2 - 1 : n2))) return;
     const int e = i / p3::kRowTw, m = i % p3::kRowTw;
-    const double N = (double)(int64_t(1) << logn);
+    const double N = (double)(int64_t(1) << log_n(logn));
     const int64_t g = pairs ? 1 << (n1 - 4) : 1 << (n1 - 5);
     const double a = pairs ? (double)(g * 2 * e * m) / N : (double)(g * e * m) / N;
     const double b = pairs ? (double)(g * (2 * e + 1) * m) / N : a + (double)m / 32.0;
@@ -360,12 +360,21 @@ __global__ void k_row_twiddles(float4 *t, int logn) {
 }  // namespace
 
 int64_t row_twiddle_entries(int logn) {
-    const int n1 = logn / 2, n2 = logn - n1;
+    const int n1 = log_n1(logn), n2 = log_n2(logn);
     return n1 < 6 || n1 > 10 ? 0 : (int64_t)p3::kRowTw << (n1 <= 8 ? n2 - 1 : n2);
 }
 
 void launch_row_twiddles(float4 *t, int logn, cudaStream_t s) {
     k_row_twiddles<<<(unsigned)((row_twiddle_entries(logn) + 255) / 256), 256, 0, s>>>(t, logn);
+}
+
+// 2^19 points as 512-point columns and 1024-point rows: the columns move in 128-byte runs
+// where 1024-point columns have 64, and the packed 1024-point rows cost less than that.
+// Measured per 2^18 points, both passes: 0.977 + 0.627 -> 0.755 + 0.735 us (n <= 3N/8), 1.081 +
+// 0.627 -> 0.860 + 0.734 (n > 3N/8).
+int search_key_f32(const Plan &p, int logn) {
+    const bool tall = logn == 19 && p.engine == 2 && !p.interbin && !p.fused && p.packed >= 1 && p.tma && p.p2_threads == 128;
+    return tall ? kTall + logn : logn;
 }
 
 bool interbin_supported(int logn) { return logn - 1 >= 12 && logn - 1 <= 19; }
@@ -399,7 +408,9 @@ int launch_search_cells_f32(const Plan &p, int band_idx, const BandDev &b, int64
             case 16: return launch_search2<16>(p, band_idx, b, s0, c0, nc, s, mid, cb);
             case 17: return launch_search2<17>(p, band_idx, b, s0, c0, nc, s, mid, cb);
             case 18: return launch_search2<18>(p, band_idx, b, s0, c0, nc, s, mid, cb);
-            case 19: return launch_search2<19>(p, band_idx, b, s0, c0, nc, s, mid, cb);
+            case 19:
+                return search_key_f32(p, 19) == 19 ? launch_search2<19>(p, band_idx, b, s0, c0, nc, s, mid, cb)
+                                                   : launch_search2<kTall + 19>(p, band_idx, b, s0, c0, nc, s, mid, cb);
             case 20: return launch_search2<20>(p, band_idx, b, s0, c0, nc, s, mid, cb);
             default: break;
         }

@@ -93,6 +93,9 @@ def test_upsample(fs, n, U):
     (393216, 1 << 20, 2, 2, dict(dt=0.5, window=2000, full=True)),          # n = 3N/8
     (393217, 1 << 20, 2, 2, dict(dt=0.5, window=2000, full_range=True)),    # half of a column, both spectrum halves
     (524288, 1 << 20, 1, 2, dict(dt=0.5, window=2000, f_off=0.0)),          # n = N / 2
+    (172328, 1 << 19, 2, 3, dict(window=2000)),                             # 512-point columns
+    (196608, 1 << 19, 2, 2, dict(window=2000, full=True)),                  # n = 3N/8
+    (196609, 1 << 19, 2, 2, dict(window=2000, full_range=True)),
 ])
 def test_fp32_1024_point_rows(fs, n, n_fft, n_sky, n_spin, kw):
     _check(fs, fs.FP32_BATCHED, n, n_fft, n_sky, n_spin, **kw)
