@@ -935,13 +935,13 @@ void parallel_for_threads(int nt, Fn f) {
     for (auto &x : th) x.join();
 }
 
-// Sorts n records by (cell, bin), cells from cell0, in `rec` with `tmp` as the other
+// Sorts n records by (cell, bin), cells from cell0, bins from bin0, in `rec` with `tmp` as the other
 // buffer: least-significant-digit counting passes of up to 11 bits over the key bits of
 // the searched range.
-void sort_records(fstat::CandRecord *rec, fstat::CandRecord *tmp, int64_t n, uint32_t cell0, int bin_bits,
-                  int key_bits) {
+void sort_records(fstat::CandRecord *rec, fstat::CandRecord *tmp, int64_t n, uint32_t cell0, uint32_t bin0,
+                  int bin_bits, int key_bits) {
     using fstat::CandRecord;
-    auto key = [&](const CandRecord &r) { return ((uint64_t)(r.cell - cell0) << bin_bits) | r.bin; };
+    auto key = [&](const CandRecord &r) { return ((uint64_t)(r.cell - cell0) << bin_bits) | (r.bin - bin0); };
     if (n < 64) {
         std::sort(rec, rec + n, [&](const CandRecord &a, const CandRecord &b) { return key(a) < key(b); });
         return;
@@ -1024,8 +1024,14 @@ fstat_status fstat_candidates_get(fstat_plan *p, fstat_candidate *buf, int64_t c
         if (n_total) *n_total = p->last_total;
         if (cap == 0) return p->last_total > 0 ? FSTAT_ERR_OVERFLOW : FSTAT_OK;   // count only
         const int64_t kept = std::min<int64_t>(p->last_total, p->cand_capacity);
-        int bin_bits = 0, cell_bits = 0;
-        while ((int64_t(1) << bin_bits) < p->n_fft_max) ++bin_bits;
+        // sort key: the cell within the searched range, then the bin within the bands' bin range
+        int64_t bin0 = p->n_fft_max, bin1 = 0;
+        for (const BandDev &b : p->bands) {
+            bin0 = std::min(bin0, b.lo);
+            bin1 = std::max(bin1, b.hi);
+        }
+        int bin_bits = 1, cell_bits = 0;
+        while ((bin1 - bin0) >> bin_bits) ++bin_bits;
         const uint64_t span = (uint64_t)(p->cand_end - p->cand_begin);
         while ((span > 0 ? span - 1 : 0) >> cell_bits) ++cell_bits;
         // few records came to the host with the search's status
@@ -1068,7 +1074,7 @@ fstat_status fstat_candidates_get(fstat_plan *p, fstat_candidate *buf, int64_t c
         }
         if (dev_sort && !p->cand_sorted) {
             p->cand_sorted = launch_cand_sort(p->cand, p->cand_tmp, p->sort_hist, kept, (uint32_t)p->cand_begin,
-                                              cell_bits + bin_bits, bin_bits, p->stream, &p->launches);
+                                              (uint32_t)bin0, cell_bits + bin_bits, bin_bits, p->stream, &p->launches);
             check(cudaGetLastError(), "candidate sort");
         }
         if (kept > kEagerRecords && (dev_sort || !p->host_sorted)) {
@@ -1079,7 +1085,7 @@ fstat_status fstat_candidates_get(fstat_plan *p, fstat_candidate *buf, int64_t c
         }
         if (!dev_sort && kept > 0 && !p->host_sorted) {
             if ((int64_t)p->h_tmp.size() < kept) p->h_tmp.resize((size_t)kept);
-            sort_records(rec, p->h_tmp.data(), kept, (uint32_t)p->cand_begin, bin_bits, cell_bits + bin_bits);
+            sort_records(rec, p->h_tmp.data(), kept, (uint32_t)p->cand_begin, (uint32_t)bin0, bin_bits, cell_bits + bin_bits);
             p->host_sorted = true;
         }
         const int64_t nw = std::min<int64_t>(kept, cap);

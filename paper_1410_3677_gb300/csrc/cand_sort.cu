@@ -1,6 +1,6 @@
 // Candidate records put in (cell, bin) order on the device before they are read
 // back: a stable least-significant-digit radix sort, 8-bit digits, over the key
-// (cell - cell0) << bin_bits | bin of the searched range.  One pass is a digit
+// (cell - cell0) << bin_bits | (bin - bin0) of the searched range.  One pass is a digit
 // histogram per tile of 1024 or 4096 records, an exclusive scan of the histograms in
 // digit-major order (the tile's first slot for each digit), and a scatter that
 // ranks each record among the equal digits before it in its tile (warp match,
@@ -23,14 +23,14 @@ constexpr int kThreads = 256;
 constexpr int kRoundsLong = 16, kRoundsShort = 4;
 constexpr int64_t kShort = int64_t(1) << 20;
 
-__device__ __forceinline__ uint32_t digit_of(const CandRecord &r, uint32_t cell0, int bin_bits, int shift) {
-    const uint64_t key = ((uint64_t)(r.cell - cell0) << bin_bits) | r.bin;
+__device__ __forceinline__ uint32_t digit_of(const CandRecord &r, uint32_t cell0, uint32_t bin0, int bin_bits, int shift) {
+    const uint64_t key = ((uint64_t)(r.cell - cell0) << bin_bits) | (r.bin - bin0);
     return (uint32_t)(key >> shift) & 255u;
 }
 
 template <int kRounds>
 __global__ void __launch_bounds__(kThreads) k_digit_hist(const CandRecord *__restrict__ in, int64_t n,
-                                                         uint32_t cell0, int bin_bits, int shift,
+                                                         uint32_t cell0, uint32_t bin0, int bin_bits, int shift,
                                                          uint32_t *__restrict__ hist, int64_t nblk) {
     __shared__ uint32_t h[256];
     h[threadIdx.x] = 0;
@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(kThreads) k_digit_hist(const CandRecord *__res
 #pragma unroll 4
     for (int i = 0; i < kRounds; ++i) {
         const int64_t idx = base + i * kThreads + threadIdx.x;
-        if (idx < n) atomicAdd(&h[digit_of(in[idx], cell0, bin_bits, shift)], 1u);
+        if (idx < n) atomicAdd(&h[digit_of(in[idx], cell0, bin0, bin_bits, shift)], 1u);
     }
     __syncthreads();
     hist[(int64_t)threadIdx.x * nblk + blockIdx.x] = h[threadIdx.x];
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(1024) k_scan_rows(uint32_t *__restrict__ h, in
 template <int kRounds>
 __global__ void __launch_bounds__(kThreads) k_digit_scatter(const CandRecord *__restrict__ in,
                                                             CandRecord *__restrict__ out, int64_t n,
-                                                            uint32_t cell0, int bin_bits, int shift,
+                                                            uint32_t cell0, uint32_t bin0, int bin_bits, int shift,
                                                             const uint32_t *__restrict__ off, int64_t nblk,
                                                             const uint32_t *__restrict__ tot) {
     __shared__ uint32_t run[256];             // slots of each digit used by earlier rounds
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kThreads) k_digit_scatter(const CandRecord *__
         uint32_t d = 256;   // past the end: a digit no record has
         if (ok) {
             r = in[idx];
-            d = digit_of(r, cell0, bin_bits, shift);
+            d = digit_of(r, cell0, bin0, bin_bits, shift);
         }
         const unsigned peers = __match_any_sync(0xffffffffu, d);
         const int rank = __popc(peers & below);
@@ -142,16 +142,16 @@ __global__ void __launch_bounds__(kThreads) k_digit_scatter(const CandRecord *__
 }
 
 template <int kRounds>
-CandRecord *sort_t(CandRecord *a, CandRecord *b, uint32_t *hist, int64_t n, uint32_t cell0, int key_bits, int bin_bits,
-                   cudaStream_t s, int64_t *launches) {
+CandRecord *sort_t(CandRecord *a, CandRecord *b, uint32_t *hist, int64_t n, uint32_t cell0, uint32_t bin0, int key_bits,
+                   int bin_bits, cudaStream_t s, int64_t *launches) {
     const int passes = (key_bits + 7) / 8;
     const int64_t tile = kThreads * kRounds, nblk = (n + tile - 1) / tile;
     CandRecord *src = a, *dst = b;
     for (int p = 0; p < passes; ++p) {
         const int shift = 8 * p;
-        k_digit_hist<kRounds><<<(unsigned)nblk, kThreads, 0, s>>>(src, n, cell0, bin_bits, shift, hist, nblk);
+        k_digit_hist<kRounds><<<(unsigned)nblk, kThreads, 0, s>>>(src, n, cell0, bin0, bin_bits, shift, hist, nblk);
         k_scan_rows<<<256, 1024, 0, s>>>(hist, nblk, hist + 256 * nblk);
-        k_digit_scatter<kRounds><<<(unsigned)nblk, kThreads, 0, s>>>(src, dst, n, cell0, bin_bits, shift, hist, nblk,
+        k_digit_scatter<kRounds><<<(unsigned)nblk, kThreads, 0, s>>>(src, dst, n, cell0, bin0, bin_bits, shift, hist, nblk,
                                                                      hist + 256 * nblk);
         *launches += 3;
         CandRecord *x = src;
@@ -171,10 +171,10 @@ int64_t cand_sort_hist(int64_t n) {
 
 // Sorts n records of `a` (using b as the other buffer of the ping-pong); returns the buffer
 // that holds the result.
-CandRecord *launch_cand_sort(CandRecord *a, CandRecord *b, uint32_t *hist, int64_t n, uint32_t cell0, int key_bits,
-                             int bin_bits, cudaStream_t s, int64_t *launches) {
-    return n < kShort ? sort_t<kRoundsShort>(a, b, hist, n, cell0, key_bits, bin_bits, s, launches)
-                      : sort_t<kRoundsLong>(a, b, hist, n, cell0, key_bits, bin_bits, s, launches);
+CandRecord *launch_cand_sort(CandRecord *a, CandRecord *b, uint32_t *hist, int64_t n, uint32_t cell0, uint32_t bin0,
+                             int key_bits, int bin_bits, cudaStream_t s, int64_t *launches) {
+    return n < kShort ? sort_t<kRoundsShort>(a, b, hist, n, cell0, bin0, key_bits, bin_bits, s, launches)
+                      : sort_t<kRoundsLong>(a, b, hist, n, cell0, bin0, key_bits, bin_bits, s, launches);
 }
 
 }  // namespace fstat
