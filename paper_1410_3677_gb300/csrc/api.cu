@@ -650,8 +650,7 @@ void band_prologue(Plan &p, BandDev &b) {
     const bool t = stat_launch(p, idx, 0.0, (double)b.n * 8.0 * (1 + p.desc.upsample));
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (t) { e0 = ev_get(p); e1 = ev_get(p); rec_timing(e0, p.stream); }
-    p.launches += launch_band_inputs(b, p.sigma_parts, p.stream);
-    p.launches += launch_upsample(p, b, p.desc.upsample, b.xu, fp32, p.stream);
+    p.launches += launch_prologue(p, b, p.desc.upsample, b.xu, fp32, p.stream);
     if (t) { rec_timing(e1, p.stream); p.pending.push_back({idx, e0, e1}); }
 }
 

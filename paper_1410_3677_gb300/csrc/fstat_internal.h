@@ -252,11 +252,6 @@ struct CellBufs {
 // ---------------------------------------------------------------- launchers
 // Each returns the number of kernels it launched (for the plan's counter).
 
-// Per band and search: partial sums of x^2 (kSigmaParts doubles; the variance is
-// finished with the norms) and, in the FP32 form, the ephemeris as double-float
-// pairs (b.r2).
-int launch_band_inputs(const BandDev &b, double *sigma_parts, cudaStream_t s);
-
 // The upsample's tables for a series of n samples: log2 of its half length, the
 // double2 of scratch that building and running need, and the build itself (t.logh
 // and the w pointers set; ab holds 2 (U - 1) 2^logh, tw 2^logh double2).
@@ -265,9 +260,10 @@ int64_t upsample_scratch(int logh, int U);
 int launch_upsample_tables(int64_t n, int U, UpsampleTables &t, double2 *ab, double2 *tw, void *scratch,
                            cudaStream_t s);
 
-// U-fold FFT upsample of x[n] (double) into xu[U n] (double or float).
-int launch_upsample(const Plan &p, const BandDev &b, int U, void *xu, bool xu_fp32,
-                    cudaStream_t s);
+// Per band and search: the U-fold FFT upsample of x[n] into xu[U n] (double or float), the
+// partial sums of x^2 (p.sigma_parts; the variance is finished with the norms) and, in the
+// FP32 form, the ephemeris as double-float pairs (b.r2).
+int launch_prologue(const Plan &p, const BandDev &b, int U, void *xu, bool xu_fp32, cudaStream_t s);
 
 // Geometry + resampling + phase demodulation for skies [s0, s0+ns) of band b.
 // FP32 form writes w as float4 (y a, y b); FP64 form writes double2 wa, wb.

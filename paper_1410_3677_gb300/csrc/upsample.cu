@@ -21,7 +21,7 @@
 // hold each other's partners: k1 -> l1, the product, and straight back l1 -> k1;
 // columns (l2 -> k2) and the interleaved store.
 // The FP64 units (1/64 of the FP32 rate) bound the three.
-// Measured on GB300 for a band of a search (with k_band_inputs), U = 2, against a
+// Measured on GB300 for a band of a search (with BandInputs), U = 2, against a
 // Bluestein transform each way (23 launches): n = 86 164 390 -> 54 us, n = 344 656
 // 1521 -> 186 us, n = 4096 113 -> 26 us.
 #include <math.h>
@@ -129,6 +129,43 @@ __device__ __forceinline__ void dft_seq(int j, const double2 *__restrict__ w, do
     }
 }
 
+// The band's other inputs, by kSigmaParts blocks beside the first upsample kernel's (or alone
+// when U = 1; a launch of their own took 5 us): part `part` of the sum of x^2 (compensated)
+// and of the ephemeris split into double-float pairs (r2 null in the FP64 form).
+struct BandInputs {
+    const double *x;
+    int64_t n;
+    double *parts;
+    const double *r;
+    DF *r2;
+    __device__ __forceinline__ void run(int part) const {
+        __shared__ double sh[32];
+        const int T = (int)blockDim.x;
+        const int64_t first = (int64_t)part * T + threadIdx.x, step = (int64_t)kSigmaParts * T;
+        if (r2)
+            for (int64_t i = first; i < n; i += step)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) r2[c * n + i] = df_from_double(r[3 * i + c]);
+        KahanD k;
+        for (int64_t i = first; i < n; i += step) k.add(x[i] * x[i]);
+        const double v = warp_sum(k.s - k.c);
+        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double t = 0.0;
+            for (int w = 0; w < (T + 31) / 32; ++w) t += sh[w];
+            parts[part] = t;
+        }
+    }
+};
+
+template <typename TO>
+__global__ void k_copy_series(BandInputs in, TO *__restrict__ xu) {
+    in.run(blockIdx.x);
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < in.n; k += (int64_t)gridDim.x * blockDim.x)
+        xu[k] = (TO)in.x[k];
+}
+
 __device__ __forceinline__ double2 *up_smem() {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     return reinterpret_cast<double2 *>(smem_raw);
@@ -138,8 +175,9 @@ __device__ __forceinline__ double2 *up_smem() {
 template <int LOGH>
 __global__ void __launch_bounds__(CfgU<LOGH, 1>::THREADS)
 k_up_columns(const double *__restrict__ x, int64_t n, double2 *__restrict__ A, const double2 *__restrict__ tw,
-             const double2 *__restrict__ w) {
+             const double2 *__restrict__ w, BandInputs in) {
     using C = CfgU<LOGH, 1>;
+    if (blockIdx.x >= C::TILES) return in.run(blockIdx.x - C::TILES);
     const int f = (int)threadIdx.x % C::F, j = (int)threadIdx.x / C::F;   // consecutive threads: adjacent columns
     const int c = blockIdx.x * C::F + f;
     auto ld = [&](int i) {
@@ -238,12 +276,6 @@ k_up_output(const double2 *__restrict__ B, const double *__restrict__ x, TO *__r
     dft_seq<C::M, 1>(j, w, up_smem() + f * C::LD, false, [&](int i) { return in[(int64_t)i * C::N1]; }, st);
 }
 
-template <typename TO>
-__global__ void k_copy_series(const double *__restrict__ x, int64_t n, TO *__restrict__ xu) {
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k < n) xu[k] = (TO)x[k];
-}
-
 // The convolution kernel d(m + s/U) on the M-point circle: h[m], m < n, and (linear
 // convolution, M > n) h[M - m] for the negative lags.  |m + s/U| <= n/2 by the
 // periodicity of d, so that sin(pi t / n) keeps its relative precision.
@@ -295,25 +327,6 @@ __global__ void k_up_twiddle(double2 *__restrict__ t, int logh) {
     t[i] = make_double2(c, -s);
 }
 
-// Partial sums of x^2 (compensated), one per block of the first kSigmaParts, and
-// the ephemeris as double-float pairs (FP32 form; r2 null otherwise): both only
-// read the band's inputs, one launch.
-__global__ void __launch_bounds__(256) k_band_inputs(const double *__restrict__ x, int64_t n,
-                                                     double *__restrict__ partials, const double *__restrict__ r,
-                                                     DF *__restrict__ r2) {
-    __shared__ double sh[8];
-    if (r2)
-        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) r2[c * n + i] = df_from_double(r[3 * i + c]);
-    if (blockIdx.x >= kSigmaParts) return;
-    KahanD k;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)kSigmaParts * blockDim.x)
-        k.add(x[i] * x[i]);
-    const double s = block_sum256(k.s - k.c, sh);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
 inline unsigned blocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 template <class K>
@@ -322,19 +335,21 @@ void smem_limit(K k, size_t bytes) {
 }
 
 template <int LOGH>
-void forward_columns(const double *x, int64_t n, double2 *A, const UpsampleTables &t, cudaStream_t s) {
+void forward_columns(const double *x, int64_t n, double2 *A, const UpsampleTables &t, const BandInputs *in,
+                     cudaStream_t s) {
     using C1 = CfgU<LOGH, 1>;
     auto k1 = k_up_columns<LOGH>;
     smem_limit(k1, C1::SMEM);
-    k1<<<C1::TILES, C1::THREADS, C1::SMEM, s>>>(x, n, A, t.tw, t.w_cols);
+    k1<<<C1::TILES + (in ? kSigmaParts : 0), C1::THREADS, C1::SMEM, s>>>(x, n, A, t.tw, t.w_cols, in ? *in : BandInputs{});
 }
 
 template <int LOGH>
-int run_t(const BandDev &b, int U, void *xu, bool fp32, const UpsampleTables &t, double2 *scratch, cudaStream_t s) {
+int run_t(const BandDev &b, int U, void *xu, bool fp32, const UpsampleTables &t, double2 *scratch,
+          const BandInputs &in, cudaStream_t s) {
     using C1 = CfgU<LOGH, 1>;
     using C2 = CfgU<LOGH, 2>;
     double2 *A = scratch, *B = scratch + C1::H;
-    forward_columns<LOGH>(b.x, b.n, A, t, s);
+    forward_columns<LOGH>(b.x, b.n, A, t, &in, s);
     auto k2 = k_up_rows<LOGH>;
     smem_limit(k2, C2::SMEM);
     k2<<<dim3(C2::TILES, 1, (unsigned)(U - 1)), C2::THREADS, C2::SMEM, s>>>(A, B, t.ab, t.tw, t.w_rows);
@@ -364,7 +379,7 @@ int tables_t(int64_t n, int U, UpsampleTables &t, double2 *ab, double2 *tw, doub
     smem_limit(k2, C2::SMEM);
     for (int sub = 1; sub < U; ++sub) {
         k_up_kernel<<<blocks(2 * H, 256), 256, 0, s>>>(h, n, 2 * H, U, sub);
-        forward_columns<LOGH>(h, 2 * H, A, t, s);
+        forward_columns<LOGH>(h, 2 * H, A, t, nullptr, s);
         k2<<<C2::TILES, C2::THREADS, C2::SMEM, s>>>(A, Z, t.w_rows);
         k_up_alpha_beta<<<blocks(H, 256), 256, 0, s>>>(Z, ab + 2 * H * (sub - 1), LOGH);
     }
@@ -385,8 +400,9 @@ struct RunOp {
     bool fp32;
     const UpsampleTables &t;
     double2 *scratch;
+    const BandInputs &in;
     cudaStream_t s;
-    template <int L> int operator()() const { return run_t<L>(b, U, xu, fp32, t, scratch, s); }
+    template <int L> int operator()() const { return run_t<L>(b, U, xu, fp32, t, scratch, in, s); }
 };
 struct TablesOp {
     int64_t n;
@@ -413,19 +429,14 @@ int launch_upsample_tables(int64_t n, int U, UpsampleTables &t, double2 *ab, dou
     return dispatch<kMinLogH>(t.logh, TablesOp{n, U, t, ab, tw, reinterpret_cast<double2 *>(scratch), s});
 }
 
-int launch_band_inputs(const BandDev &b, double *sigma_parts, cudaStream_t s) {
-    const unsigned grid = b.r2 ? std::max<unsigned>(kSigmaParts, std::min<unsigned>(1024, blocks(b.n, 256))) : kSigmaParts;
-    k_band_inputs<<<grid, 256, 0, s>>>(b.x, b.n, sigma_parts, b.r, static_cast<DF *>(b.r2));
-    return 1;
-}
-
-int launch_upsample(const Plan &p, const BandDev &b, int U, void *xu, bool xu_fp32, cudaStream_t s) {
+int launch_prologue(const Plan &p, const BandDev &b, int U, void *xu, bool xu_fp32, cudaStream_t s) {
+    const BandInputs in{b.x, b.n, p.sigma_parts, b.r, static_cast<DF *>(b.r2)};
     if (U == 1) {
-        if (xu_fp32) k_copy_series<float><<<blocks(b.n, 256), 256, 0, s>>>(b.x, b.n, (float *)xu);
-        else k_copy_series<double><<<blocks(b.n, 256), 256, 0, s>>>(b.x, b.n, (double *)xu);
+        if (xu_fp32) k_copy_series<float><<<kSigmaParts, 256, 0, s>>>(in, (float *)xu);
+        else k_copy_series<double><<<kSigmaParts, 256, 0, s>>>(in, (double *)xu);
         return 1;
     }
-    return dispatch<kMinLogH>(b.up.logh, RunOp{b, U, xu, xu_fp32, b.up, reinterpret_cast<double2 *>(p.scratch), s});
+    return dispatch<kMinLogH>(b.up.logh, RunOp{b, U, xu, xu_fp32, b.up, reinterpret_cast<double2 *>(p.scratch), in, s});
 }
 
 }  // namespace fstat
