@@ -220,9 +220,10 @@ def run_reference(args, rank, world):
 # ----------------------------------------------------------------------------- our arm
 # Files that define the FFT/F-statistic kernels (host orchestration excluded): a
 # change to any of them voids the recorded DRAM traffic.
-KERNEL_SOURCES = ("fft_engine.cuh", "fft_engine2.cuh", "passes.cuh", "passes2.cuh", "packed.cuh",
-                  "passes3.cuh", "search_launch.cuh", "search_f32.cu", "search_f64.cu", "geometry.cu",
-                  "search_persistent.cu", "sync_ptx.cuh", "fstat_internal.h")
+KERNEL_SOURCES = ("fft_codelets.cuh", "fft_engine.cuh", "fft_engine2.cuh", "passes.cuh", "passes2.cuh",
+                  "packed.cuh", "passes3.cuh", "passes64.cuh", "unit_phase.cuh", "search_launch.cuh",
+                  "search_f32.cu", "search_f64.cu", "geometry.cu", "search_persistent.cu", "sync_ptx.cuh",
+                  "fstat_internal.h")
 
 
 def traffic_record(kernel_name, flops_per_launch):

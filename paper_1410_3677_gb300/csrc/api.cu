@@ -436,7 +436,7 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
     p.sigma_parts = dalloc<double>(p, kSigmaParts, n_alloc);
     for (int q = 0; q < 2; ++q) p.normbuf[q] = dalloc<double>(p, kNormStride * p.sky_batch, n_alloc);
 
-    // FFT scratch: cell slots of 2 transforms; also hosts the generic FFT of the upsample
+    // FFT scratch: cell slots of 2 transforms; also the upsample's intermediate arrays
     const size_t tsz = fp32 ? sizeof(float2) : sizeof(double2);
     if (fp32) {
         // several worker streams, each running launch pairs of a batch of cells on its

@@ -103,6 +103,19 @@ struct BandDev {
     UpsampleTables up;
 };
 
+// Row tiles (f rows l2 each) of a pass 2 that hold the bins l = l2 + n2 l1 of the searched range:
+// tiles tile0 .. tile0 + tiles - 1 modulo n2 / f, all of them when the range spans n2 bins.
+struct RowRange {
+    int tile0, tiles;
+};
+inline RowRange searched_rows(const BandDev &b, int n2, int f) {
+    const int64_t span = b.hi - b.lo, all = n2 / f;
+    if (span >= n2 - 1) return {0, (int)all};
+    const int64_t r0 = b.lo & (n2 - 1), t0 = r0 / f, cnt = (r0 + span) / f - t0 + 1;
+    if (cnt >= all) return {0, (int)all};
+    return {(int)t0, (int)cnt};
+}
+
 struct Plan {
     fstat_plan_desc desc{};
     std::vector<BandDev> bands;
@@ -171,7 +184,7 @@ struct Plan {
     int64_t pf_dist_pk = 0;        // the same for the paired pass 2 (measured best off)
     bool share_chirp = true;       // pass 1: spindown phase shared by the lanes of a column
     int p2_ts = 32;                // paired pass 2: CTA size (32, 64 or 128: one warp per row)
-    bool p2_rows = true;           // 256-point rows (2^16, 2^17): two rows per warp, packed
+    bool p2_rows = true;           // rows of 64 .. 256 points: packed in pairs (k_pass2rows)
     bool tma = true;               // two-stage pass 2: rows staged by bulk copies
     int p2_threads = 128;          // two-stage pass 2 with bulk copies: CTA size 256 or 128
 

@@ -169,10 +169,11 @@ struct InterTw {
 // cell's scratch slot.  Scratch is written and read through L2 only
 // (st.global.cg / ld.global.cg): it is streamed once each way, and a slot reused
 // within one launch never meets a stale L1 line.
-template <class C>
+template <class C, bool ROWS = false>
 struct ScratchStore2 {
     static constexpr bool kStoreEarly = true;
     float2 *scratch;
+    int row0, rows;      // ROWS: only the rows l2 = row0 .. row0 + rows - 1 (mod N2) are stored
     float2 *base;
     int k1_0;
     __device__ void init(int tile, int64_t, int64_t slot) {
@@ -184,7 +185,7 @@ struct ScratchStore2 {
         float2 *dst = base + 2 * ((int64_t)q.j * C::N1 + k1_0 + q.f) + q.t;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            __stcg(dst, float2{re[r], im[r]});
+            if (!ROWS || ((q.j + r * JPF - row0) & (C::N2 - 1)) < rows) __stcg(dst, float2{re[r], im[r]});
             dst += 2 * JPF * C::N1;
         }
     }
@@ -330,6 +331,7 @@ struct SearchEpi2 {
     float na, nb, nab, thr_half;
     uint32_t cell;
     int l2_0;
+    int tile0;               // first row tile of a launch over some of the rows (packed pass 2)
     __device__ void init(int tile, int64_t cl, int64_t) {
         const int64_t c = c0 + cl;
         const int64_t sky = (int64_t)((uint32_t)c / (uint32_t)n_spin);   // cells < 2^32: 32-bit divide

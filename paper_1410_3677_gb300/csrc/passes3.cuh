@@ -1,9 +1,9 @@
-// The FP32 search passes in packed arithmetic (packed.cuh) for passes of length
-// 512: both passes at N_fft = 2^18 (N1 = N2 = 512, the two-sidereal-day
-// segments), the shorter rows of 2^12 .. 2^17; and
-// the 1024-point rows of 2^19 and 2^20 and the 1024-point columns of 2^20.  Same four-step split, scratch layout, tiles and
-// launch shapes as the second engine's passes (passes2.cuh); what changes is how
-// a thread's 32 elements are transformed:
+// The FP32 search passes in packed arithmetic (packed.cuh): the 512-point rows
+// (N_fft = 2^18, N1 = N2 = 512, the two-sidereal-day segments; as an option its
+// columns too), the shorter rows of 2^12 .. 2^17 and of the interbinning form, the
+// 1024-point rows of 2^19 and 2^20 and the 1024-point columns of 2^20.  Same
+// four-step split and scratch layout as the second engine's passes (passes2.cuh);
+// what changes is how a thread's 32 elements are transformed, for 512 points:
 //
 //  - the radix-32 first stage of a pass is split by one decimation-in-frequency
 //    step into two 16-point DFTs, a_m = x_m + x_{m+16} and
@@ -167,9 +167,9 @@ k_pass1h(SearchLoad2<Cfg2<LOGN, 1>> ld, ScratchStore2<Cfg2<LOGN, 1>> st, const f
 // per thread) with its twiddle folded into the split as in k_pass2q below.
 // Measured per 2^18 points: 1.056 -> 0.961 us (a third fewer instructions than the scalar pass;
 // the 64-byte runs of its loads and stores cost it the rest against the 512-point columns).
-template <int LOGN, int Z1>
+template <int LOGN, int Z1, bool ROWS>
 __global__ void __launch_bounds__(256, 3)
-k_pass1q(SearchLoad2S<Cfg2<LOGN, 1>> ld, ScratchStore2<Cfg2<LOGN, 1>> st, const float4 *__restrict__ tws,
+k_pass1q(SearchLoad2S<Cfg2<LOGN, 1>> ld, ScratchStore2<Cfg2<LOGN, 1>, ROWS> st, const float4 *__restrict__ tws,
          const float2 *__restrict__ w1024) {
     using C = Cfg2<LOGN, 1>;
     static_assert(C::M == 1024 && C::SEQ == 8 && C::THREADS == 256, "1024-point columns, 8 sequences");
@@ -360,7 +360,9 @@ __device__ __forceinline__ void epilogue(const SearchEpi2<C, LOWER> &ep, int t, 
 // F, threshold and compaction.  A warp per row (F_a in the even lanes, F_b in
 // the odd ones), TS / 32 rows per CTA; with one row per CTA (TS = 32, the
 // default) 24 CTAs share an SM and each waits only for its own 8 KiB copy.
-template <int LOGN, bool LOWER, int TS = 32>
+// ROWS: a launch over the row tiles from ep.tile0 on (modulo their number); a form of its own,
+// as the two instructions before the copy is issued cost a launch over all rows 0.7 %.
+template <int LOGN, bool LOWER, int TS, bool ROWS>
 __global__ void __launch_bounds__(TS, 768 / TS)
 k_pass2p(RowsTMA<Cfg2<LOGN, 2, TS>> ld, SearchEpi2<Cfg2<LOGN, 2, TS>, LOWER> ep,
          const float4 *__restrict__ tws) {
@@ -368,9 +370,10 @@ k_pass2p(RowsTMA<Cfg2<LOGN, 2, TS>> ld, SearchEpi2<Cfg2<LOGN, 2, TS>, LOWER> ep,
     static_assert(C::M == kM && C::F == TS / 32 && C::SEQ == 2 * C::F && C::TPF == 16, "512-point rows, a warp per row");
     static_assert(2 * kR1 * kR1 * 16 == 2 * C::N1 * sizeof(float2), "a warp's exchange fills its staged row");
     ld.prefetch_ahead();
-    ld.init(blockIdx.x, blockIdx.y, blockIdx.y);
+    const int tile = ROWS ? ((int)blockIdx.x + ep.tile0) & (C::TILES - 1) : (int)blockIdx.x;
+    ld.init(tile, blockIdx.y, blockIdx.y);
     const int w = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
-    ep.init(blockIdx.x, blockIdx.y, blockIdx.y);
+    ep.init(tile, blockIdx.y, blockIdx.y);
     ld.stage();
     // lane 2j + t: a warp's loads from the staged row cover 32 consecutive
     // complex floats (F_a and F_b of 16 k1), free of bank conflicts
@@ -457,7 +460,7 @@ struct RowGeom {
     static_assert(N1 >= 64 && N1 <= 256, "short rows");
 };
 
-template <int LOGN, bool LOWER, bool IB, int W>
+template <int LOGN, bool LOWER, bool IB, int W, bool ROWS>
 __global__ void __launch_bounds__(32 * W, 24 / W)
 k_pass2rows(const float2 *__restrict__ scratch, InterTw<LOGN / 2> tw, const float4 *__restrict__ row_tw,
             const float2 *__restrict__ s1, uint32_t *err, SearchEpi2<Cfg2<LOGN, 2, 32>, LOWER> ep) {
@@ -467,7 +470,9 @@ k_pass2rows(const float2 *__restrict__ scratch, InterTw<LOGN / 2> tw, const floa
     unsigned char *sm = eng2::dyn_smem();
     const int w = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
     const int t = lane & 1, g = (lane >> 1) & (G - 1), j = lane / (2 * G);
-    const int pair0 = blockIdx.x * (IB ? Q::STEP : Q::PAIRS) + w * G;   // the warp's first pair
+    // the warp's first pair
+    const int tile = ROWS ? ((int)blockIdx.x + ep.tile0) & (Q::TILES - 1) : (int)blockIdx.x;
+    const int pair0 = tile * (IB ? Q::STEP : Q::PAIRS) + w * G;
     float2 *stage = reinterpret_cast<float2 *>(sm + w * Q::WARP_BYTES);
     float4 *tws = reinterpret_cast<float4 *>(sm + W * Q::WARP_BYTES) + w * G * kRowTw;
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + W * Q::WARP_BYTES + Q::PAIRS * Q::TW_BYTES) + w;
@@ -594,14 +599,15 @@ k_pass2rows(const float2 *__restrict__ scratch, InterTw<LOGN / 2> tw, const floa
 // W_1024^{m(q+32)} come from one packed table.  A whole row per CTA (16 KiB, twelve
 // CTAs per SM) instead of the radix-8 engine's three stages and two exchanges.
 // Measured at N = 344 656 (768 cells): pass 2 5.36 -> 2.93 us a cell.
-template <int LOGN, bool LOWER>
+template <int LOGN, bool LOWER, bool ROWS>
 __global__ void __launch_bounds__(64, 12)
 k_pass2q(RowsTMA<Cfg2<LOGN, 2, 64>> ld, SearchEpi2<Cfg2<LOGN, 2, 64>, LOWER> ep,
          const float4 *__restrict__ tws, const float2 *__restrict__ w1024) {
     using C = Cfg2<LOGN, 2, 64>;
     static_assert(C::M == 1024 && C::F == 1 && C::THREADS == 64, "1024-point rows, one per CTA");
-    ld.init(blockIdx.x, blockIdx.y, blockIdx.y);
-    ep.init(blockIdx.x, blockIdx.y, blockIdx.y);
+    const int tile = ROWS ? ((int)blockIdx.x + ep.tile0) & (C::TILES - 1) : (int)blockIdx.x;
+    ld.init(tile, blockIdx.y, blockIdx.y);
+    ep.init(tile, blockIdx.y, blockIdx.y);
     ld.stage();
     const int t = (int)threadIdx.x & 1, j = (int)threadIdx.x >> 1;
     const int l2 = ld.l2_0;

@@ -155,6 +155,7 @@ struct Epi64 {
     int64_t c0, s0;
     uint32_t cell_base;
     int64_t bin_lo, bin_hi;
+    int tile0;   // first row tile of a launch over some of the rows
     double thr;
     CandRecord *out;
     unsigned long long *count;
@@ -225,8 +226,10 @@ struct Epi64 {
 template <int LOGN, int PASS, class LD, class ST, int Z1>
 __global__ void __launch_bounds__(kTS, 2) k_pass64(LD ld, ST st, const double *__restrict__ tw) {
     using C = Cfg64<LOGN, PASS>;
-    ld.init(blockIdx.x, blockIdx.y);
-    st.init(blockIdx.x, blockIdx.y);
+    int tile = (int)blockIdx.x;
+    if constexpr (PASS == 2) tile = (tile + st.tile0) & (C::TILES - 1);
+    ld.init(tile, blockIdx.y);
+    st.init(tile, blockIdx.y);
     eng2::run_pass<double, C::M, C::SEQ, C::EH, -1, eng2::kMapFJ, LD, ST, PASS == 1 ? Z1 : 8, true>(ld, st, tw);
 }
 

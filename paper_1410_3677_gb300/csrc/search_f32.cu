@@ -13,8 +13,9 @@ namespace {
 
 template <int LOGN, bool LOWER, int TS = 256>
 SearchEpi2<Cfg2<LOGN, 2, TS>, LOWER> make_epi(const Plan &p, int band_idx, const BandDev &b, int64_t c0,
-                                              int64_t s0, const CellBufs &cb) {
+                                              int64_t s0, const CellBufs &cb, int tile0 = 0) {
     SearchEpi2<Cfg2<LOGN, 2, TS>, LOWER> st2{};
+    st2.tile0 = tile0;
     st2.norm = cb.norm;
     st2.n_spin = (int)p.desc.n_spin;
     st2.c0 = c0;
@@ -44,7 +45,7 @@ void launch_pass2(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int
 template <int LOGN, bool LOWER, int TS>
 void launch_pass2p(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_t c0, int64_t nc,
                    cudaStream_t s, const CellBufs &cb, const ScratchLoad2<Cfg2<LOGN, 2>> &ld2,
-                   const TwiddleSet *tw) {
+                   const TwiddleSet *tw, RowRange rr) {
     using D2 = Cfg2<LOGN, 2, TS>;
     p3::RowsTMA<D2> lt{};
     lt.scratch = ld2.scratch;
@@ -52,12 +53,14 @@ void launch_pass2p(const Plan &p, int band_idx, const BandDev &b, int64_t s0, in
     lt.pf_dist = p.pf_dist_pk;   // the paired pass gains nothing from L2 prefetch ahead
     lt.err = p.qerr;
     lt.row_tw = tw->row_tw;
-    const auto ep = make_epi<LOGN, LOWER, TS>(p, band_idx, b, c0, s0, cb);
-    auto k2 = p3::k_pass2p<LOGN, LOWER, TS>;
-    constexpr size_t smem2 = p3::RowsTMA<D2>::SMEM;
-    static bool attr2p = false;
-    if (!attr2p) { set_smem(k2, smem2); attr2p = true; }
-    k2<<<dim3(D2::TILES, (unsigned)nc), D2::THREADS, smem2, s>>>(lt, ep, tw->p512_f);
+    const auto ep = make_epi<LOGN, LOWER, TS>(p, band_idx, b, c0, s0, cb, rr.tile0);
+    auto run = [&](auto k2) {
+        constexpr size_t smem2 = p3::RowsTMA<D2>::SMEM;
+        set_smem(k2, smem2);
+        k2<<<dim3(rr.tiles, (unsigned)nc), D2::THREADS, smem2, s>>>(lt, ep, tw->p512_f);
+    };
+    if (TS == 32 && rr.tiles < D2::TILES) run(p3::k_pass2p<LOGN, LOWER, TS, TS == 32>);
+    else run(p3::k_pass2p<LOGN, LOWER, TS, false>);
 }
 
 // Short rows (64 .. 256 points) in packed pairs, zero-padded or interbinning.
@@ -65,17 +68,19 @@ bool rows_packed(const Plan &p) { return p.packed >= 1 && p.tma && p.p2_threads 
 
 template <int LOGN, bool LOWER, bool IB, int W>
 void launch_rows(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_t c0, int64_t nc, cudaStream_t s,
-                 const CellBufs &cb, const TwiddleSet *tw) {
+                 const CellBufs &cb, const TwiddleSet *tw, RowRange rr) {
     using Q = p3::RowGeom<LOGN, W>;
-    const auto ep = make_epi<LOGN, LOWER, 32>(p, band_idx, b, c0, s0, cb);
-    auto k2 = p3::k_pass2rows<LOGN, LOWER, IB, W>;
-    static bool attr = false;
-    if (!attr) { set_smem(k2, Q::SMEM); attr = true; }
+    const auto ep = make_epi<LOGN, LOWER, 32>(p, band_idx, b, c0, s0, cb, rr.tile0);
     // stage-1 twiddles [r][q], q < 16; the 64-point rows' table is in another order, they take W_64^m
     const float *s1 = Q::N1 == 64 ? tw->in1_f : tw->s1_f;
-    k2<<<dim3(IB ? Q::TILES_IB : Q::TILES, (unsigned)nc), 32 * W, Q::SMEM, s>>>(
-        reinterpret_cast<const float2 *>(cb.scratch), InterTw<LOGN / 2>{tw->lo_f, tw->hi_f}, tw->row_tw,
-        reinterpret_cast<const float2 *>(s1), p.qerr, ep);
+    auto run = [&](auto k2) {
+        set_smem(k2, Q::SMEM);
+        k2<<<dim3(rr.tiles, (unsigned)nc), 32 * W, Q::SMEM, s>>>(
+            reinterpret_cast<const float2 *>(cb.scratch), InterTw<LOGN / 2>{tw->lo_f, tw->hi_f}, tw->row_tw,
+            reinterpret_cast<const float2 *>(s1), p.qerr, ep);
+    };
+    if (!IB && rr.tiles < Q::TILES) run(p3::k_pass2rows<LOGN, LOWER, IB, W, !IB>);
+    else run(p3::k_pass2rows<LOGN, LOWER, IB, W, false>);
 }
 
 template <int LOGN, bool LOWER>
@@ -89,6 +94,20 @@ int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_
     // (512-point columns) also pass 1 with packed = 2 or 3
     const bool pk2 = (LOGN == 18 || LOGN == 19) && p.packed >= 1 && p.tma && p.p2_threads == 128 && tw->p512_f;
     const bool pk1 = pk2 && LOGN == 18 && p.packed >= 2;
+    // A bin range shorter than N2 touches some of the rows l2 = bin mod N2 only (a follow-up
+    // about known candidates): the packed pass 2 runs over their tiles, and while they are at
+    // most three quarters of the rows pass 1 stores no others.  Measured, 576 cells at 2^18, a whole
+    // search (all rows 922 us): 121 bins 1264 -> 911 us with the read-back, 256 bins 920 -> 685 us, 384
+    // bins 833 -> 797; without the pass-1 part 748 us at 258 bins.  At 2^20 the test of each
+    // store costs more than it saves beyond three quarters (768 of 1024 rows 3786 -> 3747 us,
+    // 1022 rows 4208 -> 4290).
+    int f2 = 0;   // rows per tile of the packed pass 2 (0: another pass 2, all rows)
+    if constexpr (LOGN <= 17) f2 = rows_packed(p) ? 2 * p3::RowGeom<LOGN, 1>::PAIRS : 0;
+    if constexpr (LOGN == 18 || LOGN == 19) f2 = pk2 && p.p2_ts == 32 ? 1 : 0;
+    if constexpr (C2::M == 1024) f2 = 1;
+    const RowRange rr = f2 ? searched_rows(b, C2::N2, f2) : RowRange{0, C2::N2 / std::max(1, p.p2_ts / 32)};
+    const bool few = f2 && 4 * rr.tiles * f2 <= 3 * C2::N2 && p.share_chirp;
+    ScratchStore2<C1, true> st1r{st1.scratch, rr.tile0 * f2, rr.tiles * f2};
     if constexpr (LOGN == 18) {
         if (pk1) {   // packed = 2: both stages paired; 3: scalar first stage, paired second
             const bool z3 = 8 * b.n <= 3 * (int64_t)C1::N;
@@ -107,14 +126,15 @@ int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_
         if (p.packed >= 1 && p.share_chirp && tw->p1024_f) {
             SearchLoad2S<C1> l1s{};
             static_cast<SearchLoad2<C1> &>(l1s) = ld1;
-            auto k3 = p3::k_pass1q<LOGN, 3>;
-            auto k4 = p3::k_pass1q<LOGN, 4>;
             constexpr size_t smem1 = (size_t)C1::SEQ * p3::kCol1024Ld * sizeof(float2);
-            static bool attr1q = false;
-            if (!attr1q) { set_smem(k3, smem1); set_smem(k4, smem1); attr1q = true; }
-            auto k1 = 8 * b.n <= 3 * (int64_t)C1::N ? k3 : k4;
-            k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, smem1, s>>>(l1s, st1, tw->p1024_f,
-                                                                         reinterpret_cast<const float2 *>(tw->in2_f));
+            auto run = [&](auto k1, const auto &st) {
+                set_smem(k1, smem1);
+                k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, smem1, s>>>(
+                    l1s, st, tw->p1024_f, reinterpret_cast<const float2 *>(tw->in2_f));
+            };
+            const bool z3 = 8 * b.n <= 3 * (int64_t)C1::N;
+            if (few) z3 ? run(p3::k_pass1q<LOGN, 3, true>, st1r) : run(p3::k_pass1q<LOGN, 4, true>, st1r);
+            else z3 ? run(p3::k_pass1q<LOGN, 3, false>, st1) : run(p3::k_pass1q<LOGN, 4, false>, st1);
             launched = true;
         }
     }
@@ -122,10 +142,12 @@ int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_
         if (!launched && 8 * b.n <= 3 * (int64_t)C1::N && p.share_chirp) {
             SearchLoad2S<C1> l1s{};
             static_cast<SearchLoad2<C1> &>(l1s) = ld1;
-            auto k1 = k_pass2<LOGN, 1, eng2::kMapFJ, SearchLoad2S<C1>, ScratchStore2<C1>, 256, 3>;
-            static bool attr3s = false;
-            if (!attr3s) { set_smem(k1, C1::SMEM); attr3s = true; }
-            k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, C1::SMEM, s>>>(l1s, st1, tw->s2_f);
+            auto run = [&](auto k1, const auto &st) {
+                set_smem(k1, C1::SMEM);
+                k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, C1::SMEM, s>>>(l1s, st, tw->s2_f);
+            };
+            if (few) run(k_pass2<LOGN, 1, eng2::kMapFJ, SearchLoad2S<C1>, ScratchStore2<C1, true>, 256, 3>, st1r);
+            else run(k_pass2<LOGN, 1, eng2::kMapFJ, SearchLoad2S<C1>, ScratchStore2<C1>, 256, 3>, st1);
             launched = true;
         }
         if (!launched && 8 * b.n <= 3 * (int64_t)C1::N) {
@@ -139,10 +161,12 @@ int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_
     if (!launched && p.share_chirp) {
         SearchLoad2S<C1> l1s{};
         static_cast<SearchLoad2<C1> &>(l1s) = ld1;
-        auto k1 = k_pass2<LOGN, 1, eng2::kMapFJ, SearchLoad2S<C1>, ScratchStore2<C1>, 256, 4>;
-        static bool attr1s = false;
-        if (!attr1s) { set_smem(k1, C1::SMEM); attr1s = true; }
-        k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, C1::SMEM, s>>>(l1s, st1, tw->s2_f);
+        auto run = [&](auto k1, const auto &st) {
+            set_smem(k1, C1::SMEM);
+            k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, C1::SMEM, s>>>(l1s, st, tw->s2_f);
+        };
+        if (few) run(k_pass2<LOGN, 1, eng2::kMapFJ, SearchLoad2S<C1>, ScratchStore2<C1, true>, 256, 4>, st1r);
+        else run(k_pass2<LOGN, 1, eng2::kMapFJ, SearchLoad2S<C1>, ScratchStore2<C1>, 256, 4>, st1);
         launched = true;
     }
     if (!launched) {
@@ -154,15 +178,15 @@ int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_
     if (mid) record_timing_event(mid, s);
     if constexpr (LOGN <= 17) {   // rows of 64 .. 256 points: packed in pairs
         if (rows_packed(p)) {
-            launch_rows<LOGN, LOWER, false, 1>(p, band_idx, b, s0, c0, nc, s, cb, tw);
+            launch_rows<LOGN, LOWER, false, 1>(p, band_idx, b, s0, c0, nc, s, cb, tw, rr);
             return 2;
         }
     }
     if constexpr (LOGN == 18 || LOGN == 19) {
         if (pk2) {
-            if (p.p2_ts == 32) launch_pass2p<LOGN, LOWER, 32>(p, band_idx, b, s0, c0, nc, s, cb, ld2, tw);
-            else if (p.p2_ts == 64) launch_pass2p<LOGN, LOWER, 64>(p, band_idx, b, s0, c0, nc, s, cb, ld2, tw);
-            else launch_pass2p<LOGN, LOWER, 128>(p, band_idx, b, s0, c0, nc, s, cb, ld2, tw);
+            if (p.p2_ts == 32) launch_pass2p<LOGN, LOWER, 32>(p, band_idx, b, s0, c0, nc, s, cb, ld2, tw, rr);
+            else if (p.p2_ts == 64) launch_pass2p<LOGN, LOWER, 64>(p, band_idx, b, s0, c0, nc, s, cb, ld2, tw, rr);
+            else launch_pass2p<LOGN, LOWER, 128>(p, band_idx, b, s0, c0, nc, s, cb, ld2, tw, rr);
             return 2;
         }
     }
@@ -174,13 +198,15 @@ int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_
         lt.pf_dist = 0;
         lt.err = p.qerr;
         lt.row_tw = tw->row_tw;
-        const auto ep = make_epi<LOGN, LOWER, 64>(p, band_idx, b, c0, s0, cb);
-        auto k2 = p3::k_pass2q<LOGN, LOWER>;
-        constexpr size_t smem2 = p3::RowsTMA<D2>::SMEM;
-        static bool attr2q = false;
-        if (!attr2q) { set_smem(k2, smem2); attr2q = true; }
-        k2<<<dim3(D2::TILES, (unsigned)nc), D2::THREADS, smem2, s>>>(lt, ep, tw->p1024_f,
-                                                                     reinterpret_cast<const float2 *>(tw->in1_f));
+        const auto ep = make_epi<LOGN, LOWER, 64>(p, band_idx, b, c0, s0, cb, rr.tile0);
+        auto run = [&](auto k2) {
+            constexpr size_t smem2 = p3::RowsTMA<D2>::SMEM;
+            set_smem(k2, smem2);
+            k2<<<dim3(rr.tiles, (unsigned)nc), D2::THREADS, smem2, s>>>(lt, ep, tw->p1024_f,
+                                                                         reinterpret_cast<const float2 *>(tw->in1_f));
+        };
+        if (rr.tiles < D2::TILES) run(p3::k_pass2q<LOGN, LOWER, true>);
+        else run(p3::k_pass2q<LOGN, LOWER, false>);
         return 2;
     } else if (p.tma && p.p2_threads == 128) {   // smaller tiles, six CTAs per SM
         ScratchLoadTMA<Cfg2<LOGN, 2, 128>> lt{};
@@ -308,8 +334,9 @@ int launch_interbin(const Plan &p, int band_idx, const BandDev &b, int64_t s0, i
         if (rows_packed(p)) {
             // warps per tile: few enough rows computed twice (one pair per tile) at 24 warps per SM
             constexpr int W = LOGN == 12 || LOGN == 15 ? 8 : LOGN <= 14 ? 6 : 12;
-            if (b.hi < (int64_t)C2::N) launch_rows<LOGN, true, true, W>(p, band_idx, b, s0, c0, nc, s, cb, tw);
-            else launch_rows<LOGN, false, true, W>(p, band_idx, b, s0, c0, nc, s, cb, tw);
+            constexpr RowRange all{0, p3::RowGeom<LOGN, W>::TILES_IB};
+            if (b.hi < (int64_t)C2::N) launch_rows<LOGN, true, true, W>(p, band_idx, b, s0, c0, nc, s, cb, tw, all);
+            else launch_rows<LOGN, false, true, W>(p, band_idx, b, s0, c0, nc, s, cb, tw, all);
             return 2;
         }
     }

@@ -72,7 +72,9 @@ int launch_t(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_t 
     auto k2 = p64::k_pass64<LOGN, 2, LD2, ST2, 8>;
     static bool attr2 = false;
     if (!attr2) { set_smem(k2, C2::SMEM); attr2 = true; }
-    k2<<<dim3(C2::TILES, (unsigned)nc), C2::THREADS, C2::SMEM, s>>>(ld2, st2, tw->s1_d);
+    const RowRange rr = searched_rows(b, C2::N2, C2::F);
+    st2.tile0 = rr.tile0;
+    k2<<<dim3(rr.tiles, (unsigned)nc), C2::THREADS, C2::SMEM, s>>>(ld2, st2, tw->s1_d);
     return 2;
 }
 

@@ -145,3 +145,33 @@ def test_interbin_long_series(fs, n):
     """Interbinning at n = N (no zero padding left in the half-length transform) and around
     three quarters of it."""
     _check(fs, fs.FP32_BATCHED, n, 1 << 14, 3, 2, interbin=True)
+
+
+@pytest.mark.parametrize("form,n,n_fft", [(1, n, f) for n, f in (
+    (2000, 1 << 12), (4096, 1 << 13), (5000, 1 << 14), (16000, 1 << 15), (20000, 1 << 16), (60000, 1 << 17),
+    (86164, 1 << 18), (131000, 1 << 18), (172328, 1 << 19), (250000, 1 << 19), (344656, 1 << 20),
+    (500000, 1 << 20))] + [(0, 2000, 1 << 12), (0, 20000, 1 << 16), (0, 86164, 1 << 18)])
+def test_narrow_bin_ranges(fs, form, n, n_fft):
+    """Bin ranges shorter than the N2 rows of the transform search some rows only: one bin, a
+    range across the last row and the first, half of the rows and one row more, all rows but one,
+    all; below and above N / 2."""
+    n2 = 1 << ((n_fft.bit_length() - 1 + 1) // 2)
+    alpha, delta = S.fibonacci_sky(2)
+    fdot = S.spindown_grid(2, -1e-8, 0.0)
+    b = S.make_band(n, 0.5, 17 + n, 1.0, alpha, delta, fdot, [], f_off=100.5, n_fft=n_fft)
+    prm = O.params(S.LAT_DEFAULT, S.GAMMA_DEFAULT, 2, 0.0, False, 0, False)
+    sky, spin = np.repeat(np.arange(2), 2), np.tile(np.arange(2), 2)
+    base = 3 * n2
+    ranges = [(base + 5, base + 5), (base - 3, base + 2), (base + 1, base + n2 // 2), (base + 1, base + n2 // 2 + 1),
+              (base + 2, base + n2), (base + 2, base + n2 + 1), (n_fft - n2 - 3, n_fft - n2 + 2),
+              (n_fft // 2 - 2, n_fft // 2 + 1)]
+    for lo, hi in ranges:
+        ref = O.cells_F(b, prm, alpha, delta, fdot, sky, spin, lo, hi, NTHREADS)
+        with fs.Plan([b], alpha, delta, fdot, -1.0, lat=S.LAT_DEFAULT, gamma=S.GAMMA_DEFAULT, form=form,
+                     bin_lo=lo, bin_hi=hi, cand_capacity=ref.size + 64) as p:
+            p.search()
+            c, total = p.candidates()
+        assert total == ref.size, (lo, hi)
+        assert np.array_equal(c["bin"], np.tile(np.arange(lo, hi + 1), sky.size))
+        err = np.abs(c["F"].reshape(ref.shape) - ref) / np.maximum(ref, 2.0)
+        assert err.max() <= TOL[form], (lo, hi, err.max())
