@@ -573,6 +573,8 @@ void free_all(Plan &p) {
     p.workers.clear();
     p.ev_pool.clear();
     p.pending.clear();
+    if (p.drain_stream) cudaStreamDestroy(p.drain_stream);
+    p.drain_stream = nullptr;
     if (p.own_stream && p.stream) cudaStreamDestroy(p.stream);
     p.stream = nullptr;
     p.own_stream = false;
@@ -1071,16 +1073,26 @@ fstat_status fstat_candidates_get(fstat_plan *p, fstat_candidate *buf, int64_t c
                 p->sort_cap = want;
             }
         }
+        // The search has ended on the host's side; the sort and the copy go to a stream of the highest
+        // priority: beside another plan's search each of the sort's launches would otherwise wait for
+        // the running pass's grid (milliseconds each).  Measured, ranges of 65 536 cells and
+        // 3.3e7 candidates drained while the next range is searched: 256 drains 16.6 -> 11.1 s
+        if (kept > kEagerRecords && !p->drain_stream) {
+            int least = 0, greatest = 0;
+            check(cudaDeviceGetStreamPriorityRange(&least, &greatest), "stream priority");
+            check(cudaStreamCreateWithPriority(&p->drain_stream, cudaStreamNonBlocking, greatest), "stream");
+        }
+        const cudaStream_t ds = p->drain_stream;
         if (dev_sort && !p->cand_sorted) {
             p->cand_sorted = launch_cand_sort(p->cand, p->cand_tmp, p->sort_hist, kept, (uint32_t)p->cand_begin,
-                                              (uint32_t)bin0, cell_bits + bin_bits, bin_bits, p->stream, &p->launches);
+                                              (uint32_t)bin0, cell_bits + bin_bits, bin_bits, ds, &p->launches);
             check(cudaGetLastError(), "candidate sort");
         }
         if (kept > kEagerRecords && (dev_sort || !p->host_sorted)) {
             check(cudaMemcpyAsync(rec, dev_sort ? p->cand_sorted : p->cand, kept * sizeof(CandRecord),
-                                  cudaMemcpyDeviceToHost, p->stream),
+                                  cudaMemcpyDeviceToHost, ds),
                   "candidates");
-            check(cudaStreamSynchronize(p->stream), "candidates");
+            check(cudaStreamSynchronize(ds), "candidates");
         }
         if (!dev_sort && kept > 0 && !p->host_sorted) {
             if ((int64_t)p->h_tmp.size() < kept) p->h_tmp.resize((size_t)kept);

@@ -123,6 +123,7 @@ struct Plan {
     int64_t n_cells = 0, f_evals = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
+    cudaStream_t drain_stream = nullptr;   // read-back: device sort and copy, made on first use
     bool poisoned = false;
     std::string err;
     int64_t launches = 0;
