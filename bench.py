@@ -394,7 +394,7 @@ def run_large(args, stream, flush, peak):
                          "basis": "2 x 5 N log2 N FLOP per cell over the sustained wall time"},
             "fp64_plain": {"value": fp64, "unit": UNIT, "dtype": "f64",
                            "sample": f"{sub_sky} sky x {sub_spin} spindown subgrid (spindowns spread "
-                                     f"over the range), one cell per launch pair",
+                                     f"over the range), cells in batches",
                            "roofline_frac": round(flop_cell * ev64 / nb / (ms64 / 1e3) / 1e12 / peak, 6)},
             "speedup_vs_fp64_plain": sustained / fp64,
             "note": "wall time of the 256 range searches and their candidate drains to the host "
@@ -530,7 +530,7 @@ def run_ours(args, rank, world, dist):
         p64.close()
         fp64 = {"value": ev64 / (ms64 / 1e3), "unit": UNIT, "dtype": "f64",
                 "sample": f"{sub} sky x {w.n_spin} spindown subgrid of the same workload, "
-                          f"one cell per launch pair"}
+                          f"cells in batches"}
 
     # ---------------------------------------------------------------- interbinning form, same grid
     interbin = None
