@@ -657,8 +657,6 @@ void band_prologue(Plan &p, BandDev &b) {
 }
 
 void enqueue_search(Plan &p, int64_t begin, int64_t end) {
-    p.cand_begin = begin;
-    p.cand_end = end;
     const fstat_plan_desc &d = p.desc;
     const bool fp32 = d.form == FSTAT_FP32_BATCHED;
     cudaStream_t s = p.stream;
@@ -794,12 +792,15 @@ void enqueue_search(Plan &p, int64_t begin, int64_t end) {
     check(cudaGetLastError(), "search launch");
 }
 
-// Waits for the search; its error word and candidate count are in pinned memory then.
-void finish_search(Plan &p, bool recycle_events) {
+// Waits for the search of cells [begin, end), launched plainly or replayed; its error word
+// and candidate count are in pinned memory then.
+void finish_search(Plan &p, int64_t begin, int64_t end, bool recycle_events) {
     check(cudaStreamSynchronize(p.stream), "search");
     collect_timing(p, recycle_events);
     if ((uint32_t)p.h_status[1] != 0) throw TimeoutError{};
     p.last_total = (int64_t)p.h_status[0];
+    p.cand_begin = begin;
+    p.cand_end = end;
     p.host_sorted = false;
     p.searched = true;
     p.cand_sorted = nullptr;
@@ -828,7 +829,7 @@ void search_impl(Plan &p, int64_t begin, int64_t end) {
     p.prev_timing = p.timing_every;
     if (!p.use_graph || (!hit && !repeat)) {
         enqueue_search(p, begin, end);
-        finish_search(p, true);
+        finish_search(p, begin, end, true);
         return;
     }
     if (!hit) {
@@ -873,7 +874,7 @@ void search_impl(Plan &p, int64_t begin, int64_t end) {
         for (auto &pe : p.pending) pe.stat = stat_index(p, g.dk[(size_t)pe.stat].name.c_str());
     }
     check(cudaGraphLaunch(g.exec, p.stream), "graph launch");
-    finish_search(p, false);
+    finish_search(p, begin, end, false);
 }
 
 template <class F>
@@ -1250,7 +1251,7 @@ fstat_status fstat_plan_autotune(fstat_plan *p, int64_t sample_cells, fstat_tuni
             check(cudaEventRecord(e0, p->stream), "event");
             enqueue_search(*p, 0, nc);
             check(cudaEventRecord(e1, p->stream), "event");
-            finish_search(*p, true);
+            finish_search(*p, 0, nc, true);
             float ms = 0.f;
             check(cudaEventElapsedTime(&ms, e0, e1), "cudaEventElapsedTime");
             return ms;

@@ -1,0 +1,52 @@
+"""Read-backs whose order depends on more than the last launch: searches replayed as a CUDA
+graph after another range."""
+import numpy as np
+import pytest
+
+from paper_1410_3677_gb300 import synth as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fs():
+    from paper_1410_3677_gb300 import fstat
+    return fstat
+
+
+def _plan(fs, w, form, n_bins, **kw):
+    return fs.Plan(w.bands, w.alpha, w.delta, w.fdot, -1.0, lat=w.lat, gamma=w.gamma, form=form, bin_lo=100,
+                   bin_hi=99 + n_bins, cand_capacity=1 << 17, **kw)
+
+
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("n_sky,n_spin,n_bins,sub", [
+    (5, 4, 2, (8, 13)),         # 40 records: comparison sort
+    (70, 8, 7, (8, 300)),       # 3920: records that come with the search
+    (70, 8, 14, (8, 300)),      # 7840: a copy and the host sort
+    (70, 8, 20, (8, 300)),      # 11 200: device sort
+    (70, 8, 120, (8, 300)),     # 67 200
+])
+def test_order_after_a_replay_of_another_range(fs, form, n_sky, n_spin, n_bins, sub):
+    """The whole grid twice (the second search is captured), a part of it once (searched
+    plainly, the graph is kept), and the whole again, replayed: the records come in (sky, spin,
+    bin) order and a limited read returns the first ones, as from a plan of its own."""
+    w = S.workload(1, n_sky=n_sky, n_spin=n_spin)
+    n = n_sky * n_spin * n_bins
+    with _plan(fs, w, form, n_bins) as q:
+        q.search()
+        ref, total = q.candidates()
+    assert total == n
+    assert np.array_equal(ref["sky"] * n_spin + ref["spin"], np.repeat(np.arange(n_sky * n_spin), n_bins))
+    with _plan(fs, w, form, n_bins) as p:
+        p.search()
+        p.search()
+        p.search(*sub)
+        part, total = p.candidates()
+        assert np.array_equal(part, ref[sub[0] * n_bins:sub[1] * n_bins])
+        p.search()
+        few, total = p.candidates(cap=7)
+        assert total == n and np.array_equal(few, ref[:7])
+        assert np.array_equal(p.candidates()[0], ref)
+        p.search(*sub)                    # and the other way round: the part after the whole
+        assert np.array_equal(p.candidates()[0], part)
