@@ -309,9 +309,29 @@ struct ScratchLoadTMA {
     }
 };
 
+// First slot of this lane's `own` hits among the candidate records, the warp's hits taken
+// with one atomic.  All atomics of a launch meet in one word of L2: with one for each output
+// that had hits (about one per record at a few hundred records a cell) the word saturated at
+// 0.8e9 a second, and pass 2 collapsed instead of slowing down a little.  Measured, 65 536
+// cells at 2^18: without records 90.1 ms; 3.0e7 records 92.9 -> 92.4 ms; 3.5e7 from 94 to 132,
+// by the GPU and the buffers' addresses, -> 92.5; 5.7e7 159 -> 93.3.  Grids with few records
+// run as before (within 0.2 %).
+__device__ __forceinline__ unsigned long long warp_slots(int own, unsigned long long *count) {
+    const int lane = threadIdx.x & 31;
+    int sum = own;   // inclusive over the lanes
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, sum, d);
+        if (lane >= d) sum += y;
+    }
+    unsigned long long first = 0;
+    if (lane == 31) first = atomicAdd(count, (unsigned long long)sum);
+    return __shfl_sync(0xffffffffu, first, 31) + (unsigned)(sum - own);
+}
+
 // Pass 2 output: F = |F_a|^2/(sigma^2 S_aa) + |F_b|^2/(sigma^2 S_bb) per bin
 // (Fig. 1, "F-statistics calculation"), strict 2F > thr, appended with one
-// atomic per warp and output slot.  Lanes l (F_a) and l ^ 16 (F_b) hold the same
+// atomic per warp (warp_slots).  Lanes l (F_a) and l ^ 16 (F_b) hold the same
 // bins; each forms |.|^2 of its own values and trades half of them with its
 // partner, so the a lane evaluates F on the first half of the outputs and the b
 // lane on the second.  LOWER: the bin range lies below N/2, so only the outputs
@@ -346,7 +366,6 @@ struct SearchEpi2 {
     template <int R, int JPF>
     __device__ __forceinline__ void store(const eng2::Job &q, float *re, float *im) const {
         constexpr int H = (LOWER ? R / 2 : R) / 2;   // values per lane
-        const int lane = threadIdx.x & 31;
         float Fv[H];
         bool pr[H];
         bool any = false;
@@ -376,20 +395,16 @@ struct SearchEpi2 {
             any |= pr[r];
         }
         if (!__any_sync(0xffffffffu, any)) return;
+        int own = 0;
 #pragma unroll
-        for (int r = 0; r < H; ++r) {
-            const unsigned m = __ballot_sync(0xffffffffu, pr[r]);
-            if (m) {
-                const int leader = __ffs(m) - 1;
-                unsigned long long b0 = 0;
-                if (lane == leader) b0 = atomicAdd(count, (unsigned long long)__popc(m));
-                b0 = __shfl_sync(0xffffffffu, b0, leader);
-                if (pr[r]) {
-                    const unsigned long long idx = b0 + __popc(m & ((1u << lane) - 1u));
-                    if (idx < cap) out[idx] = CandRecord{cell, (uint32_t)(bin0 + r * C::N2 * JPF), (double)Fv[r]};
-                }
+        for (int r = 0; r < H; ++r) own += pr[r] ? 1 : 0;
+        unsigned long long idx = warp_slots(own, count);
+#pragma unroll
+        for (int r = 0; r < H; ++r)
+            if (pr[r]) {
+                if (idx < cap) out[idx] = CandRecord{cell, (uint32_t)(bin0 + r * C::N2 * JPF), (double)Fv[r]};
+                ++idx;
             }
-        }
     }
 };
 

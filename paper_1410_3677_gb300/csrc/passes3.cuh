@@ -289,7 +289,6 @@ template <class C, bool LOWER, class Off>
 __device__ __forceinline__ void epilogue(const SearchEpi2<C, LOWER> &ep, int t, int bin0, Off off, int step_e,
                                          const PC *Y, bool own = true) {
     constexpr int H = epi_half<LOWER>();
-    const int lane = (int)threadIdx.x & 31;
     const bool full = ep.nab != 0.f;
     float2 Fv[H];
 #pragma unroll
@@ -334,25 +333,19 @@ __device__ __forceinline__ void epilogue(const SearchEpi2<C, LOWER> &ep, int t, 
             any |= pr[2 * u + e];
         }
     if (!__any_sync(0xffffffffu, any)) return;
+    unsigned hits = 0;
+#pragma unroll
+    for (int u = 0; u < 2 * H; ++u) hits |= pr[u] ? 1u << u : 0u;
+    unsigned long long idx = warp_slots(__popc(hits), ep.count);
 #pragma unroll
     for (int u = 0; u < H; ++u)
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const bool hit = pr[2 * u + e];
-            const unsigned m = __ballot_sync(0xffffffffu, hit);
-            if (m) {
-                const int leader = __ffs(m) - 1;
-                unsigned long long b0 = 0;
-                if (lane == leader) b0 = atomicAdd(ep.count, (unsigned long long)__popc(m));
-                b0 = __shfl_sync(0xffffffffu, b0, leader);
-                if (hit) {
-                    const unsigned long long idx = b0 + __popc(m & ((1u << lane) - 1u));
-                    const float f = e ? Fv[u].y : Fv[u].x;
-                    if (idx < ep.cap)
-                        ep.out[idx] = CandRecord{ep.cell, (uint32_t)(bin0 + off(u) + step_e * e), (double)f};
-                }
+        for (int e = 0; e < 2; ++e)
+            if (hits & (1u << (2 * u + e))) {
+                const float f = e ? Fv[u].y : Fv[u].x;
+                if (idx < ep.cap) ep.out[idx] = CandRecord{ep.cell, (uint32_t)(bin0 + off(u) + step_e * e), (double)f};
+                ++idx;
             }
-        }
 }
 
 // Rows l2 of the scratch, staged by a bulk copy (ScratchLoadTMA's copy and
