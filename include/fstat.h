@@ -34,6 +34,9 @@
  *     work they queue has finished); a plan is not thread-safe, but different
  *     plans (each on its own stream) may be used from different host threads at
  *     the same time (their graph captures are thread-local);
+ *   - a plan belongs to the CUDA device that was current when it was created: its
+ *     calls run there whatever device the calling thread has current, and leave
+ *     that one current; the entry points without a plan use the current device;
  *   - the caller owns every array it passes and may free it after the call that
  *     received it returns; the plan owns all device memory it allocates;
  *   - after FSTAT_ERR_CUDA or FSTAT_ERR_TIMEOUT a plan is poisoned: later calls

@@ -13,6 +13,7 @@
 #include <system_error>
 #include <vector>
 
+#include "device_guard.h"
 #include "dfloat.cuh"
 #include "fft_engine2.cuh"
 #include "fstat_internal.h"
@@ -43,6 +44,11 @@ void check(cudaError_t e, const char *what) {
 
 struct OomError {};
 struct TimeoutError {};
+
+struct CudaDevice {
+    static bool get(int *d) { return cudaGetDevice(d) == cudaSuccess; }
+    static bool set(int d) { return cudaSetDevice(d) == cudaSuccess; }
+};
 
 // Device memory of the plan.  Small arrays are cut from 1 MiB slabs: a cudaMalloc takes
 // about 10 us, and a plan holds some thirty tables and counters.  own: an allocation of its
@@ -282,6 +288,7 @@ void copy_in(void *dst, const void *src, size_t bytes, bool on_device, cudaStrea
 void create_impl(Plan &p, const fstat_plan_desc *d) {
     int n_alloc = 0;
     p.desc = *d;
+    check(cudaGetDevice(&p.device), "current device");
     const bool dev = d->inputs_on_device == 1;
     const bool fp32 = d->form == FSTAT_FP32_BATCHED;
     p.interbin = d->interpolation == FSTAT_INTERP_INTERBIN;
@@ -882,7 +889,9 @@ fstat_status guarded(fstat_plan *p, F &&f) {
     if (!p) return FSTAT_ERR_ARG;
     if (p->poisoned) return FSTAT_ERR_STATE;
     p->err.clear();
+    const DeviceGuard<CudaDevice> on_device(p->device);
     try {
+        if (!on_device.ok()) throw CudaError{cudaGetLastError(), "the plan's device"};
         return f();
     } catch (const CudaError &e) {
         p->err = std::string(e.what) + ": " + cudaGetErrorString(e.e);
@@ -1350,6 +1359,7 @@ fstat_status fstat_plan_get_info(const fstat_plan *p, fstat_plan_info *info) {
 
 void fstat_plan_destroy(fstat_plan *p) {
     if (!p) return;
+    const DeviceGuard<CudaDevice> on_device(p->device);
     free_all(*p);
     delete p;
 }

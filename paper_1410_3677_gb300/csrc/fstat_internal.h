@@ -121,6 +121,7 @@ struct Plan {
     std::vector<BandDev> bands;
     std::vector<fstat_band> host_bands;
     int64_t n_cells = 0, f_evals = 0;
+    int device = -1;   // current at creation; every call runs on it
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     cudaStream_t drain_stream = nullptr;   // read-back: device sort and copy, made on first use
