@@ -365,7 +365,12 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
         ++p.launches;
         t.row_tw = rt;
     }
-    if (!fp32) {   // tables of the FP64 passes, for the lengths the bands search
+    if (fp32) {   // unit phases of the per-sky stage
+        float4 *tt = dalloc<float4>(p, (size_t)turn_table_entries(), n_alloc);
+        launch_turn_table(tt, s);
+        ++p.launches;
+        p.turn_tab = tt;
+    } else {   // tables of the FP64 form, the passes' for the lengths the bands search
         double2 *ut = dalloc<double2>(p, (size_t)unit_table_entries(), n_alloc);
         launch_unit_table(ut, s);
         ++p.launches;

@@ -194,6 +194,7 @@ struct Plan {
     std::vector<TwiddleSet> tw;
     void *tw_pool = nullptr;
     const double2 *unit_tab = nullptr;   // FP64 form: e^{-2 pi i m / 2048}
+    const float4 *turn_tab = nullptr;    // FP32 form: e^{2 pi i m / 2048} in double-float pairs
 
     // candidates
     CandRecord *cand = nullptr;
@@ -299,6 +300,9 @@ CandRecord *launch_cand_sort(CandRecord *a, CandRecord *b, uint32_t *hist, int64
 // Row factors of the four-step twiddle for the packed FP32 rows (0 entries: none used).
 int64_t row_twiddle_entries(int logn);
 void launch_row_twiddles(float4 *t, int logn, cudaStream_t s);
+// Unit phases of the FP32 form's per-sky stage.
+int64_t turn_table_entries();
+void launch_turn_table(float4 *t, cudaStream_t s);
 // Tables of the FP64 form: unit phases, and the four-step twiddles of a length
 // 2^logn in the order its passes read them.
 int64_t unit_table_entries();

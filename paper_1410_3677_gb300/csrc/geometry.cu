@@ -33,6 +33,7 @@ struct GeoArgs {
     double dt, inv_dt, f_off, phi0;
     int dt_pow2;              // dt is a power of two: t / dt == t * inv_dt exactly
     const double2 *unit_tab;  // FP64 form
+    const float4 *turn_tab;   // FP32 form
     const SkyConst *sky;
     int64_t s0;
     void *w;
@@ -76,10 +77,14 @@ __global__ void __launch_bounds__(256) k_delays(const double *__restrict__ r,
 // integer, phi in FP32) and the band-offset phase on f_off d_j mod 1 plus the FP32
 // increment, as before.  A segment outside the window (an ephemeris that moves
 // by more than the margin within a tile) is evaluated directly.
-// The hour angle is a rotation by the tile's reference angle (double-float, once
-// per tile) and the small angle from it (Taylor series), instead of a sincos.
-// Bound by instruction issue.  Measured at n = 86 164 per 64 positions, f_off != 0:
-// 121 -> 82 us (delay records through memory and one sincos per sample before).
+// The hour angle is a rotation by the tile's reference angle (once per tile, its cosine
+// and sine as double-float pairs) and the small angle from it (Taylor series), instead of a sincos.
+// Rounded to FP32, the reference's error is the same for a whole tile: with the four tiles of
+// 4096 samples it modulated a(t) and b(t) in steps, and the bins beside a line of 2F = 400 were off
+// by 7.6e-6 (1.0e-5 over 128 positions); with the pairs 1.2e-6 (3.0e-6), against 2.8e-6 (4.4e-6)
+// of a sincos per sample.  It costs 1 % (63.4 -> 64.0 us per 64 positions).
+// Bound by instruction issue.  Measured at n = 86 164 per 64 positions, f_off != 0, with the
+// norms: 110 -> 64 us (delay records through memory and one sincos per sample before).
 constexpr int kGeo32 = 1024;                 // samples per tile
 constexpr int kGeoThreads = 256, kGeoPer = kGeo32 / kGeoThreads;
 constexpr int kGeoMargin = 4;                // samples before the first segment
@@ -117,6 +122,26 @@ __device__ __forceinline__ void unit_f(float c, float &cs, float &sn) {
     sn = __int_as_float(__float_as_int(b) ^ ((q & 2) << 30));
 }
 
+// cos and sin of 2 pi h as double-float pairs: the nearest of kTurnTab table entries (cos hi,
+// lo, sin hi, lo) rotated by the rest, |d| <= pi / kTurnTab (first term left out d^4/24, 3e-13).
+constexpr int kTurnTab = 2048;
+__device__ __forceinline__ void unit_df(const float4 *__restrict__ tab, DF h, DF &c, DF &s) {
+    const float x = (h.hi - rintf(h.hi)) * kTurnTab, m = rintf(x);
+    const float d = ((x - m) + h.lo * kTurnTab) * (float)(kTwoPi / kTurnTab);
+    const float4 t = __ldg(tab + ((int)m & (kTurnTab - 1)));
+    const float cm = -0.5f * d * d, sd = fmaf(d * d, d * (-1.f / 6.f), d);
+    c = df_fast_two_sum(t.x, fmaf(t.x, cm, fmaf(-t.z, sd, t.y)));
+    s = df_fast_two_sum(t.z, fmaf(t.z, cm, fmaf(t.x, sd, t.w)));
+}
+__global__ void k_turn_table(float4 *t) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= kTurnTab) return;
+    double s, c;
+    sincospi(2.0 * (double)i / (double)kTurnTab, &s, &c);
+    const DF cd = df_from_double(c), sd = df_from_double(s);
+    t[i] = make_float4(cd.hi, cd.lo, sd.hi, sd.lo);
+}
+
 // Sums over the 32 lanes of the 16 values v[0 .. 15] at once: each step halves the
 // values a lane carries by trading the other half with lane ^ mask, 16 shuffles in
 // place of 80.  Value i ends in lanes with bits 4 .. 1 equal to i (low bit: either).
@@ -136,7 +161,7 @@ __device__ __forceinline__ float warp_sum16(float *v) {
 
 __global__ void __launch_bounds__(kGeoThreads, 4) k_geometry(GeoArgs g) {
     __shared__ DF win[kGeoWin];
-    __shared__ float4 cf[3];   // A0 .. A4, B0 .. B3, cos and sin of the reference angle
+    __shared__ float4 cf[4];   // A0 .. A4, B0 .. B3, cos and sin of the reference angle: high parts, low parts
     __shared__ int s_js;
     __shared__ float sums[3][kGeoThreads / 32 * kGeoPer];
     const int n = (int)g.n, tid = threadIdx.x, sl = blockIdx.y;
@@ -168,11 +193,15 @@ __global__ void __launch_bounds__(kGeoThreads, 4) k_geometry(GeoArgs g) {
     if (tid < 9) {
         cs[tid] = tid < 5 ? (float)sc.A[tid] : (float)sc.B[tid - 5];
     } else if (tid == 32) {
-        // h = alpha - phi0 - Omega_r dt mc, reduced in turns
-        float fr;
-        df_split_floor(df_add(df_add(DF{sc.nf[6], sc.nf[7]}, df_neg(g.phi0_turns)),
-                              df_neg(df_mul(g.turn_dt, DF{(float)mc, 0.f}))), &fr);
-        sincospif(2.f * fr, &cs[10], &cs[9]);
+        // h = alpha - phi0 - Omega_r dt mc, in turns
+        const DF h = df_add(df_add(DF{sc.nf[6], sc.nf[7]}, df_neg(g.phi0_turns)),
+                            df_neg(df_mul(g.turn_dt, DF{(float)mc, 0.f})));
+        DF c, s;
+        unit_df(g.turn_tab, h, c, s);
+        cs[9] = c.hi;
+        cs[10] = s.hi;
+        cs[11] = c.lo;
+        cs[12] = s.lo;
     }
     __syncthreads();
     float sv[16];
@@ -216,16 +245,18 @@ __global__ void __launch_bounds__(kGeoThreads, 4) k_geometry(GeoArgs g) {
                            (unsigned)(i0 + 1) <= (unsigned)(g.U * (n - 1));
         // hour angle: the reference rotated by -Omega_r dt (u - mc)
         const float dl = g.w_dt * (F1 - (float)(A - mc));
-        float sd, cd;
+        float sd, cm;   // sin dl, cos dl - 1
         if (fabsf(dl) <= 0.25f) {   // first terms left out: d^9/9! and d^8/8!, below 4e-10
             const float q = dl * dl;
             sd = dl * fmaf(q, fmaf(q, fmaf(q, -1.f / 5040.f, 1.f / 120.f), -1.f / 6.f), 1.f);
-            cd = fmaf(q, fmaf(q, fmaf(q, -1.f / 720.f, 1.f / 24.f), -0.5f), 1.f);
+            cm = q * fmaf(q, fmaf(q, -1.f / 720.f, 1.f / 24.f), -0.5f);
         } else {
-            sincosf(dl, &sd, &cd);
+            sincosf(dl, &sd, &cm);
+            cm -= 1.f;
         }
         const float4 q0 = cf[0], q1 = cf[1], q2 = cf[2];
-        const float c1 = q2.y * cd - q2.z * sd, s1 = q2.z * cd + q2.y * sd;
+        const float c1 = q2.y + fmaf(q2.y, cm, fmaf(-q2.z, sd, q2.w));
+        const float s1 = q2.z + fmaf(q2.z, cm, fmaf(q2.y, sd, cf[3].x));
         const float c2 = c1 * c1 - s1 * s1, s2 = 2.f * s1 * c1;
         const float av = q0.x * c2 + q0.y * s2 + q0.z * c1 + q0.w * s1 + q1.x;
         const float bv = q1.y * c2 + q1.z * s2 + q1.w * c1 + q2.x * s1;
@@ -447,6 +478,9 @@ inline int geo_blocks(int64_t n) { return (int)blocks(n, kGeo32); }
 }  // namespace
 
 // ================================================================== launchers
+int64_t turn_table_entries() { return kTurnTab; }
+void launch_turn_table(float4 *t, cudaStream_t s) { k_turn_table<<<kTurnTab / 256, 256, 0, s>>>(t); }
+
 int launch_geometry(const Plan &p, const BandDev &b, int64_t s0, int64_t ns, bool fp32,
                     void *w, double *dbg_y, double *dbg_a, double *dbg_b, uint8_t *dbg_mask,
                     cudaStream_t s) {
@@ -468,6 +502,7 @@ int launch_geometry(const Plan &p, const BandDev &b, int64_t s0, int64_t ns, boo
     int e2 = 0;
     g.dt_pow2 = frexp(b.dt, &e2) == 0.5 && isnormal(g.inv_dt);
     g.unit_tab = p.unit_tab;
+    g.turn_tab = p.turn_tab;
     g.f_off = b.f_off;
     g.phi0 = b.phi0;
     g.sky = p.sky;

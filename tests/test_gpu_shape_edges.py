@@ -175,3 +175,30 @@ def test_narrow_bin_ranges(fs, form, n, n_fft):
         assert np.array_equal(c["bin"], np.tile(np.arange(lo, hi + 1), sky.size))
         err = np.abs(c["F"].reshape(ref.shape) - ref) / np.maximum(ref, 2.0)
         assert err.max() <= TOL[form], (lo, hi, err.max())
+
+
+@pytest.mark.parametrize("lg,n_sky,n_spin", [(13, 8, 4), (13, 128, 4), (12, 32, 2), (14, 32, 2), (15, 32, 2)])
+def test_fp32_error_beside_a_strong_line(fs, lg, n_sky, n_spin):
+    """Short segments with a line of SNR 20 (at 2^13 the tiny grid), every bin: an amplitude
+    error of the demodulated series that is common to many samples shows in the weak bins
+    beside the line.  A relative amplitude error e of the line changes a bin of F by up to
+    2 e sqrt(F F_max), relative to max(F, 2) at most 2 e sqrt(F_max / 2); the bound allows
+    e = 4 x 2^-24."""
+    if lg == 13:
+        w = S.workload(1, n_sky=n_sky, n_spin=n_spin)
+        b, alpha, delta, fdot = w.bands[0], w.alpha, w.delta, w.fdot
+    else:
+        alpha, delta = S.fibonacci_sky(n_sky)
+        fdot = S.spindown_grid(n_spin, -3e-9, 0.0)
+        inj = S.Injection(sky=5, spin=1, bin=int(0.2 * (1 << lg)), snr=20.0, cos_iota=0.3, psi=0.2, phi0=1.0)
+        b = S.make_band(1 << (lg - 1), 2.0, 1000 + lg, 1.0, alpha, delta, fdot, [inj], n_fft=1 << lg)
+    prm = O.params(S.LAT_DEFAULT, S.GAMMA_DEFAULT, 2, 0.0, False, 0)
+    sky, spin = np.repeat(np.arange(n_sky), n_spin), np.tile(np.arange(n_spin), n_sky)
+    ref = O.cells_F(b, prm, alpha, delta, fdot, sky, spin, nthreads=NTHREADS)
+    with fs.Plan([b], alpha, delta, fdot, -1.0, lat=S.LAT_DEFAULT, gamma=S.GAMMA_DEFAULT, form=fs.FP32_BATCHED,
+                 cand_capacity=ref.size) as p:
+        p.search()
+        c, total = p.candidates()
+    assert total == ref.size and ref.max() > 100.0
+    err = np.abs(c["F"].reshape(ref.shape) - ref) / np.maximum(ref, 2.0)
+    assert err.max() <= 4 * 2.0 ** -24 * 2.0 * math.sqrt(ref.max() / 2.0), (err.max(), ref.max())
