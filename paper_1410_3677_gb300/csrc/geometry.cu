@@ -102,24 +102,11 @@ __device__ __forceinline__ int df_split_near(DF x, float &f) {
     return (int)r;
 }
 
-// cos and sin of 2 pi c: the nearest quarter turn and Taylor series in the rest, |r| <= 1/8
-// (first terms left out: 2 pi r ^11/11! and ^10/10!, below 2.5e-8), |c| < 2^20.
+// cos and sin of 2 pi c by the nearest quarter turn, |c| < 2^20.
 __device__ __forceinline__ void unit_f(float c, float &cs, float &sn) {
     constexpr float magic = 12582912.f;   // 1.5 2^23: the low bits of the sum are the integer
     const float qm = fmaf(c, 4.f, magic);
-    const int q = __float_as_int(qm);
-    const float r = fmaf(qm - magic, -0.25f, c), r2 = r * r;
-    constexpr double T = 6.283185307179586476925286766559, T2 = T * T;
-    const float s = r * fmaf(r2, fmaf(r2, fmaf(r2, fmaf(r2, (float)(T * T2 * T2 * T2 * T2 / 362880.0),
-                                                        (float)(-T * T2 * T2 * T2 / 5040.0)),
-                                               (float)(T * T2 * T2 / 120.0)), (float)(-T * T2 / 6.0)), (float)T);
-    const float k = fmaf(r2, fmaf(r2, fmaf(r2, fmaf(r2, (float)(T2 * T2 * T2 * T2 / 40320.0),
-                                                    (float)(-T2 * T2 * T2 / 720.0)),
-                                           (float)(T2 * T2 / 24.0)), (float)(-T2 / 2.0)), 1.f);
-    const bool odd = q & 1;
-    const float a = odd ? s : k, b = odd ? k : s;
-    cs = __int_as_float(__float_as_int(a) ^ (((q + 1) & 2) << 30));
-    sn = __int_as_float(__float_as_int(b) ^ ((q & 2) << 30));
+    fstat::unit_f(__float_as_int(qm), fmaf(qm - magic, -0.25f, c), cs, sn);
 }
 
 // cos and sin of 2 pi h as double-float pairs: the nearest of kTurnTab table entries (cos hi,

@@ -85,10 +85,12 @@ bool setup_current_device(int L, DevState **out) {
     return true;
 }
 
-// Pass-1 input: the search's loader on one series.  The dependent launch may start at
+// Pass-1 input: the search's loader on one series, with Taylor phases: the special function
+// unit's were most of the error of F (rms over the lengths 2.8-3.9e-7 -> 1.9-2.4e-7; 2.6-4.3e-7 on
+// the radix-8 passes) and these cost a lone cell no time.  The dependent launch may start at
 // once; it waits for this grid's stores.
 template <class C>
-struct CellLoad : SearchLoad2S<C> {
+struct CellLoad : SearchLoad2S<C, true> {
     __device__ void init(int tile, int64_t, int64_t) {
         asm volatile("griddepcontrol.launch_dependents;");
         this->ws = reinterpret_cast<const float2 *>(this->w);

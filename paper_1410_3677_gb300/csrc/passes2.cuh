@@ -15,6 +15,7 @@
 #include "fft_engine2.cuh"
 #include "fstat_internal.h"
 #include "sync_ptx.cuh"
+#include "unit_phase.cuh"
 
 namespace fstat {
 
@@ -92,7 +93,9 @@ struct SearchLoad2 {
 // (column mapping: lanes 2f and 2f + 1 hold the a and b halves of the same
 // samples): each lane evaluates the phase of every other element, r = 2 i + t,
 // and both read each element's (cos, sin) from the lane that evaluated it.
-template <class C>
+// TAYLOR: phases good to 3e-8 instead of the special function unit's 4e-7, for a lone cell,
+// which is bound by latency (the search's pass 1 is bound by issue).
+template <class C, bool TAYLOR = false>
 struct SearchLoad2S : SearchLoad2<C> {
     template <int R, int JPF>
     __device__ __forceinline__ void load(const eng2::Job &q, float *re, float *im) const {
@@ -117,7 +120,13 @@ struct SearchLoad2S : SearchLoad2<C> {
                 const uint32_t k = (uint32_t)(kt + C::N1 * JPF * (r0 + 2 * i));
                 const uint64_t kk = (uint64_t)k * (uint64_t)k;
                 const int32_t top = (int32_t)((this->afx * kk) >> 32);   // cycles in [-1/2, 1/2)
-                __sincosf((float)top * 1.4629180792671596e-09f, &sn[i], &cs[i]);   // 2 pi / 2^32
+                if constexpr (TAYLOR) {   // the nearest quarter turn and the rest, exact in fixed point
+                    const uint32_t t = (uint32_t)top + 0x20000000u;
+                    const float rest = (float)((int32_t)(t & 0x3fffffffu) - 0x20000000);
+                    unit_f((int)(t >> 30), rest * 2.3283064365386963e-10f, cs[i], sn[i]);   // 2^-32
+                } else {
+                    __sincosf((float)top * 1.4629180792671596e-09f, &sn[i], &cs[i]);   // 2 pi / 2^32
+                }
             }
 #pragma unroll
             for (int r = r0; r < r0 + GR; ++r) {

@@ -1,9 +1,27 @@
-// Unit phases in FP64 from a table, for the FP64 form's kernels.
+// Unit phases: in FP64 from a table, for the FP64 form's kernels, and in FP32 by Taylor series.
 #pragma once
 
 #include <cuda_runtime.h>
 
 namespace fstat {
+
+// cos and sin of 2 pi (q / 4 + r), |r| <= 1/8, by Taylor series (first terms left out:
+// 2 pi r ^11/11! and ^10/10!, below 2.5e-8); only the low two bits of q count.
+__device__ __forceinline__ void unit_f(int q, float r, float &cs, float &sn) {
+    const float r2 = r * r;
+    constexpr double T = 6.283185307179586476925286766559, T2 = T * T;
+    const float s = r * fmaf(r2, fmaf(r2, fmaf(r2, fmaf(r2, (float)(T * T2 * T2 * T2 * T2 / 362880.0),
+                                                        (float)(-T * T2 * T2 * T2 / 5040.0)),
+                                               (float)(T * T2 * T2 / 120.0)), (float)(-T * T2 / 6.0)), (float)T);
+    const float k = fmaf(r2, fmaf(r2, fmaf(r2, fmaf(r2, (float)(T2 * T2 * T2 * T2 / 40320.0),
+                                                    (float)(-T2 * T2 * T2 / 720.0)),
+                                           (float)(T2 * T2 / 24.0)), (float)(-T2 / 2.0)), 1.f);
+    const bool odd = q & 1;
+    const float a = odd ? s : k, b = odd ? k : s;
+    cs = __int_as_float(__float_as_int(a) ^ (((q + 1) & 2) << 30));
+    sn = __int_as_float(__float_as_int(b) ^ ((q & 2) << 30));
+}
+
 namespace p64 {
 
 constexpr int kUnitTab = 2048;     // entries e^{-2 pi i m / 2048}

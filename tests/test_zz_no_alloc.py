@@ -120,3 +120,33 @@ def test_noalloc_every_length(lg, frac, whole):
     got = out.cpu().numpy()
     assert got[0] == -1.0 and got[-1] == -1.0            # nothing outside the window
     assert np.max(np.abs(got[1:-1] - ref) / np.maximum(ref, 2.0)) <= 1e-4
+
+
+@pytest.mark.parametrize("lg", range(12, 19))
+@pytest.mark.parametrize("eighths,more", [(3, 0), (3, 1), (4, 0)])
+def test_noalloc_rounding(lg, eighths, more):
+    """Rms error of F over all bins of a noise series with a spindown of many cycles, against an
+    FP64 transform.  About ten roundings of 2^-24 (uniform: 2^-24 / sqrt 3 rms) a transform value
+    make 1.1e-7 of its amplitude, twice that of F; 2.5e-7 leaves an eighth.  n = 3N/8 is the
+    longest series whose columns skip five eighths, 3N/8 + 1 the first whose do not."""
+    import torch
+    from paper_1410_3677_gb300 import fstat as fs
+    N = 1 << lg
+    n = eighths * N // 8 + more
+    rng = np.random.default_rng(100 + lg)
+    rate, na, nb, lo, hi = -1.7e-8, 1.0 / n, 2.0 / n, 1, N // 2 - 1
+    rate *= (1 << 36) / float(n) ** 2                    # 1168 cycles over the series at any length
+    k = np.arange(n, dtype=np.float64)
+    ph = np.exp(-2j * np.pi * np.mod(rate * k * k, 1.0))
+    sq, count = 0.0, 0
+    for _ in range(max(1, (1 << 17) >> lg)):
+        w = rng.standard_normal((n, 4)).astype(np.float32)
+        A = np.fft.fft((w[:, 0] + 1j * w[:, 1].astype(np.float64)) * ph, N)
+        B = np.fft.fft((w[:, 2] + 1j * w[:, 3].astype(np.float64)) * ph, N)
+        ref = (np.abs(A) ** 2 * na + np.abs(B) ** 2 * nb)[lo:hi + 1]
+        wd = torch.from_numpy(w).cuda()
+        out = torch.empty(hi - lo + 1, dtype=torch.float32, device="cuda")
+        assert fs.cell_F_noalloc(wd.data_ptr(), n, N, rate, na, nb, lo, hi, out.data_ptr()) == fs.FSTAT_OK
+        sq += float(np.sum(((out.cpu().numpy() - ref) / np.maximum(ref, 2.0)) ** 2))
+        count += ref.size
+    assert np.sqrt(sq / count) <= 2.5e-7, np.sqrt(sq / count)
