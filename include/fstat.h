@@ -157,7 +157,10 @@ typedef struct fstat_plan fstat_plan;
    the launch configuration.  On success *out receives a plan; on failure *out is
    NULL and nothing is leaked.  Errors: FSTAT_ERR_ARG (any field out of range,
    NULL where a pointer is required, x and x32 both or neither given, more than
-   2^32 - 1 cells), FSTAT_ERR_OOM, FSTAT_ERR_CUDA. */
+   2^32 - 1 cells), FSTAT_ERR_OOM, FSTAT_ERR_CUDA.  Where the usual batches do not
+   fit beside what else the device holds, smaller ones are tried (slower, the same
+   results): FP32 plans with at most 256 sky positions a batch, FP64 plans down to
+   one cell and one sky position at a time. */
 fstat_status fstat_plan_create(fstat_plan **out, const fstat_plan_desc *desc);
 
 /* Replace the data of band `band` (0-based) by the next segment of the same

@@ -38,6 +38,12 @@ int alloc_fail_at() {
     return v ? atoi(v) : 0;
 }
 
+// Test hook: FSTAT_TEST_MEM_LIMIT=b lets a plan hold at most b bytes of device memory.
+bool over_limit(const Plan &p, size_t more) {
+    const char *v = getenv("FSTAT_TEST_MEM_LIMIT");
+    return v && p.device_bytes + (int64_t)more > atoll(v);
+}
+
 void check(cudaError_t e, const char *what) {
     if (e != cudaSuccess) throw CudaError{e, what};
 }
@@ -65,6 +71,7 @@ T *dalloc(Plan &p, size_t count, int &n_alloc, bool own = false) {
     if (!small || p.slab_left < room) {
         void *ptr = nullptr;
         const size_t want = small ? kSlab : bytes;
+        if (over_limit(p, want)) throw OomError{};
         cudaError_t e = cudaMalloc(&ptr, want);
         if (e == cudaErrorMemoryAllocation) {
             cudaGetLastError();
@@ -285,7 +292,12 @@ void copy_in(void *dst, const void *src, size_t bytes, bool on_device, cudaStrea
           "input copy");
 }
 
-void create_impl(Plan &p, const fstat_plan_desc *d) {
+// A plan that does not fit is tried again with smaller batches (`step` 1, 2, ...): FP32 plans once,
+// with at most 256 sky positions a batch; FP64 plans down to one cell and one position at a
+// time, an eighth of the batch memory each step.
+constexpr int kSteps32 = 1, kSteps64 = 4;
+
+void create_impl(Plan &p, const fstat_plan_desc *d, int step) {
     int n_alloc = 0;
     p.desc = *d;
     check(cudaGetDevice(&p.device), "current device");
@@ -427,14 +439,15 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
     auto fp32_batch = [&]() -> int64_t {
         const int64_t fill = (4096 + d->n_spin - 1) / d->n_spin;
         const int64_t room = std::max<int64_t>(256, (int64_t(1) << 31) / (2 * 16 * p.w_stride));
-        const int64_t most = std::max<int64_t>(64, std::min<int64_t>(std::min<int64_t>(1024, room), fill));
+        const int64_t most = std::max<int64_t>(64, std::min<int64_t>(std::min<int64_t>(step > 0 ? 256 : 1024, room), fill));
         const int64_t batches = (d->n_sky + most - 1) / most;
         return (d->n_sky + batches - 1) / batches;
     };
+    auto batch64 = [&](int64_t bytes) { return step < kSteps64 ? bytes >> (3 * step) : 0; };
     // FP64 form: up to 64 positions whose series (32 bytes a sample) fill 128 MiB: the FP64
     // kernels are bound by their arithmetic, a batch only has to fill the SMs and hide latency
     p.sky_batch = fp32 ? fp32_batch()
-                       : std::min<int64_t>(d->n_sky, std::max<int64_t>(1, std::min<int64_t>(64, (int64_t(128) << 20) / (32 * p.w_stride))));
+                       : std::min<int64_t>(d->n_sky, std::max<int64_t>(1, std::min<int64_t>(64, batch64(int64_t(128) << 20) / (32 * p.w_stride))));
     if (fp32)
         if (const char *v = getenv("FSTAT_SKY_BATCH")) p.sky_batch = std::max<int64_t>(1, std::min<int64_t>(d->n_sky, atoll(v)));
     const size_t w_elem = fp32 ? 16 : 32;
@@ -465,7 +478,7 @@ void create_impl(Plan &p, const fstat_plan_desc *d) {
         // launches of many cells (scratch up to 512 MiB, 64 cells at 2^18): one cell of a short
         // transform fills only a few SMs, and 2^18 leaves a sixth of them idle
         p.n_workers = 1;
-        p.cell_batch = std::max<int64_t>(1, std::min<int64_t>(4096, (int64_t(512) << 20) / (2 * max_nfft * (int64_t)tsz)));
+        p.cell_batch = std::max<int64_t>(1, std::min<int64_t>(4096, batch64(int64_t(512) << 20) / (2 * max_nfft * (int64_t)tsz)));
         p.cell_batch = std::min<int64_t>(p.cell_batch, p.sky_batch * d->n_spin);
     }
     // a worker's slot holds a launch's cells, or the ring of the fused launch
@@ -991,31 +1004,30 @@ fstat_status fstat_plan_create(fstat_plan **out, const fstat_plan_desc *desc) {
         if (getenv("FSTAT_LOG")) fprintf(stderr, "fstat_plan_create: %s\n", err.c_str());
         return st;
     }
-    fstat_plan *p = new (std::nothrow) fstat_plan();
-    if (!p) return FSTAT_ERR_OOM;
-    try {
-        create_impl(*p, desc);
-    } catch (const CudaError &e) {
-        if (getenv("FSTAT_LOG")) fprintf(stderr, "fstat_plan_create: %s: %s\n", e.what, cudaGetErrorString(e.e));
+    const int steps = desc->form == FSTAT_FP32_BATCHED ? kSteps32 : kSteps64;
+    for (int step = 0;; ++step) {
+        fstat_plan *p = new (std::nothrow) fstat_plan();
+        if (!p) return FSTAT_ERR_OOM;
+        try {
+            create_impl(*p, desc, step);
+            *out = p;
+            return FSTAT_OK;
+        } catch (const CudaError &e) {
+            if (getenv("FSTAT_LOG")) fprintf(stderr, "fstat_plan_create: %s: %s\n", e.what, cudaGetErrorString(e.e));
+            st = FSTAT_ERR_CUDA;
+        } catch (const OomError &) {
+            st = FSTAT_ERR_OOM;
+        } catch (const std::bad_alloc &) {
+            st = FSTAT_ERR_OOM;
+            step = steps;   // host memory: smaller device batches would not help
+        } catch (const std::string &m) {
+            if (getenv("FSTAT_LOG")) fprintf(stderr, "fstat_plan_create: %s\n", m.c_str());
+            st = FSTAT_ERR_ARG;
+        }
         free_all(*p);
         delete p;
-        return FSTAT_ERR_CUDA;
-    } catch (const OomError &) {
-        free_all(*p);
-        delete p;
-        return FSTAT_ERR_OOM;
-    } catch (const std::bad_alloc &) {
-        free_all(*p);
-        delete p;
-        return FSTAT_ERR_OOM;
-    } catch (const std::string &m) {
-        if (getenv("FSTAT_LOG")) fprintf(stderr, "fstat_plan_create: %s\n", m.c_str());
-        free_all(*p);
-        delete p;
-        return FSTAT_ERR_ARG;
+        if (st != FSTAT_ERR_OOM || step >= steps) return st;
     }
-    *out = p;
-    return FSTAT_OK;
 }
 
 fstat_status fstat_search(fstat_plan *p, int64_t cell_begin, int64_t cell_end) {
