@@ -10,13 +10,13 @@
 #include <new>
 #include <thread>
 #include <string>
-#include <system_error>
 #include <vector>
 
 #include "device_guard.h"
 #include "dfloat.cuh"
 #include "fft_engine2.cuh"
 #include "fstat_internal.h"
+#include "host_sort.h"
 
 struct fstat_plan : public fstat::Plan {};
 
@@ -944,51 +944,10 @@ constexpr int64_t kDeviceSortMin = 8192;
 constexpr int64_t kHostSortAlways = 1 << 16;  // below, the host sorts when the device has no room
 constexpr int64_t kTileSlack = 4096;          // device positions are 32-bit
 
-// Runs f(t) for t in [0, nt) on nt threads (the calling thread takes t = 0, and what
-// the system gives no thread for).
-template <class Fn>
-void parallel_for_threads(int nt, Fn f) {
-    std::vector<std::thread> th;
-    th.reserve((size_t)nt);
-    int own = nt;   // first slice without a thread
-    for (int t = 1; t < nt; ++t) {
-        try {
-            th.emplace_back(f, t);
-        } catch (const std::system_error &) {
-            own = t;
-            break;
-        }
-    }
-    f(0);
-    for (int t = own; t < nt; ++t) f(t);
-    for (auto &x : th) x.join();
-}
-
-// Sorts n records by (cell, bin), cells from cell0, bins from bin0, in `rec` with `tmp` as the other
-// buffer: least-significant-digit counting passes of up to 11 bits over the key bits of
-// the searched range.
-void sort_records(fstat::CandRecord *rec, fstat::CandRecord *tmp, int64_t n, uint32_t cell0, uint32_t bin0,
-                  int bin_bits, int key_bits) {
-    using fstat::CandRecord;
-    auto key = [&](const CandRecord &r) { return ((uint64_t)(r.cell - cell0) << bin_bits) | (r.bin - bin0); };
-    if (n < 64) {
-        std::sort(rec, rec + n, [&](const CandRecord &a, const CandRecord &b) { return key(a) < key(b); });
-        return;
-    }
-    const int passes = std::max(1, (key_bits + 10) / 11), width = (key_bits + passes - 1) / passes;
-    const uint64_t mask = (uint64_t(1) << width) - 1;
-    std::vector<int64_t> at(size_t(1) << width);
-    CandRecord *src = rec, *dst = tmp;
-    for (int p = 0; p < passes; ++p) {
-        const int shift = p * width;
-        std::fill(at.begin(), at.end(), 0);
-        for (int64_t i = 0; i < n; ++i) ++at[(key(src[i]) >> shift) & mask];
-        int64_t sum = 0;
-        for (auto &c : at) { const int64_t v = c; c = sum; sum += v; }
-        for (int64_t i = 0; i < n; ++i) dst[at[(key(src[i]) >> shift) & mask]++] = src[i];
-        std::swap(src, dst);
-    }
-    if (src != rec) std::copy(src, src + n, rec);
+// Threads that sort or expand n records on the host: one per 65 536.
+int host_threads(int64_t n) {
+    const unsigned hc = std::max(1u, std::thread::hardware_concurrency());
+    return (int)std::min<int64_t>(std::min(hc, 64u), std::max<int64_t>(1, n >> 16));
 }
 
 }  // namespace
@@ -1123,16 +1082,16 @@ fstat_status fstat_candidates_get(fstat_plan *p, fstat_candidate *buf, int64_t c
         }
         if (!dev_sort && kept > 0 && !p->host_sorted) {
             if ((int64_t)p->h_tmp.size() < kept) p->h_tmp.resize((size_t)kept);
-            sort_records(rec, p->h_tmp.data(), kept, (uint32_t)p->cand_begin, (uint32_t)bin0, bin_bits, cell_bits + bin_bits);
+            sort_records(rec, p->h_tmp.data(), kept, (uint32_t)p->cand_begin, (uint32_t)bin0, bin_bits, cell_bits + bin_bits,
+                         host_threads(kept));
             p->host_sorted = true;
         }
         const int64_t nw = std::min<int64_t>(kept, cap);
         const fstat_plan_desc &d = p->desc;
         const int64_t per_band = d.n_sky * d.n_spin;
-        const unsigned hc = std::max(1u, std::thread::hardware_concurrency());
-        // a thread per 65 536 records: 130 us of expansion; with a thread per 16 384, starting them
-        // took up to 4 ms on a busy host
-        const int nt = (int)std::min<int64_t>(std::min(hc, 64u), std::max<int64_t>(1, nw >> 16));
+        // 130 us of expansion a thread; with a thread per 16 384 records, starting them took up to
+        // 4 ms on a busy host
+        const int nt = host_threads(nw);
         parallel_for_threads(nt, [&](int t) {
             // records come cell by cell: what depends on the cell is worked out when it changes
             double alpha = 0.0, delta = 0.0, fdot = 0.0, f_off = 0.0, span_s = 1.0;
