@@ -38,7 +38,8 @@ int alloc_fail_at() {
     return v ? atoi(v) : 0;
 }
 
-// Test hook: FSTAT_TEST_MEM_LIMIT=b lets a plan hold at most b bytes of device memory.
+// Test hook: FSTAT_TEST_MEM_LIMIT=b lets a plan hold at most b bytes of device memory, and the
+// buffers of a read-back's sort beside them.
 bool over_limit(const Plan &p, size_t more) {
     const char *v = getenv("FSTAT_TEST_MEM_LIMIT");
     return v && p.device_bytes + (int64_t)more > atoll(v);
@@ -1048,7 +1049,8 @@ fstat_status fstat_candidates_get(fstat_plan *p, fstat_candidate *buf, int64_t c
             p->sort_hist = nullptr;
             p->sort_cap = 0;
             const int64_t want = std::min<int64_t>(p->cand_capacity, kept + kept / 4);
-            if (cudaMalloc((void **)&p->cand_tmp, want * sizeof(CandRecord)) != cudaSuccess ||
+            if (over_limit(*p, want * sizeof(CandRecord)) ||
+                cudaMalloc((void **)&p->cand_tmp, want * sizeof(CandRecord)) != cudaSuccess ||
                 cudaMalloc((void **)&p->sort_hist, cand_sort_hist(want) * sizeof(uint32_t)) != cudaSuccess) {
                 cudaGetLastError();
                 if (p->cand_tmp) cudaFree(p->cand_tmp);

@@ -56,3 +56,30 @@ def test_plan_fits_in_smaller_batches(fs, form, n, n_fft, n_sky, n_spin, thr, li
     with pytest.raises(fs.FstatError) as e:
         _plan(fs, b, grid, form, thr, 10)
     assert e.value.code == fs.FSTAT_ERR_OOM
+
+
+@pytest.mark.parametrize("n_sky,n_spin,n_bins", [(4, 2, 1024), (4, 2, 4000), (70, 8, 117), (70, 8, 118)])
+def test_read_back_without_room_to_sort(fs, n_sky, n_spin, n_bins):
+    """8192 to 65 535 records are sorted on the host when the device has no room for the sort's
+    second buffer, more are FSTAT_ERR_OOM; with room again the same plan sorts on the device."""
+    w = S.workload(1, n_sky=n_sky, n_spin=n_spin)
+    n = n_sky * n_spin * n_bins
+    with fs.Plan(w.bands, w.alpha, w.delta, w.fdot, -1.0, lat=w.lat, gamma=w.gamma, bin_lo=50, bin_hi=49 + n_bins,
+                 cand_capacity=1 << 17) as p:
+        p.search()
+        os.environ["FSTAT_TEST_MEM_LIMIT"] = str(p.info()["device_bytes"])
+        try:
+            got = [p.candidates_get_status(n) for _ in range(2)]
+        finally:
+            del os.environ["FSTAT_TEST_MEM_LIMIT"]
+        rc, c, total = p.candidates_get_status(n)
+        assert rc == fs.FSTAT_OK and total == n == c.size
+        assert np.array_equal(c["sky"] * n_spin + c["spin"], np.repeat(np.arange(n_sky * n_spin), n_bins))
+        assert np.array_equal(c["bin"], np.tile(np.arange(50, 50 + n_bins), n_sky * n_spin))
+        for rc, early, total in got:
+            if n < 65536:
+                assert rc == fs.FSTAT_OK and np.array_equal(early, c)
+            else:
+                assert rc == fs.FSTAT_ERR_OOM and total == n
+        p.search()                                   # not poisoned
+        assert np.array_equal(p.candidates()[0], c)
