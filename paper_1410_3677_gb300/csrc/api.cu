@@ -929,6 +929,8 @@ fstat_status guarded(fstat_plan *p, F &&f) {
     } catch (const std::string &m) {
         p->err = m;
         return FSTAT_ERR_ARG;
+    } catch (...) {   // nothing throws across the ABI
+        return FSTAT_ERR_INTERNAL;
     }
 }
 
@@ -983,6 +985,8 @@ fstat_status fstat_plan_create(fstat_plan **out, const fstat_plan_desc *desc) {
         } catch (const std::string &m) {
             if (getenv("FSTAT_LOG")) fprintf(stderr, "fstat_plan_create: %s\n", m.c_str());
             st = FSTAT_ERR_ARG;
+        } catch (...) {
+            st = FSTAT_ERR_INTERNAL;
         }
         free_all(*p);
         delete p;

@@ -5,7 +5,6 @@
 #include <stdint.h>
 
 #include <algorithm>
-#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -21,7 +20,7 @@ void parallel_for_threads(int nt, Fn f) {
     for (int t = 1; t < nt; ++t) {
         try {
             th.emplace_back(f, t);
-        } catch (const std::system_error &) {
+        } catch (...) {   // no thread, or no memory for its state: joinable threads must not be left behind
             own = t;
             break;
         }

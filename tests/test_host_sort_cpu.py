@@ -54,3 +54,43 @@ def _run(tmp_path, prog):
 def test_host_sort_matches_a_stable_sort(tmp_path):
     runs, bad = _run(tmp_path, PROG)
     assert int(runs) == 4 * 9 * 4 * 4 and int(bad) == 0
+
+
+FAILING = r"""
+#include <cstdio>
+#include <new>
+#include "host_sort.h"
+static int made, joined, fail_at, kind;
+struct Thread {
+    bool joinable = true;
+    template <class F> Thread(F f, int t) {
+        if (t == fail_at) {
+            if (kind == 0) throw std::bad_alloc();
+            throw std::system_error(std::make_error_code(std::errc::resource_unavailable_try_again));
+        }
+        ++made;
+        f(t);
+    }
+    Thread(Thread &&o) : joinable(o.joinable) { o.joinable = false; }
+    ~Thread() { if (joinable) std::terminate(); }
+    void join() { joinable = false; ++joined; }
+};
+int main() {
+    for (kind = 0; kind < 2; ++kind)
+        for (fail_at = 1; fail_at <= 6; ++fail_at) {
+            made = joined = 0;
+            int seen[6] = {};
+            fstat::parallel_for_threads<Thread>(6, [&](int t) { ++seen[t]; });
+            int once = 0;
+            for (int v : seen) once += v == 1;
+            printf("%d %d %d\n", made, joined, once);
+        }
+}
+"""
+
+
+def test_threads_that_cannot_be_made(tmp_path):
+    """Whatever the creation of a thread throws, the threads made before are joined and every
+    slice of the loop has run once."""
+    v = [int(x) for x in _run(tmp_path, FAILING.replace("#include <new>", "#include <new>\n#include <system_error>"))]
+    assert v == 2 * [x for f in range(1, 7) for x in (f - 1 if f < 6 else 5, f - 1 if f < 6 else 5, 6)]
