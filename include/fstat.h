@@ -231,13 +231,16 @@ fstat_status fstat_plan_kernel_stats(const fstat_plan *plan, fstat_kernel_stat *
 /* Launch-shape autotuner of an FSTAT_FP32_BATCHED plan (the paper's farm has no
    counterpart; it picks the GPU-side shapes the search runs with).  It times
    whole searches over the cells [0, sample_cells) (clamped to the grid) with
-   CUDA events, changing one choice at a time -- FFT engine (two-stage radix
-   32x16 / radix-8 Stockham), pass-2 tile (128 or 256 threads; one or four rows
-   per CTA for the paired 512-point rows) and loader (bulk
-   copies or per-thread loads with L2 prefetch), cells per launch pair, one fused
-   ticket-ordered launch or two launches, and at N_fft = 2^18 the passes in
-   paired FP32 instructions (two values per instruction: none, pass 2 only, or
-   both passes) -- keeps a change only when it is at
+   CUDA events, changing one choice at a time -- FFT engine (two-stage / radix-8
+   Stockham), threads of the scalar pass 2 (128 or 256; 256 also turns the paired
+   kernels off), rows per CTA of the paired 512-point rows (one or four; N_fft =
+   2^18), loader of pass 2 (bulk copies or per-thread loads; the latter also turns
+   the paired kernels off), cells per launch pair, one fused ticket-ordered launch
+   or two launches, and paired FP32 instructions (two values per instruction: none,
+   the default set, or at N_fft = 2^18 both passes).  Paired kernels serve the rows
+   of 64 .. 512 points, the 1024-point columns and the 2^19 transforms; the
+   1024-point rows (2^20) are paired and staged by bulk copies whatever is chosen.
+   It keeps a change only when it is at
    least 1 % faster, and leaves the plan configured with the best found.  The
    candidates of the tuning searches are discarded (fstat_candidates_get then
    reports none until the next fstat_search).  *chosen (may be NULL) receives the
@@ -245,11 +248,13 @@ fstat_status fstat_plan_kernel_stats(const fstat_plan *plan, fstat_kernel_stat *
    depend on the choice beyond FP32 rounding (every shape computes the same
    transforms).  FSTAT_ERR_ARG for an FP64_PLAIN plan or sample_cells < 1. */
 typedef struct {
-    int32_t engine;          /* 2: two-stage engine, 1: radix-8 engine; 3: two-stage with
-                                pass 2 in paired FP32 instructions at N_fft = 2^18, 4: with
-                                both passes paired */
-    int32_t pass2_threads;   /* threads per pass-2 CTA: 32 (one row) or 128 for the paired
-                                512-point rows, 128 or 256 for the scalar pass 2 */
+    int32_t engine;          /* 1: radix-8 engine, 2: two-stage engine, 3: two-stage with the
+                                paired kernels, 4: at N_fft = 2^18 pass 1 paired too */
+    int32_t pass2_threads;   /* threads per pass-2 CTA of the band with the longest transform: 32
+                                (one row, or two short ones) or 128 for paired rows up to 512
+                                points, 64 for 1024-point rows, 192 to 384 for short interbinning
+                                rows, 128 or 256 for the scalar pass 2, 256 for the radix-8
+                                engine and the fused launch */
     int32_t pass2_bulk_copy; /* 1: bulk-copy staging, 0: per-thread loads */
     int32_t fused;           /* 1: one ticket-ordered launch per batch */
     int64_t cells_per_launch;

@@ -1268,8 +1268,12 @@ fstat_status fstat_plan_autotune(fstat_plan *p, int64_t sample_cells, fstat_tuni
         (void)cb0;
         { const int old = p->p2_threads;
           try_set([&] { p->p2_threads = old == 128 ? 256 : 128; }, [&] { p->p2_threads = old; }); }
-        { const int old = p->p2_ts;   // the paired rows: one or four rows per CTA
-          try_set([&] { p->p2_ts = old == 32 ? 128 : 32; }, [&] { p->p2_ts = old; }); }
+        // the paired 512-point rows of 2^18: one or four rows per CTA
+        const bool rows512 = !p->interbin && std::any_of(p->bands.begin(), p->bands.end(), [](const BandDev &b) { return b.logn == 18; });
+        if (rows512) {
+            const int old = p->p2_ts;
+            try_set([&] { p->p2_ts = old == 32 ? 128 : 32; }, [&] { p->p2_ts = old; });
+        }
         { const bool old = p->tma;
           try_set([&] { p->tma = !old; }, [&] { p->tma = old; }); }
         { const bool old = p->fused;
@@ -1289,11 +1293,10 @@ fstat_status fstat_plan_autotune(fstat_plan *p, int64_t sample_cells, fstat_tuni
         p->searched = false;
         p->prev_begin = p->prev_end = -1;
         if (chosen) {
-            // the paired pass 2 (512-point rows) runs whenever packed >= 1 with the
-            // bulk-copy loader and 128-thread scalar tiles
-            const bool paired2 = p->packed >= 1 && p->tma && p->p2_threads == 128;
-            chosen->engine = p->engine == 2 && paired2 ? 2 + p->packed : p->engine;
-            chosen->pass2_threads = paired2 ? p->p2_ts : p->p2_threads;
+            const BandDev &longest = *std::max_element(p->bands.begin(), p->bands.end(),
+                                                       [](const BandDev &a, const BandDev &b) { return a.logn < b.logn; });
+            chosen->engine = p->engine == 2 && packed_rows(*p) ? 2 + p->packed : p->engine;
+            chosen->pass2_threads = pass2_threads_f32(*p, longest);
             chosen->pass2_bulk_copy = p->tma ? 1 : 0;
             chosen->fused = p->fused ? 1 : 0;
             chosen->cells_per_launch = p->cell_batch;

@@ -331,8 +331,13 @@ inline cudaError_t record_timing_event(cudaEvent_t e, cudaStream_t s) {
 // Whether a band of transform length 2^logn (the n_fft bin grid) can run in the
 // interbinning form (a half-length transform of 2^12 .. 2^19).
 bool interbin_supported(int logn);
+// Whether the two-stage FP32 searches take the packed kernels with bulk copies (passes3.cuh): the
+// rows up to 512 points and the 2^19 split.  The 1024-point rows always do.
+inline bool packed_rows(const Plan &p) { return p.packed >= 1 && p.tma && p.p2_threads == 128; }
 // The split (log2 N, or kTall + log2 N) an FP32 search of length 2^logn runs with.
 int search_key_f32(const Plan &p, int logn);
+// Threads per CTA of the pass 2 that searches the band.
+int pass2_threads_f32(const Plan &p, const BandDev &b);
 // Whether the FP32 cells of a band of length 2^logn run as one fused launch.
 bool fused_supported(const Plan &p, int logn);
 // `mid` (may be null) is recorded between the two passes.

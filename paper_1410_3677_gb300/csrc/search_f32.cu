@@ -64,7 +64,9 @@ void launch_pass2p(const Plan &p, int band_idx, const BandDev &b, int64_t s0, in
 }
 
 // Short rows (64 .. 256 points) in packed pairs, zero-padded or interbinning.
-bool rows_packed(const Plan &p) { return p.packed >= 1 && p.tma && p.p2_threads != 256 && p.p2_rows; }
+bool rows_packed(const Plan &p) { return packed_rows(p) && p.p2_rows; }
+// Warps per interbinning tile: few enough rows computed twice (one pair per tile) at 24 warps per SM.
+constexpr int ib_warps(int logn) { return logn == 12 || logn == 15 ? 8 : logn <= 14 ? 6 : 12; }
 
 template <int LOGN, bool LOWER, bool IB, int W>
 void launch_rows(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_t c0, int64_t nc, cudaStream_t s,
@@ -92,7 +94,7 @@ int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_
     using C2 = Cfg2<LOGN, 2>;
     // 512-point rows (N_fft = 2^18, 2^19): pass 2 in paired FP32 arithmetic; at 2^18
     // (512-point columns) also pass 1 with packed = 2 or 3
-    const bool pk2 = (LOGN == 18 || LOGN == 19) && p.packed >= 1 && p.tma && p.p2_threads == 128 && tw->p512_f;
+    const bool pk2 = (LOGN == 18 || LOGN == 19) && packed_rows(p) && tw->p512_f;
     const bool pk1 = pk2 && LOGN == 18 && p.packed >= 2;
     // A bin range shorter than N2 touches some of the rows l2 = bin mod N2 only (a follow-up
     // about known candidates): the packed pass 2 runs over their tiles, and while they are at
@@ -332,8 +334,7 @@ int launch_interbin(const Plan &p, int band_idx, const BandDev &b, int64_t s0, i
     if (mid) record_timing_event(mid, s);
     if constexpr (LOGN <= 17) {
         if (rows_packed(p)) {
-            // warps per tile: few enough rows computed twice (one pair per tile) at 24 warps per SM
-            constexpr int W = LOGN == 12 || LOGN == 15 ? 8 : LOGN <= 14 ? 6 : 12;
+            constexpr int W = ib_warps(LOGN);
             constexpr RowRange all{0, p3::RowGeom<LOGN, W>::TILES_IB};
             if (b.hi < (int64_t)C2::N) launch_rows<LOGN, true, true, W>(p, band_idx, b, s0, c0, nc, s, cb, tw, all);
             else launch_rows<LOGN, false, true, W>(p, band_idx, b, s0, c0, nc, s, cb, tw, all);
@@ -400,8 +401,19 @@ void launch_row_twiddles(float4 *t, int logn, cudaStream_t s) {
 // Measured per 2^18 points, both passes: 0.977 + 0.627 -> 0.755 + 0.735 us (n <= 3N/8), 1.081 +
 // 0.627 -> 0.860 + 0.734 (n > 3N/8).
 int search_key_f32(const Plan &p, int logn) {
-    const bool tall = logn == 19 && p.engine == 2 && !p.interbin && !p.fused && p.packed >= 1 && p.tma && p.p2_threads == 128;
+    const bool tall = logn == 19 && p.engine == 2 && !p.interbin && !p.fused && packed_rows(p);
     return tall ? kTall + logn : logn;
+}
+
+int pass2_threads_f32(const Plan &p, const BandDev &b) {
+    const int lg = b.logn - (p.interbin ? 1 : 0);
+    if (p.interbin) return lg <= 17 && rows_packed(p) ? 32 * ib_warps(lg) : p.tma ? 128 : 256;
+    if (p.engine == 1 || lg < 12 || fused_supported(p, lg)) return 256;
+    const int key = search_key_f32(p, lg);
+    if (log_n1(key) == 10) return 64;
+    if (key >= 18 && packed_rows(p)) return p.p2_ts;
+    if (key <= 17 && rows_packed(p)) return 32;
+    return p.tma ? p.p2_threads : 256;
 }
 
 bool interbin_supported(int logn) { return logn - 1 >= 12 && logn - 1 <= 19; }

@@ -300,6 +300,28 @@ def test_autotune_keeps_results(fs):
         assert len(common) >= 0.99 * min(len(ref), len(c))
 
 
+@pytest.mark.parametrize("n,n_fft,interbin,paired", [
+    (4096, 1 << 13, False, (32,)), (86164, 1 << 18, False, (32, 128)), (172328, 1 << 19, False, (64,)),
+    (344656, 1 << 20, False, (64,)), (4096, 1 << 13, True, (256,)), (86164, 1 << 18, True, (384,)),
+    (172328, 1 << 19, True, (128,))])
+def test_autotune_reports_the_kernels_that_run(fs, n, n_fft, interbin, paired):
+    """pass2_threads is the CTA size of the pass 2 that searches the band, whatever was chosen."""
+    al, de = S.fibonacci_sky(16)
+    b = S.make_band(n, 2.0, 5, 1.0, al, de, np.array([0.0]), [], n_fft=n_fft)
+    with fs.Plan([b], al, de, np.array([0.0, -1e-9]), 30.0, lat=S.LAT_DEFAULT, gamma=S.GAMMA_DEFAULT,
+                 form=fs.FP32_BATCHED, interbin=interbin) as p:
+        t = p.autotune(32)
+    scalar = 128 if t["pass2_bulk_copy"] and t["pass2_threads"] != 256 else 256
+    if t["engine"] == 1 and not interbin:
+        assert t["pass2_threads"] == 256
+    elif t["fused"] and not interbin and n_fft < 1 << 20:
+        assert t["pass2_threads"] == 256
+    elif t["engine"] >= 3 or n_fft == 1 << 20:
+        assert t["pass2_threads"] in paired
+    else:
+        assert t["pass2_threads"] == scalar
+
+
 @pytest.mark.parametrize("env", [
     {"FSTAT_PERSISTENT": "1", "FSTAT_PERSIST_BATCH": "3"},     # warp-specialised persistent kernel
     {"FSTAT_FUSED": "1", "FSTAT_FUSED_BATCH": "4"},             # queue-fed persistent launch
