@@ -949,8 +949,8 @@ constexpr int64_t kTileSlack = 4096;          // device positions are 32-bit
 
 // Threads that sort or expand n records on the host: one per 65 536.
 int host_threads(int64_t n) {
-    const unsigned hc = std::max(1u, std::thread::hardware_concurrency());
-    return (int)std::min<int64_t>(std::min(hc, 64u), std::max<int64_t>(1, n >> 16));
+    if (n >> 16 <= 1) return 1;   // without asking for the number of cores
+    return (int)std::min<int64_t>(std::min(std::max(1u, std::thread::hardware_concurrency()), 64u), n >> 16);
 }
 
 }  // namespace

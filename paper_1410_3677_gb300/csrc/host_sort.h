@@ -30,38 +30,60 @@ void parallel_for_threads(int nt, Fn f) {
     for (auto &x : th) x.join();
 }
 
+// One digit of the key (cell - cell0) << bin_bits | (bin - bin0).  The loops over a run of
+// records take everything by value: through references captured for the threads every record
+// reloaded them (4032 records 32 -> 58 us).
+struct KeyDigit {
+    uint32_t cell0, bin0;
+    int bin_bits, shift;
+    uint64_t mask;
+    template <class Rec>
+    uint64_t operator()(const Rec &r) const {
+        return ((((uint64_t)(r.cell - cell0) << bin_bits) | (r.bin - bin0)) >> shift) & mask;
+    }
+};
+template <class Rec>
+void count_run(const Rec *src, int64_t n, KeyDigit d, int64_t *at) {
+    for (int64_t i = 0; i < n; ++i) ++at[d(src[i])];
+}
+template <class Rec>
+void place_run(const Rec *src, int64_t n, KeyDigit d, int64_t *at, Rec *dst) {
+    for (int64_t i = 0; i < n; ++i) dst[at[d(src[i])]++] = src[i];
+}
+
 // Sorts n records by (cell, bin), cells from cell0, bins from bin0, in `rec` with `tmp` as the other
 // buffer: least-significant-digit counting passes of up to 11 bits over the key bits of
 // the searched range, each thread counting and placing a run of the records.
 template <class Rec>
 void sort_records(Rec *rec, Rec *tmp, int64_t n, uint32_t cell0, uint32_t bin0, int bin_bits, int key_bits, int nt) {
-    auto key = [&](const Rec &r) { return ((uint64_t)(r.cell - cell0) << bin_bits) | (r.bin - bin0); };
     if (n < 64) {
-        std::sort(rec, rec + n, [&](const Rec &a, const Rec &b) { return key(a) < key(b); });
+        const KeyDigit key{cell0, bin0, bin_bits, 0, ~uint64_t(0)};
+        std::sort(rec, rec + n, [key](const Rec &a, const Rec &b) { return key(a) < key(b); });
         return;
     }
     const int passes = std::max(1, (key_bits + 10) / 11), width = (key_bits + passes - 1) / passes;
-    const uint64_t digits = uint64_t(1) << width, mask = digits - 1;
+    const uint64_t digits = uint64_t(1) << width;
     std::vector<int64_t> at((size_t)nt * digits);   // [thread][digit]
+    int64_t *const all = at.data();
     Rec *src = rec, *dst = tmp;
     for (int p = 0; p < passes; ++p) {
-        const int shift = p * width;
-        parallel_for_threads(nt, [&](int t) {
-            int64_t *c = &at[(size_t)t * digits];
-            std::fill(c, c + digits, 0);
-            for (int64_t i = n * t / nt; i < n * (t + 1) / nt; ++i) ++c[(key(src[i]) >> shift) & mask];
+        const KeyDigit d{cell0, bin0, bin_bits, p * width, digits - 1};
+        std::fill(at.begin(), at.end(), 0);
+        parallel_for_threads(nt, [=](int t) {
+            const int64_t a = n * t / nt, b = n * (t + 1) / nt;
+            count_run(src + a, b - a, d, all + (size_t)t * digits);
         });
         int64_t sum = 0;
-        for (uint64_t d = 0; d < digits; ++d)
+        for (uint64_t k = 0; k < digits; ++k)
             for (int t = 0; t < nt; ++t) {
-                int64_t &c = at[(size_t)t * digits + d];
+                int64_t &c = all[(size_t)t * digits + k];
                 const int64_t v = c;
                 c = sum;
                 sum += v;
             }
-        parallel_for_threads(nt, [&](int t) {
-            int64_t *c = &at[(size_t)t * digits];
-            for (int64_t i = n * t / nt; i < n * (t + 1) / nt; ++i) dst[c[(key(src[i]) >> shift) & mask]++] = src[i];
+        parallel_for_threads(nt, [=](int t) {
+            const int64_t a = n * t / nt, b = n * (t + 1) / nt;
+            place_run(src + a, b - a, d, all + (size_t)t * digits, dst);
         });
         std::swap(src, dst);
     }
