@@ -1276,13 +1276,15 @@ fstat_status fstat_plan_autotune(fstat_plan *p, int64_t sample_cells, fstat_tuni
         }
         { const bool old = p->tma;
           try_set([&] { p->tma = !old; }, [&] { p->tma = old; }); }
-        { const bool old = p->fused;
-          try_set([&] { p->fused = !old; }, [&] { p->fused = old; }); }
-        { const int old = p->engine;
-          try_set([&] { p->engine = old == 2 ? 1 : 2; }, [&] { p->engine = old; }); }
-        for (int pkv : {0, 2}) {   // paired arithmetic in neither pass, or in both
+        if (!p->interbin) {   // interbinning has one engine and two launches
+            const bool old = p->fused;
+            try_set([&] { p->fused = !old; }, [&] { p->fused = old; });
+            const int olde = p->engine;
+            try_set([&] { p->engine = olde == 2 ? 1 : 2; }, [&] { p->engine = olde; });
+        }
+        for (int pkv : {0, 2}) {   // paired arithmetic in neither pass, or at 2^18 in both
             const int old = p->packed;
-            if (pkv == old) continue;
+            if (pkv == old || (pkv == 2 && !rows512)) continue;
             try_set([&] { p->packed = pkv; }, [&] { p->packed = old; });
         }
         p->ev_pool.push_back(e0);
