@@ -12,6 +12,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <atomic>
+
 #include "fft_engine.cuh"
 #include "fstat_internal.h"
 
@@ -298,9 +301,31 @@ k_pass(LD ld, ST st, const T *__restrict__ tw) {
     eng::run_pass<T, C::M, C::F, C::EH, DIR, MAPM>(ld, st, tw);
 }
 
+// A kernel's limit of dynamic shared memory is a property of the device: set at every launch
+// (0.2 us on the host, nothing when a graph is replayed).
 template <class KernelPtr>
 inline void set_smem(KernelPtr k, size_t bytes) {
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
+
+// CTAs of a kernel that the current device holds at once, worked out once per device.
+struct Resident {
+    static constexpr int kDevices = 64;
+    std::atomic<int> count[kDevices] = {};
+    template <class KernelPtr>
+    int operator()(KernelPtr k, int threads, size_t smem) {
+        set_smem(k, smem);
+        int dev = 0;
+        cudaGetDevice(&dev);
+        int n = dev >= 0 && dev < kDevices ? count[dev].load(std::memory_order_relaxed) : 0;
+        if (n) return n;
+        int sms = 0, per_sm = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem);
+        n = std::max(1, per_sm) * std::max(1, sms);
+        if (dev >= 0 && dev < kDevices) count[dev].store(n, std::memory_order_relaxed);
+        return n;
+    }
+};
 
 }  // namespace fstat

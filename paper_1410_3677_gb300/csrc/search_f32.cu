@@ -36,8 +36,7 @@ void launch_pass2(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int
     using C2 = Cfg2<LOGN, 2, TS>;
     const auto st2 = make_epi<LOGN, LOWER, TS>(p, band_idx, b, c0, s0, cb);
     auto k2 = k_pass2<LOGN, 2, eng2::kMapW, LD2, SearchEpi2<C2, LOWER>, TS>;
-    static bool attr2 = false;
-    if (!attr2) { set_smem(k2, C2::SMEM + extra); attr2 = true; }
+    set_smem(k2, C2::SMEM + extra);
     k2<<<dim3(C2::TILES, (unsigned)nc), C2::THREADS, C2::SMEM + extra, s>>>(ld2, st2, tw->s1_f);
 }
 
@@ -116,9 +115,7 @@ int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_
             const bool hy = p.packed == 3;
             auto k1 = hy ? (z3 ? p3::k_pass1h<LOGN, 3> : p3::k_pass1h<LOGN, 4>)
                          : (z3 ? p3::k_pass1p<LOGN, 3> : p3::k_pass1p<LOGN, 4>);
-            static bool attr1p[4] = {false, false, false, false};
-            const int ai = (hy ? 2 : 0) + (z3 ? 1 : 0);
-            if (!attr1p[ai]) { set_smem(k1, C1::SMEM); attr1p[ai] = true; }
+            set_smem(k1, C1::SMEM);
             k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, C1::SMEM, s>>>(ld1, st1, tw->p512_f);
         }
     }
@@ -154,8 +151,7 @@ int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_
         }
         if (!launched && 8 * b.n <= 3 * (int64_t)C1::N) {
             auto k1 = k_pass2<LOGN, 1, eng2::kMapFJ, SearchLoad2<C1>, ScratchStore2<C1>, 256, 3>;
-            static bool attr3 = false;
-            if (!attr3) { set_smem(k1, C1::SMEM); attr3 = true; }
+            set_smem(k1, C1::SMEM);
             k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, C1::SMEM, s>>>(ld1, st1, tw->s2_f);
             launched = true;
         }
@@ -173,8 +169,7 @@ int launch_two(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_
     }
     if (!launched) {
         auto k1 = k_pass2<LOGN, 1, eng2::kMapFJ, SearchLoad2<C1>, ScratchStore2<C1>, 256, 4>;
-        static bool attr1 = false;
-        if (!attr1) { set_smem(k1, C1::SMEM); attr1 = true; }
+        set_smem(k1, C1::SMEM);
         k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, C1::SMEM, s>>>(ld1, st1, tw->s2_f);
     }
     if (mid) record_timing_event(mid, s);
@@ -247,16 +242,8 @@ int launch_fused(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int6
     const bool z3 = eng2::radix0(C1::M) == 32 && 8 * b.n <= 3 * (int64_t)C1::N;
     auto k = z3 ? k_search_fused<LOGN, LOWER, eng2::radix0(C1::M) == 32 ? 3 : 4>
                 : k_search_fused<LOGN, LOWER, 4>;
-    static int resident[2] = {0, 0};   // CTAs of each variant that fit on the device at once
-    int &res = resident[z3 ? 1 : 0];
-    if (!res) {
-        set_smem(k, smem);
-        int dev = 0, sms = 0, per_sm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem);
-        res = std::max(1, sms * std::max(per_sm, 1));
-    }
+    static Resident resident[2];
+    const int res = resident[z3 ? 1 : 0](k, 256, smem);
     const int64_t items = (nc + p.fused_ahead) * (int64_t)(C1::TILES / tpi + C2::TILES / tpi);
     const unsigned grid = (unsigned)std::min<int64_t>(items, res);
     k<<<grid, 256, smem, s>>>(ld1, st1, ld2, st2, tw->s1_f, tw->s2_f, ctl);
@@ -350,8 +337,7 @@ int launch_interbin(const Plan &p, int band_idx, const BandDev &b, int64_t s0, i
         ld2.err = p.qerr;
         const auto ep = make_epi<LOGN, false, 128>(p, band_idx, b, c0, s0, cb);
         auto k2 = k_pass2_ib<LOGN, 128, ScratchLoadIBTMA<D2>>;
-        static bool attr2t = false;
-        if (!attr2t) { set_smem(k2, D2::SMEM + 16); attr2t = true; }
+        set_smem(k2, D2::SMEM + 16);
         k2<<<dim3(IBGeom<LOGN, 128>::TILES, (unsigned)nc), D2::THREADS, D2::SMEM + 16, s>>>(ld2, ep, tw->in1_f);
         return 2;
     }
@@ -360,8 +346,7 @@ int launch_interbin(const Plan &p, int band_idx, const BandDev &b, int64_t s0, i
     ld2.tw = {tw->lo_f, tw->hi_f};
     const auto ep = make_epi<LOGN, false>(p, band_idx, b, c0, s0, cb);
     auto k2 = k_pass2_ib<LOGN, 256, ScratchLoadIB<C2>>;
-    static bool attr2 = false;
-    if (!attr2) { set_smem(k2, C2::SMEM); attr2 = true; }
+    set_smem(k2, C2::SMEM);
     k2<<<dim3(IBGeom<LOGN>::TILES, (unsigned)nc), C2::THREADS, C2::SMEM, s>>>(ld2, ep, tw->in1_f);
     return 2;
 }

@@ -47,8 +47,7 @@ int launch_t(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_t 
     ST1 st1{};
     st1.scratch = reinterpret_cast<double2 *>(cb.scratch);
     auto k1 = p64::k_pass64<LOGN, 1, LD1, ST1, Z1>;
-    static bool attr1 = false;
-    if (!attr1) { set_smem(k1, C1::SMEM); attr1 = true; }
+    set_smem(k1, C1::SMEM);
     k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, C1::SMEM, s>>>(ld1, st1, tw->s2_d);
     if (mid) record_timing_event(mid, s);
 
@@ -70,8 +69,7 @@ int launch_t(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_t 
     st2.count = p.cand_count;
     st2.cap = (unsigned long long)p.cand_capacity;
     auto k2 = p64::k_pass64<LOGN, 2, LD2, ST2, 8>;
-    static bool attr2 = false;
-    if (!attr2) { set_smem(k2, C2::SMEM); attr2 = true; }
+    set_smem(k2, C2::SMEM);
     const RowRange rr = searched_rows(b, C2::N2, C2::F);
     st2.tile0 = rr.tile0;
     k2<<<dim3(rr.tiles, (unsigned)nc), C2::THREADS, C2::SMEM, s>>>(ld2, st2, tw->s1_d);

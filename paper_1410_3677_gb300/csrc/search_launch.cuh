@@ -41,8 +41,7 @@ int launch_search_t(const Plan &p, int band_idx, const BandDev &b, int64_t s0, i
     st1.hi = thi;
     st1.n_tr = 2 * nc;
     auto k1 = k_pass<T, LOGN, 1, -1, eng::kMapFJ, LD1, ST1, TS, EHT>;
-    static bool attr1 = false;
-    if (!attr1) { set_smem(k1, C1::SMEM); attr1 = true; }
+    set_smem(k1, C1::SMEM);
     k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, C1::SMEM, s>>>(ld1, st1, tin2);
     if (mid) record_timing_event(mid, s);
 
@@ -63,8 +62,7 @@ int launch_search_t(const Plan &p, int band_idx, const BandDev &b, int64_t s0, i
     st2.count = p.cand_count;
     st2.cap = (unsigned long long)p.cand_capacity;
     auto k2 = k_pass<T, LOGN, 2, -1, eng::kMapW, LD2, ST2, TS, EHT>;
-    static bool attr2 = false;
-    if (!attr2) { set_smem(k2, C2::SMEM); attr2 = true; }
+    set_smem(k2, C2::SMEM);
     k2<<<dim3(C2::TILES, (unsigned)nc), C2::THREADS, C2::SMEM, s>>>(ld2, st2, tin1);
     return 2;
 }

@@ -338,16 +338,9 @@ template <int LOGN>
 int launch_t(const Plan &p, int band_idx, const BandDev &b, int64_t s0, int64_t c_lo,
              int64_t c_hi, cudaStream_t s, const CellBufs &cb) {
     using P = PC<LOGN>;
-    static int grid = 0;
+    static Resident resident;
     auto k = k_search_persistent<LOGN>;
-    if (grid == 0) {
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::SMEM);
-        int per_sm = 0, dev = 0, sms = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kThreads, P::SMEM);
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        grid = std::max(1, per_sm) * std::max(1, sms);
-    }
+    const int grid = resident(k, kThreads, P::SMEM);
     const TwiddleSet *tw = p.twiddles(LOGN);
     PArgs a;
     a.w = reinterpret_cast<const float4 *>(cb.w);

@@ -62,3 +62,11 @@ def test_every_call_on_a_plan_is_guarded():
         name, first, second = m.groups()
         assert "return guarded(p, " in first or "DeviceGuard<CudaDevice> on_device(p->device)" in second, name
     assert len(re.findall(r"return guarded\(p, ", txt)) >= 6
+
+
+def test_no_process_wide_state_stands_for_a_device():
+    """A kernel's shared-memory limit and the number of its CTAs that fit belong to a device: no
+    function-local flag or count of the process decides about them."""
+    for f in sorted(os.listdir(CSRC)):
+        txt = open(os.path.join(CSRC, f)).read()
+        assert not re.findall(r"\n +static (?:bool|int|size_t) \w+(?:\[[^\]]*\])? *[={;][^\n]*", txt), f
