@@ -202,3 +202,26 @@ def test_fp32_error_beside_a_strong_line(fs, lg, n_sky, n_spin):
     assert total == ref.size and ref.max() > 100.0
     err = np.abs(c["F"].reshape(ref.shape) - ref) / np.maximum(ref, 2.0)
     assert err.max() <= 4 * 2.0 ** -24 * 2.0 * math.sqrt(ref.max() / 2.0), (err.max(), ref.max())
+
+
+@pytest.mark.parametrize("form,n,n_fft", [(1, 2000, 1 << 12), (1, 5000, 1 << 14), (1, 60000, 1 << 17), (1, 86164, 1 << 18),
+                                          (1, 172328, 1 << 19), (1, 344656, 1 << 20), (0, 20000, 1 << 16)])
+def test_narrow_bin_ranges_full_statistic(fs, form, n, n_fft):
+    """The launches over some of the rows with the cross term give the records of a search of all
+    bins, bit for bit: one bin, a range across the last row and the first, and half of the rows."""
+    n2 = 1 << ((n_fft.bit_length() - 1 + 1) // 2)
+    alpha, delta = S.fibonacci_sky(2)
+    fdot = S.spindown_grid(2, -1e-8, 0.0)
+    b = S.make_band(n, 0.5, 19 + n, 1.0, alpha, delta, fdot, [], f_off=100.5, n_fft=n_fft)
+
+    def records(lo, hi):
+        with fs.Plan([b], alpha, delta, fdot, -1e9, lat=S.LAT_DEFAULT, gamma=S.GAMMA_DEFAULT, form=form, full=True,
+                     bin_lo=lo, bin_hi=hi, cand_capacity=4 * (hi - lo + 1)) as p:
+            p.search()
+            c, total = p.candidates()
+        assert total == c.size == 4 * (hi - lo + 1)
+        return c
+
+    whole = records(0, 6 * n2)
+    for lo, hi in ((3 * n2 + 5, 3 * n2 + 5), (3 * n2 - 3, 3 * n2 + 2), (n2 + 1, n2 + n2 // 2)):
+        assert np.array_equal(records(lo, hi), whole[(whole["bin"] >= lo) & (whole["bin"] <= hi)])
