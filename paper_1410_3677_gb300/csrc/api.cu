@@ -457,7 +457,7 @@ void create_impl(Plan &p, const fstat_plan_desc *d, int step) {
         check(cudaMemsetAsync(p.wbuf[q], 0, (size_t)p.sky_batch * p.w_stride * w_elem, s), "memset");
     }
     if (!fp32) p.dbuf = dalloc<double>(p, (size_t)p.sky_batch * p.n_max, n_alloc);   // per-sample delays
-    p.partials = dalloc<double>(p, std::max<int64_t>((int64_t)p.sky_batch * nblk * 3, 256), n_alloc);
+    p.partials = dalloc<double>(p, (size_t)p.sky_batch * nblk * 3, n_alloc);
     p.S = dalloc<double>(p, 3 * p.sky_batch, n_alloc);
     p.sigma_parts = dalloc<double>(p, kSigmaParts, n_alloc);
     for (int q = 0; q < 2; ++q) p.normbuf[q] = dalloc<double>(p, kNormStride * p.sky_batch, n_alloc);

@@ -16,13 +16,13 @@
 namespace fstat {
 namespace cod {
 
-// cos(pi m / 16)
+// cos(pi m / 16), |m| <= 8
 __host__ __device__ constexpr double cos16(int m) {
-    return m < 0 ? cos16(-m)
-         : m == 0 ? 1.0 : m == 1 ? 0.98078528040323044913 : m == 2 ? 0.92387953251128675613
-         : m == 3 ? 0.83146961230254523708 : m == 4 ? 0.70710678118654752440
-         : m == 5 ? 0.55557023301960222474 : m == 6 ? 0.38268343236508977173
-         : m == 7 ? 0.19509032201612826785 : 0.0;
+    const int a = m < 0 ? -m : m;
+    return a == 0 ? 1.0 : a == 1 ? 0.98078528040323044913 : a == 2 ? 0.92387953251128675613
+         : a == 3 ? 0.83146961230254523708 : a == 4 ? 0.70710678118654752440
+         : a == 5 ? 0.55557023301960222474 : a == 6 ? 0.38268343236508977173
+         : a == 7 ? 0.19509032201612826785 : 0.0;
 }
 __host__ __device__ constexpr double tan16(int m) { return m < 0 ? -tan16(-m) : cos16(8 - m) / cos16(m); }
 // W_32^e = i^turn (1 - i tan16(dev)) cos16(dev), |dev| <= 4

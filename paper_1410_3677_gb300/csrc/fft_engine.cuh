@@ -59,8 +59,8 @@ template <typename T, int M, int F>
 __host__ __device__ constexpr size_t smem_bytes() { return exch_bytes<T, M, F>() + 2 * sizeof(T) * (size_t)tw_entries(M); }
 
 // ------------------------------------------------------------------ small DFTs
-// Natural order in and out; DIR = -1 computes sum_j v_j e^{-2 pi i jk/R}.
-template <int DIR, typename T>
+// Natural order in and out: sum_j v_j e^{-2 pi i jk/R}.
+template <typename T>
 __device__ __forceinline__ void dft2(T *re, T *im) {
     T tr = re[0] - re[1], ti = im[0] - im[1];
     re[0] += re[1];
@@ -69,38 +69,36 @@ __device__ __forceinline__ void dft2(T *re, T *im) {
     im[1] = ti;
 }
 
-template <int DIR, typename T>
+template <typename T>
 __device__ __forceinline__ void dft4(T &r0, T &i0, T &r1, T &i1, T &r2, T &i2, T &r3, T &i3) {
     T t0r = r0 + r2, t0i = i0 + i2;
     T t1r = r0 - r2, t1i = i0 - i2;
     T t2r = r1 + r3, t2i = i1 + i3;
     T t3r = r1 - r3, t3i = i1 - i3;
-    // (DIR i) * t3
-    T ur = (DIR < 0) ? t3i : -t3i;
-    T ui = (DIR < 0) ? -t3r : t3r;
+    const T ur = t3i, ui = -t3r;   // -i t3
     r0 = t0r + t2r; i0 = t0i + t2i;
     r2 = t0r - t2r; i2 = t0i - t2i;
     r1 = t1r + ur;  i1 = t1i + ui;
     r3 = t1r - ur;  i3 = t1i - ui;
 }
 
-template <int DIR, typename T>
+template <typename T>
 __device__ __forceinline__ void dft8(T *re, T *im) {
     const T h = T(0.70710678118654752440084436210485);
     T er0 = re[0], ei0 = im[0], er1 = re[2], ei1 = im[2], er2 = re[4], ei2 = im[4], er3 = re[6], ei3 = im[6];
     T or0 = re[1], oi0 = im[1], or1 = re[3], oi1 = im[3], or2 = re[5], oi2 = im[5], or3 = re[7], oi3 = im[7];
-    dft4<DIR>(er0, ei0, er1, ei1, er2, ei2, er3, ei3);
-    dft4<DIR>(or0, oi0, or1, oi1, or2, oi2, or3, oi3);
-    // O_k *= W8^k, W8 = (1 + DIR i)/sqrt(2)
+    dft4(er0, ei0, er1, ei1, er2, ei2, er3, ei3);
+    dft4(or0, oi0, or1, oi1, or2, oi2, or3, oi3);
+    // O_k *= W8^k, W8 = (1 - i)/sqrt(2)
     T wr, wi;
-    wr = (DIR < 0) ? (or1 + oi1) : (or1 - oi1);
-    wi = (DIR < 0) ? (oi1 - or1) : (oi1 + or1);
+    wr = or1 + oi1;
+    wi = oi1 - or1;
     or1 = wr * h; oi1 = wi * h;
-    wr = (DIR < 0) ? oi2 : -oi2;
-    wi = (DIR < 0) ? -or2 : or2;
+    wr = oi2;
+    wi = -or2;
     or2 = wr; oi2 = wi;
-    wr = (DIR < 0) ? (oi3 - or3) : (-or3 - oi3);
-    wi = (DIR < 0) ? (-oi3 - or3) : (or3 - oi3);
+    wr = oi3 - or3;
+    wi = -oi3 - or3;
     or3 = wr * h; oi3 = wi * h;
     re[0] = er0 + or0; im[0] = ei0 + oi0; re[4] = er0 - or0; im[4] = ei0 - oi0;
     re[1] = er1 + or1; im[1] = ei1 + oi1; re[5] = er1 - or1; im[5] = ei1 - oi1;
@@ -108,11 +106,11 @@ __device__ __forceinline__ void dft8(T *re, T *im) {
     re[3] = er3 + or3; im[3] = ei3 + oi3; re[7] = er3 - or3; im[7] = ei3 - oi3;
 }
 
-template <int R, int DIR, typename T>
+template <int R, typename T>
 __device__ __forceinline__ void dft(T *re, T *im) {
-    if constexpr (R == 8) dft8<DIR>(re, im);
-    else if constexpr (R == 4) dft4<DIR>(re[0], im[0], re[1], im[1], re[2], im[2], re[3], im[3]);
-    else if constexpr (R == 2) dft2<DIR>(re, im);
+    if constexpr (R == 8) dft8(re, im);
+    else if constexpr (R == 4) dft4(re[0], im[0], re[1], im[1], re[2], im[2], re[3], im[3]);
+    else if constexpr (R == 2) dft2(re, im);
 }
 
 // ------------------------------------------------------------------ barriers
@@ -166,7 +164,7 @@ __device__ __forceinline__ void job_fj(int i, int &f, int &j) {
 // ------------------------------------------------------------------ the pass
 // INPLACE: the Loader reads shared memory that the stage-0 scatter overwrites,
 // so the scatter waits for every thread's gather.
-template <typename T, int M, int F, int EH, int DIR, int MAPM, int S, class LD, class ST,
+template <typename T, int M, int F, int EH, int MAPM, int S, class LD, class ST,
           class BAR = CtaBarrier, bool INPLACE = false>
 __device__ __forceinline__ void run_stage(T (&re)[2][EH], T (&im)[2][EH],
                                           typename Vec2T<T>::type *sd,
@@ -194,8 +192,8 @@ __device__ __forceinline__ void run_stage(T (&re)[2][EH], T (&im)[2][EH],
         }
 #pragma unroll
         for (int i = 0; i < NJ; ++i) {
-            dft<R, DIR>(&re[0][i * R], &im[0][i * R]);
-            dft<R, DIR>(&re[1][i * R], &im[1][i * R]);
+            dft<R>(&re[0][i * R], &im[0][i * R]);
+            dft<R>(&re[1][i * R], &im[1][i * R]);
         }
     } else {
         const V *tws = tw + tw_offset(M, S);
@@ -217,14 +215,13 @@ __device__ __forceinline__ void run_stage(T (&re)[2][EH], T (&im)[2][EH],
 #pragma unroll
             for (int r = 1; r < R; ++r) {
                 const V w = tk[(r - 1) * NS];
-                const T wr = w.x, wi = (DIR < 0) ? w.y : -w.y;
-                T xr = ra[r] * wr - ia[r] * wi, xi = ra[r] * wi + ia[r] * wr;
+                T xr = ra[r] * w.x - ia[r] * w.y, xi = ra[r] * w.y + ia[r] * w.x;
                 ra[r] = xr; ia[r] = xi;
-                xr = rb[r] * wr - ib[r] * wi; xi = rb[r] * wi + ib[r] * wr;
+                xr = rb[r] * w.x - ib[r] * w.y; xi = rb[r] * w.y + ib[r] * w.x;
                 rb[r] = xr; ib[r] = xi;
             }
-            dft<R, DIR>(ra, ia);
-            dft<R, DIR>(rb, ib);
+            dft<R>(ra, ia);
+            dft<R>(rb, ib);
         }
     }
 
@@ -252,7 +249,7 @@ __device__ __forceinline__ void run_stage(T (&re)[2][EH], T (&im)[2][EH],
             }
         }
         SB::sync();
-        run_stage<T, M, F, EH, DIR, MAPM, S + 1, LD, ST, BAR, INPLACE>(re, im, sd, tw, ld, st);
+        run_stage<T, M, F, EH, MAPM, S + 1, LD, ST, BAR, INPLACE>(re, im, sd, tw, ld, st);
     }
 }
 
@@ -274,15 +271,15 @@ __device__ __forceinline__ void fill_twiddles(typename Vec2T<T>::type *tws, cons
 
 // One tile whose input the Loader reads from shared memory that is then reused
 // in place for the stage exchanges (persistent kernels); twiddle tables filled.
-template <typename T, int M, int F, int EH, int DIR, int MAPM, class BAR, class LD, class ST>
+template <typename T, int M, int F, int EH, int MAPM, class BAR, class LD, class ST>
 __device__ __forceinline__ void run_tile_inplace(LD &ld, ST &st, typename Vec2T<T>::type *buf,
                                                  const typename Vec2T<T>::type *tw) {
     T re[2][EH], im[2][EH];
-    run_stage<T, M, F, EH, DIR, MAPM, 0, LD, ST, BAR, true>(re, im, buf, tw, ld, st);
+    run_stage<T, M, F, EH, MAPM, 0, LD, ST, BAR, true>(re, im, buf, tw, ld, st);
 }
 
 // One pass over a tile.  tw: forward twiddles e^{-2 pi i k/M}, k < M, interleaved.
-template <typename T, int M, int F, int EH, int DIR, int MAPM, class LD, class ST>
+template <typename T, int M, int F, int EH, int MAPM, class LD, class ST>
 __device__ __forceinline__ void run_pass(LD &ld, ST &st, const T *__restrict__ tw) {
     using V = typename Vec2T<T>::type;
     constexpr int THREADS = F * M / EH;
@@ -294,7 +291,7 @@ __device__ __forceinline__ void run_pass(LD &ld, ST &st, const T *__restrict__ t
     // synchronise only among themselves need a CTA barrier here
     if constexpr (MAPM == kMapW && n_stages(M) > 1) __syncthreads();
     T re[2][EH], im[2][EH];
-    run_stage<T, M, F, EH, DIR, MAPM, 0>(re, im, sd, tws, ld, st);
+    run_stage<T, M, F, EH, MAPM, 0>(re, im, sd, tws, ld, st);
 }
 
 }  // namespace eng

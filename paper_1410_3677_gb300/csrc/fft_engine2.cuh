@@ -25,51 +25,29 @@ namespace eng2 {
 
 using eng::Vec2T;
 
-// ------------------------------------------------------------------ constants
-// e^{-2 pi i k/32} from the first-octant values cos(pi m/16), sin(pi m/16).
-__host__ __device__ constexpr double oct_cos(int m) {
-    return m == 0 ? 1.0 : m == 1 ? 0.98078528040323044913 : m == 2 ? 0.92387953251128675613
-         : m == 3 ? 0.83146961230254523708 : m == 4 ? 0.70710678118654752440
-         : m == 5 ? 0.55557023301960222474 : m == 6 ? 0.38268343236508977173
-         : m == 7 ? 0.19509032201612826785 : 0.0;
-}
-__host__ __device__ constexpr double oct_sin(int m) { return oct_cos(8 - m); }
-__host__ __device__ constexpr double w32_re(int k) {
-    return (k / 8) % 4 == 0 ? oct_cos(k % 8) : (k / 8) % 4 == 1 ? -oct_sin(k % 8)
-         : (k / 8) % 4 == 2 ? -oct_cos(k % 8) : oct_sin(k % 8);
-}
-__host__ __device__ constexpr double w32_im(int k) {   // -sin(2 pi k / 32)
-    return (k / 8) % 4 == 0 ? -oct_sin(k % 8) : (k / 8) % 4 == 1 ? -oct_cos(k % 8)
-         : (k / 8) % 4 == 2 ? oct_sin(k % 8) : oct_cos(k % 8);
-}
-
 // ------------------------------------------------------------------ register DFTs
-// x <- x W_32^e (DIR = -1) or x conj(W_32^e), e known at compile time once the
-// callers' loops are unrolled: the quarter turns are swaps and negations, so
-// no multiplication by 0 or 1 is left for the compiler to keep.
-template <int DIR, typename T>
-__device__ __forceinline__ void mul_w32(int e, T &xr, T &xi) {
-    e &= 31;
-    if (e == 0) return;
-    if (e == 16) { xr = -xr; xi = -xi; return; }
-    if (e == 8 || e == 24) {   // W = -i (e = 8) or +i (e = 24); conjugated for DIR > 0
-        const bool minus_i = (e == 8) == (DIR < 0);
+// x <- x W_32^m, 0 <= m < 16, m known at compile time once the callers' loops are unrolled: the
+// quarter turn is a swap and a negation, so no multiplication by 0 or 1 is left for the
+// compiler to keep.
+template <typename T>
+__device__ __forceinline__ void mul_w32(int m, T &xr, T &xi) {
+    if (m == 0) return;
+    if (m == 8) {   // W = -i
         const T r = xr;
-        xr = minus_i ? xi : -xi;
-        xi = minus_i ? -r : r;
+        xr = xi;
+        xi = -r;
         return;
     }
-    const T wr = (T)w32_re(e);
-    const T wi = DIR < 0 ? (T)w32_im(e) : -(T)w32_im(e);
+    const T wr = (T)(m < 8 ? cod::cos16(m) : -cod::cos16(16 - m));
+    const T wi = (T)(m < 8 ? -cod::cos16(8 - m) : -cod::cos16(m - 8));   // -sin(pi m / 16)
     const T r = xr * wr - xi * wi;
     xi = xr * wi + xi * wr;
     xr = r;
 }
 
 // R-point DFT of x[0 .. NZ) on split arrays, the rest zero (fft_codelets.cuh).
-template <int R, int DIR, int NZ = R, typename T>
+template <int R, int NZ = R, typename T>
 __device__ __forceinline__ void dft(T *re, T *im) {
-    static_assert(DIR == -1, "forward transforms");
     cod::SC<T> x[R];
 #pragma unroll
     for (int r = 0; r < NZ; ++r) x[r] = {re[r], im[r]};
@@ -183,7 +161,7 @@ struct NoHook {
 // and the twiddles are read from it through L1 (one 8-byte load per element, a
 // half-warp reading 16 consecutive j); else tw is the table W_M^m, m < M, from
 // which the power-of-two rows are staged in shared memory.
-template <typename T, int M, int SEQ, int EH, int DIR, int MAPM, class LD, class ST, int ZQ = 8,
+template <typename T, int M, int SEQ, int EH, int MAPM, class LD, class ST, int ZQ = 8,
           bool TWFULL = false, class HK = NoHook>
 __device__ __forceinline__ void run_pass(LD &ld, ST &st, const T *__restrict__ tw, const HK &hk = HK{}) {
     using V = typename Vec2T<T>::type;
@@ -225,7 +203,7 @@ __device__ __forceinline__ void run_pass(LD &ld, ST &st, const T *__restrict__ t
     hk.after_loads();
 #pragma unroll
     for (int i = 0; i < NJ0; ++i) {
-        dft<R0, DIR, RL0>(&re[i * R0], &im[i * R0]);
+        dft<R0, RL0>(&re[i * R0], &im[i * R0]);
     }
     if constexpr (R1 == 1) {
 #pragma unroll
@@ -283,14 +261,14 @@ __device__ __forceinline__ void run_pass(LD &ld, ST &st, const T *__restrict__ t
                 for (int r = 1; r < R1; ++r) {
                     const V w = __ldg(row + r * R0);
                     wr[r] = w.x;
-                    wi[r] = DIR < 0 ? w.y : -w.y;
+                    wi[r] = w.y;
                 }
             } else {
 #pragma unroll
                 for (int b = 0; b < LR1; ++b) {
                     const V w = tws[b * R0 + q.j];
                     wr[1 << b] = w.x;
-                    wi[1 << b] = DIR < 0 ? w.y : -w.y;
+                    wi[1 << b] = w.y;
                 }
 #pragma unroll
                 for (int r = 3; r < R1; ++r) {
@@ -308,7 +286,7 @@ __device__ __forceinline__ void run_pass(LD &ld, ST &st, const T *__restrict__ t
                 const T a = xr[r] * wr[r] - xi[r] * wi[r], b = xr[r] * wi[r] + xi[r] * wr[r];
                 xr[r] = a; xi[r] = b;
             }
-            dft<R1, DIR>(xr, xi);
+            dft<R1>(xr, xi);
             // a store that touches no shared memory can take each job as it is done
             if constexpr (StoreEarly<ST>::value) st.template store<R1, R0>(q, xr, xi);
         }

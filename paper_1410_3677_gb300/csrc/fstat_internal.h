@@ -119,7 +119,6 @@ inline RowRange searched_rows(const BandDev &b, int n2, int f) {
 struct Plan {
     fstat_plan_desc desc{};
     std::vector<BandDev> bands;
-    std::vector<fstat_band> host_bands;
     int64_t n_cells = 0, f_evals = 0;
     int device = -1;   // current at creation; every call runs on it
     cudaStream_t stream = nullptr;
@@ -146,7 +145,7 @@ struct Plan {
     int64_t sky_batch = 0;
     void *wbuf[2] = {nullptr, nullptr};   // FP32: float4 [sky_batch][w_stride]; FP64: {y a, y b} double2 pairs
     double *dbuf = nullptr;       // FP64 form: [sky_batch][n_max] per-sample delays
-    double *partials = nullptr;   // [sky_batch][n_blocks_max][3]
+    double *partials = nullptr;   // [sky_batch][blocks of the longest band][3]
     double *S = nullptr;          // [sky_batch][3]
     double *sigma_parts = nullptr;   // [kSigmaParts] of the band being searched
     double *normbuf[2] = {nullptr, nullptr};   // [sky_batch][2]: 1/(sigma^2 S_aa), 1/(sigma^2 S_bb)
@@ -192,7 +191,6 @@ struct Plan {
 
     // twiddles, one set per transform length used
     std::vector<TwiddleSet> tw;
-    void *tw_pool = nullptr;
     const double2 *unit_tab = nullptr;   // FP64 form: e^{-2 pi i m / 2048}
     const float4 *turn_tab = nullptr;    // FP32 form: e^{2 pi i m / 2048} in double-float pairs
 
@@ -230,7 +228,6 @@ struct Plan {
         cudaEvent_t a, b;
     };
     int timing_every = 0;
-    int64_t timing_tick = 0;
     std::vector<KStat> kstats;
     std::vector<Pending> pending;
     std::vector<cudaEvent_t> ev_pool, ev_all;

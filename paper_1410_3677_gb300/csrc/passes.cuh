@@ -160,19 +160,16 @@ struct SearchLoadF64 {
 // twiddles are W^{k1 j} (W^{k1 JPF})^r: two table lookups per job, then complex
 // powers, instead of a scattered lookup per element.  A lookup of W_N^m, m < N,
 // is hi[m >> log N1] lo[m & (N1 - 1)].
-template <typename T, class C, int DIR>
+template <typename T, class C>
 struct ScratchStore {
     using V = typename Vec2<T>::type;
     V *scratch;
     const T *lo, *hi;
-    int64_t n_tr;   // generic: number of transforms (the odd one out has no b); search: 2*pairs
     V *base;
-    bool has_b;
     int k1_0;
     __device__ void init() {
         const int64_t p = blockIdx.y;
         base = scratch + p * 2 * (int64_t)C::N;
-        has_b = 2 * p + 1 < n_tr;
         k1_0 = blockIdx.x * C::F;
     }
     __device__ __forceinline__ V wn(int m) const {
@@ -188,15 +185,12 @@ struct ScratchStore {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int l2 = j + r * JPF;
-            const T wr = w.x, wi = (DIR > 0) ? -w.y : w.y;
             T xr = ra[r], xi = ia[r];
-            cmul_tw(xr, xi, wr, wi);
+            cmul_tw(xr, xi, w.x, w.y);
             base[(int64_t)l2 * C::N1 + k1] = V{xr, xi};
-            if (has_b) {
-                xr = rb[r]; xi = ib[r];
-                cmul_tw(xr, xi, wr, wi);
-                base[C::N + (int64_t)l2 * C::N1 + k1] = V{xr, xi};
-            }
+            xr = rb[r]; xi = ib[r];
+            cmul_tw(xr, xi, w.x, w.y);
+            base[C::N + (int64_t)l2 * C::N1 + k1] = V{xr, xi};
             if (r + 1 < R) w = V{w.x * st.x - w.y * st.y, w.x * st.y + w.y * st.x};
         }
     }
@@ -290,7 +284,7 @@ struct SearchEpi {
 };
 
 // ------------------------------------------------------------------ kernels
-template <typename T, int LOGN, int PASS, int DIR, int MAPM, class LD, class ST, int TS = 256,
+template <typename T, int LOGN, int PASS, int MAPM, class LD, class ST, int TS = 256,
           int EHT = 0>
 __global__ void __launch_bounds__(Cfg<T, LOGN, PASS, TS, EHT>::THREADS,
                                   Cfg<T, LOGN, PASS, TS, EHT>::MIN_BLOCKS)
@@ -298,7 +292,7 @@ k_pass(LD ld, ST st, const T *__restrict__ tw) {
     using C = Cfg<T, LOGN, PASS, TS, EHT>;
     ld.init();
     st.init();
-    eng::run_pass<T, C::M, C::F, C::EH, DIR, MAPM>(ld, st, tw);
+    eng::run_pass<T, C::M, C::F, C::EH, MAPM>(ld, st, tw);
 }
 
 // A kernel's limit of dynamic shared memory is a property of the device: set at every launch

@@ -378,7 +378,7 @@ struct SearchEpi2 {
         float Fv[H];
         bool pr[H];
         bool any = false;
-        // bins < 2^19: 32-bit arithmetic; lo <= bin <= hi as one unsigned compare
+        // bins < 2^20: 32-bit arithmetic; lo <= bin <= hi as one unsigned compare
         const int bin0 = C::N2 * (q.j + q.t * H * JPF) + l2_0 + q.f;
         const int lo = (int)bin_lo;
         const unsigned span = (unsigned)(bin_hi - bin_lo);
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(TS, 768 / TS) k_pass2(LD ld, ST st, const floa
     ld.init(blockIdx.x, blockIdx.y, blockIdx.y);
     st.init(blockIdx.x, blockIdx.y, blockIdx.y);
     if constexpr (eng2::LoaderStaged<LD>::value) ld.stage();
-    eng2::run_pass<float, C::M, C::SEQ, C::EH, -1, MAPM, LD, ST, PASS == 1 ? Z1 : 8, true>(ld, st, tw);
+    eng2::run_pass<float, C::M, C::SEQ, C::EH, MAPM, LD, ST, PASS == 1 ? Z1 : 8, true>(ld, st, tw);
 }
 
 // ------------------------------------------------------------------ interbinning
@@ -567,7 +567,7 @@ k_pass2_ib(LD ld, SearchEpi2<Cfg2<LOGN, 2, TS>, false> ep, const float *__restri
     StoreRowsSmem<C> st;
     // stage-1 twiddles from the shared power-of-two rows: the full table through
     // L1 costs this kernel registers (spills) and time
-    eng2::run_pass<float, C::M, C::SEQ, C::EH, -1, eng2::kMapW, LD, StoreRowsSmem<C>, 8, false>(ld, st, tw);
+    eng2::run_pass<float, C::M, C::SEQ, C::EH, eng2::kMapW, LD, StoreRowsSmem<C>, 8, false>(ld, st, tw);
     __syncthreads();
     const float2 *X = reinterpret_cast<const float2 *>(eng2::dyn_smem());
     constexpr int RL = eng2::row_ld(C::M);
@@ -738,7 +738,7 @@ __device__ __noinline__ void fused_tile1(const SearchLoad2<Cfg2<LOGN, 1>> *pl, c
     ScratchStore2<C1> o = *po;
     l.init(tile, cell, slot);
     o.init(tile, cell, slot);
-    eng2::run_pass<float, C1::M, C1::SEQ, C1::EH, -1, eng2::kMapFJ, SearchLoad2<C1>, ScratchStore2<C1>, Z1, true,
+    eng2::run_pass<float, C1::M, C1::SEQ, C1::EH, eng2::kMapFJ, SearchLoad2<C1>, ScratchStore2<C1>, Z1, true,
                    PublishHook>(l, o, tw, hk);
 }
 
@@ -751,7 +751,7 @@ __device__ __noinline__ void fused_tile2(const ScratchLoad2<Cfg2<LOGN, 2>> *pl,
     SearchEpi2<C2, LOWER> o = *po;
     l.init(tile, cell, slot);
     o.init(tile, cell, slot);
-    eng2::run_pass<float, C2::M, C2::SEQ, C2::EH, -1, eng2::kMapW, ScratchLoad2<C2>, SearchEpi2<C2, LOWER>, 8, true,
+    eng2::run_pass<float, C2::M, C2::SEQ, C2::EH, eng2::kMapW, ScratchLoad2<C2>, SearchEpi2<C2, LOWER>, 8, true,
                    PublishHook>(l, o, tw, hk);
 }
 

@@ -39,7 +39,7 @@ __device__ __forceinline__ PC tw1(const float4 *__restrict__ t, int r, int k) {
 }
 
 // e^{-2 pi i m / 32} on one scalar complex value
-__device__ __forceinline__ void w32_scalar(int m, float &xr, float &xi) { eng2::mul_w32<-1>(m, xr, xi); }
+__device__ __forceinline__ void w32_scalar(int m, float &xr, float &xi) { eng2::mul_w32(m, xr, xi); }
 
 // --------------------------------------------------------------------- pass 1
 // Columns k1 of the demodulated series: SearchLoad2 gives the stage-0 inputs
@@ -132,7 +132,7 @@ k_pass1h(SearchLoad2<Cfg2<LOGN, 1>> ld, ScratchStore2<Cfg2<LOGN, 1>> st, const f
     {
         float re[kR0], im[kR0];
         ld.template load<NZ, 16>(q, re, im);
-        eng2::dft<kR0, -1, NZ>(re, im);
+        eng2::dft<kR0, NZ>(re, im);
         float4 *p4 = reinterpret_cast<float4 *>(sd + s * RL + eng2::pad16(j * kR0));
 #pragma unroll
         for (int k = 0; k < 16; ++k) p4[k] = make_float4(re[2 * k], re[2 * k + 1], im[2 * k], im[2 * k + 1]);
@@ -319,7 +319,7 @@ __device__ __forceinline__ void epilogue(const SearchEpi2<C, LOWER> &ep, int t, 
             Fv[u] = pk::pfma(pa, pk::bc(ep.na), pk::pmul(pb, pk::bc(ep.nb)));
         }
     }
-    const int lo = (int)ep.bin_lo;   // bins < 2^19
+    const int lo = (int)ep.bin_lo;   // bins < 2^20
     const unsigned span = (unsigned)(ep.bin_hi - ep.bin_lo);
     bool pr[2 * H];
     bool any = false;
@@ -362,7 +362,7 @@ k_pass2p(RowsTMA<Cfg2<LOGN, 2, TS>> ld, SearchEpi2<Cfg2<LOGN, 2, TS>, LOWER> ep,
     using C = Cfg2<LOGN, 2, TS>;
     static_assert(C::M == kM && C::F == TS / 32 && C::SEQ == 2 * C::F && C::TPF == 16, "512-point rows, a warp per row");
     static_assert(2 * kR1 * kR1 * 16 == 2 * C::N1 * sizeof(float2), "a warp's exchange fills its staged row");
-    ld.prefetch_ahead();
+    if constexpr (!ROWS) ld.prefetch_ahead();   // it counts the tiles of a launch over all rows
     const int tile = ROWS ? ((int)blockIdx.x + ep.tile0) & (C::TILES - 1) : (int)blockIdx.x;
     ld.init(tile, blockIdx.y, blockIdx.y);
     const int w = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;

@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kTS, 2) k_pass64(LD ld, ST st, const double *_
     if constexpr (PASS == 2) tile = (tile + st.tile0) & (C::TILES - 1);
     ld.init(tile, blockIdx.y);
     st.init(tile, blockIdx.y);
-    eng2::run_pass<double, C::M, C::SEQ, C::EH, -1, eng2::kMapFJ, LD, ST, PASS == 1 ? Z1 : 8, true>(ld, st, tw);
+    eng2::run_pass<double, C::M, C::SEQ, C::EH, eng2::kMapFJ, LD, ST, PASS == 1 ? Z1 : 8, true>(ld, st, tw);
 }
 
 }  // namespace p64

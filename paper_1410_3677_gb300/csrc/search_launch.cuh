@@ -34,13 +34,12 @@ int launch_search_t(const Plan &p, int band_idx, const BandDev &b, int64_t s0, i
     ld1.n_spin = n_spin;
     ld1.c0 = c0;
     ld1.s0 = s0;
-    using ST1 = ScratchStore<T, C1, -1>;
+    using ST1 = ScratchStore<T, C1>;
     ST1 st1{};
     st1.scratch = reinterpret_cast<V *>(cb.scratch);
     st1.lo = tlo;
     st1.hi = thi;
-    st1.n_tr = 2 * nc;
-    auto k1 = k_pass<T, LOGN, 1, -1, eng::kMapFJ, LD1, ST1, TS, EHT>;
+    auto k1 = k_pass<T, LOGN, 1, eng::kMapFJ, LD1, ST1, TS, EHT>;
     set_smem(k1, C1::SMEM);
     k1<<<dim3(C1::TILES, (unsigned)nc), C1::THREADS, C1::SMEM, s>>>(ld1, st1, tin2);
     if (mid) record_timing_event(mid, s);
@@ -61,7 +60,7 @@ int launch_search_t(const Plan &p, int band_idx, const BandDev &b, int64_t s0, i
     st2.out = p.cand;
     st2.count = p.cand_count;
     st2.cap = (unsigned long long)p.cand_capacity;
-    auto k2 = k_pass<T, LOGN, 2, -1, eng::kMapW, LD2, ST2, TS, EHT>;
+    auto k2 = k_pass<T, LOGN, 2, eng::kMapW, LD2, ST2, TS, EHT>;
     set_smem(k2, C2::SMEM);
     k2<<<dim3(C2::TILES, (unsigned)nc), C2::THREADS, C2::SMEM, s>>>(ld2, st2, tin1);
     return 2;

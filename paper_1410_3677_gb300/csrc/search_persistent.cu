@@ -293,15 +293,13 @@ __global__ void __launch_bounds__(kThreads, 3) k_search_persistent(PArgs a) {
                 ld.n = a.n;
                 ld.k1_0 = tic * P::F1;
                 ld.afx = a.chirp[cell - sky * a.n_spin];
-                ScratchStore<float, C, -1> st;
+                ScratchStore<float, C> st;
                 st.scratch = a.scratch;
                 st.lo = a.lo;
                 st.hi = a.hi;
-                st.n_tr = 2;
                 st.base = a.scratch + ((int64_t)(inf.batch % a.S) * a.B + cib) * 2 * P::N;
-                st.has_b = true;
                 st.k1_0 = tic * P::F1;
-                eng::run_tile_inplace<float, P::N2, P::F1, kEH, -1, eng::kMapFJ, eng::NamedBarrier<kNC>>(
+                eng::run_tile_inplace<float, P::N2, P::F1, kEH, eng::kMapFJ, eng::NamedBarrier<kNC>>(
                     ld, st, bp, tw1);
             } else {
                 using C = typename P::C2;
@@ -319,7 +317,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_search_persistent(PArgs a) {
                 st.out = a.out;
                 st.count = a.count;
                 st.cap = a.cap;
-                eng::run_tile_inplace<float, P::N1, P::F2, kEH, -1, eng::kMapJ, eng::NamedBarrier<kNC>>(
+                eng::run_tile_inplace<float, P::N1, P::F2, kEH, eng::kMapJ, eng::NamedBarrier<kNC>>(
                     ld, st, bp, tw2);
             }
         }
