@@ -321,7 +321,7 @@ fstat_status fstat_lattice_grid(const fstat_lattice *lattice, double *alpha, dou
      F_out  device pointer to bin_hi - bin_lo + 1 floats, 4-byte aligned;
      cuda_stream  cudaStream_t or NULL.
    The transforms' intermediate lives in a file-scope device array of
-   2 x 2^18 complex floats (4 MiB) and twiddle tables in another (about 20 KiB);
+   2 x 2^18 complex floats (4 MiB) and twiddle tables in another (about 51 KiB);
    every GPU that loads the library holds them until the process exits.  On its
    first call on a device (and on the first call for each transform length) the
    entry point resolves the arrays' device addresses and fills the twiddle table
